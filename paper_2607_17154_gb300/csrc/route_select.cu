@@ -200,76 +200,9 @@ struct Lookahead {
   int H;                 // horizon; 1 = myopic (Phi = 0)
   size_t stride;         // bytes between consecutive layers' tables
   const float* P;        // [H-1][E][E]
-  int staged;            // lookahead_select_kernel copies layers l+1.. and P to shared memory
   int topk_only;         // H = 1 with many experts: the router writes the targets and weights,
                          // select_lanes_kernel selects
 };
-
-// A plain (generic) load: the look-ahead reads the next layers' tables either
-// from global memory or from the kernel's shared-memory copy of them.
-template <class T>
-__device__ __forceinline__ T ldt(const T* p) {
-  return *p;
-}
-
-// Cost-to-go of Eq. 42 with D future layers, from server m after executing
-// expert kx with accumulated loss qacc: sum over next targets k' (ascending)
-// of P(kx -> k') times the cheapest feasible (m', k'') of the next layer
-// (Eq. 40 from server m; a single target, no distinct-expert rule), each
-// plus its own cost-to-go. Every product and sum is one rounded fp32
-// operation, so the value is reproducible bit for bit.
-template <int D>
-__device__ float lookahead_phi(const uint8_t* __restrict__ tnext, size_t stride,
-                               const float* __restrict__ P, int E, int M, int a, int m, int kx,
-                               float qacc, float qbar) {
-  const float* Q1 = reinterpret_cast<const float*>(tnext + kOffQtab);
-  const float* C1 = reinterpret_cast<const float*>(tnext + off_cq(E));
-  const float* A1 = reinterpret_cast<const float*>(tnext + off_a(E));
-  const uint32_t* pm1 = reinterpret_cast<const uint32_t*>(tnext + kOffPmask);
-  const unsigned long long* sb1 = reinterpret_cast<const unsigned long long*>(tnext + kOffSubst);
-  float acc = 0.0f;
-  for (int kt = 0; kt < E; ++kt) {
-    const float p = ldt(P + (size_t)kx * E + kt);
-    if (p == 0.0f) continue;
-    float best = INFINITY;
-    unsigned long long cand = ldt(sb1 + kt) | (1ull << kt);  // substitutes and the target
-    while (cand) {
-      const int kk = __ffsll(static_cast<long long>(cand)) - 1;
-      cand &= cand - 1;
-      const bool exact = (kk == kt);
-      float cq = 0.0f, q2 = qacc;
-      if (!exact) {
-        const float qk = ldt(Q1 + kt * E + kk);
-        if (!(__fadd_rn(qacc, qk) <= qbar)) continue;
-        q2 = __fadd_rn(qacc, qk);
-        cq = ldt(C1 + kt * E + kk);
-      }
-      uint32_t pm = ldt(pm1 + kk);
-      while (pm) {
-        const int m2 = __ffs(pm) - 1;
-        pm &= pm - 1;
-        float c = __fadd_rn(ldt(A1 + ((size_t)a * M + m) * M + m2), cq);
-        if (D > 1)
-          c = __fadd_rn(c, lookahead_phi<(D > 1 ? D - 1 : 1)>(tnext + stride, stride, P + E * E, E,
-                                                              M, a, m2, kk, q2, qbar));
-        best = fminf(best, c);
-      }
-    }
-    acc = __fadd_rn(acc, __fmul_rn(p, best));
-  }
-  return acc;
-}
-
-__device__ __forceinline__ float lookahead_cost(const Lookahead& la, const uint8_t* tab, int E,
-                                                int M, int a, int m, int kx, float qacc,
-                                                float qbar) {
-  switch (la.H) {
-    case 2: return lookahead_phi<1>(tab + la.stride, la.stride, la.P, E, M, a, m, kx, qacc, qbar);
-    case 3: return lookahead_phi<2>(tab + la.stride, la.stride, la.P, E, M, a, m, kx, qacc, qbar);
-    case 4: return lookahead_phi<3>(tab + la.stride, la.stride, la.P, E, M, a, m, kx, qacc, qbar);
-    default: return 0.0f;
-  }
-}
 
 // A token's logits in shared memory as 16-byte chunks: chunk c holds
 // logits 4c .. 4c + 3 (-inf past E), at p[128 c] (one thread's column of a
@@ -338,8 +271,7 @@ __device__ __forceinline__ bool topk_list(const Src& src, int nc, float (&v)[ORD
 template <class Src>
 __device__ __forceinline__ void select_token(
     int t, const Src& src, int E, int k, int renorm, int M, float qbar,
-    const float* Atab, const uint8_t* __restrict__ tab, const Lookahead& la,
-    const SelSmem& sm, const float* s_Q, const float* s_Cq, int a, int s, float q,
+    const float* Atab, const SelSmem& sm, const float* s_Q, const float* s_Cq, int a, int s, float q,
     uint8_t* __restrict__ loc, float* __restrict__ qhat,
     int32_t* __restrict__ topk_idx, float* __restrict__ topk_w, int32_t* __restrict__ chosen_expert,
     uint8_t* __restrict__ chosen_server, uint8_t* __restrict__ kind_out, int (&kind_count)[4],
@@ -409,19 +341,17 @@ __device__ __forceinline__ void select_token(
     for (int ki = 0; ki <= nsub; ++ki) {
       const int kk = (ki == 0) ? r : sm.sublist[r * 64 + ki - 1];
       const bool sub = (ki != 0);
-      float cq = 0.0f, qn = q;
+      float cq = 0.0f;
       if (sub) {
         if ((taken >> kk) & 1ull) continue;
         if (!(__fadd_rn(q, s_Q[r * E + kk]) <= qbar)) continue;  // Eq. 40 budget
         cq = s_Cq[r * E + kk];
-        qn = __fadd_rn(q, s_Q[r * E + kk]);
       }
       uint32_t pm = sm.pmask[kk];
       while (pm) {
         const int m = __ffs(pm) - 1;
         pm &= pm - 1;
-        float cost = __fadd_rn(Aas[m], cq);
-        if (la.H > 1) cost = __fadd_rn(cost, lookahead_cost(la, tab, E, M, a, m, kk, qn, qbar));
+        const float cost = __fadd_rn(Aas[m], cq);
         const unsigned long long key =
             (static_cast<unsigned long long>(__float_as_uint(cost)) << 32) |
             (static_cast<unsigned long long>(sub ? 1u : 0u) << 31) |
@@ -510,8 +440,8 @@ __global__ void __launch_bounds__(128) select_kernel(
 #pragma unroll
     for (int c = 0; c < EMAX; c += 4)
       s_lg[(c / 4) * 128 + threadIdx.x] = make_float4(lg[c], lg[c + 1], lg[c + 2], lg[c + 3]);
-    select_token(t, ColLogits{s_lg + threadIdx.x}, E, k, renorm, M, qbar, Atab, tab, la, sm, s_Q,
-                 s_Cq, a, sl, q0, loc, qhat, topk_idx, topk_w, chosen_expert, chosen_server,
+    select_token(t, ColLogits{s_lg + threadIdx.x}, E, k, renorm, M, qbar, Atab, sm, s_Q, s_Cq,
+                 a, sl, q0, loc, qhat, topk_idx, topk_w, chosen_expert, chosen_server,
                  kind_out, kind_count, la.H > 1);
   }
   flush_kind_counts(sm, kind_count, counters);
@@ -657,557 +587,711 @@ __global__ void __launch_bounds__(kLaneThreads) select_lanes_kernel(
 }
 
 // ---------------------------------------------------------------------------
-// Alg. 2 with horizon H > 1 (Eq. 43), one block per token, from the targets
-// topk_idx. For each slot the block lists the slot's candidates (expert,
-// server) in shared memory, then every thread takes (candidate, next target
-// k') items: the term P(k -> k') * min(...) of Eq. 42, with the deeper levels
-// of the recursion serial in the thread. Each candidate's terms are then
-// added in ascending k' (skipping P = 0, as the serial definition does), so
-// Phi is the same fp32 value; the argmin key is reduced with atomicMin.
-template <int D>
-__device__ __forceinline__ float phi_term(const uint8_t* __restrict__ tnext, size_t stride,
-                                          const float* __restrict__ P, int E, int M, int a, int m,
-                                          int kx, int kt, float qacc, float qbar) {
-  // the k' = kt term of lookahead_phi<D> (0 when P = 0)
-  const float p = ldt(P + (size_t)kx * E + kt);
-  if (p == 0.0f) return 0.0f;
-  const float* Q1 = reinterpret_cast<const float*>(tnext + kOffQtab);
-  const float* C1 = reinterpret_cast<const float*>(tnext + off_cq(E));
-  const float* A1 = reinterpret_cast<const float*>(tnext + off_a(E));
-  const uint32_t* pm1 = reinterpret_cast<const uint32_t*>(tnext + kOffPmask);
-  const unsigned long long* sb1 = reinterpret_cast<const unsigned long long*>(tnext + kOffSubst);
-  float best = INFINITY;
-  unsigned long long cand = ldt(sb1 + kt) | (1ull << kt);
-  while (cand) {
-    const int kk = __ffsll(static_cast<long long>(cand)) - 1;
-    cand &= cand - 1;
-    const bool exact = (kk == kt);
-    float cq = 0.0f, q2 = qacc;
-    if (!exact) {
-      const float qk = ldt(Q1 + kt * E + kk);
-      if (!(__fadd_rn(qacc, qk) <= qbar)) continue;
-      q2 = __fadd_rn(qacc, qk);
-      cq = ldt(C1 + kt * E + kk);
-    }
-    uint32_t pm = ldt(pm1 + kk);
-    while (pm) {
-      const int m2 = __ffs(pm) - 1;
-      pm &= pm - 1;
-      float c = __fadd_rn(ldt(A1 + ((size_t)a * M + m) * M + m2), cq);
-      if (D > 1)
-        c = __fadd_rn(c, lookahead_phi<(D > 1 ? D - 1 : 1)>(tnext + stride, stride, P + E * E, E,
-                                                            M, a, m2, kk, q2, qbar));
-      best = fminf(best, c);
-    }
-  }
-  return __fmul_rn(p, best);
+// Alg. 2 with horizon H = D + 1 > 1 (Eq. 43) from the targets topk_idx.
+//
+// Phi^(D)(m, kx, q) depends on the token through its home a and its loss q
+// only, and on q only through the budget checks it makes. Level d counts the
+// layers left (d = D: the next layer, d = 1: the last one looked at), and
+//   Phi^(d)(m, kx, q) = sum over k' of P(kx -> k') V^(d)_q(m, k'),
+//   V^(d)_q(m, k')    = min over the feasible (m', k'') of target k' of
+//                       A[a][m][m'] + Cq[k'][k''] + Phi^(d-1)(m', k'', q'),
+// where V does not depend on kx. So a block takes tokens of one home and
+// builds, once, Phi^(d) for the two cases that most losses fall into: every
+// check below passes (Ua) and every check fails (Un, exact experts only).
+//   all pass: q plus the largest loss of each level in turn stays within Qbar;
+//   all fail: at every level q plus its smallest loss exceeds Qbar.
+// Both follow for every check from these because fadd is monotone and losses
+// are not negative, so the table holds the same fp32 value as the recursion,
+// which adds its terms in ascending k' as the tables do. A candidate in
+// neither case is evaluated by its warp, k' over the lanes, with the tables
+// read again one level down. V_q itself is read from rows that hold, for each
+// target and server, the minima over its substitutes in order of loss (the
+// ones that fit are a prefix of that order); a pair in neither case one level
+// down is evaluated by its lane, unless the bounds Ua <= Phi <= Un already
+// show that it cannot be the minimum.
+//
+// One warp per token, blocks of NW warps; the block finds its home and
+// tokens by ranking home[] (every block ranks the same way, so the blocks
+// partition the tokens without scratch memory or a sort kernel).
+//
+// Bound: latency. A block's set-up is a chain of L2 reads and block barriers,
+// a slot's argmin a chain of shared-memory reads, and the slowest token (one
+// whose loss falls between the two cases slot after slot) ends the launch.
+// One block a token, with the tables rebuilt for each and V folded into every
+// term, took 15.7 ms for 2048 tokens of 64 experts, 8 servers, top-6, H = 3,
+// and 14.6 us for 128 tokens of 8 experts, 4 servers, top-2 (ncu); this takes
+// 351 us and 12.4 us.
+constexpr int kLaMaxTok = 512;   // tokens of a block
+constexpr int kLaMaxLoss = 512;  // losses of the last level that the class table takes
+// Up to 16 experts a block has 8 warps and no class table: its set-up (2 us)
+// is longer than the few evaluations it would shorten (14.5 against 12.4 us
+// for 128 tokens of 8 experts). For 64 experts the table took the 2048-token
+// call below from 4620 to 351 us.
+constexpr int kLaNarrow = 16;
+// bytes of a class's row of counts, one a target: an odd number of words, so
+// that lanes reading one word of different rows hit distinct banks
+__host__ __device__ inline int la_class_pitch(int E) { return 4 * (((E + 3) / 4) | 1); }
+__host__ __device__ inline int la_max_loss(int E) {
+  return E <= kLaNarrow ? 0 : E * (E - 1) < kLaMaxLoss ? E * (E - 1) : kLaMaxLoss;
 }
 
-// H = 3: the term of Eq. 42 with the deepest cost-to-go Phi^(1)(m2, k2, q2)
-// read from a per-token table U[m2][k2] whenever no budget check of that level
-// can fail: U was evaluated with q2 = 0, and with Qmax[k2] the largest loss of
-// a substitute that level can consider (targets k' with P(k2 -> k') != 0),
-// fadd(q2, Qmax[k2]) <= Qbar means every check passes for q2 as for 0 (fadd
-// is monotone and q2 >= 0), so the value is the same; otherwise it is
-// evaluated directly.
-__device__ __forceinline__ float phi_term2_memo(const uint8_t* __restrict__ tnext, size_t stride,
-                                                const float* __restrict__ P, int E, int M, int a,
-                                                int m, int kx, int kt, float qacc, float qbar,
-                                                const float* U, const float* qmax1) {
-  const float p = ldt(P + (size_t)kx * E + kt);
-  if (p == 0.0f) return 0.0f;
-  const float* Q1 = reinterpret_cast<const float*>(tnext + kOffQtab);
-  const float* C1 = reinterpret_cast<const float*>(tnext + off_cq(E));
-  const float* A1 = reinterpret_cast<const float*>(tnext + off_a(E));
-  const uint32_t* pm1 = reinterpret_cast<const uint32_t*>(tnext + kOffPmask);
-  const unsigned long long* sb1 = reinterpret_cast<const unsigned long long*>(tnext + kOffSubst);
-  float best = INFINITY;
-  unsigned long long cand = ldt(sb1 + kt) | (1ull << kt);
-  while (cand) {
-    const int kk = __ffsll(static_cast<long long>(cand)) - 1;
-    cand &= cand - 1;
-    const bool exact = (kk == kt);
-    float cq = 0.0f, q2 = qacc;
-    if (!exact) {
-      const float qk = ldt(Q1 + kt * E + kk);
-      if (!(__fadd_rn(qacc, qk) <= qbar)) continue;
-      q2 = __fadd_rn(qacc, qk);
-      cq = ldt(C1 + kt * E + kk);
-    }
-    const bool free = __fadd_rn(q2, qmax1[kk]) <= qbar;
-    uint32_t pm = ldt(pm1 + kk);
-    while (pm) {
-      const int m2 = __ffs(pm) - 1;
-      pm &= pm - 1;
-      const float phi1 = free ? U[m2 * E + kk]
-                              : lookahead_phi<1>(tnext + stride, stride, P + E * E, E, M, a, m2, kk,
-                                                 q2, qbar);
-      const float c = __fadd_rn(__fadd_rn(ldt(A1 + ((size_t)a * M + m) * M + m2), cq), phi1);
-      best = fminf(best, c);
-    }
-  }
-  return __fmul_rn(p, best);
-}
-
-// An order-preserving map of fp32 onto uint32 (the minimum of the keys is the
-// key of the minimum), so that partial minima can be joined with atomicMin.
-__device__ __forceinline__ uint32_t min_key(float x) {
-  const uint32_t b = __float_as_uint(x);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float from_min_key(uint32_t key) {
-  return __uint_as_float((key & 0x80000000u) ? (key & 0x7FFFFFFFu) : ~key);
-}
-
-// Pairs (k'', m2) of phi_term2_memo whose Phi^(1) is not in U, listed for a
-// parallel evaluation: code = item << 16 | m2 << 8 | k'' (item: the
-// (candidate, k') term they belong to), A(a, m, m2) + Cq, and the loss q2.
-constexpr int kLaSlow = 512;         // listed pairs per pass
-constexpr int kLaSlowTerms = 2048;   // their Phi^(1) terms per sub-pass
-constexpr size_t kLaSlowBytes = (size_t)kLaSlow * 12 + (size_t)kLaSlowTerms * 4;
-struct LaSlow {
-  uint32_t* code;
-  float* base;
-  float* q2;
-  float* terms;
+// A level's tables in global memory (layout in ordermoe.h).
+struct LaLevel {
+  const uint32_t* pmask;
+  const unsigned long long* subst;
+  const float* Q;
+  const float* Cq;
+  const float* A;  // home a's [M][M]
 };
 
-// phi_term2_memo split in two: the minimum over the pairs whose Phi^(1) is
-// read from U is returned (as a min_key), and each other pair is appended to
-// the list (or, when the list is full, evaluated here). The caller joins the
-// listed pairs' costs into the minimum and multiplies by P(kx -> kt); the
-// minimum of a set does not depend on the order it is taken in, so the term
-// is the same fp32 value.
-__device__ __forceinline__ uint32_t phi_term2_split(const uint8_t* __restrict__ tnext,
-                                                    size_t stride, const float* __restrict__ P,
-                                                    int E, int M, int a, int m, int kx, int kt,
-                                                    float qacc, float qbar, const float* U,
-                                                    const float* qmax1, int item,
-                                                    const LaSlow& slow, int* ns) {
-  const float* Q1 = reinterpret_cast<const float*>(tnext + kOffQtab);
-  const float* C1 = reinterpret_cast<const float*>(tnext + off_cq(E));
-  const float* A1 = reinterpret_cast<const float*>(tnext + off_a(E));
-  const uint32_t* pm1 = reinterpret_cast<const uint32_t*>(tnext + kOffPmask);
-  const unsigned long long* sb1 = reinterpret_cast<const unsigned long long*>(tnext + kOffSubst);
+__device__ __forceinline__ LaLevel la_level(const uint8_t* tab, int E, int M, int a) {
+  LaLevel v;
+  v.pmask = reinterpret_cast<const uint32_t*>(tab + kOffPmask);
+  v.subst = reinterpret_cast<const unsigned long long*>(tab + kOffSubst);
+  v.Q = reinterpret_cast<const float*>(tab + kOffQtab);
+  v.Cq = reinterpret_cast<const float*>(tab + off_cq(E));
+  v.A = reinterpret_cast<const float*>(tab + off_a(E)) + (size_t)a * M * M;
+  return v;
+}
+
+// Everything the evaluation of Phi reads: dynamic shared memory and the
+// levels' tables. Index d - 1 is level d. A level's rows: for target k' the
+// exact expert, then its n substitutes in order of loss (equal losses by
+// expert), M entries each, at woff[k'].
+template <int D>
+struct LaCtx {
+  int E, M, pitch;      // pitch: of P and sQ rows (odd: lanes down a column hit distinct banks)
+  float qbar;
+  LaLevel lev[D];
+  const float* P[D];    // shared [E][pitch]
+  const float* Ua[D];   // shared [M][E]: Phi^(d), every check passing
+  const float* Un[D];   //                         every check failing
+  float qmax[D], qmin[D];
+  bool has[D];          // the level has substitutes at all
+  bool prune;           // no transition is negative: Phi lies between Ua and Un
+  bool rows;            // the rows below fit in shared memory
+  const float* sQ[D];   // shared [E][pitch]: the losses of each target's substitutes, ascending
+  const float* Wa[D];   // shared rows: minima over the row's entries so far, Phi^(d-1) from Ua
+  const float* Cn[D];   // shared rows (d > 1): each entry alone, Phi^(d-1) from Un
+  const int* woff[D];
+  const int* nsub[D];
+  const uint8_t* ord[D];  // shared [E][64]: the substitutes in that order
+  // level 1's losses of all targets in ascending order, and for every number
+  // of them that fit (the class of a loss q) how many of each target's do
+  bool classes;
+  int n_loss;
+  const float* loss;
+  const uint8_t* fits;  // [n_loss + 1][la_class_pitch(E)]
+};
+
+// every budget check of levels d .. 1 passes for a loss of q
+template <int D>
+__device__ __forceinline__ bool la_all(const LaCtx<D>& c, int d, float q) {
+#pragma unroll
+  for (int i = D - 1; i >= 0; --i)
+    if (i < d && c.has[i]) {
+      q = __fadd_rn(q, c.qmax[i]);
+      if (!(q <= c.qbar)) return false;
+    }
+  return true;
+}
+// every budget check of levels d .. 1 fails for a loss of q
+template <int D>
+__device__ __forceinline__ bool la_none(const LaCtx<D>& c, int d, float q) {
+#pragma unroll
+  for (int i = D - 1; i >= 0; --i)
+    if (i < d && c.has[i] && __fadd_rn(q, c.qmin[i]) <= c.qbar) return false;
+  return true;
+}
+
+template <int D, int d>
+__device__ __forceinline__ float la_phi(const LaCtx<D>& c, int m, int kx, float q);
+
+// V^(d)_q(m, kt). From the rows: the substitutes whose deeper checks all pass
+// are a prefix of the row (and the exact expert with them, its loss being
+// smaller), those that fit at all a longer one. A pair in neither case is
+// evaluated unless its cost cannot be the minimum: Phi^(d-1) lies between Ua
+// and Un, since every operation of the recursion is monotone.
+template <int D, int d>
+__device__ __forceinline__ float la_value(const LaCtx<D>& c, int m, int kt, float q) {
+  const LaLevel& v = c.lev[d - 1];
   float best = INFINITY;
-  unsigned long long cand = ldt(sb1 + kt) | (1ull << kt);
+  if (c.rows) {
+    const float* s = c.sQ[d - 1] + kt * c.pitch;
+    const float* wa = c.Wa[d - 1] + c.woff[d - 1][kt] + m;
+    const int n = c.nsub[d - 1][kt];
+    if constexpr (d == 1) {
+      int lo = 0, hi = n;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__fadd_rn(q, s[mid]) <= c.qbar) lo = mid + 1;
+        else hi = mid;
+      }
+      return wa[lo * c.M];
+    } else {
+      const float* cn = c.Cn[d - 1] + c.woff[d - 1][kt] + m;
+      int na = 0, first = n + 1, last = -1;  // entries of neither case lie in first .. last
+      float bound = INFINITY;                // some entry's cost is at most this
+      for (int i = 0; i <= n; ++i) {
+        const float q2 = i == 0 ? q : __fadd_rn(q, s[i - 1]);
+        if (i > 0 && !(q2 <= c.qbar)) break;
+        if (la_all<D>(c, d - 1, q2)) {
+          na = i + 1;
+          continue;
+        }
+        const float x = cn[i * c.M];
+        if (la_none<D>(c, d - 1, q2)) {
+          best = fminf(best, x);
+        } else {
+          bound = fminf(bound, x);
+          first = min(first, i);
+          last = i;
+        }
+      }
+      if (na > 0) best = fminf(best, wa[(na - 1) * c.M]);
+      for (int i = first; i <= last; ++i) {
+        const float q2 = i == 0 ? q : __fadd_rn(q, s[i - 1]);
+        const int kk = i == 0 ? kt : c.ord[d - 1][kt * 64 + i - 1];
+        const float cq = i == 0 ? 0.0f : v.Cq[kt * c.E + kk];
+        for (uint32_t pm = v.pmask[kk]; pm; pm &= pm - 1) {
+          const int m2 = __ffs(pm) - 1;
+          const float base = __fadd_rn(v.A[m * c.M + m2], cq);
+          const float least = __fadd_rn(base, c.Ua[d - 2][m2 * c.E + kk]);
+          if (c.prune && (least >= best || least > bound)) continue;
+          best = fminf(best, __fadd_rn(base, la_phi<D, d - 1>(c, m2, kk, q2)));
+        }
+      }
+      return best;
+    }
+  }
+  unsigned long long cand = v.subst[kt] | (1ull << kt);
   while (cand) {
     const int kk = __ffsll(static_cast<long long>(cand)) - 1;
     cand &= cand - 1;
-    const bool exact = (kk == kt);
-    float cq = 0.0f, q2 = qacc;
-    if (!exact) {
-      const float qk = ldt(Q1 + kt * E + kk);
-      if (!(__fadd_rn(qacc, qk) <= qbar)) continue;
-      q2 = __fadd_rn(qacc, qk);
-      cq = ldt(C1 + kt * E + kk);
+    float cq = 0.0f, q2 = q;
+    if (kk != kt) {
+      q2 = __fadd_rn(q, v.Q[kt * c.E + kk]);
+      if (!(q2 <= c.qbar)) continue;
+      cq = v.Cq[kt * c.E + kk];
     }
-    const bool free = __fadd_rn(q2, qmax1[kk]) <= qbar;
-    uint32_t pm = ldt(pm1 + kk);
-    while (pm) {
+    for (uint32_t pm = v.pmask[kk]; pm; pm &= pm - 1) {
       const int m2 = __ffs(pm) - 1;
-      pm &= pm - 1;
-      const float base = __fadd_rn(ldt(A1 + ((size_t)a * M + m) * M + m2), cq);
-      if (free) {
-        best = fminf(best, __fadd_rn(base, U[m2 * E + kk]));
-        continue;
-      }
-      const int e = atomicAdd(ns, 1);
-      if (e < kLaSlow) {
-        slow.code[e] = (static_cast<uint32_t>(item) << 16) | (static_cast<uint32_t>(m2) << 8) |
-                       static_cast<uint32_t>(kk);
-        slow.base[e] = base;
-        slow.q2[e] = q2;
-      } else {
-        best = fminf(best, __fadd_rn(base, lookahead_phi<1>(tnext + stride, stride, P + E * E, E,
-                                                            M, a, m2, kk, q2, qbar)));
-      }
+      float cost = __fadd_rn(v.A[m * c.M + m2], cq);
+      if constexpr (d > 1) cost = __fadd_rn(cost, la_phi<D, d - 1>(c, m2, kk, q2));
+      best = fminf(best, cost);
     }
   }
-  return min_key(best);
+  return best;
 }
 
-// lookahead_phi<2> with its deepest level read from U / qmax1 as in
-// phi_term2_memo (the same fp32 operations in the same order).
-__device__ float lookahead_phi2_memo(const uint8_t* __restrict__ tnext, size_t stride,
-                                     const float* __restrict__ P, int E, int M, int a, int m,
-                                     int kx, float qacc, float qbar, const float* U,
-                                     const float* qmax1) {
+// Phi^(d)(m, kx, q) by one thread
+template <int D, int d>
+__device__ __forceinline__ float la_phi(const LaCtx<D>& c, int m, int kx, float q) {
+  if (la_all<D>(c, d, q)) return c.Ua[d - 1][m * c.E + kx];
+  if (la_none<D>(c, d, q)) return c.Un[d - 1][m * c.E + kx];
+  const float* Pr = c.P[d - 1] + kx * c.pitch;
   float acc = 0.0f;
-  for (int kt = 0; kt < E; ++kt) {
-    if (ldt(P + (size_t)kx * E + kt) == 0.0f) continue;
-    acc = __fadd_rn(acc, phi_term2_memo(tnext, stride, P, E, M, a, m, kx, kt, qacc, qbar, U, qmax1));
+  if (d == 1 && c.rows && c.classes) {
+    int lo = 0, hi = c.n_loss;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (__fadd_rn(q, c.loss[mid]) <= c.qbar) lo = mid + 1;
+      else hi = mid;
+    }
+    const uint8_t* fits = c.fits + lo * la_class_pitch(c.E);
+    const float* wa = c.Wa[0] + m;
+    for (int k4 = 0; k4 < c.E; k4 += 4) {
+      const uint32_t n4 = *reinterpret_cast<const uint32_t*>(fits + k4);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (k4 + u >= c.E) break;
+        const float p = Pr[k4 + u];
+        const float x = wa[c.woff[0][k4 + u] + static_cast<int>((n4 >> (8 * u)) & 0xFFu) * c.M];
+        if (p != 0.0f) acc = __fadd_rn(acc, __fmul_rn(p, x));
+      }
+    }
+    return acc;
+  }
+  for (int kt = 0; kt < c.E; ++kt) {
+    const float p = Pr[kt];
+    if (p != 0.0f) acc = __fadd_rn(acc, __fmul_rn(p, la_value<D, d>(c, m, kt, q)));
   }
   return acc;
 }
 
-// H = 4: the term of Eq. 42 with Phi^(2)(m2, k2, q2) read from a per-token
-// table U2[m2][k2] (evaluated with q2 = 0) whenever no budget check inside it
-// can fail: every loss it adds at its own level is at most qmax2[k2] and every
-// loss one level deeper at most qmaxL1 (losses are not negative; -inf: none),
-// so fadd(q2, qmax2[k2]) <= Qbar and fadd(that, qmaxL1) <= Qbar mean every
-// check passes for q2 as for 0 (fadd is monotone) and the value is the same.
-// Otherwise Phi^(2) is evaluated, its deepest level again from U1 when free.
-__device__ __forceinline__ float phi_term3_memo(const uint8_t* __restrict__ tnext, size_t stride,
-                                                const float* __restrict__ P, int E, int M, int a,
-                                                int m, int kx, int kt, float qacc, float qbar,
-                                                const float* U2, const float* qmax2, float qmaxL1,
-                                                const float* U1, const float* qmax1) {
-  const float p = ldt(P + (size_t)kx * E + kt);
-  if (p == 0.0f) return 0.0f;
-  const float* Q1 = reinterpret_cast<const float*>(tnext + kOffQtab);
-  const float* C1 = reinterpret_cast<const float*>(tnext + off_cq(E));
-  const float* A1 = reinterpret_cast<const float*>(tnext + off_a(E));
-  const uint32_t* pm1 = reinterpret_cast<const uint32_t*>(tnext + kOffPmask);
-  const unsigned long long* sb1 = reinterpret_cast<const unsigned long long*>(tnext + kOffSubst);
-  float best = INFINITY;
-  unsigned long long cand = ldt(sb1 + kt) | (1ull << kt);
-  while (cand) {
-    const int kk = __ffsll(static_cast<long long>(cand)) - 1;
-    cand &= cand - 1;
-    const bool exact = (kk == kt);
-    float cq = 0.0f, q2 = qacc;
-    if (!exact) {
-      const float qk = ldt(Q1 + kt * E + kk);
-      if (!(__fadd_rn(qacc, qk) <= qbar)) continue;
-      q2 = __fadd_rn(qacc, qk);
-      cq = ldt(C1 + kt * E + kk);
-    }
-    const float qa = __fadd_rn(q2, qmax2[kk]);
-    const float q3max = (qmax2[kk] == -INFINITY) ? q2 : qa;  // largest loss entering level 1
-    const bool free = qa <= qbar && __fadd_rn(q3max, qmaxL1) <= qbar;
-    uint32_t pm = ldt(pm1 + kk);
-    while (pm) {
-      const int m2 = __ffs(pm) - 1;
-      pm &= pm - 1;
-      const float phi2 = free ? U2[m2 * E + kk]
-                              : lookahead_phi2_memo(tnext + stride, stride, P + E * E, E, M, a, m2,
-                                                    kk, q2, qbar, U1, qmax1);
-      const float c = __fadd_rn(__fadd_rn(ldt(A1 + ((size_t)a * M + m) * M + m2), cq), phi2);
-      best = fminf(best, c);
-    }
+// Phi^(D)(m, kx, q) by the whole warp, k' over the lanes; the same value in
+// every lane. The terms are added in ascending k' (a term with P = 0 adds an
+// exact 0, which leaves the sum as it is). term: 64 floats of the warp's own.
+template <int D>
+__device__ __forceinline__ float la_phi_warp(const LaCtx<D>& c, float* term, int lane, int m, int kx,
+                                             float q) {
+  const float* Prow = c.P[D - 1] + kx * c.pitch;
+#pragma unroll 1
+  for (int kt = lane; kt < 64; kt += 32) {
+    const float p = kt < c.E ? Prow[kt] : 0.0f;
+    term[kt] = p != 0.0f ? __fmul_rn(p, la_value<D, D>(c, m, kt, q)) : 0.0f;
   }
-  return __fmul_rn(p, best);
-}
-
-// tn: the tables of layer l + 1 (the deeper layers follow, stride bytes
-// apart), Pn: the transitions l -> l + 1 (the deeper ones follow).
-__device__ __forceinline__ float phi_term_h(int H, const uint8_t* tn, size_t stride,
-                                            const float* Pn, int E, int M, int a, int m, int kx,
-                                            int kt, float qacc, float qbar) {
-  switch (H) {
-    case 2: return phi_term<1>(tn, stride, Pn, E, M, a, m, kx, kt, qacc, qbar);
-    case 3: return phi_term<2>(tn, stride, Pn, E, M, a, m, kx, kt, qacc, qbar);
-    case 4: return phi_term<3>(tn, stride, Pn, E, M, a, m, kx, kt, qacc, qbar);
-    default: return 0.0f;
+  __syncwarp();
+  float acc = 0.0f;
+  const float4* t4 = reinterpret_cast<const float4*>(term);
+#pragma unroll 4
+  for (int i = 0; i < (c.E + 3) / 4; ++i) {
+    const float4 x = t4[i];
+    acc = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(acc, x.x), x.y), x.z), x.w);
   }
+  __syncwarp();  // the terms are rewritten by the next evaluation
+  return acc;
 }
 
-// Shared-memory copy of the next layers' tables and transitions for the
-// look-ahead (bytes after the E x E tables and the H = 4 extras).
-__host__ __device__ inline size_t la_stage_offset(int E, int H) {
-  const size_t f = 2 * (size_t)E * E + (H == 4 ? 33 * (size_t)E : 0);
-  return (f * sizeof(float) + 15) & ~size_t(15);
+// Dynamic shared memory for servers up to Mcap, NW warps, level rows of wcap
+// floats (Wa of every level, Cn of all but the last).
+__host__ __device__ inline size_t la_smem_fixed(int E, int D, int Mcap, int NW) {
+  return sizeof(float) * ((size_t)64 * NW + 2 * D * E * (E | 1) + (size_t)(2 * D + 2) * Mcap * E +
+                          la_max_loss(E)) +
+         (size_t)(la_max_loss(E) + 1) * la_class_pitch(E);
 }
-__host__ __device__ inline size_t la_stage_bytes(int E, int H, size_t stride) {
-  return (size_t)(H - 1) * stride + (size_t)(H - 1) * E * E * sizeof(float);
-}
-// H = 3: the pairs listed by phi_term2_split follow the tables (and their
-// shared-memory copy, when there is one); kLaSlowBytes long.
-__host__ __device__ inline size_t la_slow_offset(int E, int H, size_t stride, int staged) {
-  const size_t end = staged ? la_stage_offset(E, H) + la_stage_bytes(E, H, stride)
-                            : 2 * (size_t)E * E * sizeof(float);
-  return (end + 15) & ~size_t(15);
+__host__ __device__ inline size_t la_smem_bytes(int E, int D, int Mcap, int NW, int wcap) {
+  return la_smem_fixed(E, D, Mcap, NW) + sizeof(float) * (size_t)(2 * D - 1) * wcap;
 }
 
-constexpr int kLaThreads = 128;
-constexpr int kLaMaxCand = 65 * 32;  // (target + 64 substitutes) x 32 servers
-constexpr int kLaTerms = 2048;       // (candidate, k') terms per pass
-
-struct LaSmem {
-  uint32_t code[kLaMaxCand];  // expert | server << 8 | substitute << 16
-  float cost0[kLaMaxCand];    // A(a, s, m) + Cq: Eq. 43 without Phi
-  float qn[kLaMaxCand];       // accumulated loss after this candidate (Eq. 44)
-  float terms[kLaTerms];
-  float U[32 * 64];           // H = 3, 4: Phi^(1)(m2, k2) with every budget check passing
-  float qmax1[64];            // H = 3, 4: largest substitute loss Phi^(1)(., k2) can consider
-  unsigned long long best;
-  int n;
-  int ns;                     // H = 3: pairs listed by phi_term2_split
-};
-
-__global__ void __launch_bounds__(kLaThreads) lookahead_select_kernel(
+template <int D, int NW>
+__global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
     const int32_t* __restrict__ topk_idx, int T, int E, int k, const uint8_t* __restrict__ tab,
-    Lookahead la, const uint8_t* __restrict__ home, uint8_t* __restrict__ loc,
-    float* __restrict__ qhat, int32_t* __restrict__ chosen_expert,
+    Lookahead la, int Mcap, int wcap, int tpb, const uint8_t* __restrict__ home,
+    uint8_t* __restrict__ loc, float* __restrict__ qhat, int32_t* __restrict__ chosen_expert,
     uint8_t* __restrict__ chosen_server, uint8_t* __restrict__ kind_out,
     int32_t* __restrict__ counters) {
+  constexpr int kThreads = 32 * NW;
   pdl_trigger();  // launched with launch_pdl: no global access before pdl_wait
   pdl_wait();
-  __shared__ SelSmem sm;
-  __shared__ LaSmem cs;
-  extern __shared__ __align__(16) float s_dyn[];
-  float* s_Q = s_dyn;
-  float* s_Cq = s_dyn + E * E;
-  const int t = blockIdx.x;
-  if (t >= T) return;
-  if (!load_tables(tab, E, sm, s_Q, s_Cq)) return;
-  // the next H - 1 layers' tables and transitions: read in place, or from a
-  // shared-memory copy (every Phi term reads them along serial chains)
-  const uint8_t* tn = tab + la.stride;
-  const float* Pn = la.P;
-  if (la.staged && la.H > 1) {
-    uint8_t* st_tab = reinterpret_cast<uint8_t*>(s_dyn) + la_stage_offset(E, la.H);
-    float* st_P = reinterpret_cast<float*>(st_tab + (size_t)(la.H - 1) * la.stride);
-    const size_t tb = (size_t)(la.H - 1) * la.stride;  // a multiple of 16
-    const size_t pn = (size_t)(la.H - 1) * E * E;
-    if (((reinterpret_cast<uintptr_t>(tn) | reinterpret_cast<uintptr_t>(la.P)) & 15u) == 0) {
-      const uint4* src = reinterpret_cast<const uint4*>(tn);
-#pragma unroll 4
-      for (size_t i = threadIdx.x; i < tb / 16; i += blockDim.x)
-        reinterpret_cast<uint4*>(st_tab)[i] = __ldg(src + i);
-    } else {
-      const uint32_t* src = reinterpret_cast<const uint32_t*>(tn);
-      for (size_t i = threadIdx.x; i < tb / 4; i += blockDim.x)
-        reinterpret_cast<uint32_t*>(st_tab)[i] = src[i];
-    }
-    for (size_t i = threadIdx.x; i < pn; i += blockDim.x) st_P[i] = la.P[i];
-    tn = st_tab;
-    Pn = st_P;
-  }
-  __syncthreads();
-  const int M = reinterpret_cast<const int32_t*>(tab)[2];
+  extern __shared__ __align__(16) unsigned char s_raw[];
+  __shared__ uint8_t s_ord[D][64 * 64];
+  __shared__ uint16_t s_rank[64 * 64];
+  __shared__ int s_cnt[32], s_nsub[D][64], s_woff[D][65], s_tok[kLaMaxTok];
+  __shared__ int s_part[NW], s_kind[4];
+  __shared__ int s_home, s_chunk, s_qmax[D], s_qmin[D];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int32_t* hdr = reinterpret_cast<const int32_t*>(tab);
+  const int M = hdr[2];
   const float qbar = reinterpret_cast<const float*>(tab)[5];
-  const float* gA = reinterpret_cast<const float*>(tab + off_a(E));
-  const int tid = threadIdx.x;
-  const int a = home[t];
-  const int s = (loc != nullptr) ? loc[t] : a;
-  if (a >= M || s >= M) {
-    if (tid == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, t);
+  if (hdr[1] != E || M <= 0 || M > Mcap) {
+    if (blockIdx.x == 0 && tid == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, -1);
     return;
   }
-  unsigned long long taken = 0;
-  for (int j = 0; j < k; ++j) {
-    const int r = topk_idx[(size_t)t * k + j];
-    if (r < 0 || r >= E) return;  // -1: a token whose logits held a NaN (reported)
-    taken |= 1ull << r;
+  // ---- this block's home and tokens: home a has ceil(count / tpb) blocks
+  if (tid < 32) s_cnt[tid] = 0;
+  if (tid < 4) s_kind[tid] = 0;
+  if (tid < D) {
+    s_qmax[tid] = -1;  // no substitute (losses are not negative: their bits order like values)
+    s_qmin[tid] = 0x7FFFFFFF;
   }
-  const float* Aas = gA + ((size_t)a * M + s) * M;
-  const int cpp = kLaTerms / E;  // candidates per pass
-  float q = (qhat != nullptr) ? qhat[t] : 0.0f;
-  const bool memo = (la.H == 3) && !(q < 0.0f);  // accumulated losses are never negative
-  const bool memo4 = (la.H == 4) && !(q < 0.0f);
-  float* U2 = s_dyn + 2 * E * E;  // H = 4: Phi^(2)(m2, k2) with every check passing, [32][E]
-  float* qmax2 = U2 + 32 * E;     // H = 4: largest loss Phi^(2)(., k2) adds at its level
-  float qmaxL1 = -INFINITY;       // H = 4: largest such loss one level deeper
-  LaSlow slow{};                  // H = 3: the listed pairs
-  if (memo) {
-    uint8_t* sp = reinterpret_cast<uint8_t*>(s_dyn) + la_slow_offset(E, 3, la.stride, la.staged);
-    slow.code = reinterpret_cast<uint32_t*>(sp);
-    slow.base = reinterpret_cast<float*>(sp + (size_t)kLaSlow * 4);
-    slow.q2 = slow.base + kLaSlow;
-    slow.terms = slow.q2 + kLaSlow;
+  // the layers' losses of this warp's rows, loaded ahead of their use
+  LaCtx<D> c;
+  c.E = E;
+  c.M = M;
+  c.pitch = E | 1;
+  c.qbar = qbar;
+  float* sp = reinterpret_cast<float*>(s_raw);
+  float* s_term = sp + 64 * warp;
+  sp += 64 * NW;
+  float *U[2 * D], *Wa[D], *Cn[D];
+  bool bad_p = false;
+  float* sQ[D];
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    // level i + 1: layer l + D - i, entered from the layer before it by P_{l + D - i - 1}
+    const float* g = la.P + (size_t)(D - 1 - i) * E * E;
+    for (int x = tid; x < E * E; x += kThreads) {
+      sp[x + (x / E) * (c.pitch - E)] = g[x];
+      bad_p |= !(g[x] >= 0.0f);
+    }
+    c.P[i] = sp;
+    sp += E * c.pitch;
+    c.sQ[i] = sQ[i] = sp;
+    sp += E * c.pitch;
   }
-  // the largest substitute loss lookahead_phi<1> on tables tl and transitions Pl
-  // can add for expert kx (targets with P(kx -> k') != 0; -inf: none)
-  auto qmax_of = [&](const uint8_t* tl, const float* Pl, int kx) {
-    const float* Ql = reinterpret_cast<const float*>(tl + kOffQtab);
-    const unsigned long long* sbl = reinterpret_cast<const unsigned long long*>(tl + kOffSubst);
-    float mx = -INFINITY;
-    for (int kt = 0; kt < E; ++kt) {
-      if (ldt(Pl + (size_t)kx * E + kt) == 0.0f) continue;
-      unsigned long long sb = ldt(sbl + kt);
-      while (sb) {
-        const int k3 = __ffsll(static_cast<long long>(sb)) - 1;
-        sb &= sb - 1;
-        mx = fmaxf(mx, ldt(Ql + kt * E + k3));
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    c.Ua[i] = U[2 * i] = sp;
+    c.Un[i] = U[2 * i + 1] = sp + Mcap * E;
+    sp += 2 * Mcap * E;
+  }
+  float* Va = sp;
+  float* Vn = Va + Mcap * E;
+  sp = Vn + Mcap * E;
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    c.Wa[i] = Wa[i] = sp;
+    sp += wcap;
+    c.Cn[i] = Cn[i] = nullptr;
+    if (i > 0) {
+      c.Cn[i] = Cn[i] = sp;
+      sp += wcap;
+    }
+    c.woff[i] = s_woff[i];
+    c.nsub[i] = s_nsub[i];
+    c.ord[i] = s_ord[i];
+  }
+  float* s_loss = sp;
+  uint8_t* s_fits = reinterpret_cast<uint8_t*>(sp + la_max_loss(E));
+  c.loss = s_loss;
+  c.fits = s_fits;
+  __syncthreads();
+  // thread i looks at tokens i, i + kThreads, ..., kScan of them loaded at a time
+  constexpr int kScan = 8;
+  auto scan_homes = [&](auto&& take) {
+    for (int b = 0; b < T; b += kScan * kThreads) {
+      int h[kScan];
+#pragma unroll
+      for (int u = 0; u < kScan; ++u) {
+        const int t = b + u * kThreads + tid;
+        h[u] = t < T ? home[t] : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < kScan; ++u) {
+        if (b + u * kThreads >= T) break;  // the same for the block
+        take(b + u * kThreads + tid, h[u]);
       }
     }
-    return mx;
   };
-  if (memo || memo4) {
-    // the deepest level's tables (layer l + H - 1) and transitions into it
-    const int dl = la.H - 1;
-    const uint8_t* td = tn + (dl - 1) * la.stride;
-    const float* Pd = Pn + (size_t)(dl - 1) * E * E;
-    for (int k2 = tid; k2 < E; k2 += blockDim.x) cs.qmax1[k2] = qmax_of(td, Pd, k2);
-    // U[m2][k2] = lookahead_phi<1>(m2, k2, q = 0): the E terms of every entry
-    // (one per next target k') in parallel, then each entry's terms added in
-    // ascending k', skipping P = 0, as lookahead_phi<1> adds them (the same
-    // fp32 value; one thread per entry walked all its terms before)
-    const int per = kLaTerms / E;  // entries per pass
-    for (int base = 0; base < M * E; base += per) {
-      const int ne = min(per, M * E - base);
-      for (int i = tid; i < ne * E; i += blockDim.x) {
-        const int c = base + i / E, kt = i - (i / E) * E;
-        const int m2 = c / E, k2 = c - (c / E) * E;
-        cs.terms[i] = phi_term<1>(td, la.stride, Pd, E, M, a, m2, k2, kt, 0.0f, qbar);
-      }
-      __syncthreads();
-      for (int cl = tid; cl < ne; cl += blockDim.x) {
-        const int c = base + cl, k2 = c - (c / E) * E;
-        float phi = 0.0f;
-        for (int kt = 0; kt < E; ++kt)
-          if (ldt(Pd + (size_t)k2 * E + kt) != 0.0f) phi = __fadd_rn(phi, cs.terms[cl * E + kt]);
-        cs.U[c] = phi;
-      }
-      __syncthreads();
+  scan_homes([&](int t, int a) {
+    const unsigned peers = __match_any_sync(0xffffffffu, a);
+    if (a >= 0 && a < M && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[a], __popc(peers));
+    if (a >= M && blockIdx.x == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, t);
+  });
+  __syncthreads();
+  if (warp == 0) {
+    const int nb = lane < M ? (s_cnt[lane] + tpb - 1) / tpb : 0;
+    int incl = nb;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    const int b = static_cast<int>(blockIdx.x);
+    const unsigned here = __ballot_sync(0xffffffffu, b >= incl - nb && b < incl);
+    if (here == 0) {
+      if (lane == 0) s_home = -1;
+    } else if (lane == __ffs(here) - 1) {
+      s_home = lane;
+      s_chunk = b - (incl - nb);
     }
   }
-  if (memo4) {
-    // one level up (layer l + 2): Phi^(2) at q = 0, through the U table above
-    const uint8_t* t2 = tn + la.stride;
-    const float* P2 = Pn + (size_t)E * E;
-    for (int k2 = tid; k2 < E; k2 += blockDim.x) qmax2[k2] = qmax_of(t2, P2, k2);
-    for (int i = tid; i < M * E; i += blockDim.x) {
-      const int m2 = i / E, k2 = i - (i / E) * E;
-      U2[i] = lookahead_phi2_memo(t2, la.stride, P2, E, M, a, m2, k2, 0.0f, qbar, cs.U, cs.qmax1);
-    }
-    for (int k3 = 0; k3 < E; ++k3) qmaxL1 = fmaxf(qmaxL1, cs.qmax1[k3]);
-    __syncthreads();
+  __syncthreads();
+  const int a = s_home;
+  if (a < 0) return;  // more blocks than the homes need
+  const int lo = s_chunk * tpb;
+  const int ntok = min(tpb, s_cnt[a] - lo);
+  int mine = 0;
+  scan_homes([&](int, int h) { mine += h == a ? 1 : 0; });
+  int incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int u = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += u;
   }
-  int first_server = s;
-  for (int j = 0; j < k; ++j) {
-    const int r = topk_idx[(size_t)t * k + j];
-    if (tid == 0) {
-      cs.n = 0;
-      cs.best = ~0ull;
-    }
-    __syncthreads();
-    // candidates: thread i takes the target (i = 0) or substitute i - 1
-    const int nsub = sm.nsub[r];
-    for (int ki = tid; ki <= nsub; ki += blockDim.x) {
-      const int kk = (ki == 0) ? r : sm.sublist[r * 64 + ki - 1];
-      const bool sub = (ki != 0);
-      float cq = 0.0f, qn = q;
-      bool ok = true;
-      if (sub) {
-        ok = !((taken >> kk) & 1ull) && (__fadd_rn(q, s_Q[r * E + kk]) <= qbar);
-        if (ok) {
-          cq = s_Cq[r * E + kk];
-          qn = __fadd_rn(q, s_Q[r * E + kk]);
-        }
+  if (lane == 31) s_part[warp] = incl;
+
+  // ---- the tables of home a. A warp a row: the losses in order, their extremes
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    c.lev[i] = la_level(tab + (size_t)(D - i) * la.stride, E, M, a);
+    for (int kt = warp; kt < E; kt += NW) {
+      const unsigned long long sb = c.lev[i].subst[kt];
+      if (lane == 0) s_nsub[i][kt] = __popcll(sb);
+      if (sb == 0ull) continue;
+      const int q0 = (sb >> lane) & 1ull ? __float_as_int(c.lev[i].Q[kt * E + lane]) : -1;
+      const int q1 = (sb >> (lane + 32)) & 1ull ? __float_as_int(c.lev[i].Q[kt * E + lane + 32]) : -1;
+      const int mx = __reduce_max_sync(0xffffffffu, max(q0, q1));
+      const unsigned mn = __reduce_min_sync(0xffffffffu, min(static_cast<unsigned>(q0), static_cast<unsigned>(q1)));
+      if (lane == 0) {
+        atomicMax(&s_qmax[i], mx);
+        atomicMin(&s_qmin[i], static_cast<int>(mn));
       }
-      uint32_t pm = ok ? sm.pmask[kk] : 0u;
-      int slot = atomicAdd(&cs.n, __popc(pm));
-      while (pm) {
-        const int m = __ffs(pm) - 1;
-        pm &= pm - 1;
-        cs.code[slot] = static_cast<uint32_t>(kk) | (static_cast<uint32_t>(m) << 8) |
-                        (sub ? (1u << 16) : 0u);
-        cs.cost0[slot] = __fadd_rn(ldt(Aas + m), cq);
-        cs.qn[slot] = qn;
-        ++slot;
+      int r0 = 0, r1 = 0;
+      for (unsigned long long b = sb; b; b &= b - 1) {
+        const int e = __ffsll(static_cast<long long>(b)) - 1;
+        const int o = __shfl_sync(0xffffffffu, e < 32 ? q0 : q1, e & 31);
+        r0 += (o < q0 || (o == q0 && e < lane)) ? 1 : 0;
+        r1 += (o < q1 || (o == q1 && e < lane + 32)) ? 1 : 0;
+      }
+      if (q0 >= 0) {
+        sQ[i][kt * c.pitch + r0] = __int_as_float(q0);
+        s_ord[i][kt * 64 + r0] = static_cast<uint8_t>(lane);
+      }
+      if (q1 >= 0) {
+        sQ[i][kt * c.pitch + r1] = __int_as_float(q1);
+        s_ord[i][kt * 64 + r1] = static_cast<uint8_t>(lane + 32);
       }
     }
-    __syncthreads();
-    const int n = cs.n;
-    for (int base = 0; base < n; base += cpp) {
-      const int nc = min(cpp, n - base);
-      if (memo) {
-        // H = 3: each (candidate, k') item takes its pairs whose Phi^(1) is in
-        // U and lists the others; the listed pairs' Phi^(1) is then evaluated
-        // with its E terms in parallel and added in ascending k'' as
-        // lookahead_phi<1> adds them, and each pair's cost joins its item's
-        // minimum (a token near its budget has many such pairs, which one
-        // thread used to walk one after another)
-        if (tid == 0) cs.ns = 0;
-        __syncthreads();
-        uint32_t* key = reinterpret_cast<uint32_t*>(cs.terms);
-        for (int i = tid; i < nc * E; i += blockDim.x) {
-          const int c = base + i / E, kt = i - (i / E) * E;
-          const uint32_t code = cs.code[c];
-          const int cm = static_cast<int>((code >> 8) & 0xFFu), ck = static_cast<int>(code & 0xFFu);
-          if (ldt(Pn + (size_t)ck * E + kt) != 0.0f)
-            key[i] = phi_term2_split(tn, la.stride, Pn, E, M, a, cm, ck, kt, cs.qn[c], qbar, cs.U,
-                                     cs.qmax1, i, slow, &cs.ns);
-        }
-        __syncthreads();
-        const int ns = min(cs.ns, kLaSlow);
-        const int per2 = kLaSlowTerms / E;
-        for (int sb = 0; sb < ns; sb += per2) {
-          const int ne = min(per2, ns - sb);
-          for (int j = tid; j < ne * E; j += blockDim.x) {
-            const int e = sb + j / E, k3 = j - (j / E) * E;
-            const uint32_t sc = slow.code[e];
-            slow.terms[j] = phi_term<1>(tn + la.stride, la.stride, Pn + E * E, E, M, a,
-                                        static_cast<int>((sc >> 8) & 0xFFu),
-                                        static_cast<int>(sc & 0xFFu), k3, slow.q2[e], qbar);
+  }
+  __syncthreads();
+  {  // the tokens of this block, by their rank among home a's
+    int rank = incl - mine;
+    for (int i = 0; i < warp; ++i) rank += s_part[i];
+    scan_homes([&](int t, int h) {
+      if (h != a) return;
+      if (rank >= lo && rank < lo + ntok) s_tok[rank - lo] = t;
+      ++rank;
+    });
+  }
+  // The classes of level 1: every loss is put at its rank among all of them
+  // (equal losses by target and place), and adds one to the count of its
+  // target in the rows past that rank. (A row between equal losses is never
+  // asked for: both fit or neither does.)
+  {
+    int all = 0, most = 0;
+    for (int kt = 0; kt < E; ++kt) {
+      all += s_nsub[0][kt];
+      most = max(most, s_nsub[0][kt]);
+    }
+    c.n_loss = all;
+    c.classes = E > kLaNarrow && all > 0 && all <= la_max_loss(E);
+    if (c.classes) {
+      for (int x = tid; x < E * most; x += kThreads) {
+        const int kt = x / most, n = x - kt * most;
+        if (n >= s_nsub[0][kt]) continue;
+        const float q = c.sQ[0][kt * c.pitch + n];
+        int r = n;
+        for (int k2 = 0; k2 < E; ++k2) {  // losses of target k2 that come before
+          if (k2 == kt) continue;
+          const float* s = c.sQ[0] + k2 * c.pitch;
+          int b = 0, e = s_nsub[0][k2];
+          while (b < e) {
+            const int mid = (b + e) >> 1;
+            if (s[mid] < q || (s[mid] == q && k2 < kt)) b = mid + 1;
+            else e = mid;
           }
-          __syncthreads();
-          for (int el = tid; el < ne; el += blockDim.x) {
-            const uint32_t sc = slow.code[sb + el];
-            const int kk = static_cast<int>(sc & 0xFFu);
-            const float* P2 = Pn + (size_t)E * E + (size_t)kk * E;
-            float phi1 = 0.0f;
-            for (int k3 = 0; k3 < E; ++k3)
-              if (ldt(P2 + k3) != 0.0f) phi1 = __fadd_rn(phi1, slow.terms[el * E + k3]);
-            atomicMin(&key[sc >> 16], min_key(__fadd_rn(slow.base[sb + el], phi1)));
-          }
-          __syncthreads();
+          r += b;
         }
-      } else {
-        for (int i = tid; i < nc * E; i += blockDim.x) {
-          const int c = base + i / E, kt = i - (i / E) * E;
-          const uint32_t code = cs.code[c];
-          const int cm = static_cast<int>((code >> 8) & 0xFFu), ck = static_cast<int>(code & 0xFFu);
-          cs.terms[i] = memo4 ? phi_term3_memo(tn, la.stride, Pn, E, M, a, cm, ck, kt, cs.qn[c],
-                                               qbar, U2, qmax2, qmaxL1, cs.U, cs.qmax1)
-                              : phi_term_h(la.H, tn, la.stride, Pn, E, M, a, cm, ck, kt, cs.qn[c],
-                                           qbar);
-        }
-        __syncthreads();
+        s_loss[r] = q;
+        s_rank[kt * 64 + n] = static_cast<uint16_t>(r);
       }
-      for (int cl = tid; cl < nc; cl += blockDim.x) {
-        const uint32_t code = cs.code[base + cl];
-        const int kk = static_cast<int>(code & 0xFFu), m = static_cast<int>((code >> 8) & 0xFFu);
-        const unsigned sub = (code >> 16) & 1u;
-        float phi = 0.0f;
-        for (int kt = 0; kt < E; ++kt) {
-          const float p = ldt(Pn + (size_t)kk * E + kt);
-          if (p == 0.0f) continue;
-          const float term = cs.terms[cl * E + kt];
-          phi = __fadd_rn(phi, memo ? __fmul_rn(p, from_min_key(__float_as_uint(term))) : term);
-        }
-        const float cost = __fadd_rn(cs.cost0[base + cl], phi);
-        const unsigned long long key =
-            (static_cast<unsigned long long>(__float_as_uint(cost)) << 32) |
-            (static_cast<unsigned long long>(sub) << 31) |
-            (static_cast<unsigned long long>(m != s ? 1u : 0u) << 30) |
-            (static_cast<unsigned long long>(m) << 8) | static_cast<unsigned long long>(kk);
-        atomicMin(&cs.best, key);
-      }
-      __syncthreads();
     }
-    const unsigned long long best = cs.best;
-    int kstar, mstar, kd;
-    if (best == ~0ull) {
-      if (tid == 0) report(&g_err_route, ORDERMOE_DEV_NO_CANDIDATE, t);
-      kstar = r; mstar = s; kd = 0;
+  }
+  // where each target's row starts: (1 + substitutes) M entries, an odd length
+  // (rows of equal length start in distinct banks), two targets a lane
+  if (warp < D) {
+    int* off = s_woff[warp];
+    const int* ns = s_nsub[warp];
+    const int n0 = 2 * lane < E ? ((ns[2 * lane] + 1) * M) | 1 : 0;
+    const int n1 = 2 * lane + 1 < E ? ((ns[2 * lane + 1] + 1) * M) | 1 : 0;
+    int in = n0 + n1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, in, o);
+      if (lane >= o) in += u;
+    }
+    if (2 * lane < E) off[2 * lane] = in - n0 - n1;
+    if (2 * lane + 1 < E) off[2 * lane + 1] = in - n1;
+    if (lane == 31) off[64] = in;
+  }
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    c.has[i] = s_qmax[i] >= 0;
+    c.qmax[i] = __int_as_float(s_qmax[i]);
+    c.qmin[i] = __int_as_float(s_qmin[i]);
+  }
+  c.prune = __syncthreads_or(bad_p) == 0;
+  c.rows = true;
+#pragma unroll
+  for (int i = 0; i < D; ++i) c.rows = c.rows && s_woff[i][64] <= wcap;
+  if (c.classes) {
+    const int pitch = la_class_pitch(E);
+    for (int kt = warp; kt < E; kt += NW) {
+      const int ns = s_nsub[0][kt];
+      for (int cl = lane; cl <= c.n_loss; cl += 32) {
+        int f = 0;
+        while (f < ns && s_rank[kt * 64 + f] < cl) ++f;
+        s_fits[cl * pitch + kt] = static_cast<uint8_t>(f);
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    const LaLevel& v = c.lev[i];
+    const float* ua = i > 0 ? c.Ua[i - (i > 0)] : nullptr;
+    const float* un = i > 0 ? c.Un[i - (i > 0)] : nullptr;
+    if (c.rows) {
+      // a warp a row, an entry (the exact expert or a substitute) and m a lane;
+      // then a lane an m takes the minima along the row
+      for (int kt = warp; kt < E; kt += NW) {
+        const int ns = s_nsub[i][kt];
+        float* wa = Wa[i] + s_woff[i][kt];
+        float* cn = i > 0 ? Cn[i] + s_woff[i][kt] : nullptr;
+        for (int x = lane; x < (ns + 1) * M; x += 32) {
+          const int n = x / M, m = x - n * M;
+          const int kk = n == 0 ? kt : s_ord[i][kt * 64 + n - 1];
+          const float cq = n == 0 ? 0.0f : v.Cq[kt * E + kk];
+          float all = INFINITY, none = INFINITY;
+          for (uint32_t pm = v.pmask[kk]; pm; pm &= pm - 1) {
+            const int m2 = __ffs(pm) - 1;
+            const float base = __fadd_rn(v.A[m * M + m2], cq);
+            if (i == 0) {
+              all = fminf(all, base);
+            } else {
+              all = fminf(all, __fadd_rn(base, ua[m2 * E + kk]));
+              none = fminf(none, __fadd_rn(base, un[m2 * E + kk]));
+            }
+          }
+          wa[x] = all;
+          if (i > 0) cn[x] = none;
+        }
+        __syncwarp();
+        for (int m = lane; m < M; m += 32) {
+          float best = wa[m];
+          Vn[m * E + kt] = i > 0 ? cn[m] : best;
+          for (int n = 1; n <= ns; ++n) {
+            best = fminf(best, wa[n * M + m]);
+            wa[n * M + m] = best;
+          }
+          Va[m * E + kt] = best;
+        }
+      }
     } else {
-      kstar = static_cast<int>(best & 0xFFu);
-      mstar = static_cast<int>((best >> 8) & 0xFFu);
-      const int sub = static_cast<int>((best >> 31) & 1u);
-      const int away = static_cast<int>((best >> 30) & 1u);
-      kd = 2 * away + sub;
-      if (sub) {
-        taken |= 1ull << kstar;
-        q = __fadd_rn(q, s_Q[r * E + kstar]);
+      // V of level i + 1, one (k', m) a thread
+      for (int x = tid; x < E * M; x += kThreads) {
+        const int kt = x / M, m = x - kt * M;
+        float all = INFINITY, none = INFINITY;
+        for (unsigned long long sb = v.subst[kt] | (1ull << kt); sb; sb &= sb - 1) {
+          const int kk = __ffsll(static_cast<long long>(sb)) - 1;
+          const float cq = kk == kt ? 0.0f : v.Cq[kt * E + kk];
+          for (uint32_t pm = v.pmask[kk]; pm; pm &= pm - 1) {
+            const int m2 = __ffs(pm) - 1;
+            const float base = __fadd_rn(v.A[m * M + m2], cq);
+            all = fminf(all, i > 0 ? __fadd_rn(base, ua[m2 * E + kk]) : base);
+            if (kk == kt) none = fminf(none, i > 0 ? __fadd_rn(base, un[m2 * E + kk]) : base);
+          }
+        }
+        Va[m * E + kt] = all;
+        Vn[m * E + kt] = none;
       }
     }
-    if (j == 0) first_server = mstar;
-    if (tid == 0) {
-      chosen_expert[(size_t)t * k + j] = kstar;
-      chosen_server[(size_t)t * k + j] = static_cast<uint8_t>(mstar);
-      kind_out[(size_t)t * k + j] = static_cast<uint8_t>(kd);
-      if (counters != nullptr) atomicAdd(&counters[kd], 1);
+    __syncthreads();
+    // Phi of level i + 1 in both cases, one (m, kx) a thread
+    for (int x = tid; x < M * E; x += kThreads) {
+      const int m = x / E, kx = x - m * E;
+      const float* Pr = c.P[i] + kx * c.pitch;
+      float pa = 0.0f, pn = 0.0f;
+#pragma unroll 8
+      for (int kt = 0; kt < E; ++kt) {
+        const float p = Pr[kt];
+        if (p != 0.0f) {
+          pa = __fadd_rn(pa, __fmul_rn(p, Va[m * E + kt]));
+          pn = __fadd_rn(pn, __fmul_rn(p, Vn[m * E + kt]));
+        }
+      }
+      U[2 * i][x] = pa;
+      U[2 * i + 1][x] = pn;
     }
-    __syncthreads();  // the candidate arrays are rewritten for the next slot
+    __syncthreads();
   }
-  if (tid == 0 && loc != nullptr) {
-    loc[t] = static_cast<uint8_t>(first_server);
-    qhat[t] = q;
+
+  // ---- the tokens, one a warp
+  const LaLevel own = la_level(tab, E, M, a);
+  // the servers of experts lane and lane + 32
+  const uint32_t pmask0 = lane < E ? own.pmask[lane] : 0u;
+  const uint32_t pmask1 = lane + 32 < E ? own.pmask[lane + 32] : 0u;
+  int kind_count[4] = {0, 0, 0, 0};
+  for (int i = warp; i < ntok; i += NW) {
+    const int t = s_tok[i];
+    const int s = (loc != nullptr) ? loc[t] : a;
+    float q = (qhat != nullptr) ? qhat[t] : 0.0f;
+    const int idx = lane < k ? topk_idx[(size_t)t * k + lane] : 0;
+    if (s >= M) {
+      if (lane == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, t);
+      continue;
+    }
+    if (__any_sync(0xffffffffu, idx < 0 || idx >= E)) continue;  // -1: a NaN token (reported)
+    unsigned long long taken = 0;
+    for (int j = 0; j < k; ++j) taken |= 1ull << __shfl_sync(0xffffffffu, idx, j);
+    const float* As = own.A + s * M;
+    int first_server = s;
+    for (int j = 0; j < k; ++j) {
+      const int r = __shfl_sync(0xffffffffu, idx, j);
+      const unsigned long long sb = own.subst[r] & ~taken;
+      unsigned long long best = ~0ull;
+#pragma unroll 1
+      for (int h = 0; 32 * h < E; ++h) {
+        const int e = lane + 32 * h;
+        const bool sub = (sb >> e) & 1ull;
+        float cq = 0.0f, qn = q;
+        uint32_t pm = (sub || e == r) ? (h ? pmask1 : pmask0) : 0u;
+        if (sub) {
+          qn = __fadd_rn(q, own.Q[r * E + e]);
+          cq = own.Cq[r * E + e];
+          if (!(qn <= qbar)) pm = 0u;  // Eq. 40 budget
+        }
+        const float* Ut = la_all<D>(c, D, qn) ? c.Ua[D - 1] : la_none<D>(c, D, qn) ? c.Un[D - 1] : nullptr;
+        auto key_of = [&](int m, float phi) {
+          const float cost = __fadd_rn(__fadd_rn(As[m], cq), phi);
+          return (static_cast<unsigned long long>(__float_as_uint(cost)) << 32) |
+                 (static_cast<unsigned long long>(sub ? 1u : 0u) << 31) |
+                 (static_cast<unsigned long long>(m != s ? 1u : 0u) << 30) |
+                 (static_cast<unsigned long long>(m) << 8) | static_cast<unsigned long long>(e);
+        };
+        if (Ut != nullptr)
+          for (; pm; pm &= pm - 1) {
+            const int m = __ffs(pm) - 1;
+            const unsigned long long key = key_of(m, Ut[m * E + e]);
+            best = key < best ? key : best;
+          }
+        // candidates in neither case, one after another by the whole warp, but
+        // those that cost more than another at best (Ua is the least of Phi)
+        for (unsigned todo = __ballot_sync(0xffffffffu, pm != 0u); todo; todo &= todo - 1) {
+          const int src = __ffs(todo) - 1;
+          const uint32_t pms = __shfl_sync(0xffffffffu, pm, src);
+          const float qs = __shfl_sync(0xffffffffu, qn, src), cqs = __shfl_sync(0xffffffffu, cq, src);
+          for (uint32_t x = pms; x; x &= x - 1) {
+            const int m = __ffs(x) - 1;
+            const float least = __fadd_rn(__fadd_rn(As[m], cqs), c.Ua[D - 1][m * E + src + 32 * h]);
+            if (__any_sync(0xffffffffu, c.prune && best != ~0ull && least > __uint_as_float(static_cast<unsigned>(best >> 32)))) continue;
+            const float phi = la_phi_warp<D>(c, s_term, lane, m, src + 32 * h, qs);
+            if (lane == src) {
+              const unsigned long long key = key_of(m, phi);
+              best = key < best ? key : best;
+            }
+          }
+        }
+      }
+      // the smallest key of the warp: high words, then the low words among those
+      const unsigned hi = static_cast<unsigned>(best >> 32);
+      const unsigned mhi = __reduce_min_sync(0xffffffffu, hi);
+      const unsigned mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? static_cast<unsigned>(best) : 0xffffffffu);
+      int kstar, mstar, kd;
+      if (mhi == 0xffffffffu && mlo == 0xffffffffu) {
+        if (lane == 0) report(&g_err_route, ORDERMOE_DEV_NO_CANDIDATE, t);
+        kstar = r; mstar = s; kd = 0;
+      } else {
+        kstar = static_cast<int>(mlo & 0xFFu);
+        mstar = static_cast<int>((mlo >> 8) & 0xFFu);
+        const int sub = static_cast<int>((mlo >> 31) & 1u);
+        kd = 2 * static_cast<int>((mlo >> 30) & 1u) + sub;
+        if (sub) {
+          taken |= 1ull << kstar;
+          q = __fadd_rn(q, own.Q[r * E + kstar]);
+        }
+      }
+      if (j == 0) first_server = mstar;
+      if (lane == 0) {
+        chosen_expert[(size_t)t * k + j] = kstar;
+        chosen_server[(size_t)t * k + j] = static_cast<uint8_t>(mstar);
+        kind_out[(size_t)t * k + j] = static_cast<uint8_t>(kd);
+      }
+#pragma unroll
+      for (int x = 0; x < 4; ++x) kind_count[x] += kd == x ? 1 : 0;
+    }
+    if (lane == 0 && loc != nullptr) {
+      loc[t] = static_cast<uint8_t>(first_server);
+      qhat[t] = q;
+    }
   }
+  if (counters == nullptr) return;
+  if (lane == 0)
+    for (int x = 0; x < 4; ++x)
+      if (kind_count[x]) atomicAdd(&s_kind[x], kind_count[x]);
+  __syncthreads();
+  if (tid < 4 && s_kind[tid]) atomicAdd(&counters[tid], s_kind[tid]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1462,8 +1546,8 @@ __global__ void __launch_bounds__(rt::THREADS, 1) router_select_kernel(
         col[(c / 4) * 128] = make_float4(lg[c], lg[c + 1], lg[c + 2], lg[c + 3]);
       const int M = reinterpret_cast<const int32_t*>(tab)[2];
       const float qbar = reinterpret_cast<const float*>(tab)[5];
-      select_token(t, ColLogits{col}, E, k, renorm, M, qbar, Atab, tab, la, sm, s_Q, s_Cq, pre_a,
-                   pre_s, pre_q, loc, qhat, topk_idx, topk_w, chosen_expert, chosen_server,
+      select_token(t, ColLogits{col}, E, k, renorm, M, qbar, Atab, sm, s_Q, s_Cq, pre_a, pre_s,
+                   pre_q, loc, qhat, topk_idx, topk_w, chosen_expert, chosen_server,
                    kind_out, kind_count, !rt::selects<NE>() || la.H > 1 || la.topk_only);
     }
     flush_kind_counts(sm, kind_count, counters);
@@ -1522,29 +1606,56 @@ extern "C" int ordermoe_build_tables(const float* sim, const int32_t* group,
   return ORDERMOE_OK;
 }
 
+template <int D, int NW>
+static cudaError_t lookahead_launch(int T, int E, int Mcap, int k, const int32_t* topk_idx,
+                                    const uint8_t* tb, const Lookahead& la, const uint8_t* home,
+                                    uint8_t* loc, float* qhat, int32_t* chosen_expert,
+                                    uint8_t* chosen_server, uint8_t* kind, int32_t* counters,
+                                    cudaStream_t stream) {
+  // rows for every substitute set there can be, or as many as fit beside the
+  // rest of a block's shared memory (200 KB of the 227; the static arrays
+  // take up to 16 KB more)
+  const size_t fixed = la_smem_fixed(E, D, Mcap, NW);
+  long long wcap = (long long)E * ((E * Mcap) | 1);
+  const long long room = (200 * 1024 - (long long)fixed) / ((2 * D - 1) * (long long)sizeof(float));
+  if (wcap > room) wcap = room > 0 ? room : 0;
+  const size_t smem = la_smem_bytes(E, D, Mcap, NW, static_cast<int>(wcap));
+  cudaFuncSetAttribute(lookahead_select_kernel<D, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)smem);
+  // a token a warp until the blocks of one wave (one an SM) are full, then
+  // more tokens a block, which share its tables
+  const long long wave = (long long)num_sms() * NW;
+  long long tpb = NW * ((T + wave - 1) / wave);
+  if (tpb > kLaMaxTok) tpb = kLaMaxTok;
+  // a home's last block may be partly filled: at most one more block a home
+  const long long blocks = T / tpb + Mcap;
+  return launch_pdl(lookahead_select_kernel<D, NW>, dim3(static_cast<unsigned>(blocks)),
+                    dim3(32 * NW), smem, stream, topk_idx, T, E, k, tb, la, Mcap,
+                    static_cast<int>(wcap), static_cast<int>(tpb), home, loc, qhat, chosen_expert,
+                    chosen_server, kind, counters);
+}
+
 static int launch_lookahead_select(const int32_t* topk_idx, int T, int E, int k,
                                    const uint8_t* tb, Lookahead la, const uint8_t* home,
                                    uint8_t* loc, float* qhat, int32_t* chosen_expert,
                                    uint8_t* chosen_server, uint8_t* kind, int32_t* counters,
-                                   size_t tab_smem, cudaStream_t stream) {
+                                   cudaStream_t stream) {
   if (T <= 0) return ORDERMOE_OK;
-  if (la.H == 4) tab_smem += sizeof(float) * (32 * E + E);  // the Phi^(2) table and its bounds
-  // the next layers' tables and transitions in shared memory when they fit
-  la.staged = 0;
-  if (la.H > 1) {
-    const size_t staged = la_stage_offset(E, la.H) + la_stage_bytes(E, la.H, la.stride);
-    if (staged <= 160 * 1024) {
-      tab_smem = staged;
-      la.staged = 1;
-    }
-  }
-  if (la.H == 3) tab_smem = la_slow_offset(E, 3, la.stride, la.staged) + kLaSlowBytes;
-  cudaFuncSetAttribute(lookahead_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)tab_smem);
-  OM_LAUNCH_PDL("lookahead_select_kernel", lookahead_select_kernel, dim3(T), dim3(kLaThreads),
-                tab_smem, stream, topk_idx, T, E, k, tb, la, home, loc, qhat, chosen_expert,
-                chosen_server, kind, counters);
-  return ORDERMOE_OK;
+  // the most servers whose tables fit the stride (the device header has the
+  // number; one that does not fit is reported)
+  int Mcap = 1;
+  while (Mcap < ORDERMOE_MAX_SERVERS && om::tables_bytes(E, Mcap + 1) <= la.stride) ++Mcap;
+  cudaError_t e;
+#define OM_LA_LAUNCH(D)                                                                         \
+  (E > kLaNarrow ? lookahead_launch<D, 16>(T, E, Mcap, k, topk_idx, tb, la, home, loc, qhat,           \
+                                    chosen_expert, chosen_server, kind, counters, stream)       \
+          : lookahead_launch<D, 8>(T, E, Mcap, k, topk_idx, tb, la, home, loc, qhat,            \
+                                   chosen_expert, chosen_server, kind, counters, stream))
+  if (la.H == 2) e = OM_LA_LAUNCH(1);
+  else if (la.H == 3) e = OM_LA_LAUNCH(2);
+  else e = OM_LA_LAUNCH(3);
+#undef OM_LA_LAUNCH
+  return e == cudaSuccess ? ORDERMOE_OK : cuda_fail(e, "lookahead_select_kernel");
 }
 
 static int launch_select_lanes(const int32_t* topk_idx, int T, int E, int k, const uint8_t* tb,
@@ -1609,8 +1720,7 @@ static int route_select_impl(const uint16_t* X, const uint16_t* W_r, const float
 #undef OM_SEL_LAUNCH
     if (sel_err != cudaSuccess) return cuda_fail(sel_err, "select_kernel");
     return la.H > 1 ? launch_lookahead_select(topk_idx, T, E, k, tb, la, home, loc, qhat,
-                                              chosen_expert, chosen_server, kind, counters,
-                                              tab_smem, stream)
+                                              chosen_expert, chosen_server, kind, counters, stream)
                     : ORDERMOE_OK;
   }
   // many experts (long candidate lists per slot): the router writes the
@@ -1660,7 +1770,7 @@ static int route_select_impl(const uint16_t* X, const uint16_t* W_r, const float
   OM_LAUNCHED("router_select_kernel");
   if (la.H > 1)
     return launch_lookahead_select(topk_idx, T, E, k, tb, la, home, loc, qhat, chosen_expert,
-                                   chosen_server, kind, counters, tab_smem, stream);
+                                   chosen_server, kind, counters, stream);
   if (lanes)
     return launch_select_lanes(topk_idx, T, E, k, tb, home, loc, qhat, chosen_expert,
                                chosen_server, kind, counters, tab_smem, stream);

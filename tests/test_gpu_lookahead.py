@@ -102,6 +102,43 @@ def test_route_select_lookahead_given_logits_bit_exact(E, M, k, H, cheap):
         print("decisions changed by the look-ahead:", int((myo[0] != ref[0]).sum() + (myo[1] != ref[1]).sum()))
 
 
+@pytest.mark.parametrize("T,E,M,k,H,skew", [
+    (5001, 8, 4, 2, 3, True),     # several tokens a warp, one home with most of them, a ragged last block
+    (6, 64, 8, 6, 3, False),      # two experts a lane, every loss regime, prefix minima in the table
+    (40, 64, 32, 2, 2, False),    # prefix minima too many for the table: the direct minimum
+    (4, 33, 32, 3, 3, True), (60, 1, 1, 1, 4, False), (17, 13, 2, 8, 4, False)])
+def test_lookahead_tokens_by_home_bit_exact(T, E, M, k, H, skew):
+    """Losses spread over the whole budget, so that candidates fall on the
+    tables with every check passing, on those with every check failing and
+    between; homes uneven, some servers without tokens."""
+    rng = np.random.default_rng(T + E + M)
+    qbar = 0.3
+    buf, stride, otabs = stack_tables(rng, H, E, M, qbar, True)
+    P = rng.random((H - 1, E, E)).astype(np.float32)
+    P[P < 0.3] = 0
+    P = (P / np.maximum(P.sum(axis=2, keepdims=True), 1e-9)).astype(np.float32)
+    logits = rng.standard_normal((T, E)).astype(np.float32)
+    home = rng.integers(0, M, T).astype(np.uint8)
+    if skew:
+        home[rng.random(T) < 0.8] = M // 2
+    loc = np.where(rng.random(T) < 0.5, home, rng.integers(0, M, T)).astype(np.uint8)
+    qhat = (rng.random(T) * 1.1 * qbar).astype(np.float32)
+    g = [torch.empty(T, k, dtype=dt, device=DEV)
+         for dt in (torch.int32, torch.float32, torch.int32, torch.uint8, torch.uint8)]
+    gl = torch.as_tensor(loc).to(DEV); gq = torch.as_tensor(qhat).to(DEV)
+    cnt = torch.zeros(4, dtype=torch.int32, device=DEV)
+    B.ordermoe_route_select_lookahead(None, None, torch.as_tensor(logits).to(DEV), T, E, 0, k, 1, buf,
+                                      stride, H, torch.as_tensor(P).to(DEV),
+                                      torch.as_tensor(home).to(DEV), gl, gq, None, *g, cnt)
+    idx, _ = oracle.topk(logits, k)
+    ref = oracle.select_lookahead(idx, otabs[:H], P, home, loc, qhat)
+    for name, got, want in zip(("chosen", "server", "kind"), (g[2], g[3], g[4]), ref[:3]):
+        np.testing.assert_array_equal(got.cpu().numpy(), want, err_msg=name)
+    np.testing.assert_array_equal(gl.cpu().numpy(), ref[3])
+    np.testing.assert_array_equal(gq.cpu().numpy(), ref[4])
+    np.testing.assert_array_equal(cnt.cpu().numpy(), np.bincount(ref[2].ravel(), minlength=4))
+
+
 def test_lookahead_horizon_one_equals_route_select():
     rng = np.random.default_rng(5)
     E, M, k, T = 8, 4, 2, 200
