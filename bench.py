@@ -54,9 +54,9 @@ def gate_up_traffic(workload):
 
 def gate_up_kernel_name(R, E, dff):
     """The gate/up kernel the library picks for R permuted rows (grouped_gemm.cu)."""
-    if R < 256 * E:
-        return "ffn_gemm_kernel<gate_up> (tcgen05, one CTA, 128-row tiles)"
-    return "ffn_gemm_pair_kernel<gate_up> (tcgen05 CTA pairs)"
+    if R < 112 * E:
+        return "ffn_gemm_kernel<gate_up> (tcgen05, one CTA, up to 128 rows)"
+    return "ffn_gemm_kernel<gate_up, pair> (tcgen05 CTA pairs)"
 
 
 def parse():

@@ -1,24 +1,18 @@
 // Grouped SwiGLU expert FFN on sm_103a tensor cores (tcgen05 + TMEM + TMA).
 //
-// Persistent warp-specialised kernels over the expert-contiguous rows of
-// ordermoe_dispatch, with the per-expert row ranges read on the device: a
-// one-CTA kernel for small batches (described here) and a CTA-pair kernel
-// with the weights on the MMA's M side for large ones (its own section below).
-// One-CTA kernel:
-//   gate/up: H[rows of e, n0:n0+128] = bf16(silu(X W1_e^T) * (X W3_e^T)) for a
-//            128-column slice n0 of d_ff. One tcgen05.mma of N = 256 computes
-//            the gate (TMEM columns 0..127) and up (128..255) projections from
-//            a B tile whose first 128 rows are W1_e rows and last 128 rows are
-//            W3_e rows; the epilogue fuses SwiGLU.
-//   down:    Y[rows of e, n0:n0+256] = bf16(H W2_e^T).
-// Tile = 128 rows x 256 accumulator columns, K step 64 (one 128-byte
-// swizzled TMA box per operand row), 4-stage shared-memory ring, two TMEM
-// accumulators (2 x 256 columns = all 512) so the epilogue of one tile
-// overlaps the main loop of the next.
-// Warp roles (192 threads): warp 0 = TMA producer, warp 1 = MMA issuer and
-// TMEM owner, warps 2-5 = epilogue (warp w reads TMEM lanes 32 (w % 4) ...).
-// Tile order: expert, then N slice, then M tile, so CTAs running at the same
-// time share the same weight slice through L2.
+// ffn_gemm_kernel: persistent warp-specialised kernels over the
+// expert-contiguous rows of ordermoe_dispatch, with the per-expert row ranges
+// read on the device: the weights on the MMA's M side, on CTA pairs for large
+// batches and on single CTAs for small ones (its own section below).
+//   gate/up: H = bf16(silu(X W1_e^T) * (X W3_e^T)), fused in the epilogue;
+//   down:    Y = bf16(H W2_e^T).
+// logits_gemm_kernel: the router logits of the offline similarity where the
+// tensor-core path of sim_gemm.cu does not apply. Tile = 128 rows x 256
+// accumulator columns, K step 64 (one 128-byte swizzled TMA box per operand
+// row), 4-stage shared-memory ring, two TMEM accumulators (2 x 256 columns =
+// all 512) so the epilogue of one tile overlaps the main loop of the next.
+// Warp roles: warp 0 = TMA producer, warp 1 = MMA issuer and TMEM owner, the
+// others = epilogue (warp w reads TMEM lanes 32 (w % 4) ...).
 // Every wait is bounded (globaltimer); a wait that runs out reports
 // ORDERMOE_DEV_WAIT_TIMEOUT, makes the other roles stop, drains the copies
 // and MMAs in flight (bounded too), frees TMEM and returns.
@@ -61,12 +55,13 @@ struct Smem {
   uint32_t tmem_base;
   int abort;
   int zero;
+  int max_rows;  // the largest row tile
   int mt_start[ORDERMOE_MAX_EXPERTS + 1];
   int offs[ORDERMOE_MAX_EXPERTS + 1];
 };
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + static_cast<int>(sizeof(Smem));
 
-enum { GATEUP = 0, DOWN = 1, LOGITS = 2 };
+enum { GATEUP = 0, DOWN = 1 };
 
 struct Args {
   const int32_t* offsets;  // [E+1] row ranges (0 <= ... <= rows); null: one group of `rows` rows
@@ -81,6 +76,7 @@ struct Args {
   int ldo;           // row length of out
   uint64_t limit_ns; // bounded-wait limit
   int m_major;       // 1: all N slices of an M tile back to back (A read once from HBM)
+  int fast_div;      // gate/up: SwiGLU's quotient by the fast reciprocal
 };
 
 struct Tile {
@@ -119,6 +115,8 @@ __device__ __forceinline__ void load_row_tiles(S& s, const Args& args, int bm, i
   }
   i1 += __shfl_sync(0xffffffffu, i0, 31);
   if (bad) i0 = i1 = 0;
+  const int most = __reduce_max_sync(0xffffffffu, max(n0 - o0, n1 - o1));
+  if (lane == 0) s.max_rows = bad ? 0 : min(most, bm);
   if (lane <= E) {
     s.offs[lane] = o0;
     s.mt_start[lane] = bad ? 0 : i0 - t0;
@@ -160,10 +158,9 @@ __device__ __forceinline__ Tile decode(int tile, const Smem& s, int E, int n_til
   return t;
 }
 
-template <int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
-    ffn_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
-                    const __grid_constant__ CUtensorMap mapB1, Args args) {
+    logits_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
+                       Args args) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -177,7 +174,6 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp == 0 && lane == 0) {
     tma_prefetch_map(&mapA);
     tma_prefetch_map(&mapB0);
-    if (MODE == GATEUP) tma_prefetch_map(&mapB1);
   }
 
   if (tid == 0) {
@@ -221,7 +217,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       uint32_t phase = 0;
       for (int tile = blockIdx.x; tile < total && !*abort; tile += gridDim.x) {
         const Tile t = decode(tile, s, args.E, args.n_tiles, args.m_major);
-        const int brow = t.e * args.b_rows + t.n * (MODE == GATEUP ? 128 : 256);  // LOGITS: e == 0
+        const int brow = t.n * 256;
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait(&s.empty[stage], phase ^ 1u, args.limit_ns, abort)) {
             if (!*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 1);
@@ -232,13 +228,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           uint8_t* sb = sa + A_BYTES;
           mbar_arrive_expect_tx(&s.full[stage], STAGE_BYTES);
           tma_load_2d(sa, &mapA, &s.full[stage], kb * BK, t.m0);
-          if (MODE == GATEUP) {
-            tma_load_2d(sb, &mapB0, &s.full[stage], kb * BK, brow);
-            tma_load_2d(sb + BOX_BYTES, &mapB1, &s.full[stage], kb * BK, brow);
-          } else {
-            tma_load_2d(sb, &mapB0, &s.full[stage], kb * BK, brow);
-            tma_load_2d(sb + BOX_BYTES, &mapB0, &s.full[stage], kb * BK, brow + 128);
-          }
+          tma_load_2d(sb, &mapB0, &s.full[stage], kb * BK, brow);
+          tma_load_2d(sb + BOX_BYTES, &mapB0, &s.full[stage], kb * BK, brow + 128);
           issued_mask |= 1u << stage;
           last_phase_bits = (last_phase_bits & ~(1u << stage)) | (phase << stage);
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -305,71 +296,27 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int row = t.m0 + lrow;
       const bool valid = row < t.m_end;
       const uint32_t tb = tmem_base + slot * BN + (static_cast<uint32_t>(q * 32) << 16);
-      if (MODE == GATEUP) {
-        uint16_t* orow = args.out + (size_t)row * args.ldo + t.n * 128;
+      const int col0 = t.n * 256;
+      float* orow = args.out_f32 + (size_t)row * args.n_valid;
+      const bool vec = (args.n_valid & 3) == 0;
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-          uint32_t g[32], u[32];
-          tmem_ld32(tb + c * 32, g);
-          tmem_ld32(tb + 128 + c * 32, u);
-          tmem_ld_wait();
-          if (valid) {
-            uint32_t pk[16];
+      for (int c = 0; c < 8; ++c) {
+        if (col0 + c * 32 >= args.n_valid) break;  // warp-uniform
+        uint32_t v[32];
+        tmem_ld32(tb + c * 32, v);
+        tmem_ld_wait();
+        if (valid) {
+          const int cb = col0 + c * 32;
+          if (vec && cb + 32 <= args.n_valid) {
+            float4* dst = reinterpret_cast<float4*>(orow + cb);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float g0 = __uint_as_float(g[2 * i]), g1 = __uint_as_float(g[2 * i + 1]);
-              const float u0 = __uint_as_float(u[2 * i]), u1 = __uint_as_float(u[2 * i + 1]);
-              const float h0 = g0 / (1.0f + __expf(-g0)) * u0;
-              const float h1 = g1 / (1.0f + __expf(-g1)) * u1;
-              pk[i] = pack_bf16x2(h0, h1);
-            }
-            uint4* dst = reinterpret_cast<uint4*>(orow + c * 32);
+            for (int i = 0; i < 8; ++i)
+              dst[i] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
+                                   __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+          } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-              dst[i] = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
-          }
-        }
-      } else if (MODE == LOGITS) {
-        const int col0 = t.n * 256;
-        float* orow = args.out_f32 + (size_t)row * args.n_valid;
-        const bool vec = (args.n_valid & 3) == 0;
-#pragma unroll 1
-        for (int c = 0; c < 8; ++c) {
-          if (col0 + c * 32 >= args.n_valid) break;  // warp-uniform
-          uint32_t v[32];
-          tmem_ld32(tb + c * 32, v);
-          tmem_ld_wait();
-          if (valid) {
-            const int cb = col0 + c * 32;
-            if (vec && cb + 32 <= args.n_valid) {
-              float4* dst = reinterpret_cast<float4*>(orow + cb);
-#pragma unroll
-              for (int i = 0; i < 8; ++i)
-                dst[i] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
-                                     __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
-            } else {
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                if (cb + i < args.n_valid) orow[cb + i] = __uint_as_float(v[i]);
-            }
-          }
-        }
-      } else {
-        uint16_t* orow = args.out + (size_t)row * args.ldo + t.n * 256;
-#pragma unroll 1
-        for (int c = 0; c < 8; ++c) {
-          uint32_t v[32];
-          tmem_ld32(tb + c * 32, v);
-          tmem_ld_wait();
-          if (valid) {
-            uint32_t pk[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-              pk[i] = pack_bf16x2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
-            uint4* dst = reinterpret_cast<uint4*>(orow + c * 32);
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              dst[i] = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+            for (int i = 0; i < 32; ++i)
+              if (cb + i < args.n_valid) orow[cb + i] = __uint_as_float(v[i]);
           }
         }
       }
@@ -399,9 +346,9 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
-// ------------------------------------------------- CTA-pair variant (gate/up, down)
+// ------------------------------------------------------------- gate/up and down
 //
-// A pair of CTAs on 2 SMs computes, with tcgen05.mma.cta_group::2 issued
+// Pairs (PAIR): a pair of CTAs on 2 SMs computes, with tcgen05.mma.cta_group::2 issued
 // by the even CTA, a tile of 256 weight rows (the MMA's M side; 128 in each
 // CTA's shared memory and TMEM lanes) by up to 256 permuted rows of one expert
 // (the N side, split evenly between the two CTAs' shared memory). The weight
@@ -420,6 +367,12 @@ __global__ void __launch_bounds__(THREADS, 1)
 // coalesced stores, skipping rows beyond the expert's range.
 // Each cluster is one CTA pair, and each CTA loads its own operand boxes from
 // this GPU's memory (no multicast loads).
+// Single CTAs: the same tile halved, 128 weight rows by up to 128 permuted
+// rows, with cta_group::1 MMAs, for batches whose weights are streamed once:
+// bound by HBM. A tile moves 16 KB of weights and the expert's own rows (16 to
+// 128) a K step; rows on the M side moved 128 row boxes whatever the expert
+// had and 256 columns a tile: gate/up of 1 token on 8 experts 126 against 72
+// us, of 128 tokens 285 against 275; 64 experts x 8 tokens 74 and 62 us.
 // Barriers: full[s] (even CTA, one arrive with the pair's bytes; both CTAs'
 // TMA loads complete on it), empty[s] and tfull[b] (both CTAs, arrived by the
 // even CTA's MMA commits signalled to the pair), tempty[b] (even CTA, one
@@ -430,7 +383,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 // shared-memory exchange, and the decision to stop is a barrier reduction over
 // all epilogue warps (barrier 3), so they always leave together.
 constexpr int P_BM = 256;            // permuted rows (N side) per tile
-constexpr int P_MAX_STAGES = 6;
+constexpr int P_MAX_STAGES = 20;
 constexpr int P_W_BYTES = 128 * BK * 2;   // 128 weight rows per CTA and K block
 constexpr int P_T_BYTES = 128 * BK * 2;   // one box of 128 permuted rows per CTA
 constexpr int P_STAGE_BYTES = P_W_BYTES + P_T_BYTES;
@@ -449,27 +402,31 @@ struct PSmem {
   uint32_t tmem_base;
   int abort;
   int zero;
+  int max_rows;  // the largest row tile
   int mt_start[ORDERMOE_MAX_EXPERTS + 1];
   int offs[ORDERMOE_MAX_EXPERTS + 1];
 };
-// Per projection: gate/up (SwiGLU exchange in the epilogue) runs two epilogue
-// groups of four warps and five stages; down (a plain conversion) one group
-// and six stages. Five stages time the same as six for gate/up, and a second
-// group made down slower.
-template <int MODE>
+// Per projection: a pair's gate/up (SwiGLU exchange in the epilogue) runs two
+// epilogue groups of four warps and five stages; down (a plain conversion) one
+// group and six stages. Five stages time the same as six for gate/up, and a
+// second group made down slower. A single CTA, bound by the weights' bytes,
+// runs one group and six stages.
+template <int MODE, bool PAIR>
 struct PCfg {
-  static constexpr int GROUPS = MODE == GATEUP ? 2 : 1;
+  static constexpr int GROUPS = MODE == GATEUP && PAIR ? 2 : 1;
   static constexpr int EPI_WARPS = 4 * GROUPS;
   static constexpr int THREADS = 64 + 32 * EPI_WARPS;
-  static constexpr int STAGES = MODE == GATEUP ? 5 : 6;
+  static constexpr int STAGES = MODE == GATEUP && PAIR ? 5 : 6;  // stages of full rows
+  static constexpr int MAX_STAGES = PAIR ? STAGES : P_MAX_STAGES;
+  static constexpr int ROWS = PAIR ? P_BM : P_BM / 2;  // permuted rows per tile
   static constexpr int EPI_BYTES = GROUPS * P_EPI_GROUP_BYTES;
   static constexpr int SMEM_BYTES =
       STAGES * P_STAGE_BYTES + EPI_BYTES + 1024 + static_cast<int>(sizeof(PSmem));
-  static_assert(STAGES <= P_MAX_STAGES, "stage barriers");
-  static_assert(SMEM_BYTES <= 227 * 1024, "pair kernel shared memory");
+  static_assert(MAX_STAGES <= P_MAX_STAGES, "stage barriers");
+  static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of the FFN kernels");
 };
 
-__device__ __forceinline__ Tile decode_pair(int tile, const PSmem& s, int E, int n_tiles) {
+__device__ __forceinline__ Tile decode_pair(int tile, const PSmem& s, int E, int n_tiles, int bm) {
   // the last expert whose first tile is <= tile (binary search: the row-tile
   // starts never decrease; empty experts share their successor's start)
   int e = 0, hi = E - 1;
@@ -483,14 +440,14 @@ __device__ __forceinline__ Tile decode_pair(int tile, const PSmem& s, int E, int
   Tile t;
   t.e = e;
   t.n = local / n_mt;
-  t.m0 = s.offs[e] + (local - t.n * n_mt) * P_BM;
+  t.m0 = s.offs[e] + (local - t.n * n_mt) * bm;
   t.m_end = s.offs[e + 1];
   return t;
 }
 
 // rows of the tile rounded up to the MMA's N granularity (16)
-__device__ __forceinline__ int tile_n(const Tile& t) {
-  const int rows = min(P_BM, t.m_end - t.m0);
+__device__ __forceinline__ int tile_n(const Tile& t, int bm) {
+  const int rows = min(bm, t.m_end - t.m0);
   return (rows + 15) & ~15;
 }
 
@@ -518,30 +475,32 @@ __device__ __forceinline__ bool epi_all(bool p) {
 // full 128-row box, since it is the row boxes, not the MMAs, that bound a
 // cut tile (an expert's last one).
 struct RowMaps {
-  CUtensorMap m[8];  // m[i]: box of 16 (i + 1) rows
+  CUtensorMap m[8];  // m[i]: box of 16 (i + 1) rows; single CTAs: m[0..3], 16 << i rows
 };
-
-// One cluster = one CTA pair.
-template <int MODE>
-__global__ void __launch_bounds__(PCfg<MODE>::THREADS, 1)
-    ffn_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapW0,
-                         const __grid_constant__ CUtensorMap mapW1,
-                         const __grid_constant__ RowMaps mapT, Args args) {
+// A single CTA's box for n rows (16 .. 128): the next power of two, so that a
+// launch prepares four maps (each costs about 0.1 us of the host's time).
+__device__ __forceinline__ int single_box(int n) { return n <= 16 ? 16 : 1 << (32 - __clz(n - 1)); }
+// PAIR: one cluster = one CTA pair. Otherwise a CTA alone computes the tile's
+// 128 weight rows by up to 128 permuted rows with cta_group::1 MMAs.
+template <int MODE, bool PAIR>
+__global__ void __launch_bounds__(PCfg<MODE, PAIR>::THREADS, 1)
+    ffn_gemm_kernel(const __grid_constant__ CUtensorMap mapW0,
+                    const __grid_constant__ CUtensorMap mapW1,
+                    const __grid_constant__ RowMaps mapT, Args args) {
+  using Cfg = PCfg<MODE, PAIR>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  constexpr int P_STAGES = PCfg<MODE>::STAGES;
-  uint8_t* epi = tiles + P_STAGES * P_STAGE_BYTES;
-  PSmem& s = *reinterpret_cast<PSmem*>(epi + PCfg<MODE>::EPI_BYTES);
+  uint8_t* epi = tiles + Cfg::STAGES * P_STAGE_BYTES;
+  PSmem& s = *reinterpret_cast<PSmem*>(epi + Cfg::EPI_BYTES);
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const int lane = tid & 31;
-  const uint32_t rank = cluster_ctarank();
-  const uint32_t rp = rank & 1u;     // rank within the pair
-  const uint32_t lead = 0;           // the pair's even CTA (MMA issuer)
+  const uint32_t rp = PAIR ? cluster_ctarank() & 1u : 0u;  // rank within the pair
+  const uint32_t lead = 0;                                  // the pair's even CTA (MMA issuer)
   const bool even = (rp == 0);
-  const int cluster = blockIdx.x / 2;
-  const int n_clusters = gridDim.x / 2;
+  const int cluster = PAIR ? blockIdx.x / 2 : blockIdx.x;
+  const int n_clusters = PAIR ? gridDim.x / 2 : gridDim.x;
   // launched with launch_pdl: barriers, TMEM and tensor-map prefetches are set
   // up while the previous kernel finishes; global memory only after pdl_wait
   pdl_trigger();
@@ -549,17 +508,17 @@ __global__ void __launch_bounds__(PCfg<MODE>::THREADS, 1)
     tma_prefetch_map(&mapW0);
     if (MODE == GATEUP) tma_prefetch_map(&mapW1);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) tma_prefetch_map(&mapT.m[i]);
+    for (int i = 0; i < (PAIR ? 8 : 4); ++i) tma_prefetch_map(&mapT.m[i]);
   }
 
   if (tid == 0) {
-    for (int i = 0; i < P_STAGES; ++i) {
+    for (int i = 0; i < Cfg::MAX_STAGES; ++i) {
       mbar_init(&s.full[i], 1);
       mbar_init(&s.empty[i], 1);  // one MMA commit of the pair
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&s.tfull[i], 1);
-      mbar_init(&s.tempty[i], 2 * PCfg<MODE>::EPI_WARPS);  // every epilogue warp of both CTAs
+      mbar_init(&s.tempty[i], (PAIR ? 2 : 1) * Cfg::EPI_WARPS);  // every epilogue warp (of both CTAs)
     }
     mbar_init(&s.drain, 1);
     s.abort = 0;
@@ -567,25 +526,38 @@ __global__ void __launch_bounds__(PCfg<MODE>::THREADS, 1)
     fence_mbar_init();
   }
   if (warp == 1) {
-    tmem_alloc_pair(&s.tmem_base, TMEM_COLS);
-    tmem_relinquish_pair();
+    if (PAIR) {
+      tmem_alloc_pair(&s.tmem_base, TMEM_COLS);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(&s.tmem_base, TMEM_COLS);
+      tmem_relinquish();
+    }
   }
   if (warp == 2) {
     pdl_wait();  // the offsets come from the permutation
-    load_row_tiles(s, args, P_BM, lane);
+    load_row_tiles(s, args, Cfg::ROWS, lane);
   }
   tc_fence_before();
-  cluster_sync();  // barriers of both CTAs initialised, TMEM allocated
+  if (PAIR) cluster_sync();  // barriers of both CTAs initialised, TMEM allocated
+  else __syncthreads();
   tc_fence_after();
   pdl_wait();  // every thread: the previous kernel's outputs are visible
   const uint32_t tmem_base = s.tmem_base;
+  // A single CTA's ring holds as many stages as its largest row tile leaves
+  // room for: it is bound by the weights' bytes, and the fewer the rows, the
+  // more of the weights are in flight. (Wide gate/up of 128 tokens, 8 experts,
+  // d 4096, d_ff 14336: 286 us with six stages of 128 rows, 273 with nine of
+  // 48; 64 experts, d 2048, d_ff 1408: 120.8 and 117.0 us.)
+  const int stage_bytes = PAIR ? P_STAGE_BYTES : P_W_BYTES + single_box(s.max_rows) * BK * 2;
+  const int n_stages = PAIR ? Cfg::STAGES : min(Cfg::MAX_STAGES, Cfg::STAGES * P_STAGE_BYTES / stage_bytes);
   const int total = s.mt_start[args.E] * args.n_tiles;
   const int kblocks = args.K / BK;
   volatile int* abort = &s.abort;
   uint32_t issued_mask = 0, last_phase_bits = 0;
   bool mma_issued = false;
   // tile -> (expert, column slice, row range)
-  auto tile_of = [&](int tile) { return decode_pair(tile, s, args.E, args.n_tiles); };
+  auto tile_of = [&](int tile) { return decode_pair(tile, s, args.E, args.n_tiles, Cfg::ROWS); };
 
   if (warp == 0) {
     if (lane == 0) {
@@ -593,33 +565,36 @@ __global__ void __launch_bounds__(PCfg<MODE>::THREADS, 1)
       uint32_t phase = 0;
       for (int tile = cluster; tile < total && !*abort; tile += n_clusters) {
         const Tile t = tile_of(tile);
-        const int trow = t.m0 + static_cast<int>(rp) * (tile_n(t) >> 1);  // N/2 rows per CTA
-        const int hb = ((tile_n(t) >> 1) + 15) & ~15;  // rows per CTA's box (16 .. 128)
-        const CUtensorMap* mrow = &mapT.m[(hb >> 4) - 1];
-        const uint32_t stage_tx = 2u * static_cast<uint32_t>(P_W_BYTES + hb * BK * 2);
-        const int wrow = (MODE == GATEUP)
-                             ? t.e * args.b_rows + t.n * 128 + 64 * static_cast<int>(rp)
-                             : t.e * args.b_rows + t.n * 256 + 128 * static_cast<int>(rp);
+        const int nr = tile_n(t, Cfg::ROWS) >> (PAIR ? 1 : 0);  // N/2 rows per CTA of a pair
+        const int trow = t.m0 + static_cast<int>(rp) * nr;
+        const int hb = PAIR ? (nr + 15) & ~15 : single_box(nr);  // rows per CTA's box (16 .. 128)
+        const CUtensorMap* mrow = &mapT.m[PAIR ? (hb >> 4) - 1 : 27 - __clz(hb)];
+        const uint32_t stage_tx = (PAIR ? 2u : 1u) * static_cast<uint32_t>(P_W_BYTES + hb * BK * 2);
+        // the CTA's rows of the weights: 64 of W1 and of W3, or 128 of W2
+        const int wrow = t.e * args.b_rows +
+                         (PAIR ? 2 * t.n + static_cast<int>(rp) : t.n) * (MODE == GATEUP ? 64 : 128);
         for (int kb = 0; kb < kblocks; ++kb) {
           if (!mbar_wait(&s.empty[stage], phase ^ 1u, args.limit_ns, abort)) {
             if (!*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 11);
             *abort = 1;
             break;
           }
-          uint8_t* sw = tiles + stage * P_STAGE_BYTES;
+          uint8_t* sw = tiles + stage * stage_bytes;
           uint8_t* st = sw + P_W_BYTES;
-          const uint32_t full_even = mapa_shared(smem_u32(&s.full[stage]), lead);
           if (even) mbar_arrive_expect_tx(&s.full[stage], stage_tx);
-          if (MODE == GATEUP) {
-            tma_load_2d_pair(sw, &mapW0, full_even, kb * BK, wrow);             // W1: lanes 0..63
-            tma_load_2d_pair(sw + P_W_BYTES / 2, &mapW1, full_even, kb * BK, wrow);  // W3: 64..127
+          if (PAIR) {
+            const uint32_t full_even = mapa_shared(smem_u32(&s.full[stage]), lead);
+            tma_load_2d_pair(sw, &mapW0, full_even, kb * BK, wrow);  // gate/up: W1, lanes 0..63
+            if (MODE == GATEUP) tma_load_2d_pair(sw + P_W_BYTES / 2, &mapW1, full_even, kb * BK, wrow);  // W3: 64..127
+            tma_load_2d_pair(st, mrow, full_even, kb * BK, trow);
           } else {
-            tma_load_2d_pair(sw, &mapW0, full_even, kb * BK, wrow);
+            tma_load_2d(sw, &mapW0, &s.full[stage], kb * BK, wrow);
+            if (MODE == GATEUP) tma_load_2d(sw + P_W_BYTES / 2, &mapW1, &s.full[stage], kb * BK, wrow);
+            tma_load_2d(st, mrow, &s.full[stage], kb * BK, trow);
           }
-          tma_load_2d_pair(st, mrow, full_even, kb * BK, trow);
           issued_mask |= 1u << stage;
           last_phase_bits = (last_phase_bits & ~(1u << stage)) | (phase << stage);
-          if (++stage == P_STAGES) { stage = 0; phase ^= 1u; }
+          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
       }
     }
@@ -638,7 +613,7 @@ __global__ void __launch_bounds__(PCfg<MODE>::THREADS, 1)
         }
         tc_fence_after();
         const Tile t = tile_of(tile);
-        const uint32_t idesc = idesc_bf16_f32(256, tile_n(t));
+        const uint32_t idesc = idesc_bf16_f32(PAIR ? 256 : 128, tile_n(t, Cfg::ROWS));
         const uint32_t d_tmem = tmem_base + slot * BN;
         bool ok = true;
         for (int kb = 0; kb < kblocks; ++kb) {
@@ -649,18 +624,24 @@ __global__ void __launch_bounds__(PCfg<MODE>::THREADS, 1)
             break;
           }
           tc_fence_after();
-          const uint32_t a0 = smem_u32(tiles + stage * P_STAGE_BYTES);
+          const uint32_t a0 = smem_u32(tiles + stage * stage_bytes);
           const uint32_t b0 = a0 + P_W_BYTES;
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk)
-            mma_bf16_pair(d_tmem, sdesc_kmajor_sw128(a0 + kk * 32),
-                          sdesc_kmajor_sw128(b0 + kk * 32), idesc, (kb | kk) != 0 ? 1u : 0u);
+            if (PAIR)
+              mma_bf16_pair(d_tmem, sdesc_kmajor_sw128(a0 + kk * 32),
+                            sdesc_kmajor_sw128(b0 + kk * 32), idesc, (kb | kk) != 0 ? 1u : 0u);
+            else
+              mma_bf16(d_tmem, sdesc_kmajor_sw128(a0 + kk * 32), sdesc_kmajor_sw128(b0 + kk * 32),
+                       idesc, (kb | kk) != 0 ? 1u : 0u);
           mma_issued = true;
-          mma_commit_pair(&s.empty[stage], 0x3);
-          if (++stage == P_STAGES) { stage = 0; phase ^= 1u; }
+          if (PAIR) mma_commit_pair(&s.empty[stage], 0x3);
+          else mma_commit(&s.empty[stage]);
+          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        mma_commit_pair(&s.tfull[slot], 0x3);
+        if (PAIR) mma_commit_pair(&s.tfull[slot], 0x3);
+        else mma_commit(&s.tfull[slot]);
       }
     }
   } else {
@@ -678,19 +659,19 @@ __global__ void __launch_bounds__(PCfg<MODE>::THREADS, 1)
       const int slot = it & 1;
       const uint32_t acc_phase = (it >> 1) & 1;
       const bool waited = (*abort == 0) && mbar_wait(&s.tfull[slot], acc_phase, args.limit_ns, abort);
-      if (!epi_all<PCfg<MODE>::EPI_WARPS * 32>(waited)) {  // the same decision in every epilogue warp
+      if (!epi_all<Cfg::EPI_WARPS * 32>(waited)) {  // the same decision in every epilogue warp
         if (!waited && lane == 0 && !*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 14);
         *abort = 1;
         break;
       }
       tc_fence_after();
       const Tile t = tile_of(tile);
-      const int rows = min(P_BM, t.m_end - t.m0);
+      const int rows = min(Cfg::ROWS, t.m_end - t.m0);
       const int nchunks = (rows + 31) >> 5;
       const uint32_t tb = tmem_base + slot * BN + (static_cast<uint32_t>(q * 32) << 16);
 #pragma unroll 1
-      for (int c = grp; c < nchunks; c += PCfg<MODE>::GROUPS) {
-        const int buf = (c / PCfg<MODE>::GROUPS) & 1;
+      for (int c = grp; c < nchunks; c += Cfg::GROUPS) {
+        const int buf = (c / Cfg::GROUPS) & 1;
         uint32_t v[32];
         tmem_ld32(tb + c * 32, v);  // TMEM column = row c*32 + i of the tile
         tmem_ld_wait();
@@ -716,16 +697,18 @@ __global__ void __launch_bounds__(PCfg<MODE>::THREADS, 1)
               const float oth = other[i + j];
               const float g = gate ? own : oth;
               const float u = gate ? oth : own;
-              // silu(g) u = g u / (1 + e^-g); the quotient by the fast reciprocal
-              // (2 ulp in fp32, far below the bf16 rounding of h)
-              h[j] = __fdividef(g * u, 1.0f + __expf(-g));
+              // silu(g) u = g u / (1 + e^-g); for full row tiles, whose epilogue
+              // the MMAs wait for, the quotient by the fast reciprocal (2 ulp in
+              // fp32, far below the bf16 rounding of h)
+              h[j] = PAIR && args.fast_div ? __fdividef(g * u, 1.0f + __expf(-g))
+                                           : g / (1.0f + __expf(-g)) * u;
             }
             const uint32_t pk = pack_bf16x2(h[0], h[1]);
             ob[(keep + i) * 64 + col] = static_cast<uint16_t>(pk & 0xFFFFu);
             ob[(keep + i + 1) * 64 + col] = static_cast<uint16_t>(pk >> 16);
           }
           epi_sync(grp);
-          uint16_t* gcol = args.out + t.n * 128 + 64 * static_cast<int>(rp) + (et & 7) * 8;
+          uint16_t* gcol = args.out + (PAIR ? 2 * t.n + static_cast<int>(rp) : t.n) * 64 + (et & 7) * 8;
 #pragma unroll
           for (int p = 0; p < 2; ++p) {
             const int r = p * 16 + (et >> 3);
@@ -744,7 +727,7 @@ __global__ void __launch_bounds__(PCfg<MODE>::THREADS, 1)
             yb[(i + 1) * 128 + col] = static_cast<uint16_t>(pk >> 16);
           }
           epi_sync(grp);
-          uint16_t* gcol = args.out + t.n * 256 + 128 * static_cast<int>(rp) + (et & 15) * 8;
+          uint16_t* gcol = args.out + (PAIR ? 2 * t.n + static_cast<int>(rp) : t.n) * 128 + (et & 15) * 8;
 #pragma unroll
           for (int p = 0; p < 4; ++p) {
             const int r = p * 8 + (et >> 4);
@@ -757,7 +740,10 @@ __global__ void __launch_bounds__(PCfg<MODE>::THREADS, 1)
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_remote(mapa_shared(smem_u32(&s.tempty[slot]), lead));
+      if (lane == 0) {
+        if (PAIR) mbar_arrive_remote(mapa_shared(smem_u32(&s.tempty[slot]), lead));
+        else mbar_arrive(&s.tempty[slot]);
+      }
     }
   }
 
@@ -765,19 +751,24 @@ __global__ void __launch_bounds__(PCfg<MODE>::THREADS, 1)
   if (s.abort) {
     volatile int* never = &s.zero;
     if (warp == 0 && lane == 0 && even) {
-      for (int st = 0; st < P_STAGES; ++st)
+      for (int st = 0; st < n_stages; ++st)
         if ((issued_mask >> st) & 1u)
           mbar_wait(&s.full[st], (last_phase_bits >> st) & 1u, args.limit_ns, never);
     }
     if (warp == 1 && lane == 0 && even && mma_issued) {
-      mma_commit_pair(&s.drain, static_cast<uint16_t>(1u << rank));
+      if (PAIR) mma_commit_pair(&s.drain, 0x1);
+      else mma_commit(&s.drain);
       mbar_wait(&s.drain, 0, args.limit_ns, never);
     }
   }
   tc_fence_before();
-  cluster_sync();  // every CTA finished: no more arrivals or copies into any
+  if (PAIR) cluster_sync();  // every CTA finished: no more arrivals or copies into any
+  else __syncthreads();
   tc_fence_after();
-  if (warp == 1) tmem_dealloc_pair(tmem_base, TMEM_COLS);
+  if (warp == 1) {
+    if (PAIR) tmem_dealloc_pair(tmem_base, TMEM_COLS);
+    else tmem_dealloc(tmem_base, TMEM_COLS);
+  }
 }
 
 // ------------------------------------------------------------------- host
@@ -822,41 +813,36 @@ int make_tmap_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t c
   return ORDERMOE_OK;
 }
 
-template <int MODE>
-static cudaError_t pair_attr() {
-  return cudaFuncSetAttribute(gg::ffn_gemm_pair_kernel<MODE>,
+template <int MODE, bool PAIR>
+static cudaError_t ffn_attr() {
+  return cudaFuncSetAttribute(gg::ffn_gemm_kernel<MODE, PAIR>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              gg::PCfg<MODE>::SMEM_BYTES);
+                              gg::PCfg<MODE, PAIR>::SMEM_BYTES);
 }
 
 static int ffn_attrs() {
   using namespace gg;
   static PerDevice cache;
   const cudaError_t attr_err = static_cast<cudaError_t>(per_device(cache, [] {
-    cudaError_t e = pair_attr<GATEUP>();
-    if (e == cudaSuccess) e = pair_attr<DOWN>();
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(ffn_gemm_kernel<GATEUP>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(ffn_gemm_kernel<DOWN>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    cudaError_t e = ffn_attr<GATEUP, true>();
+    if (e == cudaSuccess) e = ffn_attr<DOWN, true>();
+    if (e == cudaSuccess) e = ffn_attr<GATEUP, false>();
+    if (e == cudaSuccess) e = ffn_attr<DOWN, false>();
     return static_cast<int>(e);
   }));
-  if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(ffn_gemm_pair_kernel)");
+  if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(ffn_gemm_kernel)");
   return ORDERMOE_OK;
 }
 
-template <int MODE>
-static cudaLaunchConfig_t pair_config(int grid, int cl, cudaStream_t stream,
-                                      cudaLaunchAttribute* attr) {
+template <int MODE, bool PAIR>
+static cudaLaunchConfig_t ffn_config(int grid, cudaStream_t stream, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid, 1, 1);
-  cfg.blockDim = dim3(gg::PCfg<MODE>::THREADS, 1, 1);
-  cfg.dynamicSmemBytes = gg::PCfg<MODE>::SMEM_BYTES;
+  cfg.blockDim = dim3(gg::PCfg<MODE, PAIR>::THREADS, 1, 1);
+  cfg.dynamicSmemBytes = gg::PCfg<MODE, PAIR>::SMEM_BYTES;
   cfg.stream = stream;
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cl;
+  attr[0].val.clusterDim.x = PAIR ? 2 : 1;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // waits in the kernel
@@ -874,10 +860,10 @@ static int max_resident_clusters() {
   static PerDevice cache;
   return per_device(cache, [] {
     cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = pair_config<MODE>(2 * (num_sms() / 2), 2, nullptr, attr);
+    cudaLaunchConfig_t cfg = ffn_config<MODE, true>(2 * (num_sms() / 2), nullptr, attr);
     cfg.numAttrs = 1;  // the cluster shape alone decides residency
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gg::ffn_gemm_pair_kernel<MODE>, &cfg) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveClusters(&n, gg::ffn_gemm_kernel<MODE, true>, &cfg) != cudaSuccess ||
         n <= 0) {
       cudaGetLastError();
       n = num_sms() / 2;
@@ -886,40 +872,44 @@ static int max_resident_clusters() {
   });
 }
 
-// One launch of the CTA-pair kernel over `tiles` pair tiles.
-template <int MODE>
-static int launch_pair(const CUtensorMap& w0, const CUtensorMap& w1, const gg::RowMaps& t,
-                       const gg::Args& a, long long tiles, cudaStream_t stream, const char* what) {
-  const long long cmax = max_resident_clusters<MODE>();
-  const long long clusters = tiles < cmax ? tiles : cmax;
+// One launch over the row tiles of R permuted rows; a.n_tiles weight tiles
+// (of a pair, or of a CTA) per expert.
+template <int MODE, bool PAIR>
+static int launch_ffn(const CUtensorMap& w0, const CUtensorMap& w1, const gg::RowMaps& t,
+                      const gg::Args& a, int R, cudaStream_t stream, const char* what) {
+  constexpr int rows = gg::PCfg<MODE, PAIR>::ROWS;
+  const long long row_tiles = (long long)R / rows + (R < a.E ? R : a.E);  // at least as many as there are
+  const long long tiles = row_tiles * a.n_tiles;
+  const long long most = PAIR ? max_resident_clusters<MODE>() : num_sms();
+  const int units = static_cast<int>(tiles < most ? tiles : most);
   cudaLaunchAttribute attr[2];
-  cudaLaunchConfig_t cfg =
-      pair_config<MODE>(static_cast<int>(2 * (clusters > 0 ? clusters : 1)), 2, stream, attr);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, gg::ffn_gemm_pair_kernel<MODE>, w0, w1, t, a);
+  cudaLaunchConfig_t cfg = ffn_config<MODE, PAIR>(PAIR ? 2 * units : units, stream, attr);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, gg::ffn_gemm_kernel<MODE, PAIR>, w0, w1, t, a);
   if (e != cudaSuccess) return cuda_fail(e, what);
   OM_LAUNCHED(what);
   return ORDERMOE_OK;
 }
 
 // The row maps of a [rows][cols] bf16 tensor, boxes of 16 .. 128 rows.
-static int make_row_maps(gg::RowMaps* rm, const void* base, uint64_t rows, uint64_t cols) {
-  for (int i = 0; i < 8; ++i) {
-    const int rc = make_tmap_bf16(&rm->m[i], base, rows, cols, static_cast<uint32_t>(16 * (i + 1)));
+static int make_row_maps(gg::RowMaps* rm, const void* base, uint64_t rows, uint64_t cols, bool pairs) {
+  for (int i = 0; i < (pairs ? 8 : 4); ++i) {
+    const int rc = make_tmap_bf16(&rm->m[i], base, rows, cols,
+                                  static_cast<uint32_t>(pairs ? 16 * (i + 1) : 16 << i));
     if (rc) return rc;
   }
   return ORDERMOE_OK;
 }
 
-// Tile shape: CTA pairs (256 weight rows x up to 256 permuted rows) when experts average at least 256 rows; otherwise single
-// CTAs with 128-row tiles and the rows on the M side (a decode step: ~32 rows
-// per expert, where the weights are streamed once and the MMA shape hardly
-// matters).
-static bool use_pairs(int R, int E) { return (long long)R >= 256LL * E; }
-
-static int single_grid(long long tiles) {
-  const int sms = num_sms();
-  return static_cast<int>(tiles < sms ? tiles : sms);
-}
+// Tile shape: CTA pairs when experts average at least kPairRows rows, single
+// CTAs of up to 128 rows below, where an expert is one row tile and the
+// weights are read once. Measured, single against pairs (gate/up + down, us):
+// 64 experts, d 2048, d_ff 1408: 96 rows an expert on average (at most 122)
+// 128 + 67 against 133 + 69, 112 rows (139) 125 + 73 against 135 + 70, 131
+// rows (156) 157 + 85 against 136 + 72; 8 experts, d 4096, d_ff 14336: 107
+// rows (119) 287 + 155 against 302 + 161, 127 rows (142) 370 + 210 against
+// 305 + 162: the line is where the fuller experts pass 128 rows.
+constexpr int kPairRows = 112;
+static bool use_pairs(int R, int E) { return (long long)R >= (long long)kPairRows * E; }
 
 // H = SwiGLU(X_perm W1^T, X_perm W3^T) over the expert row ranges.
 int gate_up_launch(const uint16_t* X_perm, const int32_t* offsets, int R, const uint16_t* W1,
@@ -927,28 +917,18 @@ int gate_up_launch(const uint16_t* X_perm, const int32_t* offsets, int R, const 
   using namespace gg;
   int rc;
   if ((rc = ffn_attrs())) return rc;
+  const bool pairs = use_pairs(R, E);
   Args a{};
   a.offsets = offsets; a.rows = R; a.E = E; a.limit_ns = wait_limit_ns();
-  a.K = d; a.n_tiles = dff / 128; a.b_rows = dff; a.out = H; a.ldo = dff;
-  CUtensorMap mX, mW1, mW3;
-  if ((rc = make_map(&mX, X_perm, R, d))) return rc;
-  if (use_pairs(R, E)) {
-    // weights on the MMA's M side in 64-row boxes of W1 and W3
-    if ((rc = make_tmap_bf16(&mW1, W1, (uint64_t)E * dff, d, 64))) return rc;
-    if ((rc = make_tmap_bf16(&mW3, W3, (uint64_t)E * dff, d, 64))) return rc;
-    const long long row_tiles = (long long)(R + P_BM - 1) / P_BM + E;
-    gg::RowMaps rX;
-    if ((rc = make_row_maps(&rX, X_perm, R, d))) return rc;
-    return launch_pair<GATEUP>(mW1, mW3, rX, a, row_tiles * a.n_tiles, stream,
-                               "ffn_gemm_pair_kernel<gate_up>");
-  } else {
-    if ((rc = make_map(&mW1, W1, (uint64_t)E * dff, d))) return rc;
-    if ((rc = make_map(&mW3, W3, (uint64_t)E * dff, d))) return rc;
-    const long long tiles = ((long long)(R + BM - 1) / BM + E) * a.n_tiles;
-    OM_LAUNCH_PDL("ffn_gemm_kernel<gate_up>", ffn_gemm_kernel<GATEUP>, dim3(single_grid(tiles)),
-                  dim3(THREADS), SMEM_BYTES, stream, mX, mW1, mW3, a);
-  }
-  return ORDERMOE_OK;
+  a.K = d; a.n_tiles = dff / (pairs ? 128 : 64); a.b_rows = dff; a.out = H; a.ldo = dff;
+  a.fast_div = (long long)R >= (long long)P_BM * E;  // row tiles full on average
+  CUtensorMap mW1, mW3;
+  RowMaps mX;
+  if ((rc = make_tmap_bf16(&mW1, W1, (uint64_t)E * dff, d, 64))) return rc;
+  if ((rc = make_tmap_bf16(&mW3, W3, (uint64_t)E * dff, d, 64))) return rc;
+  if ((rc = make_row_maps(&mX, X_perm, R, d, pairs))) return rc;
+  return pairs ? launch_ffn<GATEUP, true>(mW1, mW3, mX, a, R, stream, "ffn_gemm_kernel<gate_up, pair>")
+               : launch_ffn<GATEUP, false>(mW1, mW3, mX, a, R, stream, "ffn_gemm_kernel<gate_up>");
 }
 
 // Y_perm = H W2^T over the expert row ranges.
@@ -957,24 +937,16 @@ int down_launch(const uint16_t* H, const int32_t* offsets, int R, const uint16_t
   using namespace gg;
   int rc;
   if ((rc = ffn_attrs())) return rc;
+  const bool pairs = use_pairs(R, E);
   Args a{};
   a.offsets = offsets; a.rows = R; a.E = E; a.limit_ns = wait_limit_ns();
-  a.K = dff; a.n_tiles = d / 256; a.b_rows = d; a.out = Y; a.ldo = d;
-  CUtensorMap mH, mW2;
-  if ((rc = make_map(&mW2, W2, (uint64_t)E * d, dff))) return rc;
-  if ((rc = make_map(&mH, H, R, dff))) return rc;
-  if (use_pairs(R, E)) {
-    const long long row_tiles = (long long)(R + P_BM - 1) / P_BM + E;
-    gg::RowMaps rH;
-    if ((rc = make_row_maps(&rH, H, R, dff))) return rc;
-    return launch_pair<DOWN>(mW2, mW2, rH, a, row_tiles * a.n_tiles, stream,
-                             "ffn_gemm_pair_kernel<down>");
-  } else {
-    const long long tiles = ((long long)(R + BM - 1) / BM + E) * a.n_tiles;
-    OM_LAUNCH_PDL("ffn_gemm_kernel<down>", ffn_gemm_kernel<DOWN>, dim3(single_grid(tiles)),
-                  dim3(THREADS), SMEM_BYTES, stream, mH, mW2, mW2, a);
-  }
-  return ORDERMOE_OK;
+  a.K = dff; a.n_tiles = d / (pairs ? 256 : 128); a.b_rows = d; a.out = Y; a.ldo = d;
+  CUtensorMap mW2;
+  RowMaps mH;
+  if ((rc = make_tmap_bf16(&mW2, W2, (uint64_t)E * d, dff, 128))) return rc;
+  if ((rc = make_row_maps(&mH, H, R, dff, pairs))) return rc;
+  return pairs ? launch_ffn<DOWN, true>(mW2, mW2, mH, a, R, stream, "ffn_gemm_kernel<down, pair>")
+               : launch_ffn<DOWN, false>(mW2, mW2, mH, a, R, stream, "ffn_gemm_kernel<down>");
 }
 
 int ffn_launch(const uint16_t* X_perm, const int32_t* offsets, int R, const uint16_t* W1,
@@ -992,7 +964,7 @@ int logits_gemm_launch(const uint16_t* X, int N, const uint16_t* W, int C, int d
   using namespace gg;
   static PerDevice cache;
   const cudaError_t attr_err = static_cast<cudaError_t>(per_device(cache, [] {
-    return static_cast<int>(cudaFuncSetAttribute(ffn_gemm_kernel<LOGITS>,
+    return static_cast<int>(cudaFuncSetAttribute(logits_gemm_kernel,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  SMEM_BYTES));
   }));
@@ -1015,8 +987,8 @@ int logits_gemm_launch(const uint16_t* X, int N, const uint16_t* W, int C, int d
   const long long tiles = (long long)((N + BM - 1) / BM) * a.n_tiles;
   const int sms = num_sms();
   const int grid = static_cast<int>(tiles < sms ? tiles : sms);
-  ffn_gemm_kernel<LOGITS><<<grid, THREADS, SMEM_BYTES, stream>>>(mX, mW, mW, a);
-  OM_LAUNCHED("ffn_gemm_kernel<logits>");
+  logits_gemm_kernel<<<grid, THREADS, SMEM_BYTES, stream>>>(mX, mW, a);
+  OM_LAUNCHED("logits_gemm_kernel");
   return ORDERMOE_OK;
 }
 

@@ -1675,6 +1675,12 @@ static int launch_select_lanes(const int32_t* topk_idx, int T, int E, int k, con
   return ORDERMOE_OK;
 }
 
+template <int NE>
+static cudaError_t router_attr() {
+  return cudaFuncSetAttribute(router_select_kernel<NE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              rt::smem_bytes<NE>(NE));
+}
+
 static int route_select_impl(const uint16_t* X, const uint16_t* W_r, const float* logits_in, int T,
                              int E, int d, int k, int renorm, const void* tables,
                              size_t tables_bytes_, Lookahead la, const uint8_t* home, uint8_t* loc,
@@ -1739,6 +1745,15 @@ static int route_select_impl(const uint16_t* X, const uint16_t* W_r, const float
   int split = 1;
   while (split * 2 <= smax && (long long)blocks * split * 2 <= num_sms() && split * 2 <= kblocks)
     split *= 2;
+  // once per device, for the most experts of each width (not at every launch)
+  static PerDevice attr_cache;
+  const cudaError_t ae = static_cast<cudaError_t>(per_device(attr_cache, [] {
+    cudaError_t e = router_attr<16>();
+    if (e == cudaSuccess) e = router_attr<32>();
+    if (e == cudaSuccess) e = router_attr<64>();
+    return static_cast<int>(e);
+  }));
+  if (ae != cudaSuccess) return cuda_fail(ae, "cudaFuncSetAttribute(router_select_kernel)");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(blocks * split, 1, 1);
   cfg.blockDim = dim3(rt::THREADS, 1, 1);
@@ -1756,8 +1771,6 @@ static int route_select_impl(const uint16_t* X, const uint16_t* W_r, const float
 #define OM_RT_LAUNCH(N)                                                                          \
   do {                                                                                           \
     cfg.dynamicSmemBytes = rt::smem_bytes<N>(E);                                                 \
-    cudaFuncSetAttribute(router_select_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                         (int)cfg.dynamicSmemBytes);                                             \
     le = cudaLaunchKernelEx(&cfg, router_select_kernel<N>, mX, mW, T, E, d, k, renorm, tb, home, \
                             loc, qhat, logits_out, topk_idx, topk_w, chosen_expert,              \
                             chosen_server, kind, counters, lim, split, la);                      \

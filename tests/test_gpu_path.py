@@ -271,6 +271,11 @@ def run_gpu_ffn(E, R, off, Xp, W1, W3, W2, d, dff):
     # and 256 columns of the transposed accumulator
     ([257, 384, 600, 300, 512, 1], 256, 512),
     ([129, 255, 256, 384], 512, 384),
+    # single CTAs (under 112 rows on average): 1-row to 16-row experts (a deep
+    # ring), 64 experts with empty ones, an expert of two row tiles; and either
+    # side of the line to pairs
+    ([1], 256, 128), ([15, 1, 16, 2], 256, 256), ([(7 * e) % 33 for e in range(64)], 256, 128),
+    ([0] * 60 + [130, 0, 17, 129], 512, 256), ([111, 112, 111], 256, 256), ([112, 112], 256, 128),
 ])
 def test_expert_ffn_matches_oracle(rows, d, dff):
     E, R, off, row_e, Xp, W1, W3, W2 = ffn_case(rows, d, dff, seed=sum(rows) + d)
