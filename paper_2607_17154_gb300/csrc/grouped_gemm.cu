@@ -352,11 +352,11 @@ __global__ void __launch_bounds__(THREADS, 1)
 // by the even CTA, a tile of 256 weight rows (the MMA's M side; 128 in each
 // CTA's shared memory and TMEM lanes) by up to 256 permuted rows of one expert
 // (the N side, split evenly between the two CTAs' shared memory). The weight
-// side is always full; an expert's last row tile is cut to the next multiple of
+// side is always full; an expert's rows are cut into even tiles of a multiple of
 // 16 rows (the N granularity of the instruction), so at most 15 padding rows
 // are computed per expert instead of up to 255 for a 256-row M tile. Each CTA
-// loads its rows as one 128-row TMA box (of which the MMA reads the first N/2):
-// a stage of 5-6 smaller boxes starved the tensor pipe.
+// loads its N/2 rows as one TMA box: a stage of 5-6 boxes starved the tensor
+// pipe.
 //   gate/up: CTA r holds W1_e rows f..f+63 (TMEM lanes 0..63) and the same
 //            rows of W3_e (lanes 64..127), f = 128 n + 64 r; the epilogue
 //            warps of the gate and up lanes exchange half of their values
@@ -426,7 +426,7 @@ struct PCfg {
   static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of the FFN kernels");
 };
 
-__device__ __forceinline__ Tile decode_pair(int tile, const PSmem& s, int E, int n_tiles, int bm) {
+__device__ __forceinline__ Tile decode_pair(int tile, const PSmem& s, int E, int n_tiles) {
   // the last expert whose first tile is <= tile (binary search: the row-tile
   // starts never decrease; empty experts share their successor's start)
   int e = 0, hi = E - 1;
@@ -440,16 +440,20 @@ __device__ __forceinline__ Tile decode_pair(int tile, const PSmem& s, int E, int
   Tile t;
   t.e = e;
   t.n = local / n_mt;
-  t.m0 = s.offs[e] + (local - t.n * n_mt) * bm;
-  t.m_end = s.offs[e + 1];
+  // an expert's rows in even shares: tiles of one expert take the same time, so
+  // the CTAs that share its weights stay at the same K and find them in L2.
+  // (Full tiles and a small last one: 2.47 and 2.23 GB of DRAM reads in the wide
+  // layer's gate/up and down, 4096 tokens x 8 experts, against 1.97 and 1.81.)
+  const int rows = s.offs[e + 1] - s.offs[e];
+  const int per = ((rows + n_mt - 1) / n_mt + 15) & ~15;  // <= bm, and (n_mt - 1) per < rows
+  const int first = (local - t.n * n_mt) * per;
+  t.m0 = s.offs[e] + first;
+  t.m_end = s.offs[e] + min(first + per, rows);
   return t;
 }
 
 // rows of the tile rounded up to the MMA's N granularity (16)
-__device__ __forceinline__ int tile_n(const Tile& t, int bm) {
-  const int rows = min(bm, t.m_end - t.m0);
-  return (rows + 15) & ~15;
-}
+__device__ __forceinline__ int tile_n(const Tile& t) { return (t.m_end - t.m0 + 15) & ~15; }
 
 // the 128 threads of epilogue group grp (named barriers 1 and 2)
 __device__ __forceinline__ void epi_sync(int grp) {
@@ -471,9 +475,8 @@ __device__ __forceinline__ bool epi_all(bool p) {
 }
 
 // Tensor maps of the permuted rows with boxes of 16, 32, ..., 128 rows: a
-// tile cut to N rows loads N/2 rows per CTA (rounded up to 16) instead of a
-// full 128-row box, since it is the row boxes, not the MMAs, that bound a
-// cut tile (an expert's last one).
+// tile of N rows loads N/2 rows per CTA (rounded up to 16) instead of a full
+// 128-row box.
 struct RowMaps {
   CUtensorMap m[8];  // m[i]: box of 16 (i + 1) rows; single CTAs: m[0..3], 16 << i rows
 };
@@ -556,31 +559,35 @@ __global__ void __launch_bounds__(PCfg<MODE, PAIR>::THREADS, 1)
   volatile int* abort = &s.abort;
   uint32_t issued_mask = 0, last_phase_bits = 0;
   bool mma_issued = false;
+  bool leader = false;  // the MMA warp's issuing lane
   // tile -> (expert, column slice, row range)
-  auto tile_of = [&](int tile) { return decode_pair(tile, s, args.E, args.n_tiles, Cfg::ROWS); };
+  auto tile_of = [&](int tile) { return decode_pair(tile, s, args.E, args.n_tiles); };
 
   if (warp == 0) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      for (int tile = cluster; tile < total && !*abort; tile += n_clusters) {
-        const Tile t = tile_of(tile);
-        const int nr = tile_n(t, Cfg::ROWS) >> (PAIR ? 1 : 0);  // N/2 rows per CTA of a pair
-        const int trow = t.m0 + static_cast<int>(rp) * nr;
-        const int hb = PAIR ? (nr + 15) & ~15 : single_box(nr);  // rows per CTA's box (16 .. 128)
-        const CUtensorMap* mrow = &mapT.m[PAIR ? (hb >> 4) - 1 : 27 - __clz(hb)];
-        const uint32_t stage_tx = (PAIR ? 2u : 1u) * static_cast<uint32_t>(P_W_BYTES + hb * BK * 2);
-        // the CTA's rows of the weights: 64 of W1 and of W3, or 128 of W2
-        const int wrow = t.e * args.b_rows +
-                         (PAIR ? 2 * t.n + static_cast<int>(rp) : t.n) * (MODE == GATEUP ? 64 : 128);
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(&s.empty[stage], phase ^ 1u, args.limit_ns, abort)) {
-            if (!*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 11);
-            *abort = 1;
-            break;
-          }
-          uint8_t* sw = tiles + stage * stage_bytes;
-          uint8_t* st = sw + P_W_BYTES;
+    const bool issuer = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    for (int tile = cluster; tile < total; tile += n_clusters) {
+      const Tile t = tile_of(tile);
+      const int nr = tile_n(t) >> (PAIR ? 1 : 0);  // N/2 rows per CTA of a pair
+      const int trow = t.m0 + static_cast<int>(rp) * nr;
+      const int hb = PAIR ? (nr + 15) & ~15 : single_box(nr);  // rows per CTA's box (16 .. 128)
+      const CUtensorMap* mrow = &mapT.m[PAIR ? (hb >> 4) - 1 : 27 - __clz(hb)];
+      const uint32_t stage_tx = (PAIR ? 2u : 1u) * static_cast<uint32_t>(P_W_BYTES + hb * BK * 2);
+      // the CTA's rows of the weights: 64 of W1 and of W3, or 128 of W2
+      const int wrow = t.e * args.b_rows +
+                       (PAIR ? 2 * t.n + static_cast<int>(rp) : t.n) * (MODE == GATEUP ? 64 : 128);
+      bool ok = true;
+      for (int kb = 0; kb < kblocks; ++kb) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&s.empty[stage], phase ^ 1u, args.limit_ns, abort))) {
+          if (issuer && !*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 11);
+          *abort = 1;
+          ok = false;
+          break;
+        }
+        uint8_t* sw = tiles + stage * stage_bytes;
+        uint8_t* st = sw + P_W_BYTES;
+        if (issuer) {
           if (even) mbar_arrive_expect_tx(&s.full[stage], stage_tx);
           if (PAIR) {
             const uint32_t full_even = mapa_shared(smem_u32(&s.full[stage]), lead);
@@ -592,56 +599,68 @@ __global__ void __launch_bounds__(PCfg<MODE, PAIR>::THREADS, 1)
             if (MODE == GATEUP) tma_load_2d(sw + P_W_BYTES / 2, &mapW1, &s.full[stage], kb * BK, wrow);
             tma_load_2d(st, mrow, &s.full[stage], kb * BK, trow);
           }
-          issued_mask |= 1u << stage;
-          last_phase_bits = (last_phase_bits & ~(1u << stage)) | (phase << stage);
-          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
+        issued_mask |= 1u << stage;
+        last_phase_bits = (last_phase_bits & ~(1u << stage)) | (phase << stage);
+        if (++stage == n_stages) { stage = 0; phase ^= 1u; }
       }
+      if (!ok) break;
     }
   } else if (warp == 1) {
-    if (lane == 0 && even) {
+    // The whole warp walks the stages, so that its control flow and the
+    // descriptors stay uniform, and one elected lane issues (the producer warp
+    // alike). A lane walking them alone held the issue back, whatever the tile:
+    // gate/up of 8192 tokens x 64 experts (top-6, d 2048, d_ff 1408) 372 -> 347
+    // us, down 197 -> 180; of 4096 x 8 (top-2, d 4096, d_ff 14336) gate/up 1144
+    // -> 1030 (ncu, with even row tiles); single CTAs' down of 1 token x 8 experts 65 -> 46, of 128 152 ->
+    // 146 us.
+    if (even) {
+      leader = elect_one();
+      const uint64_t desc0 = sdesc_kmajor_sw128(smem_u32(tiles));
       int stage = 0;
       uint32_t phase = 0;
       int it = 0;
-      for (int tile = cluster; tile < total && !*abort; tile += n_clusters, ++it) {
+      for (int tile = cluster; tile < total; tile += n_clusters, ++it) {
         const int slot = it & 1;
         const uint32_t acc_phase = (it >> 1) & 1;
-        if (!mbar_wait(&s.tempty[slot], acc_phase ^ 1u, args.limit_ns, abort)) {
-          if (!*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 12);
+        if (!__all_sync(0xffffffffu, mbar_wait(&s.tempty[slot], acc_phase ^ 1u, args.limit_ns, abort))) {
+          if (leader && !*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 12);
           *abort = 1;
           break;
         }
         tc_fence_after();
         const Tile t = tile_of(tile);
-        const uint32_t idesc = idesc_bf16_f32(PAIR ? 256 : 128, tile_n(t, Cfg::ROWS));
+        const uint32_t idesc = idesc_bf16_f32(PAIR ? 256 : 128, tile_n(t));
         const uint32_t d_tmem = tmem_base + slot * BN;
         bool ok = true;
         for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(&s.full[stage], phase, args.limit_ns, abort)) {
-            if (!*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 13);
+          if (!__all_sync(0xffffffffu, mbar_wait(&s.full[stage], phase, args.limit_ns, abort))) {
+            if (leader && !*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 13);
             *abort = 1;
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t a0 = smem_u32(tiles + stage * stage_bytes);
-          const uint32_t b0 = a0 + P_W_BYTES;
+          const uint64_t da = desc0 + static_cast<uint64_t>((stage * stage_bytes) >> 4);
+          const uint64_t db = da + (P_W_BYTES >> 4);
+          if (leader) {
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk)
-            if (PAIR)
-              mma_bf16_pair(d_tmem, sdesc_kmajor_sw128(a0 + kk * 32),
-                            sdesc_kmajor_sw128(b0 + kk * 32), idesc, (kb | kk) != 0 ? 1u : 0u);
-            else
-              mma_bf16(d_tmem, sdesc_kmajor_sw128(a0 + kk * 32), sdesc_kmajor_sw128(b0 + kk * 32),
-                       idesc, (kb | kk) != 0 ? 1u : 0u);
+            for (int kk = 0; kk < BK / 16; ++kk) {  // 16 elements = 32 bytes on
+              if (PAIR) mma_bf16_pair(d_tmem, da + 2 * kk, db + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+              else mma_bf16(d_tmem, da + 2 * kk, db + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
+            }
+            if (PAIR) mma_commit_pair(&s.empty[stage], 0x3);
+            else mma_commit(&s.empty[stage]);
+          }
           mma_issued = true;
-          if (PAIR) mma_commit_pair(&s.empty[stage], 0x3);
-          else mma_commit(&s.empty[stage]);
           if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        if (PAIR) mma_commit_pair(&s.tfull[slot], 0x3);
-        else mma_commit(&s.tfull[slot]);
+        if (leader) {
+          if (PAIR) mma_commit_pair(&s.tfull[slot], 0x3);
+          else mma_commit(&s.tfull[slot]);
+        }
+        __syncwarp();
       }
     }
   } else {
@@ -666,7 +685,7 @@ __global__ void __launch_bounds__(PCfg<MODE, PAIR>::THREADS, 1)
       }
       tc_fence_after();
       const Tile t = tile_of(tile);
-      const int rows = min(Cfg::ROWS, t.m_end - t.m0);
+      const int rows = t.m_end - t.m0;
       const int nchunks = (rows + 31) >> 5;
       const uint32_t tb = tmem_base + slot * BN + (static_cast<uint32_t>(q * 32) << 16);
 #pragma unroll 1
@@ -755,7 +774,7 @@ __global__ void __launch_bounds__(PCfg<MODE, PAIR>::THREADS, 1)
         if ((issued_mask >> st) & 1u)
           mbar_wait(&s.full[st], (last_phase_bits >> st) & 1u, args.limit_ns, never);
     }
-    if (warp == 1 && lane == 0 && even && mma_issued) {
+    if (leader && mma_issued) {  // the lane that issued the MMAs
       if (PAIR) mma_commit_pair(&s.drain, 0x1);
       else mma_commit(&s.drain);
       mbar_wait(&s.drain, 0, args.limit_ns, never);
