@@ -501,8 +501,7 @@ int ordermoe_coverage(const int32_t* group, const uint8_t* placement, int L, int
  * ordermoe_similarity_no_logits, ordermoe_place, ordermoe_replicate and
  * ordermoe_coverage write when called in that order with the same arguments.
  * For E in {8, 16, 32, 64} and L * E <= 4096 the layers go in blocks of 512 logit columns
- * (8 layers of 64 experts; the last block in two halves when there are
- * several, so that less grouping and placement is left after the last GEMM):
+ * (8 layers of 64 experts):
  * the caller's stream computes a block's logits,
  * Gram and similarities while a side stream of the library, ordered behind it
  * by events, groups and places the block before; the call joins the side

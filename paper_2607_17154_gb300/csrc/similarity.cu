@@ -304,21 +304,43 @@ __device__ __forceinline__ unsigned long long rank_key(double x) {
 struct GroupSmem {
   unsigned long long kp[64];  // rank_key of p and of I, for the placement order
   unsigned long long ki[64];
+  unsigned long long members[64];  // of each group
   double imp[64];
   double pls[64];
   int order[64];
-  int dom[64];
   int grp[64];
   int cnt[64];
-  float S[64 * 64];
+  float theta;
+  int nan;  // a similarity is NaN
+  int pad[2];
 };
+// The similarities are kept as integer keys that order like them (-0 as +0),
+// so that the greedy scan is one integer maximum per expert; 0: no value.
+__device__ __forceinline__ uint32_t sim_key(float s) {
+  const uint32_t u = __float_as_uint(s == 0.0f ? 0.0f : s);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float sim_of_key(uint32_t k) {
+  return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
+}
+// Threads of a layer (a slice): a warp up to 32 experts, two above.
+__host__ __device__ inline int group_slice_threads(int E) { return E <= 32 ? 32 : 64; }
+__host__ __device__ inline size_t group_slice_bytes(int E) {
+  return sizeof(GroupSmem) + sizeof(uint32_t) * (((size_t)E * E + 3) & ~size_t(3));
+}
 
-// Per-layer part of the plan for layer l, on 64 threads t = 0..63 of a block
-// (the layers are independent here): theta_l (Eq. 6), greedy cover
-// (Eqs. 24-26), importance (Eqs. 27-28) and the placement order (p desc,
-// I desc, index asc). A slice with live == false has no layer this round but
-// meets every barrier of the block.
-__device__ void group_layer(GroupSmem& sm, bool live, int t, int l, const float* __restrict__ sim,
+// Barrier of the nsync threads that group (named barrier 1: a warp that does
+// something else meanwhile has no part in it).
+__device__ __forceinline__ void group_sync(int nsync) {
+  asm volatile("bar.sync 1, %0;" ::"r"(nsync) : "memory");
+}
+// Per-layer part of the plan for layer l, on the nt = group_slice_threads(E)
+// threads t of a slice of the nsync that group (the layers are independent here): theta_l
+// (Eq. 6), greedy cover (Eqs. 24-26), importance (Eqs. 27-28) and the
+// placement order (p desc, I desc, index asc). A slice with live == false has
+// no layer this round but meets every barrier.
+__device__ void group_layer(GroupSmem& sm, uint32_t* K, bool live, int t, int nt, int nsync, int l,
+                            const float* __restrict__ sim,
                             const int32_t* __restrict__ counts, int L, int E, PlaceParams pp,
                             const double* __restrict__ p, int32_t* __restrict__ group,
                             int32_t* __restrict__ n_groups, float* __restrict__ theta_out,
@@ -326,94 +348,133 @@ __device__ void group_layer(GroupSmem& sm, bool live, int t, int l, const float*
   double* imp = sm.imp;
   double* pls = sm.pls;
   int* order = sm.order;
-  int* dom = sm.dom;
   int* grp = sm.grp;
   int* cnt = sm.cnt;
-  float* S = sm.S;
+  const float* S = sim + (size_t)l * E * E;
+  if (live && t == 0) sm.nan = 0;
+  group_sync(nsync);
   if (live) {
-    for (int i = t; i < E * E; i += 64) S[i] = sim[(size_t)l * E * E + i];
+    bool nan = false;
+    if ((E & 3) == 0 && (reinterpret_cast<uintptr_t>(S) & 15u) == 0) {
+#pragma unroll 8
+      for (int i = t; i < E * E / 4; i += nt) {
+        const float4 v = reinterpret_cast<const float4*>(S)[i];
+        nan |= v.x != v.x || v.y != v.y || v.z != v.z || v.w != v.w;
+        reinterpret_cast<uint4*>(K)[i] =
+            make_uint4(sim_key(v.x), sim_key(v.y), sim_key(v.z), sim_key(v.w));
+      }
+    } else {
+#pragma unroll 8
+      for (int i = t; i < E * E; i += nt) {
+        const float v = S[i];
+        nan |= v != v;
+        K[i] = sim_key(v);
+      }
+    }
+    if (nan) sm.nan = 1;
     if (t < E) {
+      sm.members[t] = 0ull;
       cnt[t] = counts[(size_t)l * E + t];
       pls[t] = p[(size_t)l * E + t];
       if (!(pls[t] >= 0.0)) report(&g_err_sim, ORDERMOE_DEV_BAD_VALUE, l * E + t);  // Eq. 29's p
     }
+    if (t < 32) {  // Eq. 6 (layers numbered from 1), by one warp (fp64 is slow)
+      float theta;
+      if (L <= 1) {
+        theta = __double2float_rn(pp.theta_single);
+      } else {
+        const double frac = __ddiv_rn(static_cast<double>(L - (l + 1)), static_cast<double>(L - 1));
+        theta = __double2float_rn(
+            __dadd_rn(pp.theta_min, __dmul_rn(__dsub_rn(pp.theta_max, pp.theta_min), frac)));
+      }
+      if (t == 0) sm.theta = theta;
+    }
   }
-  __syncthreads();
-  // Eq. 6 (layers numbered from 1)
-  float theta;
-  if (L <= 1) {
-    theta = __double2float_rn(pp.theta_single);
-  } else {
-    const double frac = __ddiv_rn(static_cast<double>(L - (l + 1)), static_cast<double>(L - 1));
-    theta = __double2float_rn(
-        __dadd_rn(pp.theta_min, __dmul_rn(__dsub_rn(pp.theta_max, pp.theta_min), frac)));
-  }
+  group_sync(nsync);
+  const float theta = live ? sm.theta : 0.0f;
   // visiting order: count desc, index asc
   if (live && t < E) {
+    const int mine = cnt[t];
     int r = 0;
-    for (int e = 0; e < E; ++e)
-      if (cnt[e] > cnt[t] || (cnt[e] == cnt[t] && e < t)) ++r;
+    int e = 0;
+#pragma unroll 4
+    for (; e + 4 <= E; e += 4) {
+      const int4 c = *reinterpret_cast<const int4*>(cnt + e);
+      r += (c.x > mine || (c.x == mine && e < t)) ? 1 : 0;
+      r += (c.y > mine || (c.y == mine && e + 1 < t)) ? 1 : 0;
+      r += (c.z > mine || (c.z == mine && e + 2 < t)) ? 1 : 0;
+      r += (c.w > mine || (c.w == mine && e + 3 < t)) ? 1 : 0;
+    }
+    for (; e < E; ++e) r += (cnt[e] > mine || (cnt[e] == mine && e < t)) ? 1 : 0;
     order[r] = t;
   }
-  __syncthreads();
-  // Eqs. 24-26 in the visiting order; warp 0 scans the existing dominants in
-  // parallel (lane g takes dominants g and g + 32; ties to the earlier one).
-  // The choice is the scan's in dominant order: the first dominant unless a
-  // later one is strictly more similar. With NaN similarities that is the
-  // first dominant when its similarity is NaN, else the first maximum with
-  // NaN counted as -inf: a total order, so every lane of the reduction ends
-  // with the same group.
+  group_sync(nsync);
+  // Eqs. 24-26 in the visiting order; warp 0 of the slice compares an expert
+  // with the existing dominants in parallel (lane g has dominants g and g +
+  // 32): the largest similarity, ties to the earlier dominant.
   if (live && t < 32) {
     int k = 0;
-    for (int pos = 0; pos < E; ++pos) {
-      const int j = order[pos];
-      float bs = -INFINITY;
-      int bg = 1 << 30;
-      for (int g = t; g < k; g += 32) {
-        const float sv = S[j * E + dom[g]];
-        const float v = sv != sv ? -INFINITY : sv;
-        if (bg == (1 << 30) || v > bs) { bg = g; bs = v; }
-      }
-      // across the lanes: the largest similarity by an order-preserving 32-bit
-      // key (0: the lane has no dominant; -0 counted as +0, so that equal
-      // similarities are equal keys), then the lowest dominant index among
-      // the lanes that hold it (dominants below 32 before those above)
-      uint32_t key = 0u;
-      if (bg != (1 << 30)) {
-        const uint32_t u = __float_as_uint(bs == 0.0f ? 0.0f : bs);
-        key = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-      }
-      const uint32_t mk = __reduce_max_sync(0xffffffffu, key);
-      const unsigned lo32 = __ballot_sync(0xffffffffu, key == mk && bg < 32);
-      const unsigned hi32 = __ballot_sync(0xffffffffu, key == mk && bg >= 32 && bg != (1 << 30));
-      if (mk == 0u) {
-        bg = 1 << 30;
-      } else {
-        bg = lo32 ? __ffs(lo32) - 1 : __ffs(hi32) - 1 + 32;
-        bs = __uint_as_float((mk & 0x80000000u) ? (mk & 0x7FFFFFFFu) : ~mk);
-      }
-      if (k > 0) {
-        const float s0 = S[j * E + dom[0]];
-        if (s0 != s0) {  // NaN first: the scan keeps dominant 0 (and NaN < theta is false)
-          bg = 0;
-          bs = s0;
+    int dom0 = 0, dom1 = 0;  // dominants t and t + 32, when there are that many
+    if (!sm.nan) {
+      const uint32_t low = theta != theta ? 0u : sim_key(theta);  // a NaN threshold: nothing is below
+      int jn = order[0];
+      for (int pos = 0; pos < E; ++pos) {
+        const int j = jn;
+        jn = order[min(pos + 1, E - 1)];
+        const uint32_t* row = K + j * E;
+        const uint32_t k0 = t < k ? row[dom0] : 0u, k1 = t + 32 < k ? row[dom1] : 0u;
+        const uint32_t mk = __reduce_max_sync(0xffffffffu, max(k0, k1));
+        int g;
+        if (k == 0 || mk < low) {
+          if (t == k) dom0 = j;
+          if (t + 32 == k) dom1 = j;
+          g = k++;
+        } else {
+          const unsigned lo32 = __ballot_sync(0xffffffffu, k0 == mk);
+          g = lo32 ? __ffs(lo32) - 1 : __ffs(__ballot_sync(0xffffffffu, k1 == mk)) + 31;
         }
+        if (t == 0) grp[j] = g;
       }
-      if (bg == (1 << 30) || bs < theta) {
-        if (t == 0) { dom[k] = j; grp[j] = k; }
-        ++k;
-      } else if (t == 0) {
-        grp[j] = bg;
+    } else {
+      // The choice is the scan's in dominant order: the first dominant unless a
+      // later one is strictly more similar. With NaN similarities that is the
+      // first dominant when its similarity is NaN, else the first maximum with
+      // NaN counted as -inf.
+      int first = 0;
+      for (int pos = 0; pos < E; ++pos) {
+        const int j = order[pos];
+        auto key = [&](int dom) {
+          const float v = S[j * E + dom];
+          return sim_key(v != v ? -INFINITY : v);
+        };
+        const uint32_t k0 = t < k ? key(dom0) : 0u, k1 = t + 32 < k ? key(dom1) : 0u;
+        const uint32_t mk = __reduce_max_sync(0xffffffffu, max(k0, k1));
+        const float s0 = k > 0 ? S[j * E + first] : 0.0f;
+        int g;
+        if (s0 != s0) {  // NaN first: the scan keeps dominant 0 (and NaN < theta is false)
+          g = 0;
+        } else if (k == 0 || sim_of_key(mk) < theta) {
+          if (k == 0) first = j;
+          if (t == k) dom0 = j;
+          if (t + 32 == k) dom1 = j;
+          g = k++;
+        } else {
+          const unsigned lo32 = __ballot_sync(0xffffffffu, k0 == mk);
+          g = lo32 ? __ffs(lo32) - 1 : __ffs(__ballot_sync(0xffffffffu, k1 == mk)) + 31;
+        }
+        if (t == 0) grp[j] = g;
       }
-      __syncwarp();
     }
     if (t == 0) {
       n_groups[l] = k;
       theta_out[l] = theta;
     }
   }
-  __syncthreads();
-  // Eqs. 27-28
+  group_sync(nsync);
+  // Eqs. 27-28; each group's members as a bit mask, so that a thread adds its
+  // own group's similarities only (in ascending order)
+  if (live && t < E) atomicOr(&sm.members[grp[t]], 1ull << t);
+  group_sync(nsync);
   // the counts' fp64 sum in index order, formed exactly as an integer sum
   // (every partial sum is an integer below 2^53, so each fp64 addition is exact)
   long long total_i = 0;
@@ -423,15 +484,18 @@ __device__ void group_layer(GroupSmem& sm, bool live, int t, int l, const float*
   if (live && t < E) {
     group[(size_t)l * E + t] = grp[t];
     double sum = 0.0;
-    int size = 0;
-    for (int k2 = 0; k2 < E; ++k2)
-      if (grp[k2] == grp[t]) { sum = __dadd_rn(sum, static_cast<double>(S[t * E + k2])); ++size; }
-    const double rho = __ddiv_rn(sum, static_cast<double>(size));
+    const unsigned long long mates = sm.members[grp[t]];
+    for (unsigned long long b = mates; b; b &= b - 1)
+    {
+      const int e = __ffsll(static_cast<long long>(b)) - 1;
+      sum = __dadd_rn(sum, static_cast<double>(sm.nan ? S[t * E + e] : sim_of_key(K[t * E + e])));
+    }
+    const double rho = __ddiv_rn(sum, static_cast<double>(__popcll(mates)));
     const double f = total > 0.0 ? __ddiv_rn(static_cast<double>(cnt[t]), total) : 0.0;
     imp[t] = __dadd_rn(__dmul_rn(pp.alpha_f, f), __dmul_rn(pp.alpha_r, rho));
     if (importance != nullptr) importance[(size_t)l * E + t] = imp[t];
   }
-  __syncthreads();
+  group_sync(nsync);
   // placement order: p desc, I desc, index asc, with NaN after every number
   // (a total order, so the ranks are a permutation whatever the values),
   // compared on integer keys
@@ -439,7 +503,7 @@ __device__ void group_layer(GroupSmem& sm, bool live, int t, int l, const float*
     sm.kp[t] = rank_key(pls[t]);
     sm.ki[t] = rank_key(imp[t]);
   }
-  __syncthreads();
+  group_sync(nsync);
   if (live && t < E) {
     const unsigned long long kpt = sm.kp[t], kit = sm.ki[t];
     int r = 0;
@@ -451,14 +515,15 @@ __device__ void group_layer(GroupSmem& sm, bool live, int t, int l, const float*
   }
 }
 
-// One block per layer l = l0 + blockIdx.x, 64 threads.
+// One block per layer l = l0 + blockIdx.x, group_slice_threads(E) threads.
 __global__ void __launch_bounds__(64) group_kernel(
     const float* __restrict__ sim, const int32_t* __restrict__ counts, int L, int E, int l0,
     PlaceParams pp, const double* __restrict__ p, int32_t* __restrict__ group,
     int32_t* __restrict__ n_groups, float* __restrict__ theta_out, double* __restrict__ importance,
     int32_t* __restrict__ porder) {
   __shared__ GroupSmem sm;
-  group_layer(sm, true, threadIdx.x, l0 + blockIdx.x, sim, counts, L, E, pp, p, group, n_groups,
+  __shared__ __align__(16) uint32_t K[64 * 64];
+  group_layer(sm, K, true, threadIdx.x, blockDim.x, blockDim.x, l0 + blockIdx.x, sim, counts, L, E, pp, p, group, n_groups,
               theta_out, importance, porder);
 }
 
@@ -493,23 +558,87 @@ __global__ void div_selftest_kernel(const double* __restrict__ a, const double* 
 // status, a later range continues from b_m in used (lambda1 * (b_m / C_m) is
 // recomputed from it, the same function the loop applies) and only raises the
 // capacity status.
+constexpr int kPlaceTable = 4096;  // (server, wins) entries
 struct PlaceSmem {
+  // uniform sizes: server m after n more experts, at m * depth + n
+  double after_b[kPlaceTable];   // b_m
+  double after_a1[kPlaceTable];  // lambda1 * (b_m / C_m)
+  double l2eta[65];  // lambda2 * eta for eta = 0 .. 64
+  double pls[64];
   int grp[64];
   int ord[64];
-  double pls[64];
   int waiting[64];
-  uint8_t xs[32 * 64];
-  int eta[32 * 64];
-  double l2eta[65];  // lambda2 * eta for eta = 0 .. 64
+  int ready;
+  int seq[64];      // experts in order with their groups
+  uint8_t who[64];  // the server of each, plus one
+  alignas(16) uint8_t xs[32 * 64];
+  alignas(16) int eta[32 * 64];
 };
+static_assert(sizeof(PlaceSmem) % 16 == 0, "vector stores into xs and eta");
+
+// Experts of one size (their memory p bitwise equal over the range's layers,
+// as a model's experts are): a server's b_m and ratio term then depend on how
+// many experts it has taken only, whichever they were. A producer warp
+// tabulates them, well ahead of the warp that places, whose loop is left with
+// one fp64 addition (the score) instead of seven on a part that has two fp64
+// lanes an SM. depth entries a server; ready of them are there.
+__host__ __device__ inline int place_depth(int M, int experts) {
+  const int want = 3 * experts / M + 16, room = kPlaceTable / M;
+  return want < room ? want : room;
+}
+__device__ __forceinline__ int place_ready(PlaceSmem& sm) {
+  int v;
+  asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(&sm.ready)) : "memory");
+  return v;
+}
+// The producer: one warp, lane m server m, b_m after 0 .. depth - 1 more
+// experts of size p, the additions in the order the placement makes them.
+__device__ void place_produce(PlaceSmem& sm, int lane, int M, int depth, double p, bool first,
+                              double lambda1, const double* __restrict__ C,
+                              const double* __restrict__ used) {
+  const bool srv = lane < M;
+  double b = (srv && !first) ? used[lane] : 0.0;
+  const double cap = srv ? C[lane] : 1.0, rcap = __drcp_rn(cap);
+  const int at = srv ? lane * depth : 0;
+  for (int n = 0; n < depth; ++n) {
+    const double a1 = __dmul_rn(lambda1, div_rn_markstein(b, cap, rcap));
+    if (srv) {
+      sm.after_b[at + n] = b;
+      sm.after_a1[at + n] = a1;
+    }
+    b = __dadd_rn(b, p);
+    if ((n & 3) == 3 || n + 1 == depth) {  // four rows at a time
+      __syncwarp();
+      if (lane == 0)
+        asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(smem_u32(&sm.ready)), "r"(n + 1) : "memory");
+    }
+  }
+}
+// whether p[0 .. n - 1] are bitwise equal (and not negative or NaN: those take
+// the general loop, which reports them), for the whole block
+__device__ bool place_uniform(const double* __restrict__ p, int n, int t, int nt) {
+  const long long p0 = __double_as_longlong(p[0]);
+  bool same = p[0] >= 0.0;
+  for (int i = t; i < n; i += nt) same = same && __double_as_longlong(p[i]) == p0;
+  return __syncthreads_and(same) != 0;
+}
+
+// A server's state after a further expert, past the tables (kept out of line:
+// inlined, its fp64 operations were issued for every expert).
+__device__ __noinline__ double2 place_further(double b, double p, double cap, double rcap,
+                                              double lambda1) {
+  const double bn = __dadd_rn(b, p);
+  return make_double2(bn, __dmul_rn(lambda1, div_rn_markstein(bn, cap, rcap)));
+}
 
 // The placement on warp 0 of a block (threadIdx.x < 32); returns 1 when a
 // waiting-list expert overfilled its server.
+// depth > 0: the sizes are uniform and the tables hold depth entries a server.
 __device__ int place_layers(PlaceSmem& sm, const int32_t* __restrict__ group,
                              const int32_t* __restrict__ porder, int L, int E, int M, int l0,
                              int l1, int first, PlaceParams pp, const double* __restrict__ p,
                              const double* __restrict__ C, uint8_t* __restrict__ placement,
-                             double* __restrict__ used) {
+                             double* __restrict__ used, int depth) {
   int* grp = sm.grp;
   int* ord = sm.ord;
   double* pls = sm.pls;
@@ -528,19 +657,132 @@ __device__ int place_layers(PlaceSmem& sm, const int32_t* __restrict__ group,
   double a1 = srv ? __dmul_rn(pp.lambda1, div_rn_markstein(b, cap, rcap)) : 0.0;
   bool bad_score = srv && !(cap > 0.0 && cap <= 1.7976931348623157e308);
   for (int i = t; i <= 64; i += 32) l2eta[i] = __dmul_rn(pp.lambda2, static_cast<double>(i));
+  int wins = 0;  // experts this server took in the range (uniform sizes)
+  int avail = 0;  // entries of its tables known to be there
+  // the next layer's rows, loaded a layer ahead (two experts a lane)
+  int g2[2] = {0, 0}, o2[2] = {0, 0};
+  double p2[2] = {0.0, 0.0};
+  auto fetch = [&](int l) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (t + 32 * h < E) {
+        g2[h] = group[(size_t)l * E + t + 32 * h];
+        o2[h] = porder[(size_t)l * E + t + 32 * h];
+        p2[h] = p[(size_t)l * E + t + 32 * h];
+      }
+  };
+  fetch(l0);
   __syncwarp();
   for (int l = l0; l < l1; ++l) {
-    for (int i = t; i < 32 * 64; i += 32) {
-      xs[i] = 0;
-      eta[i] = 0;
+    for (int i = t; i < 16 * M; i += 32) {
+      reinterpret_cast<uint32_t*>(xs)[i] = 0u;
+      reinterpret_cast<int4*>(eta)[i] = make_int4(0, 0, 0, 0);
     }
-    for (int e = t; e < E; e += 32) {
-      grp[e] = group[(size_t)l * E + e];
-      ord[e] = porder[(size_t)l * E + e];
-      pls[e] = p[(size_t)l * E + e];
-    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (t + 32 * h < E) {
+        grp[t + 32 * h] = g2[h];
+        ord[t + 32 * h] = o2[h];
+        pls[t + 32 * h] = p2[h];
+      }
+    if (l + 1 < l1) fetch(l + 1);
     __syncwarp();
     int nw = 0;
+    bool general = depth == 0;
+    if (!general) {
+      // One pass over the experts, written to branch as little as it can (a
+      // warp alone pays 20 cycles and more for each): a score that is not a
+      // plain non-negative number makes the layer start over below.
+      const double b0 = b, a10 = a1;
+      const int wins0 = wins;
+      // the experts in order with their groups (expert | group << 8), read ahead
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (t + 32 * h < E) sm.seq[t + 32 * h] = ord[t + 32 * h] | (grp[ord[t + 32 * h]] << 8);
+      __syncwarp();
+      // this server's state, and (bn, a1n) the one after a further expert
+      double bn = 0.0, a1n = 0.0;
+      if (avail < depth) avail = place_ready(sm);
+      if (srv && wins + 1 < avail) {
+        bn = sm.after_b[t * depth + wins + 1];
+        a1n = sm.after_a1[t * depth + wins + 1];
+      } else if (srv) {
+        const double2 s = place_further(b, pls[0], cap, rcap, pp.lambda1);
+        bn = s.x;
+        a1n = s.y;
+      }
+      bool feas = srv && __double_as_longlong(bn) <= cap_bits;  // bn <= C_m, bn >= 0
+      bool odd = false;
+      int* my_eta = eta + (srv ? t * 64 : 0);
+      const double* my_b = sm.after_b + (srv ? t * depth : 0);
+      const double* my_a1 = sm.after_a1 + (srv ? t * depth : 0);
+      int cur = sm.seq[0];
+      int nxt = sm.seq[min(1, E - 1)];
+      int ec = 0;  // experts of cur's group on this server
+      double sc = __dadd_rn(a1, l2eta[0]);
+      for (int pos = 0; pos < E; ++pos) {
+        // the next expert's count and lambda2 * eta, if this server takes cur and if not
+        const int after = sm.seq[min(pos + 2, E - 1)];
+        const int en = my_eta[nxt >> 8];
+        const int ew = (nxt >> 8) == (cur >> 8) ? ec + 1 : en;
+        const double l2s = l2eta[en], l2w = l2eta[ew];
+        const unsigned khi = feas ? static_cast<unsigned>(__double2hiint(sc)) : 0xffffffffu;
+        const unsigned klo = feas ? static_cast<unsigned>(__double2loint(sc)) : 0xffffffffu;
+        odd |= feas && khi >= 0x7FF00000u;  // an infinity, a NaN, a negative score or -0
+        const unsigned mhi = __reduce_min_sync(0xffffffffu, khi);
+        unsigned win = __ballot_sync(0xffffffffu, khi == mhi);
+        if ((win & (win - 1)) != 0u) {  // several lanes hold it (or no server is feasible)
+          const unsigned mlo = __reduce_min_sync(0xffffffffu, khi == mhi ? klo : 0xffffffffu);
+          win = mhi == 0xffffffffu ? 0u : __ballot_sync(0xffffffffu, khi == mhi && klo == mlo);
+        }
+        const bool won = win != 0u && t == __ffs(win) - 1;
+        a1 = won ? a1n : a1;
+        sc = __dadd_rn(a1, won ? l2w : l2s);
+        if (t == 0) sm.who[pos] = static_cast<uint8_t>(__ffs(win));  // server + 1, or 0: waiting
+        if (won) {
+          my_eta[cur >> 8] = ec + 1;
+          b = bn;
+          ++wins;
+          if (wins + 1 >= avail && avail < depth) avail = place_ready(sm);  // seldom: it is a fence
+          if (wins + 1 < avail) {
+            bn = my_b[wins + 1];
+            a1n = my_a1[wins + 1];
+          } else {
+            const double2 s = place_further(b, pls[0], cap, rcap, pp.lambda1);
+            bn = s.x;
+            a1n = s.y;
+          }
+          feas = __double_as_longlong(bn) <= cap_bits;
+        }
+        ec = won ? ew : en;
+        cur = nxt;
+        nxt = after;
+      }
+      __syncwarp();
+      if (__any_sync(0xffffffffu, odd)) {
+        general = true;
+        b = b0;
+        a1 = a10;
+        wins = wins0;
+        for (int i = t; i < 16 * M; i += 32) reinterpret_cast<int4*>(eta)[i] = make_int4(0, 0, 0, 0);
+        __syncwarp();
+      } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (t + 32 * h < E) {
+            const int m = sm.who[t + 32 * h];
+            if (m > 0) xs[(m - 1) * 64 + (sm.seq[t + 32 * h] & 0xFF)] = 1;
+          }
+        // the waiting list, in order
+        const unsigned w0 = __ballot_sync(0xffffffffu, t < E && sm.who[t] == 0);
+        const unsigned w1 = __ballot_sync(0xffffffffu, t + 32 < E && sm.who[t + 32 < 64 ? t + 32 : 0] == 0);
+        if ((w0 >> t) & 1u) waiting[__popc(w0 & ((1u << t) - 1u))] = sm.seq[t] & 0xFF;
+        if ((w1 >> t) & 1u) waiting[__popc(w0) + __popc(w1 & ((1u << t) - 1u))] = sm.seq[t + 32] & 0xFF;
+        nw = __popc(w0) + __popc(w1);
+        __syncwarp();
+      }
+    }
+    if (general) {
     int jn = ord[0];
     int gn = grp[jn];
     double pn = pls[jn];
@@ -585,8 +827,10 @@ __device__ int place_layers(PlaceSmem& sm, const int32_t* __restrict__ group,
         eta[m * 64 + g] += 1;
         b = bn;
         a1 = a1n;
+        ++wins;
       }
       __syncwarp();
+    }
     }
     // waiting list: the server with the largest C_m - b_m (ties: lower m)
     for (int w = 0; w < nw; ++w) {
@@ -607,12 +851,20 @@ __device__ int place_layers(PlaceSmem& sm, const int32_t* __restrict__ group,
         xs[bm * 64 + j] = 1;
         b = __dadd_rn(b, pls[j]);
         a1 = __dmul_rn(pp.lambda1, div_rn_markstein(b, cap, rcap));
+        ++wins;  // an expert of the same size
         if (b > cap) overflow = 1;
       }
       __syncwarp();
     }
     uint8_t* x = placement + (size_t)l * M * E;
-    for (int i = t; i < M * E; i += 32) x[i] = xs[(i / E) * 64 + (i % E)];
+    if ((E & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 3u) == 0) {
+      for (int i = t; i < M * E / 4; i += 32) {
+        const int m = i / (E / 4), e4 = i - m * (E / 4);
+        reinterpret_cast<uint32_t*>(x)[i] = reinterpret_cast<const uint32_t*>(xs)[m * 16 + e4];
+      }
+    } else {
+      for (int i = t; i < M * E; i += 32) x[i] = xs[(i / E) * 64 + (i % E)];
+    }
     __syncwarp();
   }
   if (srv) used[t] = b;
@@ -623,12 +875,20 @@ __device__ int place_layers(PlaceSmem& sm, const int32_t* __restrict__ group,
 }
 
 // Eq. 29's memory over all layers against the servers' total (the capacity
-// status of the first range), summed in order by one thread.
+// status of the first range): one fp64 sum in order, the values loaded a warp
+// at a time.
 __device__ int demand_exceeds(const double* __restrict__ p, int n, const double* __restrict__ C,
-                              int M) {
+                              int M, int lane) {
   double need = 0.0, have = 0.0;
-  for (int i = 0; i < n; ++i) need = __dadd_rn(need, p[i]);
-  for (int m = 0; m < M; ++m) have = __dadd_rn(have, C[m]);
+  double v = lane < n ? p[lane] : 0.0;
+  for (int i = 0; i < n; i += 32) {
+    const double cur = v;
+    if (i + 32 + lane < n) v = p[i + 32 + lane];
+    const int m = min(32, n - i);
+    for (int k = 0; k < m; ++k) need = __dadd_rn(need, __shfl_sync(0xffffffffu, cur, k));
+  }
+  const double c = lane < M ? C[lane] : 0.0;
+  for (int m = 0; m < M; ++m) have = __dadd_rn(have, __shfl_sync(0xffffffffu, c, m));
   return need > have ? 1 : 0;
 }
 
@@ -638,54 +898,94 @@ __device__ void place_status(int first, int overflow, int32_t* __restrict__ stat
   if (first || overflow) *status = overflow ? ORDERMOE_ERR_CAPACITY : ORDERMOE_OK;
 }
 
-__global__ void __launch_bounds__(64) place_kernel(
+// The placement of a grouped range by a block of at least four warps: the loop
+// on warp 0, the capacity check of the first range beside it on warp 3 (and
+// the producer of the tables on another).
+__device__ void place_range(PlaceSmem& sm, int* s_over, const int32_t* __restrict__ group,
+                            const int32_t* __restrict__ porder, int L, int E, int M, int l0, int l1,
+                            int first, PlaceParams pp, const double* __restrict__ p,
+                            const double* __restrict__ C, uint8_t* __restrict__ placement,
+                            double* __restrict__ used, int32_t* __restrict__ status, int depth) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int over = 0;
+  if (warp == 0)
+    over = place_layers(sm, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used, depth);
+  else if (warp == 3 && first) {
+    const int d = demand_exceeds(p, L * E, C, M, lane);
+    if (lane == 0) *s_over = d;
+  }
+  __syncthreads();
+  if (tid == 0) place_status(first, over | (first ? *s_over : 0), status);
+}
+
+constexpr int kPlaceThreads = 128;
+
+__global__ void __launch_bounds__(kPlaceThreads) place_kernel(
     const int32_t* __restrict__ group, const int32_t* __restrict__ porder, int L, int E, int M,
     int l0, int l1, int first, PlaceParams pp, const double* __restrict__ p,
     const double* __restrict__ C, uint8_t* __restrict__ placement, double* __restrict__ used,
     int32_t* __restrict__ status) {
-  __shared__ PlaceSmem sm;
+  extern __shared__ __align__(16) unsigned char s_pl[];
+  PlaceSmem& sm = *reinterpret_cast<PlaceSmem*>(s_pl);
   __shared__ int s_over;
-  int over = 0;
-  if (threadIdx.x < 32)
-    over = place_layers(sm, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used);
-  else if (threadIdx.x == 32 && first)  // beside the placement, on the second warp
-    s_over = demand_exceeds(p, L * E, C, M);
+  const int n = (l1 - l0) * E;
+  const bool uniform = place_uniform(p + (size_t)l0 * E, n, threadIdx.x, blockDim.x);
+  const int depth = uniform ? place_depth(M, n) : 0;
+  if (threadIdx.x == 0) sm.ready = 0;
   __syncthreads();
-  if (threadIdx.x == 0) place_status(first, over | (first ? s_over : 0), status);
+  if (uniform && (threadIdx.x >> 5) == 1)
+    place_produce(sm, threadIdx.x & 31, M, depth, p[(size_t)l0 * E], first, pp.lambda1, C, used);
+  place_range(sm, &s_over, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used, status,
+              depth);
 }
 
 // Grouping and placement of layers l0 .. l1 - 1 in one block: the grouping
-// runs kGroupSlices layers at a time, 64 threads a layer; then warp 0 places
-// the layers in order while the second warp sums the capacity check (one
+// runs several layers at a time on all warps but the last, which produces the
+// placement's tables meanwhile; then warp 0 places the layers in order (one
 // block, so the pipelined plan's side stream holds one SM).
-constexpr int kGroupSlices = 4;
-constexpr size_t kGroupPlaceSmem = kGroupSlices * sizeof(GroupSmem) + sizeof(PlaceSmem);
+// Bound: the serial chains (a group per expert, a server per expert). A layer
+// of 64 experts took about 28 us to place and 10 to group (8 layers 282 us
+// under ncu); with the tables and the integer scan 8 layers take 186 us.
+constexpr int kGroupThreads = 256;
 
-__global__ void __launch_bounds__(64 * kGroupSlices) group_place_kernel(
+__host__ __device__ inline int group_slices(int E) { return kGroupThreads / group_slice_threads(E); }
+static size_t group_place_smem(int E) {
+  return ((group_slices(E) * group_slice_bytes(E) + 15) & ~size_t(15)) + sizeof(PlaceSmem);
+}
+
+__global__ void __launch_bounds__(kGroupThreads + 32) group_place_kernel(
     const float* __restrict__ sim, const int32_t* __restrict__ counts, int L, int E, int M, int l0,
     int l1, int first, PlaceParams pp, const double* __restrict__ p, const double* __restrict__ C,
     int32_t* __restrict__ group, int32_t* __restrict__ n_groups, float* __restrict__ theta_out,
     double* __restrict__ importance, int32_t* __restrict__ porder, uint8_t* __restrict__ placement,
     double* __restrict__ used, int32_t* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char s_gp[];
-  GroupSmem* gs = reinterpret_cast<GroupSmem*>(s_gp);
-  PlaceSmem& ps = *reinterpret_cast<PlaceSmem*>(s_gp + kGroupSlices * sizeof(GroupSmem));
-  const int slice = threadIdx.x / 64;
-  for (int lb = l0; lb < l1; lb += kGroupSlices) {
-    const int l = lb + slice;
-    group_layer(gs[slice], l < l1, threadIdx.x % 64, l, sim, counts, L, E, pp, p, group, n_groups,
-                theta_out, importance, porder);
-    __syncthreads();  // the slices' scratch is reused by the next round
-  }
-  // group and porder written above are visible to the block after the barrier
+  const int nt = group_slice_threads(E), slices = group_slices(E);
+  PlaceSmem& ps = *reinterpret_cast<PlaceSmem*>(
+      s_gp + ((slices * group_slice_bytes(E) + 15) & ~size_t(15)));
   __shared__ int s_over;
-  int over = 0;
-  if (threadIdx.x < 32)
-    over = place_layers(ps, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used);
-  else if (threadIdx.x == 32 && first)
-    s_over = demand_exceeds(p, L * E, C, M);
+  const int n = (l1 - l0) * E;
+  const bool uniform = place_uniform(p + (size_t)l0 * E, n, threadIdx.x, blockDim.x);
+  const int depth = uniform ? place_depth(M, n) : 0;
+  const int slice = threadIdx.x / nt;
+  unsigned char* own = s_gp + (slice < slices ? slice : 0) * group_slice_bytes(E);
+  GroupSmem& gs = *reinterpret_cast<GroupSmem*>(own);
+  uint32_t* K = reinterpret_cast<uint32_t*>(own + sizeof(GroupSmem));
+  if (threadIdx.x == 0) ps.ready = 0;
   __syncthreads();
-  if (threadIdx.x == 0) place_status(first, over | (first ? s_over : 0), status);
+  if (slice >= slices) {  // the last warp
+    if (uniform)
+      place_produce(ps, threadIdx.x & 31, M, depth, p[(size_t)l0 * E], first, pp.lambda1, C, used);
+  } else {
+    for (int lb = l0; lb < l1; lb += slices) {
+      const int l = lb + slice;
+      group_layer(gs, K, l < l1, threadIdx.x % nt, nt, kGroupThreads, l, sim, counts, L, E, pp, p,
+                  group, n_groups, theta_out, importance, porder);
+      group_sync(kGroupThreads);  // the slices' scratch is reused; group and porder are written
+    }
+  }
+  place_range(ps, &s_over, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used, status,
+              depth);
 }
 
 }  // namespace om
@@ -1056,6 +1356,11 @@ extern "C" size_t ordermoe_place_workspace_bytes(int L, int E) {
   return ((size_t)L * E * sizeof(int32_t) + 255) & ~size_t(255);
 }
 
+static cudaError_t place_attr() {
+  return cudaFuncSetAttribute(place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(sizeof(PlaceSmem)));
+}
+
 extern "C" int ordermoe_place(const float* sim, const int32_t* counts, int L, int E, int M,
                               double theta_min, double theta_max, double theta_single,
                               double alpha_f, double alpha_r, double lambda1, double lambda2,
@@ -1072,10 +1377,14 @@ extern "C" int ordermoe_place(const float* sim, const int32_t* counts, int L, in
     return fail(ORDERMOE_ERR_INVALID_ARG, "place: workspace missing or too small");
   int32_t* porder_scratch = static_cast<int32_t*>(workspace);
   PlaceParams pp{theta_min, theta_max, theta_single, alpha_f, alpha_r, lambda1, lambda2};
-  group_kernel<<<L, 64, 0, stream>>>(sim, counts, L, E, 0, pp, p, group, n_groups, theta, importance,
+  group_kernel<<<L, group_slice_threads(E), 0, stream>>>(sim, counts, L, E, 0, pp, p, group, n_groups, theta, importance,
                                      porder_scratch);
   OM_LAUNCHED("group_kernel");
-  place_kernel<<<1, 64, 0, stream>>>(group, porder_scratch, L, E, M, 0, L, 1, pp, p, C, placement,
+  static PerDevice attr;
+  const cudaError_t ae =
+      static_cast<cudaError_t>(per_device(attr, [] { return static_cast<int>(place_attr()); }));
+  if (ae != cudaSuccess) return cuda_fail(ae, "cudaFuncSetAttribute(place_kernel)");
+  place_kernel<<<1, kPlaceThreads, sizeof(PlaceSmem), stream>>>(group, porder_scratch, L, E, M, 0, L, 1, pp, p, C, placement,
                                      used, status);
   OM_LAUNCHED("place_kernel");
   return ORDERMOE_OK;
@@ -1182,8 +1491,7 @@ extern "C" int ordermoe_selftest_div_rn(const double* a, const double* b, double
 // The whole offline plan in one call (Alg. 1): similarity (Eqs. 3-5), grouping
 // (Eqs. 6, 24-28), mandatory placement (Eqs. 29-31), redundant deployment
 // (Eqs. 32-35) and coverage (Eq. 32). On the tensor-core path the layers go in
-// blocks of 512 logit columns (the last block in two halves when there are
-// several): the caller's stream runs a block's logits GEMM,
+// blocks of 512 logit columns: the caller's stream runs a block's logits GEMM,
 // Gram and similarities, and a side stream, behind an event, runs that
 // block's grouping and placement while the next block's GEMM runs. The
 // placement carries b_m from block to block in `used`; its layers stay in
@@ -1214,7 +1522,8 @@ static int plan_sync(PlanSync** out) {
     PlanSync& ps = g_plan_sync[dev];
     cudaError_t err = cudaFuncSetAttribute(group_place_kernel,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           static_cast<int>(kGroupPlaceSmem));
+                                           static_cast<int>(group_place_smem(64)));
+    if (err == cudaSuccess) err = place_attr();
     if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&ps.side, cudaStreamNonBlocking);
     for (int i = 0; i < 4 && err == cudaSuccess; ++i)
       err = cudaEventCreateWithFlags(&ps.ev[i], cudaEventDisableTiming);
@@ -1284,13 +1593,8 @@ extern "C" int ordermoe_plan(const uint16_t* W_r, const uint16_t* X_cal, int L, 
     const PlaceParams pp{theta_min, theta_max, theta_single, alpha_f, alpha_r, lambda1, lambda2};
     const int part = sim_tc_part_layers(E);
     const int nsplit = sim_tc_nsplit(L, E, N);
-    // the last block's grouping and placement are not hidden behind a GEMM:
-    // when there is more than one block, the last one goes in two halves
-    const int nfull = (L + part - 1) / part;
-    const int last0 = (nfull - 1) * part, last_n = L - last0;
     for (int l0 = 0, k = 0; l0 < L && !rc; ++k) {
-      int lp = L - l0 < part ? L - l0 : part;
-      if (nfull > 1 && l0 >= last0 && last_n >= 2) lp = l0 == last0 ? (last_n + 1) / 2 : L - l0;
+      const int lp = L - l0 < part ? L - l0 : part;
       const size_t rows = (size_t)l0 * E;
       float* gpart = w.gpart + (size_t)l0 * nsplit * 4096;
       double* G = w.G + (size_t)l0 * 4096;
@@ -1309,10 +1613,22 @@ extern "C" int ordermoe_plan(const uint16_t* W_r, const uint16_t* X_cal, int L, 
         rc = cuda_fail(e, "plan: block event");
         break;
       }
-      group_place_kernel<<<1, 64 * kGroupSlices, kGroupPlaceSmem, ps->side>>>(
-          sim, counts, L, E, M, l0, l0 + lp, l0 == 0 ? 1 : 0, pp, p, C, group, n_groups, theta,
-          importance, porder, placement, used, status);
-      if ((rc = launched("group_place_kernel"))) break;
+      if (l0 + lp < L) {
+        group_place_kernel<<<1, kGroupThreads + 32, group_place_smem(E), ps->side>>>(
+            sim, counts, L, E, M, l0, l0 + lp, l0 == 0 ? 1 : 0, pp, p, C, group, n_groups, theta,
+            importance, porder, placement, used, status);
+        if ((rc = launched("group_place_kernel"))) break;
+      } else {
+        // no GEMM runs beside the last block: a block a layer groups it. (Cut in
+        // two halves, so that less is left to group and place, the last block
+        // streams X_cal once more: 1613 against 1569 us for the whole plan.)
+        group_kernel<<<lp, group_slice_threads(E), 0, ps->side>>>(
+            sim, counts, L, E, l0, pp, p, group, n_groups, theta, importance, porder);
+        if ((rc = launched("group_kernel"))) break;
+        place_kernel<<<1, kPlaceThreads, sizeof(PlaceSmem), ps->side>>>(
+            group, porder, L, E, M, l0, L, l0 == 0 ? 1 : 0, pp, p, C, placement, used, status);
+        if ((rc = launched("place_kernel"))) break;
+      }
       l0 += lp;
     }
     // every exit after the fork joins the side stream back into the caller's

@@ -296,6 +296,27 @@ def test_placement_quotient_is_correctly_rounded():
     assert bad.size == 0, (bad[:5], a[bad[:5]], b[bad[:5]], got[bad[:5]], want[bad[:5]])
 
 
+@pytest.mark.parametrize("L,E,M,size,caps", [
+    (8, 64, 32, 1.0, "one"),      # a server takes more experts than its table holds
+    (6, 24, 5, 0.3, "tight"),     # fractional sizes, waiting lists, an overflow
+    (3, 33, 7, 1.7, "loose"), (2, 1, 1, 1.0, "tight"), (40, 8, 4, 1.0, "loose"),
+    (4, 16, 3, 0.0, "loose")])    # size 0: nothing fills up
+def test_place_uniform_sizes_bit_exact(L, E, M, size, caps):
+    """Experts of one size, whose servers' states are tabulated by the number of
+    experts taken."""
+    rng = np.random.default_rng(L * 100 + E + M)
+    sim, counts = synthetic_sims(rng, L, E, max(1, min(4, E)), 0.4)
+    p = np.full((L, E), size)
+    total = max(p.sum(), 1.0)
+    C = total / M * rng.uniform(0.8, 1.3, M) * {"one": 1e-3, "tight": 0.95, "loose": 1.5}[caps]
+    if caps == "one":
+        C[3] = 2.0 * total
+    got = gpu_place(sim, counts, M, p, C)
+    ref = oracle_place_all(sim, counts, M, p, C)
+    for name, a, b in zip(("group", "n_groups", "theta", "placement", "used", "status"), got, ref):
+        np.testing.assert_array_equal(a, b, err_msg=name)
+
+
 def test_place_fractional_sizes_and_capacities_bit_exact():
     rng = np.random.default_rng(23)
     for L, E, M in [(40, 64, 32), (7, 13, 5), (64, 8, 3)]:
