@@ -224,13 +224,8 @@ __global__ void transitions_finish_kernel(const int32_t* __restrict__ counts, in
     P[(size_t)r * E + b] = row > 0.0 ? __double2float_rn(__ddiv_rn(static_cast<double>(c[b]), row)) : 0.0f;
 }
 
-// grid (L, 16), 256 threads: block (l, b) reduces the 256 Gram entries
-// i * 64 + j in [256 b, 256 b + 256) over the chunks, in chunk order (fp64).
-__global__ void __launch_bounds__(256) gram_reduce_kernel(const float* __restrict__ gpart,
-                                                          int nchunks, double* __restrict__ G) {
-  const int l = blockIdx.x;
-  const int x = blockIdx.y * 256 + threadIdx.x;
-  const float* src = gpart + (size_t)l * nchunks * 4096 + x;
+// The partial Grams of an entry summed over the chunks, in chunk order (fp64).
+__device__ __forceinline__ double gram_entry(const float* __restrict__ src, int nchunks) {
   double s = 0.0;
   int c = 0;
   for (; c + 8 <= nchunks; c += 8) {
@@ -241,28 +236,34 @@ __global__ void __launch_bounds__(256) gram_reduce_kernel(const float* __restric
     for (int u = 0; u < 8; ++u) s += static_cast<double>(v[u]);
   }
   for (; c < nchunks; ++c) s += static_cast<double>(src[(size_t)c * 4096]);
-  G[(size_t)l * 4096 + x] = s;
+  return s;
 }
 
-// grid (L, 16): Sim(i,j) = G_ij / (sqrt(G_ii) sqrt(G_jj)) (Eq. 4), diagonal 1,
-// zero-norm 0; block y takes entries 256 y .. 256 y + 255 of layer l (the fp64
-// square roots and divides of a layer spread over 16 SMs).
-__global__ void __launch_bounds__(256) sim_finish_kernel(const double* __restrict__ Gall, int E,
-                                                         float* __restrict__ sim) {
+// Sim(i,j) = G_ij / (sqrt(G_ii) sqrt(G_jj)) (Eq. 4), diagonal 1, zero-norm 0.
+// grid (L, parts), 256 threads; block (l, b) takes the layer's entries 256 b ..
+// 256 b + 255 of the E x E that there are, and first the norms it needs (all E:
+// a quarter more sums than its own at E = 64). Bound by the fp64 additions, one
+// in 19 cycles an SM. Reduction and quotients as two launches over 64 x 64
+// entries whatever E took 24.8 + 4.0 us for 32 layers of 8 experts (37 chunks),
+// 6.5 + 4.3 for 8 of 64 (75 chunks); this takes 8.3 and 10.6.
+__global__ void __launch_bounds__(256) gram_sim_kernel(const float* __restrict__ gpart, int nchunks,
+                                                       int E, float* __restrict__ sim) {
   __shared__ double norm[64];
   const int l = blockIdx.x;
-  const double* G = Gall + (size_t)l * 4096;
-  if (threadIdx.x < E) norm[threadIdx.x] = sqrt(G[threadIdx.x * 64 + threadIdx.x]);
-  __syncthreads();
+  const float* G = gpart + (size_t)l * nchunks * 4096;
   const int x = blockIdx.y * 256 + threadIdx.x;
+  const int i = x / E, j = x - i * E;
+  // the last warps take the norms, so that a block's own sums run beside them
+  const int d = 255 - static_cast<int>(threadIdx.x);
+  if (d < E) norm[d] = sqrt(gram_entry(G + d * 65, nchunks));
+  const bool mine = x < E * E && i != j;
+  const double g = mine ? gram_entry(G + i * 64 + j, nchunks) : 0.0;
+  __syncthreads();
   if (x >= E * E) return;
-  const int i = x / E, j = x % E;
-  float v;
-  if (i == j) {
-    v = 1.0f;
-  } else {
+  float v = 1.0f;
+  if (mine) {
     const double ni = norm[i], nj = norm[j];
-    v = (ni == 0.0 || nj == 0.0) ? 0.0f : __double2float_rn(G[i * 64 + j] / (ni * nj));
+    v = (ni == 0.0 || nj == 0.0) ? 0.0f : __double2float_rn(g / (ni * nj));
   }
   sim[(size_t)l * E * E + x] = v;
 }
@@ -1056,7 +1057,6 @@ struct SimLayout {
   uint16_t* hi;
   uint16_t* lo;
   float* gpart;
-  double* G;
   int64_t ldT;
   int nchunks;
   bool tc;
@@ -1074,8 +1074,6 @@ static SimLayout similarity_layout(void* workspace, int L, int E, int64_t N, boo
   w.hi = reinterpret_cast<uint16_t*>(ws + (with_H ? up((size_t)N * L * E * sizeof(float)) : 0));
   w.lo = reinterpret_cast<uint16_t*>(reinterpret_cast<uint8_t*>(w.hi) + plane);
   w.gpart = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(w.hi) + (w.tc ? 2 * plane : 0));
-  w.G = reinterpret_cast<double*>(reinterpret_cast<uint8_t*>(w.gpart) +
-                                  up((size_t)L * sim_parts(L, E, N) * 64 * 64 * sizeof(float)));
   return w;
 }
 
@@ -1092,7 +1090,6 @@ static int similarity_impl(const uint16_t* W_r, const uint16_t* X_cal, int L, in
   uint16_t* hi = w.hi;
   uint16_t* lo = w.lo;
   float* gpart = w.gpart;
-  double* G = w.G;
   const bool tc = w.tc;
   const int64_t ldT = w.ldT;
   const int nchunks = w.nchunks;
@@ -1104,10 +1101,8 @@ static int similarity_impl(const uint16_t* W_r, const uint16_t* X_cal, int L, in
                            keep_logits ? H : nullptr, hi, lo, static_cast<int>(ldT), counts, gpart,
                            nsplit, false, stream);
     if (rc) return rc;
-    gram_reduce_kernel<<<dim3(L, 16), 256, 0, stream>>>(gpart, nsplit, G);
-    OM_LAUNCHED("gram_reduce_kernel");
-    sim_finish_kernel<<<dim3(L, 16), 256, 0, stream>>>(G, E, sim);
-    OM_LAUNCHED("sim_finish_kernel");
+    gram_sim_kernel<<<dim3(L, (E * E + 255) / 256), 256, 0, stream>>>(gpart, nsplit, E, sim);
+    OM_LAUNCHED("gram_sim_kernel");
     return ORDERMOE_OK;
   }
   int rc = logits_gemm_launch(X_cal, static_cast<int>(N), W_r, L * E, d, H, stream);
@@ -1123,10 +1118,8 @@ static int similarity_impl(const uint16_t* W_r, const uint16_t* X_cal, int L, in
   OM_LAUNCHED("counts_kernel");
   gram_kernel<<<dim3(L, nchunks), 256, 0, stream>>>(H, N, L, E, gpart);
   OM_LAUNCHED("gram_kernel");
-  gram_reduce_kernel<<<dim3(L, 16), 256, 0, stream>>>(gpart, nchunks, G);
-  OM_LAUNCHED("gram_reduce_kernel");
-  sim_finish_kernel<<<dim3(L, 16), 256, 0, stream>>>(G, E, sim);
-  OM_LAUNCHED("sim_finish_kernel");
+  gram_sim_kernel<<<dim3(L, (E * E + 255) / 256), 256, 0, stream>>>(gpart, nchunks, E, sim);
+  OM_LAUNCHED("gram_sim_kernel");
   return ORDERMOE_OK;
 }
 
@@ -1597,15 +1590,12 @@ extern "C" int ordermoe_plan(const uint16_t* W_r, const uint16_t* X_cal, int L, 
       const int lp = L - l0 < part ? L - l0 : part;
       const size_t rows = (size_t)l0 * E;
       float* gpart = w.gpart + (size_t)l0 * nsplit * 4096;
-      double* G = w.G + (size_t)l0 * 4096;
       rc = sim_tc_launch(X_cal, static_cast<int>(N), W_r + rows * d, lp, E, d, k_freq, nullptr,
                          w.hi + rows * w.ldT, w.lo + rows * w.ldT, static_cast<int>(w.ldT),
                          counts + rows, gpart, nsplit, true, S);
       if (rc) break;
-      gram_reduce_kernel<<<dim3(lp, 16), 256, 0, S>>>(gpart, nsplit, G);
-      if ((rc = launched("gram_reduce_kernel"))) break;
-      sim_finish_kernel<<<dim3(lp, 16), 256, 0, S>>>(G, E, sim + rows * E);
-      if ((rc = launched("sim_finish_kernel"))) break;
+      gram_sim_kernel<<<dim3(lp, (E * E + 255) / 256), 256, 0, S>>>(gpart, nsplit, E, sim + rows * E);
+      if ((rc = launched("gram_sim_kernel"))) break;
       cudaEvent_t ev = ps->ev[1 + (k & 1)];
       cudaError_t e = cudaEventRecord(ev, S);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(ps->side, ev, 0);
