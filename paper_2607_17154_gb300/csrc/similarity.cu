@@ -25,57 +25,58 @@ int read_clear_err_sim(unsigned long long* out) {
 constexpr int kSimChunk = 1024;  // calibration tokens per partial Gram
 constexpr int kSub = 64;         // tokens staged in shared memory at a time
 
-// Rank order used for top-k: larger logit first, equal logits by lower index.
-__device__ __forceinline__ void add_topk_counts(const float* l, int E, int kf, int* counts) {
-  unsigned long long used = 0;
-  for (int j = 0; j < kf; ++j) {
-    int best = -1;
-    float bv = 0.0f;
-    for (int e = 0; e < E; ++e) {
-      if ((used >> e) & 1ull) continue;
-      if (best < 0 || l[e] > bv) { best = e; bv = l[e]; }
-    }
-    used |= 1ull << best;
-    atomicAdd(&counts[best], 1);
-  }
-}
-
-// grid (chunks, L), 256 threads. Partial Gram of layer l over one chunk of
-// tokens: thread (ti, tj) of a 16 x 16 grid accumulates the 4 x 4 block
-// G[4 ti .. 4 ti + 3][4 tj .. 4 tj + 3] in fp32; each staged token costs two
-// float4 shared loads per 16 FMAs.
+// grid (L, chunks), 256 threads. Partial Gram of layer l over one chunk of
+// tokens in 8 x 4 blocks of experts G[8 ti .. 8 ti + 7][4 tj .. 4 tj + 3], one a
+// thread in fp32 (each staged token costs three float4 shared loads per 32 FMAs:
+// the loads bound it). The ceil(E / 8) ceil(E / 4) blocks leave threads over, so
+// copies of them take every copies-th token (40 experts: 50 blocks, five
+// copies), and the copies are added in order. 4 x 4 blocks without copies, 100
+// of 256 threads at work, took 55.9 us for 32768 tokens, 8 layers of 40 experts,
+// this 31.7.
 __global__ void __launch_bounds__(256) gram_kernel(const float* __restrict__ H, int64_t N, int L,
                                                    int E, float* __restrict__ gpart) {
   __shared__ __align__(16) float sh[kSub][64];
+  __shared__ float part[256 * 17];  // the copies' blocks (pitch 17: no bank conflicts)
   // the layers of one chunk are neighbouring blocks, so each token's record
   // of L * E logits is read from DRAM once and shared through L2
   const int l = blockIdx.x, chunk = blockIdx.y;
   const int nchunks = gridDim.y;
   const int tid = threadIdx.x;
-  const int ti = tid >> 4, tj = tid & 15;
+  const int side = (E + 3) >> 2, nblk = ((E + 7) >> 3) * side;
+  const int copies = 256 / nblk;  // >= 2: at most 8 x 16 blocks
+  const int copy = tid / nblk, blk = tid - copy * nblk;
+  const int ti = blk / side, tj = blk - ti * side;
+  const bool active = copy < copies;
   const int LE = L * E;
-  float acc[4][4];
+  float acc[8][4];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 8; ++a)
 #pragma unroll
     for (int b = 0; b < 4; ++b) acc[a][b] = 0.0f;
   const int64_t n_begin = (int64_t)chunk * kSimChunk;
   int64_t n_end = n_begin + kSimChunk;
   if (n_end > N) n_end = N;
-  const bool active = 4 * ti < E && 4 * tj < E;
+  // the next kSub tokens are loaded into registers while these are multiplied
+  const bool vec = (E & 3) == 0 && (LE & 3) == 0;
+  float4 ahead[4];
+  auto fetch = [&](int64_t n0) {  // 16 float4 per token row, 4 of the 1024 a thread
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int x = tid + 256 * u;
+      const int c4 = (x & 15) * 4;
+      const int64_t n = n0 + (x >> 4);
+      ahead[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (n < n_end && c4 < E) ahead[u] = *reinterpret_cast<const float4*>(H + n * LE + (int64_t)l * E + c4);
+    }
+  };
+  if (vec) fetch(n_begin);
   for (int64_t n0 = n_begin; n0 < n_end; n0 += kSub) {
     __syncthreads();
-    if ((E & 3) == 0 && (LE & 3) == 0) {
-      // 16 float4 per token row; each thread stages 4 of the 1024 float4
+    if (vec) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int x = tid + 256 * u;
-        const int r = x >> 4, c4 = (x & 15) * 4;
-        const int64_t n = n0 + r;
-        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (n < n_end && c4 < E)
-          v = *reinterpret_cast<const float4*>(H + n * LE + (int64_t)l * E + c4);
-        *reinterpret_cast<float4*>(&sh[r][c4]) = v;
+        *reinterpret_cast<float4*>(&sh[x >> 4][(x & 15) * 4]) = ahead[u];
       }
     } else {
       for (int x = tid; x < kSub * 64; x += 256) {
@@ -85,10 +86,12 @@ __global__ void __launch_bounds__(256) gram_kernel(const float* __restrict__ H, 
       }
     }
     __syncthreads();
+    if (vec && n0 + kSub < n_end) fetch(n0 + kSub);
     if (active) {
 #pragma unroll 4
-      for (int r = 0; r < kSub; ++r) {
-        const float4 a = *reinterpret_cast<const float4*>(&sh[r][4 * ti]);
+      for (int r = copy; r < kSub; r += copies) {
+        const float4 a = *reinterpret_cast<const float4*>(&sh[r][8 * ti]);
+        const float4 d = *reinterpret_cast<const float4*>(&sh[r][8 * ti + 4]);
         const float4 b = *reinterpret_cast<const float4*>(&sh[r][4 * tj]);
 #define OM_GRAM_ROW(p, ap)                       \
   acc[p][0] = fmaf(ap, b.x, acc[p][0]);          \
@@ -96,132 +99,240 @@ __global__ void __launch_bounds__(256) gram_kernel(const float* __restrict__ H, 
   acc[p][2] = fmaf(ap, b.z, acc[p][2]);          \
   acc[p][3] = fmaf(ap, b.w, acc[p][3]);
         OM_GRAM_ROW(0, a.x) OM_GRAM_ROW(1, a.y) OM_GRAM_ROW(2, a.z) OM_GRAM_ROW(3, a.w)
+        OM_GRAM_ROW(4, d.x) OM_GRAM_ROW(5, d.y) OM_GRAM_ROW(6, d.z) OM_GRAM_ROW(7, d.w)
 #undef OM_GRAM_ROW
       }
     }
   }
   float* gp = gpart + ((size_t)l * nchunks + chunk) * 64 * 64;
-  if (active)
 #pragma unroll
-    for (int p = 0; p < 4; ++p)
+  for (int h = 0; h < 2; ++h) {  // the blocks' upper and lower four rows in turn
+    __syncthreads();
 #pragma unroll
-      for (int q = 0; q < 4; ++q) gp[(4 * ti + p) * 64 + 4 * tj + q] = acc[p][q];
+    for (int x = 0; x < 16; ++x) part[tid * 17 + x] = acc[4 * h + (x >> 2)][x & 3];
+    __syncthreads();
+    for (int x = tid; x < nblk * 16; x += 256) {
+      const int k = x >> 4, e = x & 15;  // block and entry
+      float s = part[k * 17 + e];
+      for (int c = 1; c < copies; ++c) s += part[(c * nblk + k) * 17 + e];
+      gp[(8 * (k / side) + 4 * h + (e >> 2)) * 64 + 4 * (k % side) + (e & 3)] = s;
+    }
+  }
 }
 
-// Eq. 5 counts from the token-major logits H[n][l E + e]: one thread per
-// (token, layer) holds the layer's E logits in registers and takes k_freq
-// passes (larger logit first, lower index on ties). Block totals are added
-// with integer atomics, so the result does not depend on the order.
-template <int EMAX>
-__global__ void __launch_bounds__(256) counts_kernel(const float* __restrict__ H, int64_t N, int L,
-                                                     int E, int kf, int32_t* __restrict__ counts) {
+// Top-kf experts of a token's E logits as a bit set (rank order: larger first,
+// lower index on ties). KN > 0: a descending min/max network keeps the KN >= kf
+// largest values with multiplicity, T is the kf-th of them, every logit >= T is
+// taken, and where equal logits straddle the boundary the surplus equal to T
+// goes back from the highest index down. KN = 0 (kf > 8), or a NaN among the
+// logits: kf passes, each taking the first unused maximum.
+template <int KN>
+__device__ __forceinline__ unsigned long long topk_set(const float* row, int E, int kf) {
+  unsigned long long used = 0;
+  if constexpr (KN > 0) {
+    float v[KN];
+#pragma unroll
+    for (int p = 0; p < KN; ++p) v[p] = -INFINITY;
+    bool nan = false;
+#pragma unroll 8
+    for (int e = 0; e < E; ++e) {
+      const float c = row[e];
+      nan |= c != c;
+#pragma unroll
+      for (int p = KN - 1; p >= 1; --p) v[p] = fminf(v[p - 1], fmaxf(v[p], c));
+      v[0] = fmaxf(v[0], c);
+    }
+    if (!nan) {
+      float T = v[0];
+#pragma unroll
+      for (int p = 1; p < KN; ++p) T = p < kf ? fminf(T, v[p]) : T;
+      uint32_t m[2] = {0u, 0u};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int n = min(32, E - 32 * h);
+#pragma unroll 8
+        for (int e = 0; e < n; ++e) m[h] |= row[32 * h + e] >= T ? 1u << e : 0u;
+      }
+      used = (static_cast<unsigned long long>(m[1]) << 32) | m[0];
+      int extra = __popcll(used) - kf;
+      for (int e = E - 1; extra > 0; --e)
+        if (((used >> e) & 1ull) && row[e] == T) {
+          used &= ~(1ull << e);
+          --extra;
+        }
+      return used;
+    }
+  }
+  for (int j = 0; j < kf; ++j) {
+    int best = -1;
+    float bv = 0.0f;
+    for (int e = 0; e < E; ++e) {
+      if ((used >> e) & 1ull) continue;
+      const float c = row[e];
+      if (best < 0 || c > bv) {
+        best = e;
+        bv = c;
+      }
+    }
+    used |= 1ull << best;
+  }
+  return used;
+}
+
+// The logits of a tile of kTopkTokens tokens at one layer, through shared memory
+// (rows of E floats in global memory, read coalesced; an odd pitch, so that a
+// thread a token reads its row without bank conflicts). Every thread of the
+// block calls it; rows past n_end are left as they are.
+constexpr int kTopkTokens = 256;
+constexpr int kTransTiles = 8;  // tiles of a transitions block, at most
+__host__ __device__ inline int topk_pitch(int E) { return E | 1; }
+__device__ __forceinline__ void load_logit_tile(float* s, const float* __restrict__ logits, int64_t n0,
+                                                int64_t n_end, int E, int64_t sn) {
+  const int rows = static_cast<int>(n_end - n0 < kTopkTokens ? n_end - n0 : kTopkTokens);
+  const int pitch = topk_pitch(E);
+  const float* src = logits + n0 * sn;
+  if (((E | sn) & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15u) == 0) {
+    const int q = E >> 2;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < rows * q; i += kTopkTokens) {
+      const int r = i / q, c = (i - r * q) * 4;
+      const float4 v = *reinterpret_cast<const float4*>(src + r * sn + c);
+      float* d = s + r * pitch + c;
+      d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+    }
+  } else {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < rows * E; i += kTopkTokens) {
+      const int r = i / E, c = i - r * E;
+      s[r * pitch + c] = src[r * sn + c];
+    }
+  }
+}
+
+// Eq. 5 counts of layer l = blockIdx.x: logits of token n at layer l start at
+// n * sn + l * sl (floats). Block totals are added with integer atomics, so the
+// result does not depend on the order. Bound by the loads and the top-k's
+// instructions; a thread reading its own row from global memory took 42 us for
+// 32768 tokens, 8 layers of 40 experts (top-4), this 22.2.
+template <int KN>
+__global__ void __launch_bounds__(kTopkTokens) counts_kernel(const float* __restrict__ logits,
+                                                             int64_t N, int E, int kf, int64_t sn,
+                                                             int64_t sl, int32_t* __restrict__ counts) {
+  extern __shared__ float s_tile[];
   __shared__ int cnt[64];
   const int l = blockIdx.x;  // layers of the same tokens run side by side (L2 reuse)
   if (threadIdx.x < 64) cnt[threadIdx.x] = 0;
-  __syncthreads();
-  const int LE = L * E;
-  const bool vec = (E & 3) == 0 && (LE & 3) == 0;
-  for (int64_t n = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; n < N;
-       n += (int64_t)gridDim.y * blockDim.x) {
-    const float* row = H + n * LE + (int64_t)l * E;
-    float v[EMAX];
-    if (vec) {
-#pragma unroll
-      for (int e = 0; e < EMAX; e += 4) {
-        if (e < E) {
-          const float4 q = *reinterpret_cast<const float4*>(row + e);
-          v[e] = q.x; v[e + 1] = q.y; v[e + 2] = q.z; v[e + 3] = q.w;
-        }
-      }
-    } else {
-#pragma unroll
-      for (int e = 0; e < EMAX; ++e)
-        if (e < E) v[e] = row[e];
-    }
-    unsigned long long used = 0;
-    for (int j = 0; j < kf; ++j) {
-      int best = -1;
-      float bv = 0.0f;
-#pragma unroll
-      for (int e = 0; e < EMAX; ++e) {
-        if (e < E && !((used >> e) & 1ull) && (best < 0 || v[e] > bv)) {
-          best = e;
-          bv = v[e];
-        }
-      }
-      used |= 1ull << best;
-      atomicAdd(&cnt[best], 1);
+  for (int64_t n0 = (int64_t)blockIdx.y * kTopkTokens; n0 < N; n0 += (int64_t)gridDim.y * kTopkTokens) {
+    __syncthreads();
+    load_logit_tile(s_tile, logits + l * sl, n0, N, E, sn);
+    __syncthreads();
+    if (n0 + threadIdx.x < N) {
+      const float* row = s_tile + threadIdx.x * topk_pitch(E);
+      for (unsigned long long b = topk_set<KN>(row, E, kf); b; b &= b - 1)
+        atomicAdd(&cnt[__ffsll(static_cast<long long>(b)) - 1], 1);
     }
   }
   __syncthreads();
   if (threadIdx.x < E && cnt[threadIdx.x]) atomicAdd(&counts[(size_t)l * E + threadIdx.x], cnt[threadIdx.x]);
 }
 
-// Top-kf of one token's E logits (rank order: larger first, lower index on
-// ties) as a bit set.
-template <int EMAX>
-__device__ __forceinline__ unsigned long long topk_set(const float* __restrict__ row, int E, int kf) {
-  float v[EMAX];
-#pragma unroll
-  for (int e = 0; e < EMAX; ++e) v[e] = (e < E) ? row[e] : 0.0f;
-  unsigned long long used = 0;
-  for (int j = 0; j < kf; ++j) {
-    int best = -1;
-    float bv = 0.0f;
-#pragma unroll
-    for (int e = 0; e < EMAX; ++e)
-      if (e < E && !((used >> e) & 1ull) && (best < 0 || v[e] > bv)) {
-        best = e;
-        bv = v[e];
+// Transition counts of Eq. 41 for the layer pairs (l, l + 1), l in [per *
+// blockIdx.y, + per): each token adds one to n_l(k -> k') for every k in its
+// top-kf at layer l and k' in its top-kf at layer l + 1 (integer atomics:
+// order-independent). A block walks the layers of its tokens and keeps each
+// layer's sets for the next, so that a row is read and ranked once (twice at a
+// range's ends); logits of token n at layer l start at n * sn + l * sl. Ranked
+// per pair, with a thread reading its own rows, it took 101 us for 32768 tokens,
+// 8 layers of 40 experts (top-4), this 33.2.
+template <int KN>
+__global__ void __launch_bounds__(kTopkTokens) transitions_kernel(const float* __restrict__ logits,
+                                                                  int64_t N, int L, int E, int kf,
+                                                                  int64_t sn, int64_t sl, int per,
+                                                                  int tiles,
+                                                                  int32_t* __restrict__ counts) {
+  extern __shared__ float s_tile[];  // the tile, then E * E counts
+  __shared__ unsigned long long s_prev[kTransTiles][kTopkTokens];  // each thread's own
+  int* h = reinterpret_cast<int*>(s_tile + kTopkTokens * topk_pitch(E));
+  const int l0 = blockIdx.y * per, l1 = min(l0 + per, L - 1);  // pairs l0 .. l1 - 1
+  const int64_t first = (int64_t)blockIdx.x * tiles * kTopkTokens;
+  const float* row = s_tile + threadIdx.x * topk_pitch(E);
+  for (int l = l0; l <= l1; ++l) {
+    for (int i = threadIdx.x; i < E * E; i += kTopkTokens) h[i] = 0;
+    for (int tl = 0; tl < tiles; ++tl) {
+      const int64_t n0 = first + (int64_t)tl * kTopkTokens;
+      if (n0 >= N) break;
+      load_logit_tile(s_tile, logits + l * sl, n0, N, E, sn);
+      __syncthreads();
+      const unsigned long long set = n0 + threadIdx.x < N ? topk_set<KN>(row, E, kf) : 0ull;
+      if (l > l0) {
+        for (unsigned long long a = s_prev[tl][threadIdx.x]; a; a &= a - 1) {
+          int* hr = h + (__ffsll(static_cast<long long>(a)) - 1) * E - 1;
+          for (unsigned long long b = set; b; b &= b - 1) atomicAdd(&hr[__ffsll(static_cast<long long>(b))], 1);
+        }
       }
-    used |= 1ull << best;
-  }
-  return used;
-}
-
-// Transition counts of Eq. 41 for the layer pair (l, l + 1) = blockIdx.y:
-// each token adds one to n_l(k -> k') for every k in its top-kf at layer l
-// and k' in its top-kf at layer l + 1 (integer atomics: order-independent).
-template <int EMAX>
-// logits of token n at layer l start at n * sn + l * sl (floats).
-__global__ void __launch_bounds__(256) transitions_kernel(const float* __restrict__ logits,
-                                                          int64_t N, int L, int E, int kf,
-                                                          int64_t sn, int64_t sl,
-                                                          int32_t* __restrict__ counts) {
-  __shared__ int h[64 * 64];
-  const int l = blockIdx.y;
-  for (int i = threadIdx.x; i < E * E; i += blockDim.x) h[i] = 0;
-  __syncthreads();
-  for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N;
-       n += (int64_t)gridDim.x * blockDim.x) {
-    unsigned long long a = topk_set<EMAX>(logits + n * sn + l * sl, E, kf);
-    const unsigned long long b = topk_set<EMAX>(logits + n * sn + (l + 1) * sl, E, kf);
-    while (a) {
-      const int x = __ffsll(static_cast<long long>(a)) - 1;
-      a &= a - 1;
-      unsigned long long bb = b;
-      while (bb) {
-        const int y = __ffsll(static_cast<long long>(bb)) - 1;
-        bb &= bb - 1;
-        atomicAdd(&h[x * E + y], 1);
-      }
+      s_prev[tl][threadIdx.x] = set;
+      __syncthreads();  // the tile is rewritten; the counts are complete
+    }
+    if (l > l0) {
+      for (int i = threadIdx.x; i < E * E; i += kTopkTokens)
+        if (h[i]) atomicAdd(&counts[(size_t)(l - 1) * E * E + i], h[i]);
+      __syncthreads();
     }
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < E * E; i += blockDim.x)
-    if (h[i]) atomicAdd(&counts[(size_t)l * E * E + i], h[i]);
+}
+
+// The list length for kf (0: the passes), and dynamic shared memory.
+inline int topk_list_len(int kf) { return kf <= 2 ? 2 : kf <= 4 ? 4 : kf <= 6 ? 6 : kf <= 8 ? 8 : 0; }
+inline size_t topk_tile_bytes(int E) { return sizeof(float) * kTopkTokens * topk_pitch(E); }
+
+// counts (zeroed by the caller) of L layers
+static int counts_launch(const float* logits, int64_t N, int L, int E, int kf, int64_t sn, int64_t sl,
+                         int32_t* counts, cudaStream_t stream) {
+  static PerDevice attr;
+  const cudaError_t ae = static_cast<cudaError_t>(per_device(attr, [] {
+    const int most = static_cast<int>(topk_tile_bytes(64));
+    cudaError_t e = cudaFuncSetAttribute(counts_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(counts_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(counts_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(counts_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(counts_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    return static_cast<int>(e);
+  }));
+  if (ae != cudaSuccess) return cuda_fail(ae, "cudaFuncSetAttribute(counts_kernel)");
+  int64_t blocks = (N + kTopkTokens - 1) / kTopkTokens;
+  const int64_t cap = (num_sms() * 6 + L - 1) / L;
+  if (blocks > cap) blocks = cap;
+  const dim3 grid(L, static_cast<unsigned>(blocks));
+  const size_t smem = topk_tile_bytes(E);
+  switch (topk_list_len(kf)) {
+    case 2: counts_kernel<2><<<grid, kTopkTokens, smem, stream>>>(logits, N, E, kf, sn, sl, counts); break;
+    case 4: counts_kernel<4><<<grid, kTopkTokens, smem, stream>>>(logits, N, E, kf, sn, sl, counts); break;
+    case 6: counts_kernel<6><<<grid, kTopkTokens, smem, stream>>>(logits, N, E, kf, sn, sl, counts); break;
+    case 8: counts_kernel<8><<<grid, kTopkTokens, smem, stream>>>(logits, N, E, kf, sn, sl, counts); break;
+    default: counts_kernel<0><<<grid, kTopkTokens, smem, stream>>>(logits, N, E, kf, sn, sl, counts);
+  }
+  OM_LAUNCHED("counts_kernel");
+  return ORDERMOE_OK;
 }
 
 // P_l(k -> k') = n / sum_k'' n (fp64, rounded once to fp32); 0 for an empty row.
-__global__ void transitions_finish_kernel(const int32_t* __restrict__ counts, int rows, int E,
-                                          float* __restrict__ P) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+// A warp a row; the counts' sum is an integer below 2^53, the same in fp64 in
+// any order.
+__global__ void __launch_bounds__(128) transitions_finish_kernel(const int32_t* __restrict__ counts,
+                                                                 int rows, int E,
+                                                                 float* __restrict__ P) {
+  const int r = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= rows) return;
   const int32_t* c = counts + (size_t)r * E;
-  double row = 0.0;
-  for (int b = 0; b < E; ++b) row = __dadd_rn(row, static_cast<double>(c[b]));
-  for (int b = 0; b < E; ++b)
-    P[(size_t)r * E + b] = row > 0.0 ? __double2float_rn(__ddiv_rn(static_cast<double>(c[b]), row)) : 0.0f;
+  const int c0 = lane < E ? c[lane] : 0, c1 = lane + 32 < E ? c[lane + 32] : 0;
+  long long sum = (long long)c0 + c1;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  const double row = static_cast<double>(sum);
+  float* out = P + (size_t)r * E;
+  if (lane < E) out[lane] = sum > 0 ? __double2float_rn(__ddiv_rn(static_cast<double>(c0), row)) : 0.0f;
+  if (lane + 32 < E)
+    out[lane + 32] = sum > 0 ? __double2float_rn(__ddiv_rn(static_cast<double>(c1), row)) : 0.0f;
 }
 
 // The partial Grams of an entry summed over the chunks, in chunk order (fp64).
@@ -266,21 +377,6 @@ __global__ void __launch_bounds__(256) gram_sim_kernel(const float* __restrict__
     v = (ni == 0.0 || nj == 0.0) ? 0.0f : __double2float_rn(g / (ni * nj));
   }
   sim[(size_t)l * E * E + x] = v;
-}
-
-__global__ void counts_from_logits_kernel(const float* __restrict__ logits, int64_t N, int E,
-                                          int kf, int32_t* __restrict__ counts) {
-  __shared__ int cnt[64];
-  if (threadIdx.x < 64) cnt[threadIdx.x] = 0;
-  __syncthreads();
-  for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < N;
-       n += (int64_t)gridDim.x * blockDim.x) {
-    float l[64];
-    for (int e = 0; e < E; ++e) l[e] = logits[n * E + e];
-    add_topk_counts(l, E, kf, cnt);
-  }
-  __syncthreads();
-  if (threadIdx.x < E && cnt[threadIdx.x]) atomicAdd(&counts[threadIdx.x], cnt[threadIdx.x]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1107,15 +1203,7 @@ static int similarity_impl(const uint16_t* W_r, const uint16_t* X_cal, int L, in
   }
   int rc = logits_gemm_launch(X_cal, static_cast<int>(N), W_r, L * E, d, H, stream);
   if (rc) return rc;
-  int64_t cblocks = (N + 255) / 256;
-  const int64_t ccap = (num_sms() * 8 + L - 1) / L;
-  if (cblocks > ccap) cblocks = ccap;
-  const dim3 cgrid(L, static_cast<unsigned>(cblocks));
-  if (E <= 8) counts_kernel<8><<<cgrid, 256, 0, stream>>>(H, N, L, E, k_freq, counts);
-  else if (E <= 16) counts_kernel<16><<<cgrid, 256, 0, stream>>>(H, N, L, E, k_freq, counts);
-  else if (E <= 32) counts_kernel<32><<<cgrid, 256, 0, stream>>>(H, N, L, E, k_freq, counts);
-  else counts_kernel<64><<<cgrid, 256, 0, stream>>>(H, N, L, E, k_freq, counts);
-  OM_LAUNCHED("counts_kernel");
+  if ((rc = counts_launch(H, N, L, E, k_freq, (int64_t)L * E, E, counts, stream))) return rc;
   gram_kernel<<<dim3(L, nchunks), 256, 0, stream>>>(H, N, L, E, gpart);
   OM_LAUNCHED("gram_kernel");
   gram_sim_kernel<<<dim3(L, (E * E + 255) / 256), 256, 0, stream>>>(gpart, nchunks, E, sim);
@@ -1149,11 +1237,7 @@ extern "C" int ordermoe_expert_counts(const float* logits, int64_t N, int E, int
   if (!counts || (N > 0 && !logits)) return fail(ORDERMOE_ERR_INVALID_ARG, "expert_counts: null pointer");
   OM_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * E, stream));
   if (N == 0) return ORDERMOE_OK;
-  int64_t blocks = (N + 255) / 256;
-  if (blocks > num_sms() * 4) blocks = num_sms() * 4;
-  counts_from_logits_kernel<<<static_cast<int>(blocks), 256, 0, stream>>>(logits, N, E, k_freq, counts);
-  OM_LAUNCHED("counts_from_logits_kernel");
-  return ORDERMOE_OK;
+  return counts_launch(logits, N, 1, E, k_freq, E, 0, counts, stream);
 }
 
 namespace om {
@@ -1391,18 +1475,42 @@ static int transitions_launch(const char* who, const float* logits, int64_t N, i
   if (!counts || !P || (N > 0 && !logits)) return fail(ORDERMOE_ERR_INVALID_ARG, "%s: null pointer", who);
   OM_CUDA(cudaMemsetAsync(counts, 0, sizeof(int32_t) * (size_t)(L - 1) * E * E, stream));
   if (N > 0) {
-    int64_t blocks = (N + 255) / 256;
-    const int64_t cap = (num_sms() * 4 + L - 2) / (L - 1);
-    if (blocks > cap) blocks = cap;
-    const dim3 grid(static_cast<unsigned>(blocks), L - 1);
-    if (E <= 8) transitions_kernel<8><<<grid, 256, 0, stream>>>(logits, N, L, E, k_freq, sn, sl, counts);
-    else if (E <= 16) transitions_kernel<16><<<grid, 256, 0, stream>>>(logits, N, L, E, k_freq, sn, sl, counts);
-    else if (E <= 32) transitions_kernel<32><<<grid, 256, 0, stream>>>(logits, N, L, E, k_freq, sn, sl, counts);
-    else transitions_kernel<64><<<grid, 256, 0, stream>>>(logits, N, L, E, k_freq, sn, sl, counts);
+    static PerDevice attr;
+    const cudaError_t ae = static_cast<cudaError_t>(per_device(attr, [] {
+      const int most = static_cast<int>(topk_tile_bytes(64) + sizeof(int) * 64 * 64);
+      cudaError_t e = cudaFuncSetAttribute(transitions_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(transitions_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(transitions_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(transitions_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(transitions_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+      return static_cast<int>(e);
+    }));
+    if (ae != cudaSuccess) return cuda_fail(ae, "cudaFuncSetAttribute(transitions_kernel)");
+    const int64_t tiles = (N + kTopkTokens - 1) / kTopkTokens;
+    if (tiles > INT32_MAX) return fail(ORDERMOE_ERR_UNSUPPORTED_SHAPE, "%s: too many tokens", who);
+    // tiles a block counts before it adds its E * E counts to memory, and layer
+    // pairs it walks: as many as leave two blocks an SM
+    int64_t tb = tiles / num_sms();
+    if (tb < 1) tb = 1;
+    if (tb > kTransTiles) tb = kTransTiles;
+    const int64_t cols = (tiles + tb - 1) / tb;
+    int64_t ranges = (2 * num_sms() + cols - 1) / cols;
+    if (ranges > L - 1) ranges = L - 1;
+    int per = static_cast<int>((L - 1 + ranges - 1) / ranges);
+    if ((L - 1 + per - 1) / per > 65535) per = (L - 1 + 65534) / 65535;  // the grid's y limit
+    const dim3 grid(static_cast<unsigned>(cols), (L - 1 + per - 1) / per);
+    const size_t smem = topk_tile_bytes(E) + sizeof(int) * E * E;
+    switch (topk_list_len(k_freq)) {
+      case 2: transitions_kernel<2><<<grid, kTopkTokens, smem, stream>>>(logits, N, L, E, k_freq, sn, sl, per, static_cast<int>(tb), counts); break;
+      case 4: transitions_kernel<4><<<grid, kTopkTokens, smem, stream>>>(logits, N, L, E, k_freq, sn, sl, per, static_cast<int>(tb), counts); break;
+      case 6: transitions_kernel<6><<<grid, kTopkTokens, smem, stream>>>(logits, N, L, E, k_freq, sn, sl, per, static_cast<int>(tb), counts); break;
+      case 8: transitions_kernel<8><<<grid, kTopkTokens, smem, stream>>>(logits, N, L, E, k_freq, sn, sl, per, static_cast<int>(tb), counts); break;
+      default: transitions_kernel<0><<<grid, kTopkTokens, smem, stream>>>(logits, N, L, E, k_freq, sn, sl, per, static_cast<int>(tb), counts);
+    }
     OM_LAUNCHED("transitions_kernel");
   }
   const int rows = (L - 1) * E;
-  transitions_finish_kernel<<<(rows + 127) / 128, 128, 0, stream>>>(counts, rows, E, P);
+  transitions_finish_kernel<<<(rows + 3) / 4, 128, 0, stream>>>(counts, rows, E, P);
   OM_LAUNCHED("transitions_finish_kernel");
   return ORDERMOE_OK;
 }

@@ -37,6 +37,47 @@ def test_transitions_given_logits_bit_exact(N, L, E, kf):
     np.testing.assert_array_equal(P.cpu().numpy(), rP)
 
 
+@pytest.mark.parametrize("N,L,E,kf", [
+    (78500, 2, 12, 3),   # two tiles of tokens a block, the last one ragged
+    (257, 9, 17, 1), (700, 3, 64, 8), (300, 3, 33, 9), (1, 2, 1, 1), (513, 4, 40, 5)])
+def test_topk_sets_with_ties_infinities_and_nan(N, L, E, kf):
+    """The counts and transitions against the rule itself (kf passes, each
+    taking the first unused maximum): equal logits across the boundary, -inf
+    and +inf, and NaN logits, which are taken only where a pass starts on one."""
+    rng = np.random.default_rng(N + E + kf)
+    logits = np.round(rng.standard_normal((N, L, E)) * 2).astype(np.float32) / 2
+    logits[rng.random((N, L, E)) < 0.02] = -np.inf
+    logits[rng.random((N, L, E)) < 0.01] = np.inf
+    logits[::7][rng.random(logits[::7].shape) < 0.03] = np.nan
+    logits[0] = -np.inf
+    sets = np.zeros((N, L, E), bool)
+    n, l = np.ogrid[:N, :L]
+    for _ in range(kf):
+        best = np.full((N, L), -1)
+        bv = np.zeros((N, L), np.float32)
+        for e in range(E):
+            with np.errstate(invalid="ignore"):
+                take = ~sets[:, :, e] & ((best < 0) | (logits[:, :, e] > bv))
+            best[take], bv[take] = e, logits[:, :, e][take]
+        sets[n, l, best] = True
+    s = sets.astype(np.float32)  # sums below 2^24
+    want = np.stack([s[:, i].T @ s[:, i + 1] for i in range(L - 1)]).astype(np.int64)
+    cnt = torch.empty(L - 1, E, E, dtype=torch.int32, device=DEV)
+    P = torch.empty(L - 1, E, E, dtype=torch.float32, device=DEV)
+    B.ordermoe_transitions(torch.as_tensor(logits).to(DEV), N, L, E, kf, cnt, P)
+    np.testing.assert_array_equal(cnt.cpu().numpy(), want)
+    row = want.sum(2, keepdims=True)
+    np.testing.assert_array_equal(P.cpu().numpy(), (want / np.maximum(row, 1)).astype(np.float32))
+    # unaligned rows, layer by layer: E + 1 floats apart
+    wide = torch.zeros(L, N, E + 1, dtype=torch.float32, device=DEV)
+    wide[:, :, :E] = torch.as_tensor(logits).to(DEV).transpose(0, 1)
+    B.ordermoe_transitions_strided(wide, N, L, E, kf, E + 1, N * (E + 1), cnt, P)
+    np.testing.assert_array_equal(cnt.cpu().numpy(), want)
+    c = torch.empty(E, dtype=torch.int32, device=DEV)
+    B.ordermoe_expert_counts(torch.as_tensor(logits[:, 0].copy()).to(DEV), N, E, kf, c)
+    np.testing.assert_array_equal(c.cpu().numpy(), sets[:, 0].sum(0))
+
+
 def stack_tables(rng, L, E, M, qbar, cheap_links):
     """L layers' tables, random groups/placements, as one device buffer plus the
     oracle's own copies."""
