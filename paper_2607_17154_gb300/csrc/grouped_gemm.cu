@@ -41,10 +41,8 @@ constexpr int STAGES = 4;
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int B_BYTES = BN * BK * 2;
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-constexpr int BOX_BYTES = 128 * BK * 2;  // one TMA box: 128 rows x 64 columns
 constexpr int THREADS = 192;
 constexpr int TMEM_COLS = 512;
-constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN);
 
 struct Smem {
   uint64_t full[STAGES];
@@ -71,7 +69,7 @@ struct Args {
   int E;
   int K;             // reduction length
   int n_tiles;       // N slices per expert
-  int b_rows;        // weight rows per expert in the B tensor map (d_ff or d)
+  int b_rows;        // weight rows per expert (d_ff or d); logits: columns of a slice
   uint16_t* out;     // H [R][d_ff] or Y [R][d]
   int ldo;           // row length of out
   uint64_t limit_ns; // bounded-wait limit
@@ -210,70 +208,78 @@ __global__ void __launch_bounds__(THREADS, 1)
   // per-role bookkeeping for the drain after an abort
   uint32_t issued_mask = 0, last_phase_bits = 0;
   bool mma_issued = false;
+  bool leader = false;  // the MMA warp's issuing lane
 
+  const int width = args.b_rows;  // columns of a slice, its weight rows in two boxes
+  const int box_bytes = width / 2 * BK * 2;
   if (warp == 0) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      for (int tile = blockIdx.x; tile < total && !*abort; tile += gridDim.x) {
-        const Tile t = decode(tile, s, args.E, args.n_tiles, args.m_major);
-        const int brow = t.n * 256;
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(&s.empty[stage], phase ^ 1u, args.limit_ns, abort)) {
-            if (!*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 1);
-            *abort = 1;
-            break;
-          }
-          uint8_t* sa = tiles + stage * STAGE_BYTES;
-          uint8_t* sb = sa + A_BYTES;
-          mbar_arrive_expect_tx(&s.full[stage], STAGE_BYTES);
-          tma_load_2d(sa, &mapA, &s.full[stage], kb * BK, t.m0);
-          tma_load_2d(sb, &mapB0, &s.full[stage], kb * BK, brow);
-          tma_load_2d(sb + BOX_BYTES, &mapB0, &s.full[stage], kb * BK, brow + 128);
-          issued_mask |= 1u << stage;
-          last_phase_bits = (last_phase_bits & ~(1u << stage)) | (phase << stage);
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+    // producer and MMA issuer walk the stages converged, one elected lane issues
+    const bool issuer = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
+      const Tile t = decode(tile, s, args.E, args.n_tiles, args.m_major);
+      for (int kb = 0; kb < kblocks; ++kb) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&s.empty[stage], phase ^ 1u, args.limit_ns, abort))) {
+          if (issuer && !*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 1);
+          *abort = 1;
+          ok = false;
+          break;
         }
+        uint8_t* sa = tiles + stage * STAGE_BYTES;
+        uint8_t* sb = sa + A_BYTES;
+        if (issuer) {
+          mbar_arrive_expect_tx(&s.full[stage], A_BYTES + 2 * box_bytes);
+          tma_load_2d(sa, &mapA, &s.full[stage], kb * BK, t.m0);
+          tma_load_2d(sb, &mapB0, &s.full[stage], kb * BK, t.n * width);
+          tma_load_2d(sb + box_bytes, &mapB0, &s.full[stage], kb * BK, t.n * width + width / 2);
+        }
+        issued_mask |= 1u << stage;
+        last_phase_bits = (last_phase_bits & ~(1u << stage)) | (phase << stage);
+        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      int it = 0;
-      for (int tile = blockIdx.x; tile < total && !*abort; tile += gridDim.x, ++it) {
-        const int slot = it & 1;
-        const uint32_t acc_phase = (it >> 1) & 1;
-        if (!mbar_wait(&s.tempty[slot], acc_phase ^ 1u, args.limit_ns, abort)) {
-          if (!*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 2);
+    leader = elect_one();
+    const uint64_t desc0 = sdesc_kmajor_sw128(smem_u32(tiles));
+    const uint32_t idesc = idesc_bf16_f32(BM, width);
+    int stage = 0;
+    uint32_t phase = 0;
+    int it = 0;
+    for (int tile = blockIdx.x; tile < total; tile += gridDim.x, ++it) {
+      const int slot = it & 1;
+      const uint32_t acc_phase = (it >> 1) & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&s.tempty[slot], acc_phase ^ 1u, args.limit_ns, abort))) {
+        if (leader && !*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 2);
+        *abort = 1;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + slot * BN;
+      bool ok = true;
+      for (int kb = 0; kb < kblocks; ++kb) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&s.full[stage], phase, args.limit_ns, abort))) {
+          if (leader && !*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 3);
           *abort = 1;
+          ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + slot * BN;
-        bool ok = true;
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(&s.full[stage], phase, args.limit_ns, abort)) {
-            if (!*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 3);
-            *abort = 1;
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t a0 = smem_u32(tiles + stage * STAGE_BYTES);
-          const uint32_t b0 = a0 + A_BYTES;
+        const uint64_t da = desc0 + static_cast<uint64_t>((stage * STAGE_BYTES) >> 4);
+        const uint64_t db = da + (A_BYTES >> 4);
+        if (leader) {
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {
-            mma_bf16(d_tmem, sdesc_kmajor_sw128(a0 + kk * 32), sdesc_kmajor_sw128(b0 + kk * 32),
-                     IDESC, (kb | kk) != 0 ? 1u : 0u);
-          }
-          mma_issued = true;
+          for (int kk = 0; kk < BK / 16; ++kk)  // 16 elements = 32 bytes on
+            mma_bf16(d_tmem, da + 2 * kk, db + 2 * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
           mma_commit(&s.empty[stage]);
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
-        if (!ok) break;
-        mma_commit(&s.tfull[slot]);
+        mma_issued = true;
+        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
+      if (!ok) break;
+      if (leader) mma_commit(&s.tfull[slot]);
+      __syncwarp();
     }
   } else {
     // epilogue: warps 2..5 -> TMEM lane quarter (warp % 4)
@@ -296,18 +302,18 @@ __global__ void __launch_bounds__(THREADS, 1)
       const int row = t.m0 + lrow;
       const bool valid = row < t.m_end;
       const uint32_t tb = tmem_base + slot * BN + (static_cast<uint32_t>(q * 32) << 16);
-      const int col0 = t.n * 256;
+      const int col0 = t.n * width, col1 = min(col0 + width, args.n_valid);
       float* orow = args.out_f32 + (size_t)row * args.n_valid;
       const bool vec = (args.n_valid & 3) == 0;
 #pragma unroll 1
       for (int c = 0; c < 8; ++c) {
-        if (col0 + c * 32 >= args.n_valid) break;  // warp-uniform
+        if (col0 + c * 32 >= col1) break;  // warp-uniform
         uint32_t v[32];
         tmem_ld32(tb + c * 32, v);
         tmem_ld_wait();
         if (valid) {
           const int cb = col0 + c * 32;
-          if (vec && cb + 32 <= args.n_valid) {
+          if (vec && cb + 32 <= col1) {
             float4* dst = reinterpret_cast<float4*>(orow + cb);
 #pragma unroll
             for (int i = 0; i < 8; ++i)
@@ -316,7 +322,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           } else {
 #pragma unroll
             for (int i = 0; i < 32; ++i)
-              if (cb + i < args.n_valid) orow[cb + i] = __uint_as_float(v[i]);
+              if (cb + i < col1) orow[cb + i] = __uint_as_float(v[i]);
           }
         }
       }
@@ -334,7 +340,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         if ((issued_mask >> st) & 1u)
           mbar_wait(&s.full[st], (last_phase_bits >> st) & 1u, args.limit_ns, never);
     }
-    if (warp == 1 && lane == 0 && mma_issued) {
+    if (leader && mma_issued) {  // the lane that issued the MMAs
       mma_commit(&s.drain);
       mbar_wait(&s.drain, 0, args.limit_ns, never);
     }
@@ -991,7 +997,12 @@ int logits_gemm_launch(const uint16_t* X, int N, const uint16_t* W, int C, int d
   CUtensorMap mX, mW;
   int rc;
   if ((rc = make_map(&mX, X, N, d))) return rc;
-  if ((rc = make_map(&mW, W, C, d))) return rc;
+  // column slices of one width, so that every tile costs the same (with 256 and
+  // a rest, CTAs of one parity got all the full tiles: 45.7 against 33.2 us
+  // for 32768 tokens x 320 columns, d 1024)
+  const int n_tiles = (C + BN - 1) / BN;
+  const int width = ((C + n_tiles - 1) / n_tiles + 15) & ~15;
+  if ((rc = make_tmap_bf16(&mW, W, C, d, width / 2))) return rc;
   Args a{};
   a.offsets = nullptr;
   a.rows = N;
@@ -999,8 +1010,8 @@ int logits_gemm_launch(const uint16_t* X, int N, const uint16_t* W, int C, int d
   a.out_f32 = H;
   a.E = 1;
   a.K = d;
-  a.n_tiles = (C + 255) / 256;
-  a.b_rows = 0;
+  a.n_tiles = n_tiles;
+  a.b_rows = width;
   a.limit_ns = wait_limit_ns();
   a.m_major = 1;  // the stacked router rows (a few MB) stay in L2; X_cal streams once
   const long long tiles = (long long)((N + BM - 1) / BM) * a.n_tiles;
