@@ -462,6 +462,93 @@ __global__ void __launch_bounds__(128) select_kernel(
 constexpr int kLaneTokens = 4;   // tokens per warp (eight lanes each)
 constexpr int kLaneThreads = 256;
 
+// The slots of one token whose targets are idx, on eight lanes (sub 0 .. 7); Aas:
+// its row A[a][s][.] of the delay table (valid when a, s < M). Every lane of the
+// warp calls it (the butterflies need them all), inactive tokens (past T, a NaN
+// token) write nothing.
+__device__ __forceinline__ void select_slots(
+    int t, bool active, int sub, const int (&idx)[ORDERMOE_MAX_TOPK], int E, int k, int M, float qbar,
+    const float* Aas, const SelSmem& sm, const float* s_Q, const float* s_Cq, int a, int s, float q,
+    uint8_t* __restrict__ loc, float* __restrict__ qhat, int32_t* __restrict__ chosen_expert,
+    uint8_t* __restrict__ chosen_server, uint8_t* __restrict__ kind_out, int (&kind_count)[4]) {
+  unsigned long long taken = 0;
+#pragma unroll
+  for (int j = 0; j < ORDERMOE_MAX_TOPK; ++j)
+    if (j < k && active) {
+      if (idx[j] < 0 || idx[j] >= E) active = false;
+      else taken |= 1ull << idx[j];
+    }
+  if (active && (a >= M || s >= M)) {
+    if (sub == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, t);
+    active = false;
+  }
+  int first_server = s;
+#pragma unroll
+  for (int j = 0; j < ORDERMOE_MAX_TOPK; ++j) {
+    if (j >= k) break;  // k is the same for every lane
+    const int r = idx[j];
+    const int nsub = active ? sm.nsub[r] : -1;
+    unsigned long long best = ~0ull;
+    for (int ki = sub; ki <= nsub; ki += 8) {
+      const int kk = (ki == 0) ? r : sm.sublist[r * 64 + ki - 1];
+      const bool issub = (ki != 0);
+      float cq = 0.0f;
+      if (issub) {
+        if ((taken >> kk) & 1ull) continue;
+        if (!(__fadd_rn(q, s_Q[r * E + kk]) <= qbar)) continue;  // Eq. 40 budget
+        cq = s_Cq[r * E + kk];
+      }
+      uint32_t pm = sm.pmask[kk];
+      while (pm) {
+        const int m = __ffs(pm) - 1;
+        pm &= pm - 1;
+        const float cost = __fadd_rn(Aas[m], cq);
+        const unsigned long long key =
+            (static_cast<unsigned long long>(__float_as_uint(cost)) << 32) |
+            (static_cast<unsigned long long>(issub ? 1u : 0u) << 31) |
+            (static_cast<unsigned long long>(m != s ? 1u : 0u) << 30) |
+            (static_cast<unsigned long long>(m) << 8) | static_cast<unsigned long long>(kk);
+        best = key < best ? key : best;
+      }
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
+      const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
+      best = other < best ? other : best;
+    }
+    if (!active) continue;
+    int kstar, mstar, kd;
+    if (best == ~0ull) {
+      if (sub == 0) report(&g_err_route, ORDERMOE_DEV_NO_CANDIDATE, t);
+      kstar = r; mstar = s; kd = 0;
+    } else {
+      kstar = static_cast<int>(best & 0xFFu);
+      mstar = static_cast<int>((best >> 8) & 0xFFu);
+      const int bsub = static_cast<int>((best >> 31) & 1u);
+      const int away = static_cast<int>((best >> 30) & 1u);
+      kd = 2 * away + bsub;
+      if (bsub) {
+        taken |= 1ull << kstar;
+        q = __fadd_rn(q, s_Q[r * E + kstar]);
+      }
+    }
+    if (j == 0) first_server = mstar;
+    if (sub == 0) {
+      chosen_expert[(size_t)t * k + j] = kstar;
+      chosen_server[(size_t)t * k + j] = static_cast<uint8_t>(mstar);
+      kind_out[(size_t)t * k + j] = static_cast<uint8_t>(kd);
+      if (kd == 0) ++kind_count[0];  // constant indices: kind_count[] stays in registers
+      else if (kd == 1) ++kind_count[1];
+      else if (kd == 2) ++kind_count[2];
+      else ++kind_count[3];
+    }
+  }
+  if (active && sub == 0 && loc != nullptr) {
+    loc[t] = static_cast<uint8_t>(first_server);
+    qhat[t] = q;
+  }
+}
+
 __global__ void __launch_bounds__(kLaneThreads) select_lanes_kernel(
     const int32_t* __restrict__ topk_idx, int T, int E, int k, const uint8_t* __restrict__ tab,
     const uint8_t* __restrict__ home, uint8_t* __restrict__ loc, float* __restrict__ qhat,
@@ -488,9 +575,7 @@ __global__ void __launch_bounds__(kLaneThreads) select_lanes_kernel(
   for (int base = (blockIdx.x * (kLaneThreads / 32) + (threadIdx.x >> 5)) * kLaneTokens; base < T;
        base += warps_total * kLaneTokens) {
     const int t = base + grp;
-    // every lane runs every slot (the butterflies need the whole warp);
-    // inactive tokens (past T, a NaN token's -1 targets, bad servers) write nothing
-    bool active = t < T;
+    const bool active = t < T;
     // the token's state and targets, loaded together
     int a = 0, s = 0;
     float q = 0.0f;
@@ -500,85 +585,11 @@ __global__ void __launch_bounds__(kLaneThreads) select_lanes_kernel(
       q = (qhat != nullptr) ? qhat[t] : 0.0f;
     }
     int idx[ORDERMOE_MAX_TOPK];
-    unsigned long long taken = 0;
 #pragma unroll
     for (int j = 0; j < ORDERMOE_MAX_TOPK; ++j) idx[j] = (j < k && active) ? topk_idx[(size_t)t * k + j] : 0;
-#pragma unroll
-    for (int j = 0; j < ORDERMOE_MAX_TOPK; ++j)
-      if (j < k && active) {
-        if (idx[j] < 0 || idx[j] >= E) active = false;
-        else taken |= 1ull << idx[j];
-      }
-    if (active && (a >= M || s >= M)) {
-      if (sub == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, t);
-      active = false;
-    }
-    const float* Aas = Atab + (active ? (a * M + s) * M : 0);
-    int first_server = s;
-#pragma unroll
-    for (int j = 0; j < ORDERMOE_MAX_TOPK; ++j) {
-      if (j >= k) break;  // k is the same for every lane
-      const int r = idx[j];
-      const int nsub = active ? sm.nsub[r] : -1;
-      unsigned long long best = ~0ull;
-      for (int ki = sub; ki <= nsub; ki += 8) {
-        const int kk = (ki == 0) ? r : sm.sublist[r * 64 + ki - 1];
-        const bool issub = (ki != 0);
-        float cq = 0.0f;
-        if (issub) {
-          if ((taken >> kk) & 1ull) continue;
-          if (!(__fadd_rn(q, s_Q[r * E + kk]) <= qbar)) continue;  // Eq. 40 budget
-          cq = s_Cq[r * E + kk];
-        }
-        uint32_t pm = sm.pmask[kk];
-        while (pm) {
-          const int m = __ffs(pm) - 1;
-          pm &= pm - 1;
-          const float cost = __fadd_rn(Aas[m], cq);
-          const unsigned long long key =
-              (static_cast<unsigned long long>(__float_as_uint(cost)) << 32) |
-              (static_cast<unsigned long long>(issub ? 1u : 0u) << 31) |
-              (static_cast<unsigned long long>(m != s ? 1u : 0u) << 30) |
-              (static_cast<unsigned long long>(m) << 8) | static_cast<unsigned long long>(kk);
-          best = key < best ? key : best;
-        }
-      }
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xffffffffu, best, o);
-        best = other < best ? other : best;
-      }
-      if (!active) continue;
-      int kstar, mstar, kd;
-      if (best == ~0ull) {
-        if (sub == 0) report(&g_err_route, ORDERMOE_DEV_NO_CANDIDATE, t);
-        kstar = r; mstar = s; kd = 0;
-      } else {
-        kstar = static_cast<int>(best & 0xFFu);
-        mstar = static_cast<int>((best >> 8) & 0xFFu);
-        const int bsub = static_cast<int>((best >> 31) & 1u);
-        const int away = static_cast<int>((best >> 30) & 1u);
-        kd = 2 * away + bsub;
-        if (bsub) {
-          taken |= 1ull << kstar;
-          q = __fadd_rn(q, s_Q[r * E + kstar]);
-        }
-      }
-      if (j == 0) first_server = mstar;
-      if (sub == 0) {
-        chosen_expert[(size_t)t * k + j] = kstar;
-        chosen_server[(size_t)t * k + j] = static_cast<uint8_t>(mstar);
-        kind_out[(size_t)t * k + j] = static_cast<uint8_t>(kd);
-        if (kd == 0) ++kind_count[0];  // constant indices: kind_count[] stays in registers
-        else if (kd == 1) ++kind_count[1];
-        else if (kd == 2) ++kind_count[2];
-        else ++kind_count[3];
-      }
-    }
-    if (active && sub == 0 && loc != nullptr) {
-      loc[t] = static_cast<uint8_t>(first_server);
-      qhat[t] = q;
-    }
+    const float* Aas = Atab + (active && a < M && s < M ? (a * M + s) * M : 0);
+    select_slots(t, active, sub, idx, E, k, M, qbar, Aas, sm, s_Q, s_Cq, a, s, q, loc, qhat,
+                 chosen_expert, chosen_server, kind_out, kind_count);
   }
   flush_kind_counts(sm, kind_count, counters);
   __syncthreads();
@@ -1572,6 +1583,338 @@ __global__ void __launch_bounds__(rt::THREADS, 1) router_select_kernel(
   }
 }
 
+// Small batches of 17 to 64 experts: router, top-k and selection in one launch.
+// A cluster of 8 CTAs handles 128 tokens, CTA r an eighth of the K blocks (as in
+// router_select_kernel), and then the tokens 16 r .. 16 r + 15: every CTA
+// scatters its partial logits to the tokens' owners (distributed shared memory),
+// and each owner adds the eight partials in rank order and gives a token eight
+// lanes for the top-k, the softmax and the slots of Alg. 2 (select_slots, as
+// select_lanes_kernel). Bound by latency: the K share's loads, one cluster
+// barrier and the slots' serial argmins. One CTA of two with all 128 tokens, a
+// thread each, and the selection in a launch of its own took 14.2 + 9.8 us for 33
+// tokens of 64 experts, d 2048 (ncu), 14.7 + 11.2 for 1021; this takes
+// 13.4 and
+// 14.3. (The token's row of the delay table staged in shared memory: 14.2, 14.8.)
+namespace rl {
+constexpr int SPLIT = 8;
+constexpr int ROWS = 128 / SPLIT;  // tokens of a CTA
+constexpr int STAGES = 5;
+constexpr int THREADS = 192;
+// partials of one rank: [NE / 4 chunks][ROWS + 1][4] floats (the odd pitch spreads
+// the chunks that the eight lanes of a token read over the banks)
+template <int NE>
+constexpr int part_floats() { return NE / 4 * (ROWS + 1) * 4; }
+constexpr int LG_PITCH = 68;  // floats a token's logits take
+template <int NE>
+constexpr int smem_bytes(int E) {
+  return 1024 + STAGES * (rt::A_BYTES + NE * rt::BK * 2) + 256 + SPLIT * part_floats<NE>() * 4 +
+         2 * ROWS * LG_PITCH * 4 + 8 * E * E;
+}
+static_assert(smem_bytes<64>(64) + sizeof(SelSmem) <= 227 * 1024, "router shared memory");
+}  // namespace rl
+
+struct RouterLanesSmem {
+  uint64_t full[rl::STAGES];
+  uint64_t empty[rl::STAGES];
+  uint64_t tfull;
+  uint64_t drain;
+  uint32_t tmem_base;
+  int abort;
+  int zero;
+};
+
+template <int NE>
+__global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1, 1)
+    router_lanes_kernel(const __grid_constant__ CUtensorMap mapX,
+                        const __grid_constant__ CUtensorMap mapW, int T, int E, int d, int k,
+                        int renorm, const uint8_t* __restrict__ tab,
+                        const uint8_t* __restrict__ home, uint8_t* __restrict__ loc,
+                        float* __restrict__ qhat, float* __restrict__ logits_out,
+                        int32_t* __restrict__ topk_idx, float* __restrict__ topk_w,
+                        int32_t* __restrict__ chosen_expert, uint8_t* __restrict__ chosen_server,
+                        uint8_t* __restrict__ kind_out, int32_t* __restrict__ counters,
+                        uint64_t limit_ns, int topk_only) {
+  pdl_trigger();  // launched with programmatic serialization: set-up first
+  constexpr int STAGE_BYTES = rt::A_BYTES + NE * rt::BK * 2;
+  constexpr int TMEM_COLS = NE;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* tiles = reinterpret_cast<uint8_t*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  RouterLanesSmem& s = *reinterpret_cast<RouterLanesSmem*>(tiles + rl::STAGES * STAGE_BYTES);
+  float* part = reinterpret_cast<float*>(tiles + rl::STAGES * STAGE_BYTES + 256);
+  float* s_lg = part + rl::SPLIT * rl::part_floats<NE>();  // [ROWS][LG_PITCH] logits
+  float* s_ex = s_lg + rl::ROWS * rl::LG_PITCH;            // their exponentials
+  float* s_Q = s_ex + rl::ROWS * rl::LG_PITCH;
+  float* s_Cq = s_Q + E * E;
+  __shared__ SelSmem sm;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = static_cast<int>(cluster_ctarank());
+  const int m0 = static_cast<int>(blockIdx.x / rl::SPLIT) * 128;
+  const int kblocks_all = d / rt::BK;
+  const int per = (kblocks_all + rl::SPLIT - 1) / rl::SPLIT;
+  const int kb_begin = min(kblocks_all, rank * per);
+  const int kblocks = min(kblocks_all, kb_begin + per) - kb_begin;
+
+  if (tid == 0) {
+    for (int i = 0; i < rl::STAGES; ++i) {
+      mbar_init(&s.full[i], 1);
+      mbar_init(&s.empty[i], 1);
+    }
+    mbar_init(&s.tfull, 1);
+    mbar_init(&s.drain, 1);
+    s.abort = 0;
+    s.zero = 0;
+    fence_mbar_init();
+  }
+  if (warp == 0 && lane == 0) {
+    tma_prefetch_map(&mapX);
+    tma_prefetch_map(&mapW);
+  }
+  if (warp == 1) {
+    tmem_alloc(&s.tmem_base, TMEM_COLS);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_wait();  // the previous kernel's outputs (X, tables, state) are ready
+  const uint32_t tmem_base = s.tmem_base;
+  volatile int* abort = &s.abort;
+  uint32_t issued_mask = 0, last_phase_bits = 0;
+  bool mma_issued = false, leader = false;
+  bool tables_ok = true;
+  // the epilogue thread's token (eight lanes each) and its state
+  const int et = tid - 64;
+  const int row = et >> 3, sub = lane & 7;
+  const int t = m0 + rank * rl::ROWS + row;
+  int a = 0, loc0 = 0;
+  float q0 = 0.0f;
+
+  if (warp == 0) {
+    const bool issuer = elect_one();
+    for (int i = 0; i < kblocks; ++i) {
+      const int stage = i % rl::STAGES;
+      const uint32_t phase = (i / rl::STAGES) & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&s.empty[stage], phase ^ 1u, limit_ns, abort))) {
+        if (issuer && !*abort) report(&g_err_route, ORDERMOE_DEV_WAIT_TIMEOUT, 24);
+        *abort = 1;
+        break;
+      }
+      if (issuer) {
+        uint8_t* sa = tiles + stage * STAGE_BYTES;
+        mbar_arrive_expect_tx(&s.full[stage], STAGE_BYTES);
+        tma_load_2d(sa, &mapX, &s.full[stage], (kb_begin + i) * rt::BK, m0);
+        tma_load_2d(sa + rt::A_BYTES, &mapW, &s.full[stage], (kb_begin + i) * rt::BK, 0);
+      }
+      issued_mask |= 1u << stage;
+      last_phase_bits = (last_phase_bits & ~(1u << stage)) | (phase << stage);
+    }
+  } else if (warp == 1) {
+    constexpr uint32_t IDESC = idesc_bf16_f32(128, NE);
+    leader = elect_one();
+    const uint64_t desc0 = sdesc_kmajor_sw128(smem_u32(tiles));
+    bool ok = true;
+    for (int i = 0; i < kblocks; ++i) {
+      const int stage = i % rl::STAGES;
+      const uint32_t phase = (i / rl::STAGES) & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&s.full[stage], phase, limit_ns, abort))) {
+        if (leader && !*abort) report(&g_err_route, ORDERMOE_DEV_WAIT_TIMEOUT, 25);
+        *abort = 1;
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint64_t da = desc0 + static_cast<uint64_t>((stage * STAGE_BYTES) >> 4);
+      const uint64_t db = da + (rt::A_BYTES >> 4);
+      if (leader) {
+#pragma unroll
+        for (int kk = 0; kk < rt::BK / 16; ++kk)  // 16 elements = 32 bytes on
+          mma_bf16(tmem_base, da + 2 * kk, db + 2 * kk, IDESC, (i | kk) != 0 ? 1u : 0u);
+        mma_commit(&s.empty[stage]);
+      }
+      mma_issued = true;
+    }
+    if (ok && leader) {
+      if (mma_issued) mma_commit(&s.tfull);
+      else mbar_arrive(&s.tfull);  // empty K share: nothing to wait for
+    }
+  } else {
+    // the selection tables and the token's state, while the TMA and MMA warps run
+    if (et < 4) sm.kind[et] = 0;
+    if (!topk_only) {
+      if (t < T) {
+        a = home[t];
+        loc0 = (loc != nullptr) ? loc[t] : a;  // no state given: first layer (Eq. 36)
+        q0 = (qhat != nullptr) ? qhat[t] : 0.0f;
+      }
+      tables_ok = load_tables_range(tab, E, sm, s_Q, s_Cq, et, 128);
+    }
+    // this CTA's partial logits to the tokens' owners
+    const int q = warp & 3;
+    const int r128 = q * 32 + lane;
+    const bool ok = __all_sync(0xffffffffu, mbar_wait(&s.tfull, 0, limit_ns, abort));
+    if (!ok) {
+      if (lane == 0 && !*abort) report(&g_err_route, ORDERMOE_DEV_WAIT_TIMEOUT, 26);
+      *abort = 1;
+    } else {
+      tc_fence_after();
+      const uint32_t dst = mapa_shared(
+          smem_u32(part + rank * rl::part_floats<NE>() + (r128 % rl::ROWS) * 4), r128 / rl::ROWS);
+#pragma unroll
+      for (int c = 0; c < NE; c += 32) {
+        uint32_t v[32];
+        tmem_ld32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + c, v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+          const bool any = kblocks > 0;
+          asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(
+                           dst + static_cast<uint32_t>((c + i) / 4 * (rl::ROWS + 1) * 16)),
+                       "f"(any ? __uint_as_float(v[i]) : 0.0f), "f"(any ? __uint_as_float(v[i + 1]) : 0.0f),
+                       "f"(any ? __uint_as_float(v[i + 2]) : 0.0f), "f"(any ? __uint_as_float(v[i + 3]) : 0.0f)
+                       : "memory");
+        }
+      }
+      tc_fence_before();
+    }
+  }
+  cluster_sync();  // the partials of every CTA are there (and the tables, in the block)
+  if (warp >= 2 && !*abort) {
+    // the token's logits: chunks of four experts over its lanes, ranks in order
+    float* lg = s_lg + row * rl::LG_PITCH;
+    float* ex = s_ex + row * rl::LG_PITCH;
+    bool nan = false;
+    float v[NE / 8];
+#pragma unroll
+    for (int h = 0; h < NE / 32; ++h) {
+      const int c = sub + 8 * h;  // chunk
+      const float* src = part + (c * (rl::ROWS + 1) + row) * 4;
+      float4 x = *reinterpret_cast<const float4*>(src);
+#pragma unroll
+      for (int r = 1; r < rl::SPLIT; ++r) {
+        const float4 y = *reinterpret_cast<const float4*>(src + r * rl::part_floats<NE>());
+        x.x += y.x;
+        x.y += y.y;
+        x.z += y.z;
+        x.w += y.w;
+      }
+      float xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = 4 * c + u;
+        if (e >= E) xs[u] = -INFINITY;
+        else if (logits_out != nullptr && t < T) logits_out[(size_t)t * E + e] = xs[u];
+        nan |= xs[u] != xs[u];
+        v[4 * h + u] = xs[u];
+      }
+      *reinterpret_cast<float4*>(lg + 4 * c) = make_float4(xs[0], xs[1], xs[2], xs[3]);
+    }
+    const unsigned group = 0xFFu << (lane & 24);  // the token's lanes
+    nan = (__ballot_sync(0xffffffffu, nan) & group) != 0u;
+    bool active = t < T && !nan;
+    if (t < T && nan && sub == 0) {
+      report(&g_err_route, ORDERMOE_DEV_NAN_LOGIT, t);
+      for (int j = 0; j < k; ++j) {  // no targets: a later pass skips this token
+        topk_idx[(size_t)t * k + j] = -1;
+        topk_w[(size_t)t * k + j] = 0.0f;
+      }
+    }
+    // top-k by (logit desc, index asc): each pass takes the largest left, found
+    // among a lane's eight and then across the token's lanes. Lane j keeps slot j.
+    float my_v = -INFINITY, lmax = -INFINITY;
+    int my_e = 0;
+    uint32_t used = 0;  // of this lane's experts
+    int idx[ORDERMOE_MAX_TOPK];
+#pragma unroll
+    for (int j = 0; j < ORDERMOE_MAX_TOPK; ++j) {
+      idx[j] = 0;
+      if (j >= k) continue;  // the same for every lane
+      float bv = -INFINITY;
+      int be = 1 << 20, bi = 0;
+#pragma unroll
+      for (int i = 0; i < NE / 8; ++i) {
+        const int e = 4 * (sub + 8 * (i >> 2)) + (i & 3);
+        // an unused expert, a real one before the padding past E
+        if (!((used >> i) & 1u) && e < E && (be == (1 << 20) || v[i] > bv)) {
+          bv = v[i];
+          be = e;
+          bi = i;
+        }
+      }
+      const int own = be;
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int oe = __shfl_xor_sync(0xffffffffu, be, o);
+        if (oe != (1 << 20) && (be == (1 << 20) || ov > bv || (ov == bv && oe < be))) {
+          bv = ov;
+          be = oe;
+        }
+      }
+      if (own == be && own != (1 << 20)) used |= 1u << bi;
+      idx[j] = active ? be : 0;
+      if (j == 0) lmax = bv;
+      if (sub == j) {
+        my_v = bv;
+        my_e = be;
+      }
+    }
+    // softmax over all E in fp32, summed in index order (the -inf logits past E
+    // add exact zeros); gate weights of the k slots
+#pragma unroll
+    for (int h = 0; h < NE / 32; ++h) {
+      const int c = sub + 8 * h;
+      *reinterpret_cast<float4*>(ex + 4 * c) =
+          make_float4(expf(v[4 * h] - lmax), expf(v[4 * h + 1] - lmax), expf(v[4 * h + 2] - lmax),
+                      expf(v[4 * h + 3] - lmax));
+    }
+    __syncwarp();
+    float denom = 0.0f;
+    for (int c = 0; c < (E + 3) / 4; ++c) {
+      const float4 x = *reinterpret_cast<const float4*>(ex + 4 * c);
+      denom += x.x;
+      denom += x.y;
+      denom += x.z;
+      denom += x.w;
+    }
+    const float wsel = sub < k ? expf(my_v - lmax) / denom : 0.0f;
+    float ssel = 0.0f;
+    for (int j = 0; j < k; ++j) ssel += __shfl_sync(0xffffffffu, wsel, (lane & 24) + j);
+    if (active && sub < k) {
+      topk_idx[(size_t)t * k + sub] = my_e;
+      topk_w[(size_t)t * k + sub] = renorm ? wsel / ssel : wsel;
+    }
+    if (!topk_only && tables_ok) {  // the same for the warp
+      const int M = reinterpret_cast<const int32_t*>(tab)[2];
+      const float qbar = reinterpret_cast<const float*>(tab)[5];
+      const float* Aas = reinterpret_cast<const float*>(tab + off_a(E)) +
+                         (active && a < M && loc0 < M ? (a * M + loc0) * M : 0);
+      int kind_count[4] = {0, 0, 0, 0};
+      select_slots(t, active, sub, idx, E, k, M, qbar, Aas, sm, s_Q, s_Cq, a, loc0, q0, loc, qhat,
+                   chosen_expert, chosen_server, kind_out, kind_count);
+      flush_kind_counts(sm, kind_count, counters);
+    }
+  }
+
+  __syncthreads();
+  if (s.abort) {
+    volatile int* never = &s.zero;
+    if (warp == 0 && lane == 0)
+      for (int st = 0; st < rl::STAGES; ++st)
+        if ((issued_mask >> st) & 1u) mbar_wait(&s.full[st], (last_phase_bits >> st) & 1u, limit_ns, never);
+    if (leader && mma_issued) {  // the lane that issued the MMAs
+      mma_commit(&s.drain);
+      mbar_wait(&s.drain, 0, limit_ns, never);
+    }
+    __syncthreads();
+  }
+  if (counters != nullptr && tid < 4 && sm.kind[tid]) atomicAdd(&counters[tid], sm.kind[tid]);
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, TMEM_COLS);
+  }
+}
+
 }  // namespace om
 
 using namespace om;
@@ -1681,6 +2024,12 @@ static cudaError_t router_attr() {
                               rt::smem_bytes<NE>(NE));
 }
 
+template <int NE>
+static cudaError_t router_lanes_attr() {
+  return cudaFuncSetAttribute(router_lanes_kernel<NE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              rl::smem_bytes<NE>(NE));
+}
+
 static int route_select_impl(const uint16_t* X, const uint16_t* W_r, const float* logits_in, int T,
                              int E, int d, int k, int renorm, const void* tables,
                              size_t tables_bytes_, Lookahead la, const uint8_t* home, uint8_t* loc,
@@ -1751,6 +2100,8 @@ static int route_select_impl(const uint16_t* X, const uint16_t* W_r, const float
     cudaError_t e = router_attr<16>();
     if (e == cudaSuccess) e = router_attr<32>();
     if (e == cudaSuccess) e = router_attr<64>();
+    if (e == cudaSuccess) e = router_lanes_attr<32>();
+    if (e == cudaSuccess) e = router_lanes_attr<64>();
     return static_cast<int>(e);
   }));
   if (ae != cudaSuccess) return cuda_fail(ae, "cudaFuncSetAttribute(router_select_kernel)");
@@ -1768,6 +2119,31 @@ static int route_select_impl(const uint16_t* X, const uint16_t* W_r, const float
   cfg.attrs = attr;
   cfg.numAttrs = pdl_on(stream) ? 2 : 1;
   cudaError_t le;
+  // Small batches of many experts: all eight CTAs of every cluster can be
+  // resident and each has K blocks (up to 2432 tokens on 152 SMs, d >= 512).
+  // Larger ones fill the SMs with the tokens, and the selection of 128 tokens by
+  // one CTA in eight rounds would be longer than a launch over all SMs.
+  if (E > 16 && (long long)blocks * rl::SPLIT <= num_sms() && kblocks >= rl::SPLIT) {
+    cfg.gridDim = dim3(blocks * rl::SPLIT, 1, 1);
+    cfg.blockDim = dim3(rl::THREADS, 1, 1);
+    attr[0] = attr[1];  // the cluster shape is the kernel's own
+    cfg.numAttrs = pdl_on(stream) ? 1 : 0;
+    const int only = la.H > 1 ? 1 : 0;
+    if (NE == 32) {
+      cfg.dynamicSmemBytes = rl::smem_bytes<32>(E);
+      OM_CUDA(cudaLaunchKernelEx(&cfg, router_lanes_kernel<32>, mX, mW, T, E, d, k, renorm, tb, home, loc,
+                                 qhat, logits_out, topk_idx, topk_w, chosen_expert, chosen_server, kind,
+                                 counters, lim, only));
+    } else {
+      cfg.dynamicSmemBytes = rl::smem_bytes<64>(E);
+      OM_CUDA(cudaLaunchKernelEx(&cfg, router_lanes_kernel<64>, mX, mW, T, E, d, k, renorm, tb, home, loc,
+                                 qhat, logits_out, topk_idx, topk_w, chosen_expert, chosen_server, kind,
+                                 counters, lim, only));
+    }
+    return only ? launch_lookahead_select(topk_idx, T, E, k, tb, la, home, loc, qhat, chosen_expert,
+                                          chosen_server, kind, counters, stream)
+                : ORDERMOE_OK;
+  }
 #define OM_RT_LAUNCH(N)                                                                          \
   do {                                                                                           \
     cfg.dynamicSmemBytes = rt::smem_bytes<N>(E);                                                 \
