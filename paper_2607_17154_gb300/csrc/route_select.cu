@@ -614,30 +614,34 @@ __global__ void __launch_bounds__(kLaneThreads) select_lanes_kernel(
 // Both follow for every check from these because fadd is monotone and losses
 // are not negative, so the table holds the same fp32 value as the recursion,
 // which adds its terms in ascending k' as the tables do. A candidate in
-// neither case is evaluated by its warp, k' over the lanes, with the tables
-// read again one level down. V_q itself is read from rows that hold, for each
+// neither case is listed and evaluated by a warp, k' over the lanes (with more
+// levels and experts by the block, k' and its substitutes over the threads),
+// with the tables read again one level down. V_q itself is read from rows that hold, for each
 // target and server, the minima over its substitutes in order of loss (the
 // ones that fit are a prefix of that order); a pair in neither case one level
 // down is evaluated by its lane, unless the bounds Ua <= Phi <= Un already
 // show that it cannot be the minimum.
 //
-// One warp per token, blocks of NW warps; the block finds its home and
+// A warp a token and slot, blocks of NW warps; the block finds its home and
 // tokens by ranking home[] (every block ranks the same way, so the blocks
 // partition the tokens without scratch memory or a sort kernel).
 //
 // Bound: latency. A block's set-up is a chain of L2 reads and block barriers,
-// a slot's argmin a chain of shared-memory reads, and the slowest token (one
-// whose loss falls between the two cases slot after slot) ends the launch.
+// a slot's argmin a chain of shared-memory reads, and a token whose loss falls
+// between the two cases slot after slot would end the launch long after the
+// rest (one warp takes 40 us for such an evaluation at H = 3), so the tokens
+// of a block go slot by slot and all its warps share what is open.
 // One block a token, with the tables rebuilt for each and V folded into every
 // term, took 15.7 ms for 2048 tokens of 64 experts, 8 servers, top-6, H = 3,
 // and 14.6 us for 128 tokens of 8 experts, 4 servers, top-2 (ncu); this takes
-// 351 us and 12.4 us.
+// 98 us and 10.7 us (351 us with every token's evaluations left to its warp).
 constexpr int kLaMaxTok = 512;   // tokens of a block
+constexpr int kLaTasks = 512;    // evaluations listed in a step
 constexpr int kLaMaxLoss = 512;  // losses of the last level that the class table takes
 // Up to 16 experts a block has 8 warps and no class table: its set-up (2 us)
 // is longer than the few evaluations it would shorten (14.5 against 12.4 us
 // for 128 tokens of 8 experts). For 64 experts the table took the 2048-token
-// call below from 4620 to 351 us.
+// call above from 4620 to 351 us, a token's evaluations still one after another.
 constexpr int kLaNarrow = 16;
 // bytes of a class's row of counts, one a target: an odd number of words, so
 // that lanes reading one word of different rows hit distinct banks
@@ -854,6 +858,72 @@ __device__ __forceinline__ float la_phi_warp(const LaCtx<D>& c, float* term, int
   return acc;
 }
 
+// V^(D)_q(m, kt) by `width` neighbouring lanes (a power of two), lane `sub` of
+// them taking every width-th substitute; the same value in all of them. Called
+// by whole warps. (The minimum does not depend on the order.)
+template <int D>
+__device__ __forceinline__ float la_value_lanes(const LaCtx<D>& c, int m, int kt, float q, int sub,
+                                                int width) {
+  auto all_min = [&](float x) {
+    for (int o = width >> 1; o; o >>= 1) x = fminf(x, __shfl_xor_sync(0xffffffffu, x, o));
+    return x;
+  };
+  const LaLevel& v = c.lev[D - 1];
+  float best = INFINITY;
+  // entry i of the target's row: expert kk at a loss of q2
+  auto entry = [&](int kk, float cq, float q2, float bound) {
+#pragma unroll 1
+    for (uint32_t pm = v.pmask[kk]; pm; pm &= pm - 1) {
+      const int m2 = __ffs(pm) - 1;
+      const float base = __fadd_rn(v.A[m * c.M + m2], cq);
+      const float least = __fadd_rn(base, c.Ua[D - 2][m2 * c.E + kk]);
+      if (c.prune && (least >= best || least > bound)) continue;
+      best = fminf(best, __fadd_rn(base, la_phi<D, D - 1>(c, m2, kk, q2)));
+    }
+  };
+  if (c.rows) {
+    const float* s = c.sQ[D - 1] + kt * c.pitch;
+    const float* wa = c.Wa[D - 1] + c.woff[D - 1][kt] + m;
+    const float* cn = c.Cn[D - 1] + c.woff[D - 1][kt] + m;
+    const int n = c.nsub[D - 1][kt];
+    unsigned long long neither = 0;  // of this lane's entries
+    float bound = INFINITY;          // some entry's cost is at most this
+    int na = 0;
+    for (int i = sub; i <= n; i += width) {
+      const float q2 = i == 0 ? q : __fadd_rn(q, s[i - 1]);
+      if (i > 0 && !(q2 <= c.qbar)) break;
+      if (la_all<D>(c, D - 1, q2)) {
+        na = i + 1;
+      } else if (la_none<D>(c, D - 1, q2)) {
+        best = fminf(best, cn[i * c.M]);
+      } else {
+        bound = fminf(bound, cn[i * c.M]);
+        neither |= 1ull << i;
+      }
+    }
+    if (na > 0) best = fminf(best, wa[(na - 1) * c.M]);
+    best = all_min(best);
+    bound = all_min(bound);
+#pragma unroll 1
+    for (; neither; neither &= neither - 1) {
+      const int i = __ffsll(static_cast<long long>(neither)) - 1;
+      const int kk = i == 0 ? kt : c.ord[D - 1][kt * 64 + i - 1];
+      entry(kk, i == 0 ? 0.0f : v.Cq[kt * c.E + kk], i == 0 ? q : __fadd_rn(q, s[i - 1]), bound);
+    }
+  } else {
+    int i = 0;
+#pragma unroll 1
+    for (unsigned long long sb = v.subst[kt] | (1ull << kt); sb; sb &= sb - 1, ++i) {
+      if ((i & (width - 1)) != sub) continue;
+      const int kk = __ffsll(static_cast<long long>(sb)) - 1;
+      const float q2 = kk == kt ? q : __fadd_rn(q, v.Q[kt * c.E + kk]);
+      if (kk != kt && !(q2 <= c.qbar)) continue;
+      entry(kk, kk == kt ? 0.0f : v.Cq[kt * c.E + kk], q2, INFINITY);
+    }
+  }
+  return all_min(best);
+}
+
 // Dynamic shared memory for servers up to Mcap, NW warps, level rows of wcap
 // floats (Wa of every level, Cn of all but the last).
 __host__ __device__ inline size_t la_smem_fixed(int E, int D, int Mcap, int NW) {
@@ -873,11 +943,21 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
     uint8_t* __restrict__ chosen_server, uint8_t* __restrict__ kind_out,
     int32_t* __restrict__ counters) {
   constexpr int kThreads = 32 * NW;
+  constexpr int kEmax = NW > 8 ? 64 : kLaNarrow;    // experts that this many warps take
+  constexpr int kRowsPer = (kEmax + NW - 1) / NW;   // rows of a level a warp
+  constexpr int kElems = (kEmax * kEmax + kThreads - 1) / kThreads;  // elements of P a thread
   pdl_trigger();  // launched with launch_pdl: no global access before pdl_wait
   pdl_wait();
   extern __shared__ __align__(16) unsigned char s_raw[];
   __shared__ uint8_t s_ord[D][64 * 64];
-  __shared__ uint16_t s_rank[64 * 64];
+  // the losses' ranks while the tables are built, then the listed evaluations
+  __shared__ __align__(16) unsigned char s_scratch[64 * 64 * 2];
+  static_assert(sizeof(uint4) * kLaTasks <= sizeof(s_scratch), "task list");
+  uint16_t* s_rank = reinterpret_cast<uint16_t*>(s_scratch);
+  uint4* s_task = reinterpret_cast<uint4*>(s_scratch);  // cost0, q, key's low word, warp
+  __shared__ unsigned long long s_best[NW];
+  __shared__ float s_As[NW][32];  // a warp's own row of A
+  __shared__ int s_task_n[2][2];
   __shared__ int s_cnt[32], s_nsub[D][64], s_woff[D][65], s_tok[kLaMaxTok];
   __shared__ int s_part[NW], s_kind[4];
   __shared__ int s_home, s_chunk, s_qmax[D], s_qmin[D];
@@ -885,18 +965,20 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
   const int32_t* hdr = reinterpret_cast<const int32_t*>(tab);
   const int M = hdr[2];
   const float qbar = reinterpret_cast<const float*>(tab)[5];
-  if (hdr[1] != E || M <= 0 || M > Mcap) {
+  if (hdr[1] != E || E > kEmax || M <= 0 || M > Mcap) {
     if (blockIdx.x == 0 && tid == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, -1);
     return;
   }
   // ---- this block's home and tokens: home a has ceil(count / tpb) blocks
   if (tid < 32) s_cnt[tid] = 0;
-  if (tid < 4) s_kind[tid] = 0;
+  if (tid < 4) {
+    s_kind[tid] = 0;
+    s_task_n[tid >> 1][tid & 1] = 0;
+  }
   if (tid < D) {
     s_qmax[tid] = -1;  // no substitute (losses are not negative: their bits order like values)
     s_qmin[tid] = 0x7FFFFFFF;
   }
-  // the layers' losses of this warp's rows, loaded ahead of their use
   LaCtx<D> c;
   c.E = E;
   c.M = M;
@@ -908,13 +990,25 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
   float *U[2 * D], *Wa[D], *Cn[D];
   bool bad_p = false;
   float* sQ[D];
+  float pv[D][kElems];  // every load in flight before the first store
+#pragma unroll
+  for (int i = 0; i < D; ++i) {
+    const float* g = la.P + (size_t)(D - 1 - i) * E * E;
+#pragma unroll
+    for (int u = 0; u < kElems; ++u) {
+      const int x = tid + u * kThreads;
+      pv[i][u] = x < E * E ? g[x] : 0.0f;
+    }
+  }
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     // level i + 1: layer l + D - i, entered from the layer before it by P_{l + D - i - 1}
-    const float* g = la.P + (size_t)(D - 1 - i) * E * E;
-    for (int x = tid; x < E * E; x += kThreads) {
-      sp[x + (x / E) * (c.pitch - E)] = g[x];
-      bad_p |= !(g[x] >= 0.0f);
+#pragma unroll
+    for (int u = 0; u < kElems; ++u) {
+      const int x = tid + u * kThreads;
+      if (x >= E * E) break;
+      sp[x + (x / E) * (c.pitch - E)] = pv[i][u];
+      bad_p |= !(pv[i][u] >= 0.0f);
     }
     c.P[i] = sp;
     sp += E * c.pitch;
@@ -1003,38 +1097,60 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
   }
   if (lane == 31) s_part[warp] = incl;
 
-  // ---- the tables of home a. A warp a row: the losses in order, their extremes
+  // ---- the tables of home a. A warp a row: the losses in order, their extremes.
+  // The rows' sets are loaded together, then their losses.
+  {
+    unsigned long long sets[D][kRowsPer];
+    int loss0[D][kRowsPer], loss1[D][kRowsPer];
 #pragma unroll
-  for (int i = 0; i < D; ++i) {
-    c.lev[i] = la_level(tab + (size_t)(D - i) * la.stride, E, M, a);
-    for (int kt = warp; kt < E; kt += NW) {
-      const unsigned long long sb = c.lev[i].subst[kt];
-      if (lane == 0) s_nsub[i][kt] = __popcll(sb);
-      if (sb == 0ull) continue;
-      const int q0 = (sb >> lane) & 1ull ? __float_as_int(c.lev[i].Q[kt * E + lane]) : -1;
-      const int q1 = (sb >> (lane + 32)) & 1ull ? __float_as_int(c.lev[i].Q[kt * E + lane + 32]) : -1;
-      const int mx = __reduce_max_sync(0xffffffffu, max(q0, q1));
-      const unsigned mn = __reduce_min_sync(0xffffffffu, min(static_cast<unsigned>(q0), static_cast<unsigned>(q1)));
-      if (lane == 0) {
-        atomicMax(&s_qmax[i], mx);
-        atomicMin(&s_qmin[i], static_cast<int>(mn));
-      }
-      int r0 = 0, r1 = 0;
-      for (unsigned long long b = sb; b; b &= b - 1) {
-        const int e = __ffsll(static_cast<long long>(b)) - 1;
-        const int o = __shfl_sync(0xffffffffu, e < 32 ? q0 : q1, e & 31);
-        r0 += (o < q0 || (o == q0 && e < lane)) ? 1 : 0;
-        r1 += (o < q1 || (o == q1 && e < lane + 32)) ? 1 : 0;
-      }
-      if (q0 >= 0) {
-        sQ[i][kt * c.pitch + r0] = __int_as_float(q0);
-        s_ord[i][kt * 64 + r0] = static_cast<uint8_t>(lane);
-      }
-      if (q1 >= 0) {
-        sQ[i][kt * c.pitch + r1] = __int_as_float(q1);
-        s_ord[i][kt * 64 + r1] = static_cast<uint8_t>(lane + 32);
+    for (int i = 0; i < D; ++i) {
+      c.lev[i] = la_level(tab + (size_t)(D - i) * la.stride, E, M, a);
+#pragma unroll
+      for (int u = 0; u < kRowsPer; ++u) {
+        const int kt = warp + u * NW;
+        sets[i][u] = kt < E ? c.lev[i].subst[kt] : 0ull;
       }
     }
+#pragma unroll
+    for (int i = 0; i < D; ++i)
+#pragma unroll
+      for (int u = 0; u < kRowsPer; ++u) {
+        const float* Q = c.lev[i].Q + (warp + u * NW) * E;
+        loss0[i][u] = (sets[i][u] >> lane) & 1ull ? __float_as_int(Q[lane]) : -1;
+        loss1[i][u] = kEmax > 32 && ((sets[i][u] >> (lane + 32)) & 1ull) ? __float_as_int(Q[lane + 32]) : -1;
+      }
+#pragma unroll
+    for (int i = 0; i < D; ++i)
+#pragma unroll
+      for (int u = 0; u < kRowsPer; ++u) {
+        const int kt = warp + u * NW;
+        if (kt >= E) break;
+        const unsigned long long sb = sets[i][u];
+        if (lane == 0) s_nsub[i][kt] = __popcll(sb);
+        if (sb == 0ull) continue;
+        const int q0 = loss0[i][u], q1 = loss1[i][u];
+        const int mx = __reduce_max_sync(0xffffffffu, max(q0, q1));
+        const unsigned mn = __reduce_min_sync(0xffffffffu, min(static_cast<unsigned>(q0), static_cast<unsigned>(q1)));
+        if (lane == 0) {
+          atomicMax(&s_qmax[i], mx);
+          atomicMin(&s_qmin[i], static_cast<int>(mn));
+        }
+        int r0 = 0, r1 = 0;
+        for (unsigned long long b = sb; b; b &= b - 1) {
+          const int e = __ffsll(static_cast<long long>(b)) - 1;
+          const int o = __shfl_sync(0xffffffffu, e < 32 ? q0 : q1, e & 31);
+          r0 += (o < q0 || (o == q0 && e < lane)) ? 1 : 0;
+          r1 += (o < q1 || (o == q1 && e < lane + 32)) ? 1 : 0;
+        }
+        if (q0 >= 0) {
+          sQ[i][kt * c.pitch + r0] = __int_as_float(q0);
+          s_ord[i][kt * 64 + r0] = static_cast<uint8_t>(lane);
+        }
+        if (q1 >= 0) {
+          sQ[i][kt * c.pitch + r1] = __int_as_float(q1);
+          s_ord[i][kt * 64 + r1] = static_cast<uint8_t>(lane + 32);
+        }
+      }
   }
   __syncthreads();
   {  // the tokens of this block, by their rank among home a's
@@ -1047,37 +1163,44 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
     });
   }
   // The classes of level 1: every loss is put at its rank among all of them
-  // (equal losses by target and place), and adds one to the count of its
-  // target in the rows past that rank. (A row between equal losses is never
-  // asked for: both fit or neither does.)
+  // (equal losses by target and place), read as one list, which lies where the
+  // counts go once all ranks are known. (A row of counts between equal losses
+  // is never asked for: both fit or neither does.)
+  int first0, first1;  // where targets 2 lane and 2 lane + 1 start in the list
   {
-    int all = 0, most = 0;
-    for (int kt = 0; kt < E; ++kt) {
-      all += s_nsub[0][kt];
-      most = max(most, s_nsub[0][kt]);
+    const int n0 = 2 * lane < E ? s_nsub[0][2 * lane] : 0;
+    const int n1 = 2 * lane + 1 < E ? s_nsub[0][2 * lane + 1] : 0;
+    int in = n0 + n1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, in, o);
+      if (lane >= o) in += u;
     }
-    c.n_loss = all;
-    c.classes = E > kLaNarrow && all > 0 && all <= la_max_loss(E);
-    if (c.classes) {
-      for (int x = tid; x < E * most; x += kThreads) {
-        const int kt = x / most, n = x - kt * most;
-        if (n >= s_nsub[0][kt]) continue;
-        const float q = c.sQ[0][kt * c.pitch + n];
-        int r = n;
-        for (int k2 = 0; k2 < E; ++k2) {  // losses of target k2 that come before
-          if (k2 == kt) continue;
-          const float* s = c.sQ[0] + k2 * c.pitch;
-          int b = 0, e = s_nsub[0][k2];
-          while (b < e) {
-            const int mid = (b + e) >> 1;
-            if (s[mid] < q || (s[mid] == q && k2 < kt)) b = mid + 1;
-            else e = mid;
-          }
-          r += b;
-        }
-        s_loss[r] = q;
-        s_rank[kt * 64 + n] = static_cast<uint16_t>(r);
+    first0 = in - n0 - n1;
+    first1 = in - n1;
+    c.n_loss = __shfl_sync(0xffffffffu, in, 31);
+    c.classes = E > kLaNarrow && c.n_loss > 0 && c.n_loss <= la_max_loss(E);
+  }
+  auto first_of = [&](int kt) { return __shfl_sync(0xffffffffu, kt & 1 ? first1 : first0, kt >> 1); };
+  if (c.classes) {
+    float* list = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(s_fits) + 15) & ~uintptr_t(15));
+    for (int kt = warp; kt < E; kt += NW) {
+      const int f = first_of(kt);
+      for (int n = lane; n < s_nsub[0][kt]; n += 32) list[f + n] = c.sQ[0][kt * c.pitch + n];
+    }
+    if (tid < 4) list[c.n_loss + tid] = INFINITY;  // the last four's rest: after every loss
+    __syncthreads();
+    for (int x = tid; x < c.n_loss; x += kThreads) {
+      const float q = list[x];
+      int r = 0;
+#pragma unroll 4
+      for (int y = 0; y < c.n_loss; y += 4) {
+        const float4 o = *reinterpret_cast<const float4*>(list + y);
+        r += (o.x < q || (o.x == q && y < x)) + (o.y < q || (o.y == q && y + 1 < x)) +
+             (o.z < q || (o.z == q && y + 2 < x)) + (o.w < q || (o.w == q && y + 3 < x));
       }
+      s_loss[r] = q;
+      s_rank[x] = static_cast<uint16_t>(r);
     }
   }
   // where each target's row starts: (1 + substitutes) M entries, an odd length
@@ -1108,14 +1231,22 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
 #pragma unroll
   for (int i = 0; i < D; ++i) c.rows = c.rows && s_woff[i][64] <= wcap;
   if (c.classes) {
+    // a target a warp, classes lane, lane + 32, ... a lane: the losses below each
     const int pitch = la_class_pitch(E);
+    constexpr int kPer = kLaMaxLoss / 32 + 1;
     for (int kt = warp; kt < E; kt += NW) {
-      const int ns = s_nsub[0][kt];
-      for (int cl = lane; cl <= c.n_loss; cl += 32) {
-        int f = 0;
-        while (f < ns && s_rank[kt * 64 + f] < cl) ++f;
-        s_fits[cl * pitch + kt] = static_cast<uint8_t>(f);
+      const int ns = s_nsub[0][kt], f0 = first_of(kt);
+      int f[kPer];
+#pragma unroll
+      for (int u = 0; u < kPer; ++u) f[u] = 0;
+      for (int n = 0; n < ns; ++n) {
+        const int r = s_rank[f0 + n];
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) f[u] += r < lane + 32 * u ? 1 : 0;
       }
+#pragma unroll
+      for (int u = 0; u < kPer; ++u)
+        if (lane + 32 * u <= c.n_loss) s_fits[(lane + 32 * u) * pitch + kt] = static_cast<uint8_t>(f[u]);
     }
   }
 #pragma unroll
@@ -1204,76 +1335,170 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
   const uint32_t pmask0 = lane < E ? own.pmask[lane] : 0u;
   const uint32_t pmask1 = lane + 32 < E ? own.pmask[lane + 32] : 0u;
   int kind_count[4] = {0, 0, 0, 0};
-  for (int i = warp; i < ntok; i += NW) {
-    const int t = s_tok[i];
-    const int s = (loc != nullptr) ? loc[t] : a;
-    float q = (qhat != nullptr) ? qhat[t] : 0.0f;
-    const int idx = lane < k ? topk_idx[(size_t)t * k + lane] : 0;
-    if (s >= M) {
+  // NW tokens at a time, one a warp, slot by slot: each warp takes its token's
+  // candidates in the two cases and lists the others, then the warps share the
+  // listed evaluations (a few tokens have most of them), then each updates its
+  // token. Counters of a step are cleared a step ahead.
+  int step = 0;
+  for (int base = 0; base < ntok; base += NW) {
+    bool live = base + warp < ntok;
+    const int t = live ? s_tok[base + warp] : 0;
+    const int s = live && loc != nullptr ? loc[t] : a;
+    float q = live && qhat != nullptr ? qhat[t] : 0.0f;
+    const int idx = live && lane < k ? topk_idx[(size_t)t * k + lane] : 0;
+    if (live && s >= M) {
       if (lane == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, t);
-      continue;
+      live = false;
     }
-    if (__any_sync(0xffffffffu, idx < 0 || idx >= E)) continue;  // -1: a NaN token (reported)
+    if (__any_sync(0xffffffffu, idx < 0 || idx >= E)) live = false;  // -1: a NaN token (reported)
     unsigned long long taken = 0;
-    for (int j = 0; j < k; ++j) taken |= 1ull << __shfl_sync(0xffffffffu, idx, j);
-    const float* As = own.A + s * M;
-    int first_server = s;
-    for (int j = 0; j < k; ++j) {
+    for (int j = 0; j < k; ++j) taken |= 1ull << (__shfl_sync(0xffffffffu, idx, j) & 63);
+    const float* As = s_As[warp];
+    if (live && lane < M) s_As[warp][lane] = own.A[s * M + lane];
+    __syncwarp();
+    // the target's set and rows, loaded a slot ahead
+    unsigned long long sb_next = 0;
+    float q_next[2] = {0.0f, 0.0f}, cq_next[2] = {0.0f, 0.0f};
+    auto load_slot = [&](int j) {
       const int r = __shfl_sync(0xffffffffu, idx, j);
-      const unsigned long long sb = own.subst[r] & ~taken;
-      unsigned long long best = ~0ull;
-#pragma unroll 1
-      for (int h = 0; 32 * h < E; ++h) {
+      if (!live) return;
+      sb_next = own.subst[r];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
         const int e = lane + 32 * h;
-        const bool sub = (sb >> e) & 1ull;
-        float cq = 0.0f, qn = q;
-        uint32_t pm = (sub || e == r) ? (h ? pmask1 : pmask0) : 0u;
-        if (sub) {
-          qn = __fadd_rn(q, own.Q[r * E + e]);
-          cq = own.Cq[r * E + e];
-          if (!(qn <= qbar)) pm = 0u;  // Eq. 40 budget
+        if (e < E) {
+          q_next[h] = own.Q[r * E + e];
+          cq_next[h] = own.Cq[r * E + e];
         }
-        const float* Ut = la_all<D>(c, D, qn) ? c.Ua[D - 1] : la_none<D>(c, D, qn) ? c.Un[D - 1] : nullptr;
-        auto key_of = [&](int m, float phi) {
-          const float cost = __fadd_rn(__fadd_rn(As[m], cq), phi);
-          return (static_cast<unsigned long long>(__float_as_uint(cost)) << 32) |
-                 (static_cast<unsigned long long>(sub ? 1u : 0u) << 31) |
-                 (static_cast<unsigned long long>(m != s ? 1u : 0u) << 30) |
-                 (static_cast<unsigned long long>(m) << 8) | static_cast<unsigned long long>(e);
-        };
-        if (Ut != nullptr)
+      }
+    };
+    load_slot(0);
+    int first_server = s;
+    for (int j = 0; j < k; ++j, ++step) {
+      const int r = __shfl_sync(0xffffffffu, idx, j);
+      const unsigned long long sb_r = sb_next;
+      const float q_r[2] = {q_next[0], q_next[1]}, cq_r[2] = {cq_next[0], cq_next[1]};
+      if (j + 1 < k) load_slot(j + 1);
+      int* n_task = &s_task_n[step & 1][0];  // listed, taken
+      unsigned long long best = ~0ull;
+      if (live) {
+        const unsigned long long sb = sb_r & ~taken;
+#pragma unroll
+        for (int h = 0; h < kEmax / 32 + (kEmax < 32); ++h) {
+          const int e = lane + 32 * h;
+          const bool sub = (sb >> e) & 1ull;
+          float cq = 0.0f, qn = q;
+          uint32_t pm = (sub || e == r) ? (h ? pmask1 : pmask0) : 0u;
+          if (sub) {
+            qn = __fadd_rn(q, q_r[h]);
+            cq = cq_r[h];
+            if (!(qn <= qbar)) pm = 0u;  // Eq. 40 budget
+          }
+          const float* Ut = la_all<D>(c, D, qn) ? c.Ua[D - 1] : la_none<D>(c, D, qn) ? c.Un[D - 1] : nullptr;
+          // the key's low word: substitute, away, server, expert
+          auto low_of = [&](int m) {
+            return (sub ? 0x80000000u : 0u) | (m != s ? 0x40000000u : 0u) |
+                   (static_cast<uint32_t>(m) << 8) | static_cast<uint32_t>(e);
+          };
+          uint32_t left = 0u;  // not listed for want of room
           for (; pm; pm &= pm - 1) {
             const int m = __ffs(pm) - 1;
-            const unsigned long long key = key_of(m, Ut[m * E + e]);
-            best = key < best ? key : best;
-          }
-        // candidates in neither case, one after another by the whole warp, but
-        // those that cost more than another at best (Ua is the least of Phi)
-        for (unsigned todo = __ballot_sync(0xffffffffu, pm != 0u); todo; todo &= todo - 1) {
-          const int src = __ffs(todo) - 1;
-          const uint32_t pms = __shfl_sync(0xffffffffu, pm, src);
-          const float qs = __shfl_sync(0xffffffffu, qn, src), cqs = __shfl_sync(0xffffffffu, cq, src);
-          for (uint32_t x = pms; x; x &= x - 1) {
-            const int m = __ffs(x) - 1;
-            const float least = __fadd_rn(__fadd_rn(As[m], cqs), c.Ua[D - 1][m * E + src + 32 * h]);
-            if (__any_sync(0xffffffffu, c.prune && best != ~0ull && least > __uint_as_float(static_cast<unsigned>(best >> 32)))) continue;
-            const float phi = la_phi_warp<D>(c, s_term, lane, m, src + 32 * h, qs);
-            if (lane == src) {
-              const unsigned long long key = key_of(m, phi);
+            const float cost0 = __fadd_rn(As[m], cq);
+            if (Ut != nullptr) {
+              const unsigned long long key =
+                  (static_cast<unsigned long long>(__float_as_uint(__fadd_rn(cost0, Ut[m * E + e]))) << 32) | low_of(m);
               best = key < best ? key : best;
+              continue;
+            }
+            const int i = atomicAdd(n_task, 1);
+            if (i < kLaTasks) s_task[i] = make_uint4(__float_as_uint(cost0), __float_as_uint(qn), low_of(m), warp);
+            else left |= 1u << m;
+          }
+          for (unsigned todo = __ballot_sync(0xffffffffu, left != 0u); todo; todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const float qs = __shfl_sync(0xffffffffu, qn, src);
+            for (uint32_t x = __shfl_sync(0xffffffffu, left, src); x; x &= x - 1) {
+              const int m = __ffs(x) - 1;
+              const float phi = la_phi_warp<D>(c, s_term, lane, m, src + 32 * h, qs);
+              if (lane == src) {
+                const unsigned long long key =
+                    (static_cast<unsigned long long>(__float_as_uint(__fadd_rn(__fadd_rn(As[m], cq), phi))) << 32) | low_of(m);
+                best = key < best ? key : best;
+              }
             }
           }
         }
+        // the smallest key of the warp: high words, then the low words among those
+        const unsigned hi = static_cast<unsigned>(best >> 32);
+        const unsigned mhi = __reduce_min_sync(0xffffffffu, hi);
+        const unsigned mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? static_cast<unsigned>(best) : 0xffffffffu);
+        if (lane == 0) s_best[warp] = (static_cast<unsigned long long>(mhi) << 32) | mlo;
       }
-      // the smallest key of the warp: high words, then the low words among those
-      const unsigned hi = static_cast<unsigned>(best >> 32);
-      const unsigned mhi = __reduce_min_sync(0xffffffffu, hi);
-      const unsigned mlo = __reduce_min_sync(0xffffffffu, hi == mhi ? static_cast<unsigned>(best) : 0xffffffffu);
+      __syncthreads();
+      if (tid == 0) s_task_n[(step + 1) & 1][0] = s_task_n[(step + 1) & 1][1] = 0;
+      const int nt = min(n_task[0], kLaTasks);
+      // passed over when it costs more than another at best (Ua is the least of Phi)
+      auto passed_over = [&](float cost0, uint32_t low, unsigned long long so_far) {
+        const int m = static_cast<int>((low >> 8) & 0xFFu), e = static_cast<int>(low & 0xFFu);
+        return c.prune && so_far != ~0ull &&
+               __fadd_rn(cost0, c.Ua[D - 1][m * E + e]) > __uint_as_float(static_cast<unsigned>(so_far >> 32));
+      };
+      if constexpr (D > 1 && NW > 8) {
+        // all warps on one evaluation: a group of lanes a target
+        int width = 1;
+        while (2 * width * E <= kThreads && width < 8) width *= 2;
+#pragma unroll 1
+        for (int i = 0; i < nt; ++i) {
+          const uint4 task = s_task[i];
+          const float cost0 = __uint_as_float(task.x), qn = __uint_as_float(task.y);
+          if (passed_over(cost0, task.z, s_best[task.w])) continue;  // the same for the block
+          const int m = static_cast<int>((task.z >> 8) & 0xFFu), e = static_cast<int>(task.z & 0xFFu);
+          float* term = reinterpret_cast<float*>(s_raw);
+          const int sub = tid & (width - 1), kt = tid / width;
+          for (int k0 = 0; k0 < E; k0 += kThreads / width) {
+            const int kv = min(k0 + kt, E - 1);
+            const float p = c.P[D - 1][e * c.pitch + kv];
+            const float x = la_value_lanes<D>(c, m, kv, qn, sub, width);
+            if (sub == 0 && k0 + kt < E) term[k0 + kt] = p != 0.0f ? __fmul_rn(p, x) : 0.0f;
+          }
+          __syncthreads();
+          if (tid == 0) {
+            float phi = 0.0f;
+#pragma unroll 8
+            for (int kv = 0; kv < E; ++kv) phi = __fadd_rn(phi, term[kv]);
+            const unsigned long long key =
+                (static_cast<unsigned long long>(__float_as_uint(__fadd_rn(cost0, phi))) << 32) | task.z;
+            if (key < s_best[task.w]) s_best[task.w] = key;
+          }
+          __syncthreads();
+        }
+      } else {
+        // an evaluation a warp
+        while (nt > 0) {
+          int i = 0;
+          if (lane == 0) i = atomicAdd(n_task + 1, 1);
+          i = __shfl_sync(0xffffffffu, i, 0);
+          if (i >= nt) break;
+          const uint4 task = s_task[i];
+          const float cost0 = __uint_as_float(task.x);
+          const unsigned long long so_far = *static_cast<volatile unsigned long long*>(&s_best[task.w]);
+          if (__any_sync(0xffffffffu, passed_over(cost0, task.z, so_far))) continue;
+          const float phi = la_phi_warp<D>(c, s_term, lane, static_cast<int>((task.z >> 8) & 0xFFu),
+                                           static_cast<int>(task.z & 0xFFu), __uint_as_float(task.y));
+          if (lane == 0)
+            atomicMin(&s_best[task.w],
+                      (static_cast<unsigned long long>(__float_as_uint(__fadd_rn(cost0, phi))) << 32) | task.z);
+        }
+      }
+      __syncthreads();
+      if (!live) continue;
+      best = s_best[warp];
       int kstar, mstar, kd;
-      if (mhi == 0xffffffffu && mlo == 0xffffffffu) {
+      if (best == ~0ull) {
         if (lane == 0) report(&g_err_route, ORDERMOE_DEV_NO_CANDIDATE, t);
         kstar = r; mstar = s; kd = 0;
       } else {
+        const uint32_t mlo = static_cast<uint32_t>(best);
         kstar = static_cast<int>(mlo & 0xFFu);
         mstar = static_cast<int>((mlo >> 8) & 0xFFu);
         const int sub = static_cast<int>((mlo >> 31) & 1u);
@@ -1292,7 +1517,7 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
 #pragma unroll
       for (int x = 0; x < 4; ++x) kind_count[x] += kd == x ? 1 : 0;
     }
-    if (lane == 0 && loc != nullptr) {
+    if (live && lane == 0 && loc != nullptr) {
       loc[t] = static_cast<uint8_t>(first_server);
       qhat[t] = q;
     }
@@ -1957,7 +2182,7 @@ static cudaError_t lookahead_launch(int T, int E, int Mcap, int k, const int32_t
                                     cudaStream_t stream) {
   // rows for every substitute set there can be, or as many as fit beside the
   // rest of a block's shared memory (200 KB of the 227; the static arrays
-  // take up to 16 KB more)
+  // take up to 26 KB more)
   const size_t fixed = la_smem_fixed(E, D, Mcap, NW);
   long long wcap = (long long)E * ((E * Mcap) | 1);
   const long long room = (200 * 1024 - (long long)fixed) / ((2 * D - 1) * (long long)sizeof(float));

@@ -147,6 +147,8 @@ def test_route_select_lookahead_given_logits_bit_exact(E, M, k, H, cheap):
     (5001, 8, 4, 2, 3, True),     # several tokens a warp, one home with most of them, a ragged last block
     (6, 64, 8, 6, 3, False),      # two experts a lane, every loss regime, prefix minima in the table
     (40, 64, 32, 2, 2, False),    # prefix minima too many for the table: the direct minimum
+    (64, 64, 32, 2, 2, True),     # more open evaluations in a step than are listed
+    (20, 24, 3, 4, 3, True),      # an evaluation by all warps, lanes past the targets
     (4, 33, 32, 3, 3, True), (60, 1, 1, 1, 4, False), (17, 13, 2, 8, 4, False)])
 def test_lookahead_tokens_by_home_bit_exact(T, E, M, k, H, skew):
     """Losses spread over the whole budget, so that candidates fall on the
