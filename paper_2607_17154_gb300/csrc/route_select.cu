@@ -815,6 +815,7 @@ __device__ __forceinline__ float la_phi(const LaCtx<D>& c, int m, int kx, float 
     }
     const uint8_t* fits = c.fits + lo * la_class_pitch(c.E);
     const float* wa = c.Wa[0] + m;
+#pragma unroll 2
     for (int k4 = 0; k4 < c.E; k4 += 4) {
       const uint32_t n4 = *reinterpret_cast<const uint32_t*>(fits + k4);
 #pragma unroll
@@ -1188,18 +1189,22 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
       const int f = first_of(kt);
       for (int n = lane; n < s_nsub[0][kt]; n += 32) list[f + n] = c.sQ[0][kt * c.pitch + n];
     }
-    if (tid < 4) list[c.n_loss + tid] = INFINITY;  // the last four's rest: after every loss
+    if (tid < 4) list[c.n_loss + tid] = __int_as_float(0x7FFFFFFF);  // the last four's rest: after every loss
     __syncthreads();
     for (int x = tid; x < c.n_loss; x += kThreads) {
-      const float q = list[x];
+      // losses are not negative: their bits order like values. Before the four
+      // that hold x an equal loss counts, after them it does not.
+      const int q = __float_as_int(list[x]), x4 = x & ~3;
+      const int4* l4 = reinterpret_cast<const int4*>(list);
       int r = 0;
 #pragma unroll 4
       for (int y = 0; y < c.n_loss; y += 4) {
-        const float4 o = *reinterpret_cast<const float4*>(list + y);
-        r += (o.x < q || (o.x == q && y < x)) + (o.y < q || (o.y == q && y + 1 < x)) +
-             (o.z < q || (o.z == q && y + 2 < x)) + (o.w < q || (o.w == q && y + 3 < x));
+        const int4 o = l4[y >> 2];
+        const int below = y < x4 ? q + 1 : q;
+        r += (o.x < below ? 1 : 0) + (o.y < below ? 1 : 0) + (o.z < below ? 1 : 0) + (o.w < below ? 1 : 0);
       }
-      s_loss[r] = q;
+      for (int y = x4; y < x; ++y) r += __float_as_int(list[y]) == q ? 1 : 0;
+      s_loss[r] = __int_as_float(q);
       s_rank[x] = static_cast<uint16_t>(r);
     }
   }

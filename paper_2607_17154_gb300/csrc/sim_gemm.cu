@@ -1,7 +1,8 @@
 // Offline similarity on the tensor cores (Section III-B, Eqs. 3-5; Alg. 1)
 // for E in {8, 16, 32, 64}:
 //   sim_logits_kernel<E>: H = X_cal W^T for the L routers stacked (W rows =
-//     L * E), one 128-token x 256-logit tile per step of a persistent loop
+//     L * E), one 128-token x 256-logit tile (narrower when there are fewer
+//     such tiles than SMs) per step of a persistent loop
 //     (TMA ring, tcgen05.mma, two TMEM accumulators, as in the expert FFN).
 //     The epilogue writes H in fp32, token-major (the workspace contract),
 //     writes H^T as two bf16 planes, hi = bf16(h) and lo = bf16(h - hi),
@@ -54,7 +55,6 @@ constexpr int THREADS = 192;    // Gram: TMA, MMA, 4 epilogue warps
 constexpr int L_EPI_WARPS = 16;  // logits epilogue: four warps per TMEM lane quarter
 constexpr int L_THREADS = 64 + 32 * L_EPI_WARPS;  // + TMA and MMA warps
 constexpr int TMEM_COLS = 512;
-constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN);
 constexpr int MAX_HIST = 4096;  // L * E counters in shared memory
 
 constexpr int G_ROWS = 64;  // rows of H^T per Gram block
@@ -71,7 +71,7 @@ constexpr uint32_t G_IDESC = idesc_bf16_f32(128, 128);
 // memory traffic per flop), six stages deep.
 constexpr int P_STAGES = 6;
 constexpr int P_STAGE_BYTES = A_BYTES + BOX_BYTES;
-constexpr int L_MAX_STAGES = P_STAGES > STAGES ? P_STAGES : STAGES;
+constexpr int L_MAX_STAGES = 8;  // of the narrowest column slice: 24 KB a stage
 static_assert(P_STAGES * P_STAGE_BYTES <= STAGES * STAGE_BYTES, "pair ring fits the 1-CTA ring's space");
 
 struct LSmem {
@@ -101,7 +101,11 @@ struct LArgs {
   int N;            // calibration tokens (rows of X)
   int C;            // L * E logit columns
   int K;            // d
-  int n_tiles;      // 256-column slices
+  int bn;           // columns of a tile: 256, or 128 or 64 in the one-CTA variant
+  int stages;       // one-CTA variant: the ring's depth and bytes a stage
+  int stage_bytes;
+  uint32_t idesc;
+  int n_tiles;      // bn-column slices
   int L;
   int kf;           // k_freq of Eq. 5
   float* H;         // [N][C] fp32, or null: not written
@@ -187,8 +191,9 @@ template <int E, int NK, bool PAIR>
 __global__ void __launch_bounds__(L_THREADS, 1)
     sim_logits_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapW,
                       LArgs args) {
-  constexpr int KSTAGES = PAIR ? P_STAGES : STAGES;
-  constexpr int KSTAGE_BYTES = PAIR ? P_STAGE_BYTES : STAGE_BYTES;
+  const int KSTAGES = PAIR ? P_STAGES : args.stages;
+  const int KSTAGE_BYTES = PAIR ? P_STAGE_BYTES : args.stage_bytes;
+  const int bn = PAIR ? BN : args.bn;
   constexpr int TBM = PAIR ? 2 * BM : BM;  // tokens per tile
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>(
@@ -269,10 +274,11 @@ __global__ void __launch_bounds__(L_THREADS, 1)
             tma_load_2d_pair(sa, &mapX, full_even, kb * BK, mt * TBM + static_cast<int>(rp) * BM);
             tma_load_2d_pair(sa + A_BYTES, &mapW, full_even, kb * BK, n * BN + static_cast<int>(rp) * 128);
           } else {
-            mbar_arrive_expect_tx(&s.full[stage], STAGE_BYTES);
+            mbar_arrive_expect_tx(&s.full[stage], KSTAGE_BYTES);
             tma_load_2d(sa, &mapX, &s.full[stage], kb * BK, mt * BM);
-            tma_load_2d(sa + A_BYTES, &mapW, &s.full[stage], kb * BK, n * BN);
-            tma_load_2d(sa + A_BYTES + BOX_BYTES, &mapW, &s.full[stage], kb * BK, n * BN + 128);
+            tma_load_2d(sa + A_BYTES, &mapW, &s.full[stage], kb * BK, n * bn);
+            if (bn == BN)
+              tma_load_2d(sa + A_BYTES + BOX_BYTES, &mapW, &s.full[stage], kb * BK, n * bn + 128);
           }
         }
         issued_mask |= 1u << stage;
@@ -312,7 +318,7 @@ __global__ void __launch_bounds__(L_THREADS, 1)
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {  // 16 elements = 32 bytes on
               if (PAIR) mma_bf16_pair(d_tmem, da + 2 * kk, db + 2 * kk, idesc_bf16_f32(256, BN), (kb | kk) != 0 ? 1u : 0u);
-              else mma_bf16(d_tmem, da + 2 * kk, db + 2 * kk, IDESC, (kb | kk) != 0 ? 1u : 0u);
+              else mma_bf16(d_tmem, da + 2 * kk, db + 2 * kk, args.idesc, (kb | kk) != 0 ? 1u : 0u);
             }
             if (PAIR) mma_commit_pair(&s.empty[stage], 0x3);
             else mma_commit(&s.empty[stage]);
@@ -356,8 +362,8 @@ __global__ void __launch_bounds__(L_THREADS, 1)
 #pragma unroll
       for (int half = 0; half < 2; ++half) {  // the two 32-column chunks of the warp's part
         const int c = 2 * part + half;
-        const int cb = n * BN + c * 32;
-        if (cb >= args.C) break;  // warp-uniform
+        const int cb = n * bn + c * 32;
+        if (c * 32 >= bn || cb >= args.C) break;  // warp-uniform
         uint32_t v[32];
         tmem_ld32(tb + c * 32, v);
         tmem_ld_wait();
@@ -808,15 +814,38 @@ int sim_tc_launch(const uint16_t* X, int N, const uint16_t* W, int L, int E, int
   if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute(similarity)");
   CUtensorMap mX, mW, mHi, mLo;
   int rc;
+  int sms = num_sms();
+  if (reserve_sm && sms > 1) {
+    --sms;
+    const size_t whole = static_cast<size_t>(whole_sm_smem());
+    if (whole > lsmem) lsmem = whole;
+    if (whole > gsmem) gsmem = whole;
+  }
+  // One CTA a tile: a K step is bound by the bytes the CTA copies (its 128 tokens
+  // and bn weight rows), so the slice is the one with the fewest bytes a step
+  // times rounds over the SMs, the widest among equals. 4096 tokens, 32 layers x
+  // 8 experts, d 4096: 32 tiles of 256 columns 31.8 us, 128 of 64 columns 23.2 us.
+  const bool pair = E == 64 && kf <= 8;
+  const long long mtiles = (N + BM - 1) / BM;
+  int bn = BN;
+  if (!pair)
+    for (int w = 128; w >= 64; w /= 2) {
+      auto cost = [&](int x) { return (BM + x) * ((mtiles * ((C + x - 1) / x) + sms - 1) / sms); };
+      if (cost(w) < cost(bn)) bn = w;
+    }
   if ((rc = make_tmap_bf16(&mX, X, N, d, 128))) return rc;
-  if ((rc = make_tmap_bf16(&mW, W, C, d, 128))) return rc;
+  if ((rc = make_tmap_bf16(&mW, W, C, d, bn < 128 ? bn : 128))) return rc;
   if ((rc = make_map_ld(&mHi, hi, C, N, ldT))) return rc;
   if ((rc = make_map_ld(&mLo, lo, C, N, ldT))) return rc;
   LArgs la{};
   la.N = N;
   la.C = C;
   la.K = d;
-  la.n_tiles = (C + BN - 1) / BN;
+  la.bn = bn;
+  la.stage_bytes = A_BYTES + bn * BK * 2;
+  la.stages = bn == BN ? STAGES : bn == 128 ? P_STAGES : L_MAX_STAGES;
+  la.idesc = idesc_bf16_f32(128, bn);
+  la.n_tiles = (C + bn - 1) / bn;
   la.L = L;
   la.kf = kf;
   la.H = H;
@@ -825,16 +854,9 @@ int sim_tc_launch(const uint16_t* X, int N, const uint16_t* W, int L, int E, int
   la.ldT = ldT;
   la.counts = counts;
   la.limit_ns = wait_limit_ns();
-  const long long tiles = (long long)((N + BM - 1) / BM) * la.n_tiles;
-  int sms = num_sms();
-  if (reserve_sm && sms > 1) {
-    --sms;
-    const size_t whole = static_cast<size_t>(whole_sm_smem());
-    if (whole > lsmem) lsmem = whole;
-    if (whole > gsmem) gsmem = whole;
-  }
+  const long long tiles = mtiles * la.n_tiles;
   const int grid = static_cast<int>(tiles < sms ? tiles : sms);
-  if (E == 64 && kf <= 8) {
+  if (pair) {
     // CTA pairs over 256-token tiles, at most one pair per two SMs
     const long long ptiles = (long long)((N + 2 * BM - 1) / (2 * BM)) * la.n_tiles;
     const int pairs = static_cast<int>(ptiles < sms / 2 ? ptiles : sms / 2);

@@ -54,6 +54,37 @@ def test_similarity_matches_oracle(L, E, d, N, kf, K):
         assert np.abs(counts[l] - ref_counts).sum() <= max(2, N // 500), (counts[l], ref_counts)
 
 
+@pytest.mark.parametrize("L,E,d,N,kf,K", [
+    (32, 8, 128, 4096, 2, 4),     # 64-column tiles: one round of the SMs
+    (32, 8, 128, 8960, 2, 4),     # 128-column tiles
+    (32, 8, 64, 19584, 2, 4),     # 256-column tiles, two rounds
+    (5, 16, 128, 1100, 3, 4),     # a last slice with 16 of its 64 columns
+    (3, 64, 64, 700, 9, 8)])      # a layer a slice, its two halves in turn
+def test_similarity_column_slices(L, E, d, N, kf, K):
+    """The width of the logits' column tiles follows from the number of tiles:
+    the logits equal an fp64 product up to fp32 accumulation (d + 1 roundings
+    of at most the sum of the terms' magnitudes), the counts are Eq. 5 of those
+    very logits, the similarity is within the suite's bound."""
+    Wr = torch.stack([synth.router_weights(E, d, K, seed=30 + l) for l in range(L)])
+    Xcal = synth.calibration(N, d, seed=L + E)
+    ws = torch.empty(B.ordermoe_similarity_workspace_bytes(L, E, N), dtype=torch.uint8, device=DEV)
+    sim = torch.empty(L, E, E, dtype=torch.float32, device=DEV)
+    cnt = torch.empty(L, E, dtype=torch.int32, device=DEV)
+    B.ordermoe_similarity(Wr.to(DEV).contiguous(), Xcal.to(DEV), L, E, d, N, kf, sim, cnt, ws)
+    H = ws[: N * L * E * 4].view(torch.float32).view(N, L * E).cpu()
+    W2 = Wr.view(L * E, d).double()
+    ref = Xcal.double() @ W2.T
+    bound = (d + 1) * 2.0 ** -23 * (Xcal.double().abs() @ W2.abs().T)
+    assert ((H.double() - ref).abs() <= bound).all()
+    for l in range(L):
+        want = oracle.expert_counts(np.ascontiguousarray(H[:, l * E:(l + 1) * E].numpy()), kf)
+        np.testing.assert_array_equal(cnt[l].cpu().numpy(), want)
+        h = ref[:, l * E:(l + 1) * E]
+        g = h.T @ h
+        n = g.diagonal().sqrt()
+        np.testing.assert_allclose(sim[l].cpu().numpy(), (g / n[:, None] / n[None, :]).numpy(), atol=2e-5, rtol=0)
+
+
 @pytest.mark.parametrize("L,E,d,N,kf", [(3, 64, 512, 3000, 6), (2, 16, 128, 700, 3), (2, 12, 128, 1000, 3)])
 def test_similarity_no_logits_same_results(L, E, d, N, kf):
     # the entry point that skips the fp32 logits gives the same sim and counts bit for bit
