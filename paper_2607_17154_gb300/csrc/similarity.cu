@@ -1246,16 +1246,28 @@ constexpr int kRepThreads = 512;
 constexpr int kRepMaxCand = 16384;
 constexpr int kRepMaxLayers = 1024;
 
-// Redundant deployment for one server (blockIdx.x = m), Eqs. 32-35. The
-// candidates (l, j) get the key (benefit bits, then candidate id), are sorted
-// by benefit desc and id asc (bitonic sort in shared memory), and are deployed
-// in that order while the group is uncovered and the replica fits. Benefits
-// are positive fp64 values, so their bit patterns order like the values;
-// non-positive and NaN benefits get key 0 and are never taken. A server's
-// state (b_m and its covered groups) changes only when it takes a candidate,
-// so one warp tests 32 sorted candidates at a time against the current state
-// and takes the first that passes: every candidate it passes over failed
-// under the same state it would have met one at a time.
+// Redundant deployment for one server (blockIdx.x = m), Eqs. 32-35: the
+// candidates (l, j) are deployed in the order (benefit desc, candidate id asc)
+// while the group is uncovered and the replica fits. Benefits are positive
+// fp64 values, so their bit patterns order like the values; non-positive and
+// NaN benefits are never taken.
+//
+// Only candidates that can be taken are ordered. The server's load b_m never
+// falls (p > 0, and rounding is monotone) and its covered groups stay covered,
+// so a candidate that fails against the initial state fails always. Of two
+// candidates of one group, the later is never taken when its p is at least the
+// earlier's: when the earlier was taken the group is covered, and when it did
+// not fit the later does not either. Up to kRepThreads candidates are ordered
+// by counting those before each, more by a bitonic sort in shared memory. One
+// warp then tests 32 at a time against the current state and takes the first
+// that passes: every candidate it passes over failed under the same state it
+// would have met one at a time.
+//
+// Bound: latency of one block a server (barriers of the sort, fp64 chain of the
+// takes). All candidates in one bitonic sort, and a window read again after
+// each take, took 54.6 us for 24 layers x 64 experts on 8 full servers and 24.0
+// us for 32 x 8 on 4 servers with room for as many again; this takes 8.2
+// and 17.9 (ncu).
 __global__ void __launch_bounds__(kRepThreads) replicate_kernel(
     const int32_t* __restrict__ group, const double* __restrict__ importance,
     const double* __restrict__ p, const double* __restrict__ C, const double* __restrict__ pi,
@@ -1265,107 +1277,157 @@ __global__ void __launch_bounds__(kRepThreads) replicate_kernel(
   unsigned long long* key = reinterpret_cast<unsigned long long*>(s_rep);
   unsigned long long* cov = key + Np;  // [L]: bit g = group g covered (Eq. 32)
   uint32_t* cid = reinterpret_cast<uint32_t*>(cov + L);
+  __shared__ int n_cand;
   const int m = blockIdx.x;
   const int t = threadIdx.x;
+  const int lane = t & 31;
+  const unsigned full = 0xffffffffu;
   const int N = L * E;
-  for (int l = t; l < L; l += blockDim.x) {
-    unsigned long long bits = 0;
-    for (int j = 0; j < E; ++j) {
-      const int g = group[(size_t)l * E + j];
-      if (placement[((size_t)l * M + m) * E + j] && g >= 0 && g < E) bits |= 1ull << g;
-    }
-    cov[l] = bits;
+  if (t == 0) n_cand = 0;
+  for (int l = t; l < L; l += kRepThreads) cov[l] = 0ull;
+  __syncthreads();
+  for (int i = t; i < N; i += kRepThreads) {
+    const int g = group[i], l = i / E;
+    const bool here = placement[((size_t)l * M + m) * E + (i - l * E)] != 0;
+    if (here && g >= 0 && g < E) atomicOr(&cov[l], 1ull << g);
   }
   const double pim = pi[m];
-  for (int i = t; i < Np; i += blockDim.x) {
+  const double b0 = used[m], cap = C[m];
+  __syncthreads();
+  // benefits of the candidates that pass the initial state (0: none), their groups
+  for (int i = t; i < N; i += kRepThreads) {
     unsigned long long k = 0;
-    if (i < N) {
-      const int g = group[i];
-      const double pj = p[i];
-      if (g < 0 || g >= E) {
-        if (m == 0) report(&g_err_sim, ORDERMOE_DEV_BAD_INDEX, i);
-      } else if (!(pj > 0.0)) {
-        if (m == 0) report(&g_err_sim, ORDERMOE_DEV_BAD_VALUE, i);
-      } else {
-        const double ben = __ddiv_rn(__dmul_rn(pim, importance[i]), pj);  // Eq. 33, y = 0
-        if (ben > 0.0) k = static_cast<unsigned long long>(__double_as_longlong(ben));
-      }
+    const int g = group[i];
+    const double pj = p[i];
+    if (g < 0 || g >= E) {
+      if (m == 0) report(&g_err_sim, ORDERMOE_DEV_BAD_INDEX, i);
+    } else if (!(pj > 0.0)) {
+      if (m == 0) report(&g_err_sim, ORDERMOE_DEV_BAD_VALUE, i);
+    } else if (!((cov[i / E] >> g) & 1ull) && __dadd_rn(b0, pj) <= cap) {  // Eqs. 32, 35
+      const double ben = __ddiv_rn(__dmul_rn(pim, importance[i]), pj);     // Eq. 33, y = 0
+      if (ben > 0.0) k = static_cast<unsigned long long>(__double_as_longlong(ben));
     }
     key[i] = k;
-    cid[i] = i < N ? static_cast<uint32_t>(i) : 0xFFFFFFFFu;
+    cid[i] = static_cast<uint32_t>(g);
   }
   __syncthreads();
-  // bitonic sort into (key desc, cid asc)
-  for (int size = 2; size <= Np; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int i = t; i < Np; i += blockDim.x) {
-        const int o = i ^ stride;
-        if (o > i) {
-          const unsigned long long ki = key[i], ko = key[o];
-          const uint32_t ci = cid[i], co = cid[o];
-          const bool o_first = ko > ki || (ko == ki && co < ci);
-          const bool i_first = ki > ko || (ki == ko && ci < co);
-          if ((i & size) == 0 ? o_first : i_first) {
-            key[i] = ko; key[o] = ki;
-            cid[i] = co; cid[o] = ci;
+  // kept: not after another of its group that asks for no more memory
+  uint32_t keep = 0;  // bit r: candidate r kRepThreads + t
+  static_assert(kRepMaxCand <= 32 * kRepThreads, "a bit a candidate of the thread");
+  for (int i = t, r = 0; i < N; i += kRepThreads, ++r) {
+    const unsigned long long k = key[i];
+    if (k == 0) continue;
+    const uint32_t g = cid[i];
+    const double pj = p[i];
+    const int l0 = i / E * E;
+    bool stays = true;
+    for (int o = l0; o < l0 + E && stays; ++o) {
+      const unsigned long long ko = key[o];
+      if ((ko > k || (ko == k && o < i)) && cid[o] == g) stays = !(p[o] <= pj);
+    }
+    if (stays) keep |= 1u << r;
+  }
+  __syncthreads();
+  // their keys and ids moved to the front, kRepThreads candidates at a time (a
+  // round writes only where it and the rounds before it have been read)
+  for (int r = 0; r * kRepThreads < N; ++r) {
+    const bool mine = (keep >> r) & 1u;
+    const int i = r * kRepThreads + t;
+    const unsigned long long k = mine ? key[i] : 0ull;
+    const unsigned bal = __ballot_sync(full, mine);
+    int at = 0;
+    if (lane == 0 && bal != 0u) at = atomicAdd(&n_cand, __popc(bal));
+    at = __shfl_sync(full, at, 0) + __popc(bal & ((1u << lane) - 1u));
+    __syncthreads();
+    if (mine) {
+      key[at] = k;
+      cid[at] = static_cast<uint32_t>(i);
+    }
+    __syncthreads();
+  }
+  const int nc = n_cand;
+  if (nc > kRepThreads) {
+    int ns = 1;
+    while (ns < nc) ns <<= 1;  // <= Np
+    for (int i = nc + t; i < ns; i += kRepThreads) {
+      key[i] = 0ull;
+      cid[i] = 0xFFFFFFFFu;
+    }
+    __syncthreads();
+    // bitonic sort into (key desc, cid asc)
+    for (int size = 2; size <= ns; size <<= 1) {
+      for (int stride = size >> 1; stride > 0; stride >>= 1) {
+        for (int i = t; i < ns; i += kRepThreads) {
+          const int o = i ^ stride;
+          if (o > i) {
+            const unsigned long long ki = key[i], ko = key[o];
+            const uint32_t ci = cid[i], co = cid[o];
+            const bool o_first = ko > ki || (ko == ki && co < ci);
+            const bool i_first = ki > ko || (ki == ko && ci < co);
+            if ((i & size) == 0 ? o_first : i_first) {
+              key[i] = ko; key[o] = ki;
+              cid[i] = co; cid[o] = ci;
+            }
           }
         }
+        __syncthreads();
       }
-      __syncthreads();
     }
   }
-  // the candidates (key != 0) are a prefix of the sorted order; each sorted
-  // slot is repacked in place as (l, g, j) and the bits of p_{l,j}
-  __shared__ int n_cand;
-  if (t == 0) n_cand = 0;
-  __syncthreads();
-  int mine = 0;
-  for (int s = t; s < N; s += blockDim.x) {
-    if (key[s] == 0) continue;
-    ++mine;
-    const int i = static_cast<int>(cid[s]);
-    const int l = i / E, j = i - l * E;
-    cid[s] = (static_cast<uint32_t>(l) << 12) | (static_cast<uint32_t>(group[i]) << 6) |
-             static_cast<uint32_t>(j);
-    key[s] = static_cast<unsigned long long>(__double_as_longlong(p[i]));
+  // each sorted slot holds (l, g, j) and the bits of p_{l,j}
+  if (nc <= kRepThreads) {
+    int rank = 0, i = 0;
+    if (t < nc) {
+      const unsigned long long k = key[t];
+      i = static_cast<int>(cid[t]);
+#pragma unroll 4
+      for (int o = 0; o < nc; ++o) {
+        const unsigned long long ko = key[o];
+        rank += ko > k || (ko == k && cid[o] < static_cast<uint32_t>(i)) ? 1 : 0;
+      }
+    }
+    __syncthreads();
+    if (t < nc) {
+      const int l = i / E;
+      cid[rank] = (static_cast<uint32_t>(l) << 12) | (static_cast<uint32_t>(group[i]) << 6) |
+                  static_cast<uint32_t>(i - l * E);
+      key[rank] = static_cast<unsigned long long>(__double_as_longlong(p[i]));
+    }
+  } else {
+    for (int s = t; s < nc; s += kRepThreads) {
+      const int i = static_cast<int>(cid[s]), l = i / E;
+      cid[s] = (static_cast<uint32_t>(l) << 12) | (static_cast<uint32_t>(group[i]) << 6) |
+               static_cast<uint32_t>(i - l * E);
+      key[s] = static_cast<unsigned long long>(__double_as_longlong(p[i]));
+    }
   }
-  if (mine) atomicAdd(&n_cand, mine);
   __syncthreads();
   if (t < 32) {
-    const unsigned full = 0xffffffffu;
-    const int nc = n_cand;
-    double b = used[m];
-    const double cap = C[m];
+    double b = b0;
     int count = 0;
-    for (int base = 0; base < nc;) {
-      const int s = base + t;
-      uint32_t rec = 0;
-      double pj = 0.0;
-      bool take = false;
-      if (s < nc) {
-        rec = cid[s];
-        pj = __longlong_as_double(static_cast<long long>(key[s]));
-        const int l = static_cast<int>(rec >> 12), g = static_cast<int>((rec >> 6) & 63u);
-        take = !((cov[l] >> g) & 1ull) &&        // B = 0 once the group is local
-               __dadd_rn(b, pj) <= cap;          // Eq. 35
+    for (int base = 0; base < nc; base += 32) {
+      const int s = base + lane;
+      const uint32_t rec = s < nc ? cid[s] : 0u;
+      const double pj = s < nc ? __longlong_as_double(static_cast<long long>(key[s])) : 0.0;
+      const uint32_t lg = rec >> 6;  // layer and group
+      bool open = s < nc && !((cov[lg >> 6] >> (lg & 63u)) & 1ull);  // B = 0 once the group is local
+      for (;;) {
+        const double b1 = __dadd_rn(b, pj);
+        const unsigned bal = __ballot_sync(full, open && b1 <= cap);  // Eq. 35
+        if (bal == 0) break;
+        const int w = __ffs(bal) - 1;
+        b = __shfl_sync(full, b1, w);
+        const uint32_t taken = __shfl_sync(full, lg, w);
+        open = open && lane > w && lg != taken;
+        if (lane == w) {
+          placement[((size_t)(lg >> 6) * M + m) * E + static_cast<int>(rec & 63u)] = 1;
+          cov[lg >> 6] |= 1ull << (lg & 63u);
+        }
+        ++count;
       }
-      const unsigned bal = __ballot_sync(full, take);
-      if (bal == 0) {
-        base += 32;
-        continue;
-      }
-      const int w = __ffs(bal) - 1;
-      if (t == w) {
-        const int l = static_cast<int>(rec >> 12), g = static_cast<int>((rec >> 6) & 63u);
-        placement[((size_t)l * M + m) * E + static_cast<int>(rec & 63u)] = 1;
-        cov[l] |= 1ull << g;
-      }
-      b = __dadd_rn(b, __shfl_sync(full, pj, w));
-      ++count;
-      base += w + 1;
-      __syncwarp();
+      __syncwarp();  // the groups covered here are seen by the next 32
     }
-    if (t == 0) {
+    if (lane == 0) {
       used[m] = b;
       replicas[m] = count;
     }
