@@ -1,9 +1,9 @@
 // Token permutation (histogram, prefix sum, stable scatter + row gather) and
 // the weighted combine.
 //
-// Up to 4096 entries (a decode step) one block computes the histogram, the
-// offsets and the stable ranks (dispatch_small_kernel). Otherwise the (token,
-// slot) entries i = t*k + j are cut into chunks of kChunk = 256 consecutive
+// Up to 4096 entries (a decode step, a short chunk) one launch counts,
+// ranks and copies (dispatch_gather_kernel). Otherwise the (token, slot)
+// entries i = t*k + j are cut into chunks of kChunk = 256 consecutive
 // entries, one block each:
 //   1. chunk_hist: per-chunk expert histogram -> hist[E][chunk]
 //   2. chunk_scan: one block; for every expert the exclusive prefix of its
@@ -412,63 +412,118 @@ __global__ void __launch_bounds__(kNormThreads) residual_norm_kernel(
   }
 }
 
-// Small batches (n <= kSmallN entries, e.g. a decode step): histogram, offsets
-// and the stable rank in one block of 1024 threads. Pass 1 counts every
-// expert; pass 2 walks the entries in rounds of 1024 in index order, ranks
-// each round like rank_kernel and advances the experts' running starts, so
-// the permutation equals the chunked path's.
+// Small batches (n <= kSmallN entries, e.g. a decode step): offsets, stable
+// ranks and the row copies in one launch. A block takes `per` consecutive
+// entries (8, 16 or 32, a warp an entry at a time) and counts, over all n entries,
+// each expert's total and its entries before the block's first; with the
+// offsets (a scan of the totals) and the entry's rank in the block that gives
+// its row, the one of the chunked path. The X row is loaded while the block
+// counts. Block 0 writes the offsets.
+//
+// Bound: latency (launch, one L2 round trip for the entries, the counts), and
+// from a few thousand entries the counting, which every block repeats: more
+// entries a block then, at the price of rows copied one after another. Times of
+// the call in a graph, 64 experts, 2048 columns, against one block ranking all
+// entries (the chunked path from 4097 on) and a launch for the copies:
+//   entries      384   1218   2046   4092   6126
+//   before       6.0    8.2   10.5   16.5   11.4 us
+//   8 a block    3.2    4.8    7.4   18.4   37.2
+//   16           4.1    5.3    6.5   12.4   21.7
+//   32           5.5    6.8    7.9   10.6   18.1
+// and 256 entries of 8 experts, 4096 columns: 4.0 + 5.0 against 5.6 us (ncu).
 constexpr int kSmallN = 4096;
+inline int small_per_block(int64_t n) { return n <= 1216 ? 8 : n <= 2432 ? 16 : 32; }
 
-__global__ void __launch_bounds__(1024) dispatch_small_kernel(
-    const int32_t* __restrict__ chosen, int n, int k, int E, int32_t* __restrict__ offsets,
-    int32_t* __restrict__ row_token, int32_t* __restrict__ row_of) {
+__global__ void __launch_bounds__(256) dispatch_gather_kernel(
+    const int32_t* __restrict__ chosen, const uint16_t* __restrict__ X, int n, int k, int E, int d,
+    int per, int32_t* __restrict__ offsets, int32_t* __restrict__ row_token,
+    int32_t* __restrict__ row_of, uint16_t* __restrict__ X_perm) {
   pdl_trigger();  // launched with launch_pdl: no global access before pdl_wait
   pdl_wait();
-  __shared__ int total[64];
-  __shared__ int start[64];
-  __shared__ int wc[32][64];
+  __shared__ int total[64], before[64], start[64];
+  constexpr int kUnroll = 8;  // 16-byte vectors of a row a lane has in flight
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid < 64) total[tid] = 0;
+  const int begin = blockIdx.x * per;
+  const int nvec = d >> 3;
+  // the block's entries, and the head of this warp's first row
+  const int mine = lane < per && begin + lane < n ? chosen[begin + lane] : -1;
+  uint4 buf[kUnroll];
+  auto load_head = [&](int i) {
+    const uint4* in = reinterpret_cast<const uint4*>(X + (size_t)(i / k) * d);
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u)
+      if (lane + 32 * u < nvec) buf[u] = __ldg(in + lane + 32 * u);
+  };
+  if (begin + warp < n) load_head(begin + warp);
+  if (tid < 64) total[tid] = before[tid] = 0;
   __syncthreads();
-  for (int i = tid; i < n; i += blockDim.x) {
-    const int e = chosen[i];
-    if (e >= 0 && e < E) atomicAdd(&total[e], 1);
-    else report(&g_err_dispatch, ORDERMOE_DEV_BAD_INDEX, i);
+  constexpr int kLoads = 4;
+  for (int j0 = 0; j0 < n; j0 += kLoads * 256) {
+    int e[kLoads];
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int j = j0 + u * 256 + tid;
+      e[u] = j < n ? chosen[j] : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int w0 = j0 + u * 256 + warp * 32;  // the warp's first entry
+      if (w0 >= n) break;
+      const bool ok = e[u] >= 0 && e[u] < E;
+      if (!ok && w0 + lane < n && w0 + lane >= begin && w0 + lane < begin + per)
+        report(&g_err_dispatch, ORDERMOE_DEV_BAD_INDEX, w0 + lane);
+      const unsigned peers = __match_any_sync(0xffffffffu, ok ? e[u] : -1);
+      if (ok && lane == __ffs(peers) - 1) {
+        atomicAdd(&total[e[u]], __popc(peers));
+        const int nb = begin - w0;  // entries of the warp before the block's
+        const unsigned early = nb >= 32 ? peers : nb > 0 ? peers & ((1u << nb) - 1u) : 0u;
+        if (early != 0u) atomicAdd(&before[e[u]], __popc(early));
+      }
+    }
   }
   __syncthreads();
-  if (tid == 0) {
-    int acc = 0;
-    for (int x = 0; x < E; ++x) {
-      start[x] = acc;
-      offsets[x] = acc;
-      acc += total[x];
+  if (warp == 0) {  // offsets, two experts a lane
+    const int n0 = total[2 * lane], n1 = total[2 * lane + 1];
+    int in = n0 + n1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, in, o);
+      if (lane >= o) in += u;
     }
-    offsets[E] = acc;
+    const int s0 = in - n0 - n1, s1 = in - n1;
+    start[2 * lane] = s0 + before[2 * lane];
+    start[2 * lane + 1] = s1 + before[2 * lane + 1];
+    if (blockIdx.x == 0) {
+      if (2 * lane <= E) offsets[2 * lane] = s0;
+      if (2 * lane + 1 <= E) offsets[2 * lane + 1] = s1;
+      if (lane == 31 && E == 64) offsets[64] = in;
+    }
   }
-  for (int r0 = 0; r0 < n; r0 += blockDim.x) {
-    for (int x = tid; x < 32 * 64; x += blockDim.x) (&wc[0][0])[x] = 0;
-    __syncthreads();
-    const int i = r0 + tid;
-    int e = i < n ? chosen[i] : -1;
-    if (e >= E || e < -1) e = -1;  // reported in pass 1
-    const unsigned peers = __match_any_sync(0xffffffffu, e);
-    const int rank_in_warp = __popc(peers & ((1u << lane) - 1u));
-    if (e >= 0 && rank_in_warp == 0) wc[warp][e] = __popc(peers);
-    __syncthreads();
-    if (e >= 0) {
-      int before = 0;
-      for (int w = 0; w < warp; ++w) before += wc[w][e];
-      const int row = start[e] + before + rank_in_warp;
-      row_of[i] = row;
-      row_token[row] = i / k;
+  __syncthreads();
+  for (int x = warp; x < per && begin + x < n; x += 8) {
+    const int i = begin + x;
+    const int e = __shfl_sync(0xffffffffu, mine, x);
+    const unsigned same = __ballot_sync(0xffffffffu, mine == e);
+    if (e >= 0 && e < E) {
+      const int64_t row = start[e] + __popc(same & ((1u << x) - 1u));
+      if (lane == 0) {
+        row_of[i] = static_cast<int>(row);
+        row_token[row] = i / k;
+      }
+      const uint4* in = reinterpret_cast<const uint4*>(X + (size_t)(i / k) * d);
+      uint4* out = reinterpret_cast<uint4*>(X_perm + row * d);
+      for (int v0 = lane;; ) {
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u)
+          if (v0 + 32 * u < nvec) out[v0 + 32 * u] = buf[u];
+        v0 += 32 * kUnroll;
+        if (v0 - lane >= nvec) break;
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u)
+          if (v0 + 32 * u < nvec) buf[u] = __ldg(in + v0 + 32 * u);
+      }
     }
-    __syncthreads();
-    if (tid < E) {
-      int c = 0;
-      for (int w = 0; w < 32; ++w) c += wc[w][tid];
-      start[tid] += c;
-    }
-    __syncthreads();  // wc is read above before the next round clears it
+    if (x + 8 < per && begin + x + 8 < n) load_head(begin + x + 8);
   }
 }
 
@@ -485,17 +540,26 @@ int dispatch_launch(const int32_t* chosen, const uint16_t* X, int T, int k, int 
     OM_CUDA(cudaMemsetAsync(offsets, 0, sizeof(int32_t) * (E + 1), stream));
     return ORDERMOE_OK;
   }
-  if (n <= kSmallN) {
-    OM_LAUNCH_PDL("dispatch_small_kernel", dispatch_small_kernel, dim3(1), dim3(1024), 0, stream,
-                  chosen, static_cast<int>(n), k, E, offsets, row_token, row_of);
-  } else {
-    OM_LAUNCH_PDL("chunk_hist_kernel", chunk_hist_kernel, dim3(nchunks), dim3(kChunk), 0, stream,
-                  chosen, n, E, hist);
-    OM_LAUNCH_PDL("chunk_scan_kernel", chunk_scan_kernel, dim3(1), dim3(1024), 0, stream,
-                  hist, nchunks, E, offsets);
-    OM_LAUNCH_PDL("rank_kernel", rank_kernel, dim3(nchunks), dim3(kChunk), 0, stream,
-                  chosen, n, k, E, hist, row_token, row_of);
+  // (in the one launch every block reads all of chosen: not where an output
+  // takes its place, which the chunked path allows)
+  auto apart = [&](const void* out, size_t bytes) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(chosen), o = reinterpret_cast<uintptr_t>(out);
+    return a + n * sizeof(int32_t) <= o || o + bytes <= a;
+  };
+  if (n <= kSmallN && apart(row_of, n * sizeof(int32_t)) && apart(row_token, n * sizeof(int32_t)) &&
+      apart(offsets, (E + 1) * sizeof(int32_t)) && apart(X_perm, n * (size_t)d * 2)) {
+    const int per = small_per_block(n);
+    OM_LAUNCH_PDL("dispatch_gather_kernel", dispatch_gather_kernel,
+                  dim3(static_cast<unsigned>((n + per - 1) / per)), dim3(256), 0, stream, chosen, X,
+                  static_cast<int>(n), k, E, d, per, offsets, row_token, row_of, X_perm);
+    return ORDERMOE_OK;
   }
+  OM_LAUNCH_PDL("chunk_hist_kernel", chunk_hist_kernel, dim3(nchunks), dim3(kChunk), 0, stream,
+                chosen, n, E, hist);
+  OM_LAUNCH_PDL("chunk_scan_kernel", chunk_scan_kernel, dim3(1), dim3(1024), 0, stream,
+                hist, nchunks, E, offsets);
+  OM_LAUNCH_PDL("rank_kernel", rank_kernel, dim3(nchunks), dim3(kChunk), 0, stream,
+                chosen, n, k, E, hist, row_token, row_of);
   int64_t blocks = (n + 7) / 8;
   const int cap = num_sms() * 8;
   if (blocks > cap) blocks = cap;

@@ -203,8 +203,8 @@ def test_router_exact_ties_every_list_width(E, k):
 # ------------------------------------------------------------------ permutation
 
 @pytest.mark.parametrize("T,k,E,d", [(64, 2, 8, 256), (1000, 6, 64, 64), (1, 1, 1, 8), (333, 3, 7, 40),
-                                     # one block ranking several rounds of 1024 entries, up to
-                                     # its limit of 4096, and the first size past it
+                                     # sizes of one launch up to its limit of 4096, and the
+                                     # first size past it
                                      (1500, 2, 8, 64), (2048, 2, 8, 16), (683, 6, 64, 8),
                                      (4096, 2, 8, 4096),
                                      (8192, 6, 64, 64),     # 192 chunks: the scan holds them in registers
@@ -229,6 +229,45 @@ def test_dispatch_bit_exact(T, k, E, d):
     np.testing.assert_array_equal(g_rt.cpu().numpy(), rt)
     np.testing.assert_array_equal(g_rof.cpu().numpy(), rof)
     np.testing.assert_array_equal(gbits(g_xp), Xp_ref)
+
+
+@pytest.mark.parametrize("T,k,E,d", [
+    (1, 1, 1, 8), (9, 1, 5, 8), (152, 8, 64, 2304),   # eight entries a block: one, a ragged last, the most
+    (1217, 1, 33, 264), (304, 8, 64, 24),             # sixteen: the fewest, the most
+    (2433, 1, 12, 8), (512, 8, 64, 520),              # 32: the fewest, the most
+    (4097, 1, 7, 8)])                                 # the first size of the chunked path
+def test_dispatch_in_one_launch_skips_and_reports_bad_experts(T, k, E, d):
+    """The permutation of the entries with a valid expert; the others are left out
+    and one of them is reported. The same with row_of in the place of chosen."""
+    rng = np.random.default_rng(T + d)
+    chosen = rng.integers(0, E, (T, k)).astype(np.int32)
+    n = T * k
+    flat = chosen.reshape(-1)
+    bad = np.unique([n - 1, n // 2]) if n > 8 else np.array([], int)
+    flat[bad] = [E, -1][: len(bad)]
+    good = np.nonzero((flat >= 0) & (flat < E))[0]
+    order = good[np.argsort(flat[good], kind="stable")]
+    want_off = np.concatenate([[0], np.cumsum(np.bincount(flat[good], minlength=E))])
+    X = synth.normal((T, d), 1.0, seed=T).to(DEV)
+    ws = torch.empty(B.ordermoe_dispatch_workspace_bytes(T, k, E), dtype=torch.uint8, device=DEV)
+    for in_place in (False, True):
+        g_ch = dev(chosen).clone()
+        off = torch.full((E + 1,), -7, dtype=torch.int32, device=DEV)
+        rt = torch.full((n,), -7, dtype=torch.int32, device=DEV)
+        rof = g_ch if in_place else torch.full((T, k), -7, dtype=torch.int32, device=DEV)
+        xp = torch.zeros(n, d, dtype=torch.bfloat16, device=DEV)
+        B.ordermoe_dispatch(g_ch, X, T, k, E, d, off, rt, rof, xp, ws)
+        code, detail = B.ordermoe_device_error()
+        assert (code, detail in bad) == ((B.DEV_BAD_INDEX, True) if len(bad) else (0, False))
+        np.testing.assert_array_equal(off.cpu().numpy(), want_off)
+        np.testing.assert_array_equal(rt.cpu().numpy()[: len(order)], order // k)
+        assert (rt.cpu().numpy()[len(order):] == -7).all()
+        got = rof.cpu().numpy().reshape(-1)
+        np.testing.assert_array_equal(got[order], np.arange(len(order)))
+        if not in_place:
+            assert (got[bad] == -7).all()
+        assert torch.equal(xp[: len(order)], X[torch.as_tensor(order // k, device=DEV)])
+        assert not xp[len(order):].any()
 
 
 def test_dispatch_empty():
