@@ -645,8 +645,9 @@ __global__ void div_selftest_kernel(const double* __restrict__ a, const double* 
 // Mandatory placement, Eqs. 29-31 (Alg. 1): one warp, layers and
 // experts in order, b_m carried over the layers. Lane m keeps server m's
 // state in registers: b_m, C_m and lambda1 * (b_m / C_m); lambda2 * eta for
-// every count is a table. Per expert, lane m forms its score (one fp64 add of
-// the two terms, as Eq. 30 states them) and, speculatively, the ratio term it
+// every count is a table. Per expert (experts of one size take their scores
+// from tables, see below), lane m forms its score (one fp64 add of the two
+// terms, as Eq. 30 states them) and, speculatively, the ratio term it
 // would have after taking the expert; the argmin runs on integer keys
 // (scores are non-negative, so their bit patterns order like the values; ties
 // to the lower server), and the winner keeps its speculative term. A
@@ -658,8 +659,7 @@ __global__ void div_selftest_kernel(const double* __restrict__ a, const double* 
 constexpr int kPlaceTable = 4096;  // (server, wins) entries
 struct PlaceSmem {
   // uniform sizes: server m after n more experts, at m * depth + n
-  double after_b[kPlaceTable];   // b_m
-  double after_a1[kPlaceTable];  // lambda1 * (b_m / C_m)
+  double after_b[kPlaceTable];  // b_m
   double l2eta[65];  // lambda2 * eta for eta = 0 .. 64
   double pls[64];
   int grp[64];
@@ -675,36 +675,85 @@ static_assert(sizeof(PlaceSmem) % 16 == 0, "vector stores into xs and eta");
 
 // Experts of one size (their memory p bitwise equal over the range's layers,
 // as a model's experts are): a server's b_m and ratio term then depend on how
-// many experts it has taken only, whichever they were. A producer warp
-// tabulates them, well ahead of the warp that places, whose loop is left with
-// one fp64 addition (the score) instead of seven on a part that has two fp64
-// lanes an SM. depth entries a server; ready of them are there.
+// many experts it has taken only, whichever they were, and a score on that and
+// on eta. A producer warp tabulates b_m and the scores as ordered keys, ahead
+// of the warp that places, whose loop is left without fp64 (an instruction
+// holds a lone warp for 65 cycles). depth rows a server, cols scores a row
+// (eta = 0 .. cols - 1; larger ones are added up when they come); ready rows of
+// them are there. With the states alone tabulated, an fp64 addition an expert left
+// and a branch for ties, 512 experts on 8 servers took 151 us and 256 on 4 (32
+// layers) 105; this takes 101 and 79 (ncu), the second half of it per-layer work.
 __host__ __device__ inline int place_depth(int M, int experts) {
-  const int want = 3 * experts / M + 16, room = kPlaceTable / M;
+  const int want = 2 * experts / M + 16, room = kPlaceTable / M;
   return want < room ? want : room;
 }
-__device__ __forceinline__ int place_ready(PlaceSmem& sm) {
-  int v;
-  asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(&sm.ready)) : "memory");
+// Score columns: a producer warp fills a row of all servers in M cols / 32 steps,
+// and must fill rows faster than M experts are placed. Two rows more are for the
+// lanes without a server. (19 columns for 8 servers: 198 us instead of 101.)
+__host__ __device__ inline int place_cols(int M) { return M <= 4 ? 8 : 4; }
+__host__ __device__ inline size_t place_score_bytes(int M, int experts) {
+  return 8 * ((size_t)M * place_depth(M, experts) + 2) * place_cols(M);
+}
+
+constexpr unsigned long long kNoServer = ~0ull;           // the expert does not fit
+constexpr unsigned long long kOddScore = 0x7FF0ull << 48;  // not a plain non-negative number
+
+// a score as a key: non-negative finite values order like their bit patterns
+// (an infinity, a NaN, a negative score or -0 sends the layer to the general loop)
+__device__ __forceinline__ unsigned long long place_key(double sc) {
+  const unsigned long long k = static_cast<unsigned long long>(__double_as_longlong(sc));
+  return k >= kOddScore ? kOddScore : k;
+}
+// The key for an eta past the columns, from the row's eta = 0 (whose score is
+// the ratio term). Out of line: inlined, its fp64 is issued for every expert.
+__device__ __noinline__ unsigned long long place_key_past(unsigned long long base, double l2) {
+  if (base >= kOddScore) return base;
+  return place_key(__dadd_rn(__longlong_as_double(static_cast<long long>(base)), l2));
+}
+// ready rows once there are `need` of them (at most depth), or those there after
+// the limit of about 0.1 s (the producer never waits, so that is not reached).
+__device__ __noinline__ int place_wait(PlaceSmem& sm, int need, int depth) {
+  need = need < depth ? need : depth;
+  int v = 0;
+  for (int i = 0; i < (1 << 21); ++i) {
+    asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(&sm.ready)) : "memory");
+    if (v >= need) break;
+  }
   return v;
 }
+// before the producer starts, the whole block: l2eta and the spare rows
+__device__ void place_tables_init(PlaceSmem& sm, unsigned long long* score, int M, int depth, int cols,
+                                  double lambda2, int t, int nt) {
+  for (int i = t; i <= 64; i += nt) sm.l2eta[i] = __dmul_rn(lambda2, static_cast<double>(i));
+  if (depth > 0)
+    for (int i = t; i < 2 * cols; i += nt) score[(size_t)M * depth * cols + i] = kNoServer;
+  if (t == 0) sm.ready = 0;
+}
 // The producer: one warp, lane m server m, b_m after 0 .. depth - 1 more
-// experts of size p, the additions in the order the placement makes them.
-__device__ void place_produce(PlaceSmem& sm, int lane, int M, int depth, double p, bool first,
-                              double lambda1, const double* __restrict__ C,
-                              const double* __restrict__ used) {
+// experts of size p, the additions in the order the placement makes them, and
+// the keys of placing one more then.
+__device__ void place_produce(PlaceSmem& sm, unsigned long long* score, int lane, int M, int depth,
+                              int cols, double p, bool first, double lambda1,
+                              const double* __restrict__ C, const double* __restrict__ used) {
   const bool srv = lane < M;
   double b = (srv && !first) ? used[lane] : 0.0;
   const double cap = srv ? C[lane] : 1.0, rcap = __drcp_rn(cap);
   const int at = srv ? lane * depth : 0;
+  const int e = lane & (cols - 1), m0 = lane / cols;  // cols is a power of two
+  const double l2 = sm.l2eta[e];
   for (int n = 0; n < depth; ++n) {
     const double a1 = __dmul_rn(lambda1, div_rn_markstein(b, cap, rcap));
-    if (srv) {
-      sm.after_b[at + n] = b;
-      sm.after_a1[at + n] = a1;
-    }
+    if (srv) sm.after_b[at + n] = b;
     b = __dadd_rn(b, p);
-    if ((n & 3) == 3 || n + 1 == depth) {  // four rows at a time
+    const int feas = __double_as_longlong(b) <= __double_as_longlong(cap);  // b <= C_m, b >= 0
+    for (int mb = 0; mb < M; mb += 32 / cols) {
+      const int m = mb + m0;
+      const double am = __shfl_sync(0xffffffffu, a1, m & 31);
+      const int fm = __shfl_sync(0xffffffffu, feas, m & 31);
+      const unsigned long long key = place_key(__dadd_rn(am, l2));
+      if (m < M) score[((size_t)m * depth + n) * cols + e] = fm ? key : kNoServer;
+    }
+    if (n < 3 || (n & 3) == 3 || n + 1 == depth) {  // four rows at a time, the first as they come
       __syncwarp();
       if (lane == 0)
         asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(smem_u32(&sm.ready)), "r"(n + 1) : "memory");
@@ -720,18 +769,10 @@ __device__ bool place_uniform(const double* __restrict__ p, int n, int t, int nt
   return __syncthreads_and(same) != 0;
 }
 
-// A server's state after a further expert, past the tables (kept out of line:
-// inlined, its fp64 operations were issued for every expert).
-__device__ __noinline__ double2 place_further(double b, double p, double cap, double rcap,
-                                              double lambda1) {
-  const double bn = __dadd_rn(b, p);
-  return make_double2(bn, __dmul_rn(lambda1, div_rn_markstein(bn, cap, rcap)));
-}
-
 // The placement on warp 0 of a block (threadIdx.x < 32); returns 1 when a
 // waiting-list expert overfilled its server.
-// depth > 0: the sizes are uniform and the tables hold depth entries a server.
-__device__ int place_layers(PlaceSmem& sm, const int32_t* __restrict__ group,
+// depth > 0: the sizes are uniform and the tables hold depth rows a server.
+__device__ int place_layers(PlaceSmem& sm, const unsigned long long* score, int cols, const int32_t* __restrict__ group,
                              const int32_t* __restrict__ porder, int L, int E, int M, int l0,
                              int l1, int first, PlaceParams pp, const double* __restrict__ p,
                              const double* __restrict__ C, uint8_t* __restrict__ placement,
@@ -753,9 +794,8 @@ __device__ int place_layers(PlaceSmem& sm, const int32_t* __restrict__ group,
   const long long cap_bits = __double_as_longlong(cap);
   double a1 = srv ? __dmul_rn(pp.lambda1, div_rn_markstein(b, cap, rcap)) : 0.0;
   bool bad_score = srv && !(cap > 0.0 && cap <= 1.7976931348623157e308);
-  for (int i = t; i <= 64; i += 32) l2eta[i] = __dmul_rn(pp.lambda2, static_cast<double>(i));
-  int wins = 0;  // experts this server took in the range (uniform sizes)
-  int avail = 0;  // entries of its tables known to be there
+  int wins = 0;   // experts this server took in the range (uniform sizes)
+  int avail = 0;  // rows of its tables known to be there
   // the next layer's rows, loaded a layer ahead (two experts a lane)
   int g2[2] = {0, 0}, o2[2] = {0, 0};
   double p2[2] = {0.0, 0.0};
@@ -788,82 +828,70 @@ __device__ int place_layers(PlaceSmem& sm, const int32_t* __restrict__ group,
     bool general = depth == 0;
     if (!general) {
       // One pass over the experts, written to branch as little as it can (a
-      // warp alone pays 20 cycles and more for each): a score that is not a
-      // plain non-negative number makes the layer start over below.
-      const double b0 = b, a10 = a1;
+      // warp alone pays 20 cycles and more for each): an odd score, or a server
+      // past its table, makes the layer start over below.
       const int wins0 = wins;
       // the experts in order with their groups (expert | group << 8), read ahead
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
+      for (int h = 0; h < 2; ++h) {
         if (t + 32 * h < E) sm.seq[t + 32 * h] = ord[t + 32 * h] | (grp[ord[t + 32 * h]] << 8);
-      __syncwarp();
-      // this server's state, and (bn, a1n) the one after a further expert
-      double bn = 0.0, a1n = 0.0;
-      if (avail < depth) avail = place_ready(sm);
-      if (srv && wins + 1 < avail) {
-        bn = sm.after_b[t * depth + wins + 1];
-        a1n = sm.after_a1[t * depth + wins + 1];
-      } else if (srv) {
-        const double2 s = place_further(b, pls[0], cap, rcap, pp.lambda1);
-        bn = s.x;
-        a1n = s.y;
+        sm.who[t + 32 * h] = 0;
       }
-      bool feas = srv && __double_as_longlong(bn) <= cap_bits;  // bn <= C_m, bn >= 0
-      bool odd = false;
-      int* my_eta = eta + (srv ? t * 64 : 0);
-      const double* my_b = sm.after_b + (srv ? t * depth : 0);
-      const double* my_a1 = sm.after_a1 + (srv ? t * depth : 0);
-      int cur = sm.seq[0];
-      int nxt = sm.seq[min(1, E - 1)];
-      int ec = 0;  // experts of cur's group on this server
-      double sc = __dadd_rn(a1, l2eta[0]);
-      for (int pos = 0; pos < E; ++pos) {
-        // the next expert's count and lambda2 * eta, if this server takes cur and if not
-        const int after = sm.seq[min(pos + 2, E - 1)];
-        const int en = my_eta[nxt >> 8];
-        const int ew = (nxt >> 8) == (cur >> 8) ? ec + 1 : en;
-        const double l2s = l2eta[en], l2w = l2eta[ew];
-        const unsigned khi = feas ? static_cast<unsigned>(__double2hiint(sc)) : 0xffffffffu;
-        const unsigned klo = feas ? static_cast<unsigned>(__double2loint(sc)) : 0xffffffffu;
-        odd |= feas && khi >= 0x7FF00000u;  // an infinity, a NaN, a negative score or -0
-        const unsigned mhi = __reduce_min_sync(0xffffffffu, khi);
-        unsigned win = __ballot_sync(0xffffffffu, khi == mhi);
-        if ((win & (win - 1)) != 0u) {  // several lanes hold it (or no server is feasible)
-          const unsigned mlo = __reduce_min_sync(0xffffffffu, khi == mhi ? klo : 0xffffffffu);
-          win = mhi == 0xffffffffu ? 0u : __ballot_sync(0xffffffffu, khi == mhi && klo == mlo);
-        }
-        const bool won = win != 0u && t == __ffs(win) - 1;
-        a1 = won ? a1n : a1;
-        sc = __dadd_rn(a1, won ? l2w : l2s);
-        if (t == 0) sm.who[pos] = static_cast<uint8_t>(__ffs(win));  // server + 1, or 0: waiting
-        if (won) {
-          my_eta[cur >> 8] = ec + 1;
-          b = bn;
-          ++wins;
-          if (wins + 1 >= avail && avail < depth) avail = place_ready(sm);  // seldom: it is a fence
-          if (wins + 1 < avail) {
-            bn = my_b[wins + 1];
-            a1n = my_a1[wins + 1];
-          } else {
-            const double2 s = place_further(b, pls[0], cap, rcap, pp.lambda1);
-            bn = s.x;
-            a1n = s.y;
+      if (srv && wins + 1 >= avail) avail = place_wait(sm, wins + 2, depth);
+      bool odd = srv && wins + 1 >= avail;
+      __syncwarp();
+      if (!__any_sync(0xffffffffu, odd)) {
+        // this server's row, and the one after it for a further expert
+        const unsigned long long* row = score + (size_t)(srv ? t * depth + wins : M * depth) * cols;
+        int* my_eta = eta + (srv ? t * 64 : 0);
+        int cur = sm.seq[0];
+        int nxt = sm.seq[min(1, E - 1)];
+        int ec = 0;  // experts of cur's group on this server
+        unsigned long long key = row[0];
+        for (int pos = 0; pos < E; ++pos) {
+          // the next expert's count and key, if this server takes cur and if not
+          const int after = sm.seq[min(pos + 2, E - 1)];
+          const int en = my_eta[nxt >> 8];
+          const int ew = (nxt >> 8) == (cur >> 8) ? ec + 1 : en;
+          unsigned long long ks = row[min(en, cols - 1)], kw = row[cols + min(ew, cols - 1)];
+          if (ew >= cols) {  // (en <= ew)
+            if (en >= cols) ks = place_key_past(row[0], l2eta[min(en, 64)]);
+            kw = place_key_past(row[cols], l2eta[min(ew, 64)]);
           }
-          feas = __double_as_longlong(bn) <= cap_bits;
+          const unsigned khi = static_cast<unsigned>(key >> 32), klo = static_cast<unsigned>(key);
+          odd |= key == kOddScore;
+          const unsigned mhi = __reduce_min_sync(0xffffffffu, khi);
+          const unsigned mlo = __reduce_min_sync(0xffffffffu, khi == mhi ? klo : 0xffffffffu);
+          const unsigned win = __ballot_sync(0xffffffffu, khi == mhi && klo == mlo);
+          const bool won = mhi != 0xffffffffu && t == __ffs(win) - 1;  // none: it waits
+          if (won) {
+            sm.who[pos] = static_cast<uint8_t>(t + 1);
+            my_eta[cur >> 8] = ec + 1;
+            ++wins;
+            row += cols;
+            if (wins + 1 >= avail) {  // seldom
+              avail = place_wait(sm, wins + 2, depth);
+              if (wins + 1 >= avail) {
+                odd = true;
+                row -= cols;  // the rows end here
+              }
+            }
+          }
+          key = won ? kw : ks;
+          ec = won ? ew : en;
+          cur = nxt;
+          nxt = after;
         }
-        ec = won ? ew : en;
-        cur = nxt;
-        nxt = after;
       }
       __syncwarp();
       if (__any_sync(0xffffffffu, odd)) {
         general = true;
-        b = b0;
-        a1 = a10;
         wins = wins0;
+        a1 = srv ? __dmul_rn(pp.lambda1, div_rn_markstein(b, cap, rcap)) : 0.0;
         for (int i = t; i < 16 * M; i += 32) reinterpret_cast<int4*>(eta)[i] = make_int4(0, 0, 0, 0);
         __syncwarp();
       } else {
+        if (srv) b = sm.after_b[t * depth + wins];
 #pragma unroll
         for (int h = 0; h < 2; ++h)
           if (t + 32 * h < E) {
@@ -998,7 +1026,7 @@ __device__ void place_status(int first, int overflow, int32_t* __restrict__ stat
 // The placement of a grouped range by a block of at least four warps: the loop
 // on warp 0, the capacity check of the first range beside it on warp 3 (and
 // the producer of the tables on another).
-__device__ void place_range(PlaceSmem& sm, int* s_over, const int32_t* __restrict__ group,
+__device__ void place_range(PlaceSmem& sm, const unsigned long long* score, int cols, int* s_over, const int32_t* __restrict__ group,
                             const int32_t* __restrict__ porder, int L, int E, int M, int l0, int l1,
                             int first, PlaceParams pp, const double* __restrict__ p,
                             const double* __restrict__ C, uint8_t* __restrict__ placement,
@@ -1006,7 +1034,7 @@ __device__ void place_range(PlaceSmem& sm, int* s_over, const int32_t* __restric
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int over = 0;
   if (warp == 0)
-    over = place_layers(sm, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used, depth);
+    over = place_layers(sm, score, cols, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used, depth);
   else if (warp == 3 && first) {
     const int d = demand_exceeds(p, L * E, C, M, lane);
     if (lane == 0) *s_over = d;
@@ -1024,15 +1052,16 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(
     int32_t* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char s_pl[];
   PlaceSmem& sm = *reinterpret_cast<PlaceSmem*>(s_pl);
+  unsigned long long* score = reinterpret_cast<unsigned long long*>(s_pl + sizeof(PlaceSmem));
   __shared__ int s_over;
   const int n = (l1 - l0) * E;
   const bool uniform = place_uniform(p + (size_t)l0 * E, n, threadIdx.x, blockDim.x);
-  const int depth = uniform ? place_depth(M, n) : 0;
-  if (threadIdx.x == 0) sm.ready = 0;
+  const int depth = uniform ? place_depth(M, n) : 0, cols = place_cols(M);
+  place_tables_init(sm, score, M, depth, cols, pp.lambda2, threadIdx.x, blockDim.x);
   __syncthreads();
   if (uniform && (threadIdx.x >> 5) == 1)
-    place_produce(sm, threadIdx.x & 31, M, depth, p[(size_t)l0 * E], first, pp.lambda1, C, used);
-  place_range(sm, &s_over, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used, status,
+    place_produce(sm, score, threadIdx.x & 31, M, depth, cols, p[(size_t)l0 * E], first, pp.lambda1, C, used);
+  place_range(sm, score, cols, &s_over, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used, status,
               depth);
 }
 
@@ -1042,13 +1071,18 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(
 // block, so the pipelined plan's side stream holds one SM).
 // Bound: the serial chains (a group per expert, a server per expert). A layer
 // of 64 experts took about 28 us to place and 10 to group (8 layers 282 us
-// under ncu); with the tables and the integer scan 8 layers take 186 us.
+// under ncu); with the servers' states tabulated and the integer scan 8 layers
+// took 186 us, with the scores tabulated too 132.
 constexpr int kGroupThreads = 256;
 
 __host__ __device__ inline int group_slices(int E) { return kGroupThreads / group_slice_threads(E); }
-static size_t group_place_smem(int E) {
-  return ((group_slices(E) * group_slice_bytes(E) + 15) & ~size_t(15)) + sizeof(PlaceSmem);
+static size_t group_place_smem(int E, int M, int experts) {
+  return ((group_slices(E) * group_slice_bytes(E) + 15) & ~size_t(15)) + sizeof(PlaceSmem) +
+         place_score_bytes(M, experts);
 }
+constexpr int kPlaceRange = 512;  // experts of a range
+constexpr size_t kPlaceSmemMax = 200 * 1024;  // of either placing kernel, at any M
+static size_t place_smem(int M, int experts) { return sizeof(PlaceSmem) + place_score_bytes(M, experts); }
 
 __global__ void __launch_bounds__(kGroupThreads + 32) group_place_kernel(
     const float* __restrict__ sim, const int32_t* __restrict__ counts, int L, int E, int M, int l0,
@@ -1060,19 +1094,20 @@ __global__ void __launch_bounds__(kGroupThreads + 32) group_place_kernel(
   const int nt = group_slice_threads(E), slices = group_slices(E);
   PlaceSmem& ps = *reinterpret_cast<PlaceSmem*>(
       s_gp + ((slices * group_slice_bytes(E) + 15) & ~size_t(15)));
+  unsigned long long* score = reinterpret_cast<unsigned long long*>(&ps + 1);
   __shared__ int s_over;
   const int n = (l1 - l0) * E;
   const bool uniform = place_uniform(p + (size_t)l0 * E, n, threadIdx.x, blockDim.x);
-  const int depth = uniform ? place_depth(M, n) : 0;
+  const int depth = uniform ? place_depth(M, n) : 0, cols = place_cols(M);
   const int slice = threadIdx.x / nt;
   unsigned char* own = s_gp + (slice < slices ? slice : 0) * group_slice_bytes(E);
   GroupSmem& gs = *reinterpret_cast<GroupSmem*>(own);
   uint32_t* K = reinterpret_cast<uint32_t*>(own + sizeof(GroupSmem));
-  if (threadIdx.x == 0) ps.ready = 0;
+  place_tables_init(ps, score, M, depth, cols, pp.lambda2, threadIdx.x, blockDim.x);
   __syncthreads();
   if (slice >= slices) {  // the last warp
     if (uniform)
-      place_produce(ps, threadIdx.x & 31, M, depth, p[(size_t)l0 * E], first, pp.lambda1, C, used);
+      place_produce(ps, score, threadIdx.x & 31, M, depth, cols, p[(size_t)l0 * E], first, pp.lambda1, C, used);
   } else {
     for (int lb = l0; lb < l1; lb += slices) {
       const int l = lb + slice;
@@ -1081,7 +1116,7 @@ __global__ void __launch_bounds__(kGroupThreads + 32) group_place_kernel(
       group_sync(kGroupThreads);  // the slices' scratch is reused; group and porder are written
     }
   }
-  place_range(ps, &s_over, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used, status,
+  place_range(ps, score, cols, &s_over, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used, status,
               depth);
 }
 
@@ -1497,7 +1532,21 @@ extern "C" size_t ordermoe_place_workspace_bytes(int L, int E) {
 
 static cudaError_t place_attr() {
   return cudaFuncSetAttribute(place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(sizeof(PlaceSmem)));
+                              static_cast<int>(kPlaceSmemMax));
+}
+
+// The placement of grouped layers l0 .. l1 - 1 in ranges of at most 512 experts
+// (a range's tables hold its servers' states).
+static cudaError_t place_launch(const int32_t* group, const int32_t* porder, int L, int E, int M, int l0,
+                                int l1, const PlaceParams& pp, const double* p, const double* C,
+                                uint8_t* placement, double* used, int32_t* status, cudaStream_t stream) {
+  const int part = kPlaceRange / E;
+  for (int a = l0; a < l1; a += part) {
+    const int b = a + part < l1 ? a + part : l1;
+    place_kernel<<<1, kPlaceThreads, place_smem(M, (b - a) * E), stream>>>(
+        group, porder, L, E, M, a, b, a == 0 ? 1 : 0, pp, p, C, placement, used, status);
+  }
+  return cudaGetLastError();
 }
 
 extern "C" int ordermoe_place(const float* sim, const int32_t* counts, int L, int E, int M,
@@ -1523,9 +1572,8 @@ extern "C" int ordermoe_place(const float* sim, const int32_t* counts, int L, in
   const cudaError_t ae =
       static_cast<cudaError_t>(per_device(attr, [] { return static_cast<int>(place_attr()); }));
   if (ae != cudaSuccess) return cuda_fail(ae, "cudaFuncSetAttribute(place_kernel)");
-  place_kernel<<<1, kPlaceThreads, sizeof(PlaceSmem), stream>>>(group, porder_scratch, L, E, M, 0, L, 1, pp, p, C, placement,
-                                     used, status);
-  OM_LAUNCHED("place_kernel");
+  const cudaError_t e = place_launch(group, porder_scratch, L, E, M, 0, L, pp, p, C, placement, used, status, stream);
+  if (e != cudaSuccess) return cuda_fail(e, "place_kernel");
   return ORDERMOE_OK;
 }
 
@@ -1685,7 +1733,7 @@ static int plan_sync(PlanSync** out) {
     PlanSync& ps = g_plan_sync[dev];
     cudaError_t err = cudaFuncSetAttribute(group_place_kernel,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           static_cast<int>(group_place_smem(64)));
+                                           static_cast<int>(kPlaceSmemMax));
     if (err == cudaSuccess) err = place_attr();
     if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&ps.side, cudaStreamNonBlocking);
     for (int i = 0; i < 4 && err == cudaSuccess; ++i)
@@ -1774,7 +1822,7 @@ extern "C" int ordermoe_plan(const uint16_t* W_r, const uint16_t* X_cal, int L, 
         break;
       }
       if (l0 + lp < L) {
-        group_place_kernel<<<1, kGroupThreads + 32, group_place_smem(E), ps->side>>>(
+        group_place_kernel<<<1, kGroupThreads + 32, group_place_smem(E, M, lp * E), ps->side>>>(
             sim, counts, L, E, M, l0, l0 + lp, l0 == 0 ? 1 : 0, pp, p, C, group, n_groups, theta,
             importance, porder, placement, used, status);
         if ((rc = launched("group_place_kernel"))) break;
@@ -1785,9 +1833,11 @@ extern "C" int ordermoe_plan(const uint16_t* W_r, const uint16_t* X_cal, int L, 
         group_kernel<<<lp, group_slice_threads(E), 0, ps->side>>>(
             sim, counts, L, E, l0, pp, p, group, n_groups, theta, importance, porder);
         if ((rc = launched("group_kernel"))) break;
-        place_kernel<<<1, kPlaceThreads, sizeof(PlaceSmem), ps->side>>>(
-            group, porder, L, E, M, l0, L, l0 == 0 ? 1 : 0, pp, p, C, placement, used, status);
-        if ((rc = launched("place_kernel"))) break;
+        const cudaError_t pe = place_launch(group, porder, L, E, M, l0, L, pp, p, C, placement, used, status, ps->side);
+        if (pe != cudaSuccess) {
+          rc = cuda_fail(pe, "place_kernel");
+          break;
+        }
       }
       l0 += lp;
     }

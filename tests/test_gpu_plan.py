@@ -331,15 +331,19 @@ def test_placement_quotient_is_correctly_rounded():
     (8, 64, 32, 1.0, "one"),      # a server takes more experts than its table holds
     (6, 24, 5, 0.3, "tight"),     # fractional sizes, waiting lists, an overflow
     (3, 33, 7, 1.7, "loose"), (2, 1, 1, 1.0, "tight"), (40, 8, 4, 1.0, "loose"),
-    (4, 16, 3, 0.0, "loose")])    # size 0: nothing fills up
+    (4, 16, 3, 0.0, "loose"),     # size 0: nothing fills up
+    (4, 64, 1, 1.0, "mates"),     # more experts of a group on a server than it has columns
+    (20, 64, 3, 0.7, "mates")])   # ranges of 512 experts, the last one shorter
 def test_place_uniform_sizes_bit_exact(L, E, M, size, caps):
     """Experts of one size, whose servers' states are tabulated by the number of
     experts taken."""
     rng = np.random.default_rng(L * 100 + E + M)
-    sim, counts = synthetic_sims(rng, L, E, max(1, min(4, E)), 0.4)
+    sim, counts = synthetic_sims(rng, L, E, 1 if caps == "mates" else max(1, min(4, E)), 0.4)
+    if caps == "mates":
+        sim = np.maximum(sim, np.float32(0.9))  # one group a layer
     p = np.full((L, E), size)
     total = max(p.sum(), 1.0)
-    C = total / M * rng.uniform(0.8, 1.3, M) * {"one": 1e-3, "tight": 0.95, "loose": 1.5}[caps]
+    C = total / M * rng.uniform(0.8, 1.3, M) * {"one": 1e-3, "tight": 0.95, "loose": 1.5, "mates": 1.4}[caps]
     if caps == "one":
         C[3] = 2.0 * total
     got = gpu_place(sim, counts, M, p, C)
