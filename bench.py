@@ -321,9 +321,8 @@ def run_ours(args, dist):
             ("combine", lambda: B.ordermoe_combine(Yp, row_of, wts, T, k, d, y)),
         ]
 
-    # route_select 1 (2 for more than 16 experts: the lane selection kernel),
-    # dispatch 4, gate/up 1, down 1, combine 1
-    KERNELS_PER_STEP = 8 + (1 if E > 16 else 0)
+    # gate/up, down and combine 1 each
+    KERNELS_PER_STEP = route_launches(T, E, d) + dispatch_launches(T, k) + 3
     step(cnt=counters)     # one counted pass for the execution-type breakdown
     for _ in range(max(args.warmup, 3)):
         step()
@@ -708,13 +707,26 @@ def decode_timed(args, dist, w, device, S, H):
     return ms, clocks, stack, hs, xs, loc, qhat
 
 
+def route_launches(T, E, d):
+    """Kernels of one route_select call (H = 1): 1, or 2 with a lane selection
+    kernel of its own for more than 16 experts where the clusters of eight
+    (128 tokens each) do not fit on 152 SMs at once."""
+    return 1 if E <= 16 or (8 * ((T + 127) // 128) <= 152 and d // 64 >= 8) else 2
+
+
+def dispatch_launches(T, k):
+    """Kernels of one dispatch call: up to 4096 entries are counted, ranked and
+    copied in one launch."""
+    return 1 if T * k <= 4096 else 4
+
+
 def decode_launches(w, H):
-    """Kernels of one decode step: the first layer's RMSNorm, then per layer
-    route_select 1 (2 with a look-ahead horizon H > 1 or more than 16
-    experts: a separate selection kernel), dispatch 2 (one block ranks up to
-    4096 entries) or 4, gate/up 1, down 1 and the residual combine 1."""
-    route = 1 if (H == 1 and w.E <= 16) else 2
-    return 1 + (route + 3 + (2 if w.T * w.k <= 4096 else 4)) * w.L
+    """Kernels of one decode step: the first layer's RMSNorm, then per layer the
+    routing (router and look-ahead selection where the layer looks ahead, all
+    but the last when H > 1), the dispatch, gate/up, down and the residual
+    combine."""
+    route = sum(2 if min(H, w.L - l) > 1 else route_launches(w.T, w.E, w.d) for l in range(w.L))
+    return 1 + route + (dispatch_launches(w.T, w.k) + 3) * w.L
 
 
 def run_decode(args, dist, w, device):
@@ -785,10 +797,7 @@ def decode_line(args, dist, w, ms, clocks, H, S):
                      "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                      "frac": round(achieved / peak, 4), "traffic": None,
                      "peak_source": "%s hbm_gbs" % pk_kind, "bytes_per_step": wbytes},
-        # plus the look-ahead selection pass on every layer that looks ahead
-        # (all but the last when H > 1)
-        "gpu_launches": (decode_launches(w, H)
-                         + sum(min(H, w.L - l) > 1 for l in range(w.L))) * args.steps,
+        "gpu_launches": decode_launches(w, H) * args.steps,
         "clocks": clocks,
         "lookahead_H": H,
     }
@@ -796,18 +805,16 @@ def decode_line(args, dist, w, ms, clocks, H, S):
 
 def plan_launches(L, E):
     """Kernels of one ordermoe_plan call: on the tensor-core path (E in {8,
-    16, 32, 64}, L E <= 4096) the layers go in blocks of 512 logit columns,
-    the last block in two halves when there is more than one, and each block
-    launches the logits GEMM, the Gram, its reduction, the similarities and
-    one grouping + placement kernel (5); otherwise the similarity takes 5 and
-    the placement 2. Replication and coverage add 1 each."""
+    16, 32, 64}, L E <= 4096) the layers go in blocks of 512 logit columns, and
+    each block launches the logits GEMM, the Gram, the similarities and one
+    grouping + placement kernel (4; the last block's grouping is a kernel of
+    its own); otherwise the similarity takes 4, the grouping 1 and the placement
+    one for every 512 experts. Replication and coverage add 1 each."""
     if E in (8, 16, 32, 64) and L * E <= 4096:
         part = max(1, 512 // E)
-        nfull = (L + part - 1) // part
-        last_n = L - (nfull - 1) * part
-        blocks = nfull + (1 if nfull > 1 and last_n >= 2 else 0)
-        return 5 * blocks + 2
-    return 5 + 2 + 2
+        return 4 * ((L + part - 1) // part) + 1 + 2
+    part = 512 // E
+    return 4 + 1 + (L + part - 1) // part + 2
 
 
 def run_similarity(args, dist, w, device):
