@@ -435,7 +435,7 @@ __device__ __forceinline__ void group_sync(int nsync) {
 // threads t of a slice of the nsync that group (the layers are independent here): theta_l
 // (Eq. 6), greedy cover (Eqs. 24-26), importance (Eqs. 27-28) and the
 // placement order (p desc, I desc, index asc). A slice with live == false has
-// no layer this round but meets every barrier.
+// no layer this time but meets every barrier.
 __device__ void group_layer(GroupSmem& sm, uint32_t* K, bool live, int t, int nt, int nsync, int l,
                             const float* __restrict__ sim,
                             const int32_t* __restrict__ counts, int L, int E, PlaceParams pp,
