@@ -1653,56 +1653,61 @@ __global__ void __launch_bounds__(rt::THREADS, 1) router_select_kernel(
   const uint32_t tmem_base = s.tmem_base;
   volatile int* abort = &s.abort;
   uint32_t issued_mask = 0, last_phase_bits = 0;
-  bool mma_issued = false;
+  bool mma_issued = false, leader = false;
   float lg[NE];
   int kind_count[4] = {0, 0, 0, 0};
 
+  // Producer and MMA warps walk the stages converged, one elected lane issues: a
+  // lane walking them alone held the stream back (4096 tokens of 8 experts, d
+  // 4096, 14.9 us; so 12.9; 8192 of 64, d 2048, 20.5 and 19.4; 128 tokens 8.9 and
+  // 8.1, ncu).
   if (warp == 0) {
-    if (lane == 0) {
-      for (int i = 0; i < kblocks && !*abort; ++i) {
-        const int stage = i % STAGES;
-        const uint32_t phase = (i / STAGES) & 1;
-        if (!mbar_wait(&s.empty[stage], phase ^ 1u, limit_ns, abort)) {
-          if (!*abort) report(&g_err_route, ORDERMOE_DEV_WAIT_TIMEOUT, 21);
-          *abort = 1;
-          break;
-        }
-        uint8_t* sa = tiles + stage * STAGE_BYTES;
-        const int kb = kb_begin + i;
-        mbar_arrive_expect_tx(&s.full[stage], STAGE_BYTES);
-        tma_load_2d(sa, &mapX, &s.full[stage], kb * rt::BK, m0);
-        tma_load_2d(sa + rt::A_BYTES, &mapW, &s.full[stage], kb * rt::BK, 0);
-        issued_mask |= 1u << stage;
-        last_phase_bits = (last_phase_bits & ~(1u << stage)) | (phase << stage);
+    const bool issuer = elect_one();
+    for (int i = 0; i < kblocks; ++i) {
+      const int stage = i % STAGES;
+      const uint32_t phase = (i / STAGES) & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&s.empty[stage], phase ^ 1u, limit_ns, abort))) {
+        if (issuer && !*abort) report(&g_err_route, ORDERMOE_DEV_WAIT_TIMEOUT, 21);
+        *abort = 1;
+        break;
       }
+      if (issuer) {
+        uint8_t* sa = tiles + stage * STAGE_BYTES;
+        mbar_arrive_expect_tx(&s.full[stage], STAGE_BYTES);
+        tma_load_2d(sa, &mapX, &s.full[stage], (kb_begin + i) * rt::BK, m0);
+        tma_load_2d(sa + rt::A_BYTES, &mapW, &s.full[stage], (kb_begin + i) * rt::BK, 0);
+      }
+      issued_mask |= 1u << stage;
+      last_phase_bits = (last_phase_bits & ~(1u << stage)) | (phase << stage);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t IDESC = idesc_bf16_f32(128, NE);
-      bool ok = true;
-      for (int i = 0; i < kblocks && !*abort; ++i) {
-        const int stage = i % STAGES;
-        const uint32_t phase = (i / STAGES) & 1;
-        if (!mbar_wait(&s.full[stage], phase, limit_ns, abort)) {
-          if (!*abort) report(&g_err_route, ORDERMOE_DEV_WAIT_TIMEOUT, 22);
-          *abort = 1;
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t a0 = smem_u32(tiles + stage * STAGE_BYTES);
-        const uint32_t b0 = a0 + rt::A_BYTES;
+    constexpr uint32_t IDESC = idesc_bf16_f32(128, NE);
+    leader = elect_one();
+    const uint64_t desc0 = sdesc_kmajor_sw128(smem_u32(tiles));
+    bool ok = true;
+    for (int i = 0; i < kblocks; ++i) {
+      const int stage = i % STAGES;
+      const uint32_t phase = (i / STAGES) & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&s.full[stage], phase, limit_ns, abort))) {
+        if (leader && !*abort) report(&g_err_route, ORDERMOE_DEV_WAIT_TIMEOUT, 22);
+        *abort = 1;
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint64_t da = desc0 + static_cast<uint64_t>((stage * STAGE_BYTES) >> 4);
+      const uint64_t db = da + (rt::A_BYTES >> 4);
+      if (leader) {
 #pragma unroll
-        for (int kk = 0; kk < rt::BK / 16; ++kk)
-          mma_bf16(tmem_base, sdesc_kmajor_sw128(a0 + kk * 32), sdesc_kmajor_sw128(b0 + kk * 32),
-                   IDESC, (i | kk) != 0 ? 1u : 0u);
-        mma_issued = true;
+        for (int kk = 0; kk < rt::BK / 16; ++kk)  // 16 elements = 32 bytes on
+          mma_bf16(tmem_base, da + 2 * kk, db + 2 * kk, IDESC, (i | kk) != 0 ? 1u : 0u);
         mma_commit(&s.empty[stage]);
       }
-      if (ok && !*abort) {
-        if (mma_issued) mma_commit(&s.tfull);
-        else mbar_arrive(&s.tfull);  // empty K share: nothing to wait for
-      }
+      mma_issued = true;
+    }
+    if (ok && leader) {
+      if (mma_issued) mma_commit(&s.tfull);
+      else mbar_arrive(&s.tfull);  // empty K share: nothing to wait for
     }
   } else {
     // the selection tables, while the TMA and MMA warps run (named barrier 1:
@@ -1800,7 +1805,7 @@ __global__ void __launch_bounds__(rt::THREADS, 1) router_select_kernel(
     if (warp == 0 && lane == 0)
       for (int st = 0; st < STAGES; ++st)
         if ((issued_mask >> st) & 1u) mbar_wait(&s.full[st], (last_phase_bits >> st) & 1u, limit_ns, never);
-    if (warp == 1 && lane == 0 && mma_issued) {
+    if (leader && mma_issued) {  // the lane that issued the MMAs
       mma_commit(&s.drain);
       mbar_wait(&s.drain, 0, limit_ns, never);
     }
@@ -1822,8 +1827,7 @@ __global__ void __launch_bounds__(rt::THREADS, 1) router_select_kernel(
 // select_lanes_kernel). Bound by latency: the K share's loads, one cluster
 // barrier and the slots' serial argmins. One CTA of two with all 128 tokens, a
 // thread each, and the selection in a launch of its own took 14.2 + 9.8 us for 33
-// tokens of 64 experts, d 2048 (ncu), 14.7 + 11.2 for 1021; this takes
-// 13.4 and
+// tokens of 64 experts, d 2048 (ncu), 14.7 + 11.2 for 1021; this takes 13.4 and
 // 14.3. (The token's row of the delay table staged in shared memory: 14.2, 14.8.)
 namespace rl {
 constexpr int SPLIT = 8;
