@@ -715,9 +715,9 @@ def route_launches(T, E, d):
 
 
 def dispatch_launches(T, k):
-    """Kernels of one dispatch call: up to 4096 entries are counted, ranked and
+    """Kernels of one dispatch call: up to 9728 entries are counted, ranked and
     copied in one launch."""
-    return 1 if T * k <= 4096 else 4
+    return 1 if T * k <= 9728 else 4
 
 
 def decode_launches(w, H):

@@ -1,7 +1,7 @@
 // Token permutation (histogram, prefix sum, stable scatter + row gather) and
 // the weighted combine.
 //
-// Up to 4096 entries (a decode step, a short chunk) one launch counts,
+// Up to 9728 entries (a decode step, a chunk) one launch counts,
 // ranks and copies (dispatch_gather_kernel). Otherwise the (token, slot)
 // entries i = t*k + j are cut into chunks of kChunk = 256 consecutive
 // entries, one block each:
@@ -422,25 +422,34 @@ __global__ void __launch_bounds__(kNormThreads) residual_norm_kernel(
 //
 // Bound: latency (launch, one L2 round trip for the entries, the counts), and
 // from a few thousand entries the counting, which every block repeats: more
-// entries a block then, at the price of rows copied one after another. Times of
-// the call in a graph, 64 experts, 2048 columns, against one block ranking all
+// entries a block then, at the price of rows copied one after another. Counters
+// in eight copies: one copy took 17.5 us for 9216 entries of one expert, ranking
+// equal lanes by a match instruction 10.6 for 4092 of 64 experts.
+// Times of the call in a graph, 2048 columns, against one block ranking all
 // entries (the chunked path from 4097 on) and a launch for the copies:
-//   entries      384   1218   2046   4092   6126
-//   before       6.0    8.2   10.5   16.5   11.4 us
-//   8 a block    3.2    4.8    7.4   18.4   37.2
-//   16           4.1    5.3    6.5   12.4   21.7
-//   32           5.5    6.8    7.9   10.6   18.1
-// and 256 entries of 8 experts, 4096 columns: 4.0 + 5.0 against 5.6 us (ncu).
-constexpr int kSmallN = 4096;
-inline int small_per_block(int64_t n) { return n <= 1216 ? 8 : n <= 2432 ? 16 : 32; }
+//   entries, experts  198 64   1218 64   2046 64   4092 64   6126 64   9216 64   9216 1
+//   before            5        8.2       10.5      16.5      11.7      13.6      13.2 us
+//   8 a block         2.5      3.1       4.0       6.4       10.4      15.0      16.2
+//   16                3.3      3.4       3.8       5.7       8.9       12.0      13.0
+//   32                4.7      4.9       5.1       5.8       8.4       9.5       10.3
+// (12288: 14.7 of 32 a block, 14.6 chunked.) The lines lie at 152 blocks of 8, of 32
+// and two of those an SM (64 entries).
+constexpr int kSmallN = 9728;
+static_assert(kSmallN < 65536, "counts in 16 bits");
+inline int small_per_block(int64_t n) { return n <= 1216 ? 8 : n <= 4864 ? 16 : 32; }
 
-__global__ void __launch_bounds__(256) dispatch_gather_kernel(
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) dispatch_gather_kernel(
     const int32_t* __restrict__ chosen, const uint16_t* __restrict__ X, int n, int k, int E, int d,
     int per, int32_t* __restrict__ offsets, int32_t* __restrict__ row_token,
     int32_t* __restrict__ row_of, uint16_t* __restrict__ X_perm) {
   pdl_trigger();  // launched with launch_pdl: no global access before pdl_wait
   pdl_wait();
-  __shared__ int total[64], before[64], start[64];
+  // entries of an expert, those before the block's << 16, in copies (lanes of a
+  // warp on one counter take turns, so on one expert they are split over eight)
+  constexpr int kCopies = 8, kPitch = 65;
+  __shared__ unsigned count[kCopies * kPitch];
+  __shared__ int start[64];
   constexpr int kUnroll = 8;  // 16-byte vectors of a row a lane has in flight
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int begin = blockIdx.x * per;
@@ -454,36 +463,35 @@ __global__ void __launch_bounds__(256) dispatch_gather_kernel(
     for (int u = 0; u < kUnroll; ++u)
       if (lane + 32 * u < nvec) buf[u] = __ldg(in + lane + 32 * u);
   };
-  if (begin + warp < n) load_head(begin + warp);
-  if (tid < 64) total[tid] = before[tid] = 0;
+  if (warp < per && begin + warp < n) load_head(begin + warp);
+  for (int i = tid; i < kCopies * kPitch; i += THREADS) count[i] = 0;
   __syncthreads();
+  unsigned* mine_count = count + (lane & (kCopies - 1)) * kPitch;
   constexpr int kLoads = 4;
-  for (int j0 = 0; j0 < n; j0 += kLoads * 256) {
+  for (int j0 = tid; j0 < n; j0 += kLoads * THREADS) {
     int e[kLoads];
 #pragma unroll
     for (int u = 0; u < kLoads; ++u) {
-      const int j = j0 + u * 256 + tid;
-      e[u] = j < n ? chosen[j] : -1;
+      const int j = j0 + u * THREADS;
+      e[u] = j < n ? chosen[j] : 0;
     }
 #pragma unroll
     for (int u = 0; u < kLoads; ++u) {
-      const int w0 = j0 + u * 256 + warp * 32;  // the warp's first entry
-      if (w0 >= n) break;
-      const bool ok = e[u] >= 0 && e[u] < E;
-      if (!ok && w0 + lane < n && w0 + lane >= begin && w0 + lane < begin + per)
-        report(&g_err_dispatch, ORDERMOE_DEV_BAD_INDEX, w0 + lane);
-      const unsigned peers = __match_any_sync(0xffffffffu, ok ? e[u] : -1);
-      if (ok && lane == __ffs(peers) - 1) {
-        atomicAdd(&total[e[u]], __popc(peers));
-        const int nb = begin - w0;  // entries of the warp before the block's
-        const unsigned early = nb >= 32 ? peers : nb > 0 ? peers & ((1u << nb) - 1u) : 0u;
-        if (early != 0u) atomicAdd(&before[e[u]], __popc(early));
-      }
+      const int j = j0 + u * THREADS;
+      if (j >= n) break;
+      if (e[u] >= 0 && e[u] < E) atomicAdd(&mine_count[e[u]], j < begin ? 0x10001u : 1u);
+      else if (j >= begin && j < begin + per) report(&g_err_dispatch, ORDERMOE_DEV_BAD_INDEX, j);
     }
   }
   __syncthreads();
   if (warp == 0) {  // offsets, two experts a lane
-    const int n0 = total[2 * lane], n1 = total[2 * lane + 1];
+    unsigned c0 = 0, c1 = 0;  // sums of at most kSmallN in either half
+#pragma unroll
+    for (int c = 0; c < kCopies; ++c) {
+      c0 += count[c * kPitch + 2 * lane];
+      c1 += count[c * kPitch + 2 * lane + 1];
+    }
+    const int n0 = static_cast<int>(c0 & 0xFFFFu), n1 = static_cast<int>(c1 & 0xFFFFu);
     int in = n0 + n1;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -491,8 +499,8 @@ __global__ void __launch_bounds__(256) dispatch_gather_kernel(
       if (lane >= o) in += u;
     }
     const int s0 = in - n0 - n1, s1 = in - n1;
-    start[2 * lane] = s0 + before[2 * lane];
-    start[2 * lane + 1] = s1 + before[2 * lane + 1];
+    start[2 * lane] = s0 + static_cast<int>(c0 >> 16);
+    start[2 * lane + 1] = s1 + static_cast<int>(c1 >> 16);
     if (blockIdx.x == 0) {
       if (2 * lane <= E) offsets[2 * lane] = s0;
       if (2 * lane + 1 <= E) offsets[2 * lane + 1] = s1;
@@ -500,7 +508,8 @@ __global__ void __launch_bounds__(256) dispatch_gather_kernel(
     }
   }
   __syncthreads();
-  for (int x = warp; x < per && begin + x < n; x += 8) {
+  constexpr int kWarps = THREADS / 32;
+  for (int x = warp; x < per && begin + x < n; x += kWarps) {
     const int i = begin + x;
     const int e = __shfl_sync(0xffffffffu, mine, x);
     const unsigned same = __ballot_sync(0xffffffffu, mine == e);
@@ -523,7 +532,7 @@ __global__ void __launch_bounds__(256) dispatch_gather_kernel(
           if (v0 + 32 * u < nvec) buf[u] = __ldg(in + v0 + 32 * u);
       }
     }
-    if (x + 8 < per && begin + x + 8 < n) load_head(begin + x + 8);
+    if (x + kWarps < per && begin + x + kWarps < n) load_head(begin + x + kWarps);
   }
 }
 
@@ -549,9 +558,13 @@ int dispatch_launch(const int32_t* chosen, const uint16_t* X, int T, int k, int 
   if (n <= kSmallN && apart(row_of, n * sizeof(int32_t)) && apart(row_token, n * sizeof(int32_t)) &&
       apart(offsets, (E + 1) * sizeof(int32_t)) && apart(X_perm, n * (size_t)d * 2)) {
     const int per = small_per_block(n);
-    OM_LAUNCH_PDL("dispatch_gather_kernel", dispatch_gather_kernel,
-                  dim3(static_cast<unsigned>((n + per - 1) / per)), dim3(256), 0, stream, chosen, X,
-                  static_cast<int>(n), k, E, d, per, offsets, row_token, row_of, X_perm);
+    const dim3 grid(static_cast<unsigned>((n + per - 1) / per));
+    if (per <= 8)
+      OM_LAUNCH_PDL("dispatch_gather_kernel", dispatch_gather_kernel<256>, grid, dim3(256), 0, stream, chosen,
+                    X, static_cast<int>(n), k, E, d, per, offsets, row_token, row_of, X_perm);
+    else
+      OM_LAUNCH_PDL("dispatch_gather_kernel", dispatch_gather_kernel<512>, grid, dim3(512), 0, stream, chosen,
+                    X, static_cast<int>(n), k, E, d, per, offsets, row_token, row_of, X_perm);
     return ORDERMOE_OK;
   }
   OM_LAUNCH_PDL("chunk_hist_kernel", chunk_hist_kernel, dim3(nchunks), dim3(kChunk), 0, stream,

@@ -203,8 +203,7 @@ def test_router_exact_ties_every_list_width(E, k):
 # ------------------------------------------------------------------ permutation
 
 @pytest.mark.parametrize("T,k,E,d", [(64, 2, 8, 256), (1000, 6, 64, 64), (1, 1, 1, 8), (333, 3, 7, 40),
-                                     # sizes of one launch up to its limit of 4096, and the
-                                     # first size past it
+                                     # sizes of one launch
                                      (1500, 2, 8, 64), (2048, 2, 8, 16), (683, 6, 64, 8),
                                      (4096, 2, 8, 4096),
                                      (8192, 6, 64, 64),     # 192 chunks: the scan holds them in registers
@@ -233,9 +232,9 @@ def test_dispatch_bit_exact(T, k, E, d):
 
 @pytest.mark.parametrize("T,k,E,d", [
     (1, 1, 1, 8), (9, 1, 5, 8), (152, 8, 64, 2304),   # eight entries a block: one, a ragged last, the most
-    (1217, 1, 33, 264), (304, 8, 64, 24),             # sixteen: the fewest, the most
-    (2433, 1, 12, 8), (512, 8, 64, 520),              # 32: the fewest, the most
-    (4097, 1, 7, 8)])                                 # the first size of the chunked path
+    (1217, 1, 33, 264), (608, 8, 64, 24),             # sixteen: the fewest, the most
+    (4865, 1, 12, 8), (1216, 8, 64, 520), (9000, 1, 1, 8),  # 32: the fewest, the most, one expert
+    (9729, 1, 7, 8)])                                 # the first size of the chunked path
 def test_dispatch_in_one_launch_skips_and_reports_bad_experts(T, k, E, d):
     """The permutation of the entries with a valid expert; the others are left out
     and one of them is reported. The same with row_of in the place of chosen."""
