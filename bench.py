@@ -709,9 +709,9 @@ def decode_timed(args, dist, w, device, S, H):
 
 def route_launches(T, E, d):
     """Kernels of one route_select call (H = 1): 1, or 2 with a lane selection
-    kernel of its own for more than 16 experts where the clusters of eight
-    (128 tokens each) do not fit on 152 SMs at once."""
-    return 1 if E <= 16 or (8 * ((T + 127) // 128) <= 152 and d // 64 >= 8) else 2
+    kernel of its own for more than 16 experts where one CTA for every 16
+    tokens does not fit on 152 SMs at once."""
+    return 1 if E <= 16 or ((T + 15) // 16 <= 152 and d // 64 >= 8) else 2
 
 
 def dispatch_launches(T, k):

@@ -1841,32 +1841,46 @@ __global__ void __launch_bounds__(rt::THREADS, 1) router_select_kernel(
 }
 
 // Small batches of 17 to 64 experts: router, top-k and selection in one launch.
-// A cluster of 8 CTAs handles 128 tokens, CTA r an eighth of the K blocks (as in
-// router_select_kernel), and then the tokens 16 r .. 16 r + 15: every CTA
-// scatters its partial logits to the tokens' owners (distributed shared memory),
-// and each owner adds the eight partials in rank order and gives a token eight
+// A cluster of S CTAs (two for more than 32 experts, else four) handles 16 S
+// tokens, CTA r the r-th of S shares of the K blocks, and then the tokens 16 r ..
+// 16 r + 15: every CTA stores its partial logits of a token into the shared memory
+// of the CTA that owns it, which adds them in rank order and gives the token eight
 // lanes for the top-k, the softmax and the slots of Alg. 2 (select_slots, as
-// select_lanes_kernel). Bound by latency: the K share's loads, one cluster
-// barrier and the slots' serial argmins. One CTA of two with all 128 tokens, a
-// thread each, and the selection in a launch of its own took 14.2 + 9.8 us for 33
-// tokens of 64 experts, d 2048 (ncu), 14.7 + 11.2 for 1021; this takes 13.4 and
-// 14.3. (The token's row of the delay table staged in shared memory: 14.2, 14.8.)
+// select_lanes_kernel). The shares are router_select_kernel's at its largest
+// split, so a token's logits are the same bits from either kernel.
+// The MMA's M side is 128 rows, of which the tokens' 16 S are loaded; it reads the
+// rest from the stage's own weights and from padding that nothing writes, and
+// those rows of the accumulator are not read.
+// Bound by latency: the K share's loads, two cluster barriers and the slots'
+// serial argmins. In a graph of calls, tokens x experts, d 2048: one CTA of two
+// with all 128 tokens, a thread each, and the selection in a launch of its own took
+// 19.5 us for 33 x 64 and 20.2 for 1021 x 64, this takes 11.6 and 12.0 (d 4096:
+// 27.0 and 15.9); 12.4 and 8.5 for 33 x 24, d 1024. Stages of one K block, ten of
+// them: 12.1 and 12.5. (Eight shares of K for 128 tokens took 11.1 and 11.4 us, but
+// their logits differ from the other kernel's in the last bits.)
 namespace rl {
-constexpr int SPLIT = 8;
-constexpr int ROWS = 128 / SPLIT;  // tokens of a CTA
-constexpr int STAGES = 5;
+constexpr int ROWS = 16;  // tokens of a CTA
+constexpr int STAGES = 5;  // of two K blocks each
 constexpr int THREADS = 192;
+template <int NE>
+constexpr int split() { return rt::max_split<NE>(); }
+template <int NE>
+constexpr int a_bytes() { return split<NE>() * ROWS * rt::BK * 2; }  // the tokens' rows
+constexpr int BLOCK_BYTES = rt::A_BYTES;  // what an MMA's 128 rows span
 // partials of one rank: [NE / 4 chunks][ROWS + 1][4] floats (the odd pitch spreads
 // the chunks that the eight lanes of a token read over the banks)
 template <int NE>
 constexpr int part_floats() { return NE / 4 * (ROWS + 1) * 4; }
-constexpr int LG_PITCH = 68;  // floats a token's logits take
+constexpr int LG_PITCH = 68;  // floats a token's exponentials take
 template <int NE>
 constexpr int smem_bytes(int E) {
-  return 1024 + STAGES * (rt::A_BYTES + NE * rt::BK * 2) + 256 + SPLIT * part_floats<NE>() * 4 +
-         2 * ROWS * LG_PITCH * 4 + 8 * E * E;
+  return 1024 + STAGES * 2 * BLOCK_BYTES + 256 + split<NE>() * part_floats<NE>() * 4 + ROWS * LG_PITCH * 4 +
+         8 * E * E;
 }
+static_assert(smem_bytes<32>(32) + sizeof(SelSmem) <= 227 * 1024, "router shared memory");
 static_assert(smem_bytes<64>(64) + sizeof(SelSmem) <= 227 * 1024, "router shared memory");
+static_assert(a_bytes<32>() + 32 * rt::BK * 2 <= BLOCK_BYTES, "rows and weights of a K block");
+static_assert(a_bytes<64>() + 64 * rt::BK * 2 <= BLOCK_BYTES, "rows and weights of a K block");
 }  // namespace rl
 
 struct RouterLanesSmem {
@@ -1880,7 +1894,7 @@ struct RouterLanesSmem {
 };
 
 template <int NE>
-__global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1, 1)
+__global__ void __launch_bounds__(rl::THREADS, 1)
     router_lanes_kernel(const __grid_constant__ CUtensorMap mapX,
                         const __grid_constant__ CUtensorMap mapW, int T, int E, int d, int k,
                         int renorm, const uint8_t* __restrict__ tab,
@@ -1891,23 +1905,25 @@ __global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1,
                         uint8_t* __restrict__ kind_out, int32_t* __restrict__ counters,
                         uint64_t limit_ns, int topk_only) {
   pdl_trigger();  // launched with programmatic serialization: set-up first
-  constexpr int STAGE_BYTES = rt::A_BYTES + NE * rt::BK * 2;
+  constexpr int SPLIT = rl::split<NE>();
+  constexpr int TILE = SPLIT * rl::ROWS;  // tokens of the cluster
+  constexpr int BLOCK_BYTES = rl::BLOCK_BYTES, STAGE_BYTES = 2 * BLOCK_BYTES;
+  constexpr int A_BYTES = rl::a_bytes<NE>(), B_BYTES = NE * rt::BK * 2;
   constexpr int TMEM_COLS = NE;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   RouterLanesSmem& s = *reinterpret_cast<RouterLanesSmem*>(tiles + rl::STAGES * STAGE_BYTES);
   float* part = reinterpret_cast<float*>(tiles + rl::STAGES * STAGE_BYTES + 256);
-  float* s_lg = part + rl::SPLIT * rl::part_floats<NE>();  // [ROWS][LG_PITCH] logits
-  float* s_ex = s_lg + rl::ROWS * rl::LG_PITCH;            // their exponentials
+  float* s_ex = part + SPLIT * rl::part_floats<NE>();  // [ROWS][LG_PITCH] the logits' exponentials
   float* s_Q = s_ex + rl::ROWS * rl::LG_PITCH;
   float* s_Cq = s_Q + E * E;
   __shared__ SelSmem sm;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = static_cast<int>(cluster_ctarank());
-  const int m0 = static_cast<int>(blockIdx.x / rl::SPLIT) * 128;
+  const int m0 = static_cast<int>(blockIdx.x / SPLIT) * TILE;
   const int kblocks_all = d / rt::BK;
-  const int per = (kblocks_all + rl::SPLIT - 1) / rl::SPLIT;
+  const int per = (kblocks_all + SPLIT - 1) / SPLIT;
   const int kb_begin = min(kblocks_all, rank * per);
   const int kblocks = min(kblocks_all, kb_begin + per) - kb_begin;
 
@@ -1931,7 +1947,7 @@ __global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1,
     tmem_relinquish();
   }
   tc_fence_before();
-  __syncthreads();
+  cluster_sync();  // every CTA of the cluster runs: its shared memory may be written
   tc_fence_after();
   pdl_wait();  // the previous kernel's outputs (X, tables, state) are ready
   const uint32_t tmem_base = s.tmem_base;
@@ -1948,8 +1964,8 @@ __global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1,
 
   if (warp == 0) {
     const bool issuer = elect_one();
-    for (int i = 0; i < kblocks; ++i) {
-      const int stage = i % rl::STAGES;
+    for (int kb = 0, i = 0; kb < kblocks; kb += 2, ++i) {
+      const int stage = i % rl::STAGES, n = min(2, kblocks - kb);
       const uint32_t phase = (i / rl::STAGES) & 1;
       if (!__all_sync(0xffffffffu, mbar_wait(&s.empty[stage], phase ^ 1u, limit_ns, abort))) {
         if (issuer && !*abort) report(&g_err_route, ORDERMOE_DEV_WAIT_TIMEOUT, 24);
@@ -1958,9 +1974,11 @@ __global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1,
       }
       if (issuer) {
         uint8_t* sa = tiles + stage * STAGE_BYTES;
-        mbar_arrive_expect_tx(&s.full[stage], STAGE_BYTES);
-        tma_load_2d(sa, &mapX, &s.full[stage], (kb_begin + i) * rt::BK, m0);
-        tma_load_2d(sa + rt::A_BYTES, &mapW, &s.full[stage], (kb_begin + i) * rt::BK, 0);
+        mbar_arrive_expect_tx(&s.full[stage], n * (A_BYTES + B_BYTES));
+        for (int j = 0; j < n; ++j, sa += BLOCK_BYTES) {
+          tma_load_2d(sa, &mapX, &s.full[stage], (kb_begin + kb + j) * rt::BK, m0);
+          tma_load_2d(sa + A_BYTES, &mapW, &s.full[stage], (kb_begin + kb + j) * rt::BK, 0);
+        }
       }
       issued_mask |= 1u << stage;
       last_phase_bits = (last_phase_bits & ~(1u << stage)) | (phase << stage);
@@ -1970,8 +1988,8 @@ __global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1,
     leader = elect_one();
     const uint64_t desc0 = sdesc_kmajor_sw128(smem_u32(tiles));
     bool ok = true;
-    for (int i = 0; i < kblocks; ++i) {
-      const int stage = i % rl::STAGES;
+    for (int kb = 0, i = 0; kb < kblocks; kb += 2, ++i) {
+      const int stage = i % rl::STAGES, n = min(2, kblocks - kb);
       const uint32_t phase = (i / rl::STAGES) & 1;
       if (!__all_sync(0xffffffffu, mbar_wait(&s.full[stage], phase, limit_ns, abort))) {
         if (leader && !*abort) report(&g_err_route, ORDERMOE_DEV_WAIT_TIMEOUT, 25);
@@ -1980,12 +1998,14 @@ __global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1,
         break;
       }
       tc_fence_after();
-      const uint64_t da = desc0 + static_cast<uint64_t>((stage * STAGE_BYTES) >> 4);
-      const uint64_t db = da + (rt::A_BYTES >> 4);
+      const uint64_t da0 = desc0 + static_cast<uint64_t>((stage * STAGE_BYTES) >> 4);
       if (leader) {
+        for (int j = 0; j < n; ++j) {
+          const uint64_t da = da0 + static_cast<uint64_t>((j * BLOCK_BYTES) >> 4), db = da + (A_BYTES >> 4);
 #pragma unroll
-        for (int kk = 0; kk < rt::BK / 16; ++kk)  // 16 elements = 32 bytes on
-          mma_bf16(tmem_base, da + 2 * kk, db + 2 * kk, IDESC, (i | kk) != 0 ? 1u : 0u);
+          for (int kk = 0; kk < rt::BK / 16; ++kk)  // 16 elements = 32 bytes on
+            mma_bf16(tmem_base, da + 2 * kk, db + 2 * kk, IDESC, (kb | j | kk) != 0 ? 1u : 0u);
+        }
         mma_commit(&s.empty[stage]);
       }
       mma_issued = true;
@@ -2007,15 +2027,15 @@ __global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1,
     }
     // this CTA's partial logits to the tokens' owners
     const int q = warp & 3;
-    const int r128 = q * 32 + lane;
-    const bool ok = __all_sync(0xffffffffu, mbar_wait(&s.tfull, 0, limit_ns, abort));
+    const int r = q * 32 + lane;  // TMEM lane: row of the tile
+    const bool ok = q * 32 >= TILE || __all_sync(0xffffffffu, mbar_wait(&s.tfull, 0, limit_ns, abort));
     if (!ok) {
       if (lane == 0 && !*abort) report(&g_err_route, ORDERMOE_DEV_WAIT_TIMEOUT, 26);
       *abort = 1;
-    } else {
+    } else if (q * 32 < TILE) {
       tc_fence_after();
       const uint32_t dst = mapa_shared(
-          smem_u32(part + rank * rl::part_floats<NE>() + (r128 % rl::ROWS) * 4), r128 / rl::ROWS);
+          smem_u32(part + rank * rl::part_floats<NE>() + (r % rl::ROWS) * 4), r / rl::ROWS);
 #pragma unroll
       for (int c = 0; c < NE; c += 32) {
         uint32_t v[32];
@@ -2037,7 +2057,6 @@ __global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1,
   cluster_sync();  // the partials of every CTA are there (and the tables, in the block)
   if (warp >= 2 && !*abort) {
     // the token's logits: chunks of four experts over its lanes, ranks in order
-    float* lg = s_lg + row * rl::LG_PITCH;
     float* ex = s_ex + row * rl::LG_PITCH;
     bool nan = false;
     float v[NE / 8];
@@ -2047,7 +2066,7 @@ __global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1,
       const float* src = part + (c * (rl::ROWS + 1) + row) * 4;
       float4 x = *reinterpret_cast<const float4*>(src);
 #pragma unroll
-      for (int r = 1; r < rl::SPLIT; ++r) {
+      for (int r = 1; r < SPLIT; ++r) {
         const float4 y = *reinterpret_cast<const float4*>(src + r * rl::part_floats<NE>());
         x.x += y.x;
         x.y += y.y;
@@ -2063,7 +2082,6 @@ __global__ void __launch_bounds__(rl::THREADS, 1) __cluster_dims__(rl::SPLIT, 1,
         nan |= xs[u] != xs[u];
         v[4 * h + u] = xs[u];
       }
-      *reinterpret_cast<float4*>(lg + 4 * c) = make_float4(xs[0], xs[1], xs[2], xs[3]);
     }
     const unsigned group = 0xFFu << (lane & 24);  // the token's lanes
     nan = (__ballot_sync(0xffffffffu, nan) & group) != 0u;
@@ -2341,11 +2359,19 @@ static int route_select_impl(const uint16_t* X, const uint16_t* W_r, const float
   CUtensorMap mX, mW;
   int rc;
   const int NE = E <= 16 ? 16 : (E <= 32 ? 32 : 64);
-  if ((rc = make_tmap_bf16(&mX, X, T, d, 128))) return rc;
-  if ((rc = make_tmap_bf16(&mW, W_r, E, d, NE))) return rc;
   const uint64_t lim = wait_limit_ns();
-  // split K over a cluster so that about one CTA per SM streams X
   const int kblocks = d / rt::BK;
+  // Small batches of many experts: one CTA for every 16 tokens, all resident at
+  // once (up to 2432 tokens on 152 SMs). Larger ones fill the SMs with the tokens,
+  // and the selection in rounds would be longer than a launch over all SMs.
+  // (d >= 512: narrower routers are a few K blocks.)
+  const int rl_split = NE == 32 ? rl::split<32>() : rl::split<64>();
+  const int rl_tile = rl_split * rl::ROWS;
+  const long long rl_tiles = (T + rl_tile - 1) / rl_tile;
+  const bool small = E > 16 && rl_tiles * rl_split <= num_sms() && kblocks >= 8;
+  if ((rc = make_tmap_bf16(&mX, X, T, d, small ? rl_tile : 128))) return rc;
+  if ((rc = make_tmap_bf16(&mW, W_r, E, d, NE))) return rc;
+  // split K over a cluster so that about one CTA per SM streams X
   const int smax = NE == 16 ? rt::max_split<16>() : (NE == 32 ? rt::max_split<32>() : rt::max_split<64>());
   int split = 1;
   while (split * 2 <= smax && (long long)blocks * split * 2 <= num_sms() && split * 2 <= kblocks)
@@ -2375,15 +2401,10 @@ static int route_select_impl(const uint16_t* X, const uint16_t* W_r, const float
   cfg.attrs = attr;
   cfg.numAttrs = pdl_on(stream) ? 2 : 1;
   cudaError_t le;
-  // Small batches of many experts: all eight CTAs of every cluster can be
-  // resident and each has K blocks (up to 2432 tokens on 152 SMs, d >= 512).
-  // Larger ones fill the SMs with the tokens, and the selection of 128 tokens by
-  // one CTA in eight rounds would be longer than a launch over all SMs.
-  if (E > 16 && (long long)blocks * rl::SPLIT <= num_sms() && kblocks >= rl::SPLIT) {
-    cfg.gridDim = dim3(blocks * rl::SPLIT, 1, 1);
+  if (small) {
+    cfg.gridDim = dim3(static_cast<unsigned>(rl_tiles * rl_split), 1, 1);
     cfg.blockDim = dim3(rl::THREADS, 1, 1);
-    attr[0] = attr[1];  // the cluster shape is the kernel's own
-    cfg.numAttrs = pdl_on(stream) ? 1 : 0;
+    attr[0].val.clusterDim.x = rl_split;
     const int only = la.H > 1 ? 1 : 0;
     if (NE == 32) {
       cfg.dynamicSmemBytes = rl::smem_bytes<32>(E);

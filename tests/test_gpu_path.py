@@ -200,6 +200,62 @@ def test_router_exact_ties_every_list_width(E, k):
     np.testing.assert_array_equal(outs[4].cpu().numpy(), kd)
 
 
+@pytest.mark.parametrize("T,d,E,k,renorm", [
+    (40, 576, 24, 3, 1),    # nine K blocks in four shares: 3, 3, 3 and none; tokens missing in the tile
+    (33, 576, 64, 6, 0),    # in two shares: 5 and 4; one token in the last tile
+    (65, 1024, 17, 1, 0), (130, 2048, 64, 8, 1)])
+def test_router_small_batch_sums_the_larger_batches_shares(T, d, E, k, renorm):
+    """A batch whose clusters fit on the SMs splits K into the shares that
+    every router launch of so few tokens takes (two above 32 experts, else
+    four): its logits are the partial logits of the shares, which a batch of a
+    128-token tile an SM accumulates whole, added in order, bit for bit. Targets,
+    weights and selection follow from those logits; a token with a NaN has none
+    and is reported."""
+    S = 2 if E > 32 else 4
+    w = synth.workload("tiny", T=T, d=d, E=E, n_clusters=1)
+    inp = synth.layer_inputs(w, seed=T, with_ffn=False)
+    X, Wr, home, M = inp["X"].to(DEV), inp["Wr"].to(DEV), inp["home"], w.M
+    sim, group, x = random_tables_case(np.random.default_rng(E + k), E, M, 2)
+    sp = synth.server_params(M, d, w.dff, 0)
+    tab = build_tables(sim, group, x, 0.3, 0.1, sp, DEV)
+
+    def route(X, W, home):
+        n = X.shape[0]
+        logits = torch.empty(n, E, dtype=torch.float32, device=DEV)
+        outs = [torch.empty(n, k, dtype=dt, device=DEV)
+                for dt in (torch.int32, torch.float32, torch.int32, torch.uint8, torch.uint8)]
+        loc, q = dev(home), torch.zeros(n, device=DEV)
+        B.ordermoe_route_select(X, W, None, n, E, X.shape[1], k, renorm, tab, dev(home), loc, q, logits,
+                                *outs)
+        return [logits.cpu().numpy()] + [o.cpu().numpy() for o in outs] + [loc.cpu().numpy(), q.cpu().numpy()]
+
+    big = 128 * torch.cuda.get_device_properties(0).multi_processor_count
+    per = -(-(d // 64) // S) * 64
+    want = None
+    for k0 in range(0, d, per):
+        Xs, Ws = X[:, k0:k0 + per], Wr[:, k0:k0 + per].contiguous()
+        part = route(Xs.repeat(-(-big // T), 1)[:big].contiguous(), Ws, np.resize(home, big))[0][:T]
+        want = part if want is None else want + part
+    nan_row = T - 1
+    for bad in (False, True):
+        Xb = X.clone()
+        if bad:
+            Xb[nan_row, d // 2] = float("nan")
+        got, idx, wt, ch, sv, kd, loc, q = route(Xb, Wr, home)
+        ok = np.arange(T) != (nan_row if bad else -1)
+        assert B.ordermoe_device_error() == ((B.DEV_NAN_LOGIT, nan_row) if bad else (0, 0))
+        np.testing.assert_array_equal(got[ok], want[ok])
+        o_idx, o_w = oracle.topk(got[ok], k, renorm)
+        np.testing.assert_array_equal(idx[ok], o_idx)
+        np.testing.assert_allclose(wt[ok], o_w, rtol=1e-5, atol=1e-7)
+        if bad:
+            assert (idx[nan_row] == -1).all() and (wt[nan_row] == 0).all()
+        otab = oracle.tables(sim, group, x, 0.3, 0.1, sp.F, sp.B, sp.tau, sp.z, sp.c, sp.omega_T, sp.omega_Q)
+        h = home[ok]
+        for a, b in zip((ch, sv, kd, loc, q), oracle.select(o_idx, otab, h, h.copy(), np.zeros(len(h), np.float32))):
+            np.testing.assert_array_equal(a[ok], b)
+
+
 # ------------------------------------------------------------------ permutation
 
 @pytest.mark.parametrize("T,k,E,d", [(64, 2, 8, 256), (1000, 6, 64, 64), (1, 1, 1, 8), (333, 3, 7, 40),
