@@ -1669,7 +1669,8 @@ __global__ void __launch_bounds__(rt::THREADS, 1) router_select_kernel(
   int pre_a = 0, pre_s = 0;  // the token's home and location, loaded during the main loop
   float pre_q = 0.0f;
   tc_fence_before();
-  __syncthreads();
+  if (split > 1) cluster_sync();  // rank 0 runs: its shared memory may be written
+  else __syncthreads();
   tc_fence_after();
   pdl_wait();  // the previous kernel's outputs (X, tables, state) are ready
   const uint32_t tmem_base = s.tmem_base;

@@ -200,18 +200,20 @@ def test_router_exact_ties_every_list_width(E, k):
     np.testing.assert_array_equal(outs[4].cpu().numpy(), kd)
 
 
-@pytest.mark.parametrize("T,d,E,k,renorm", [
-    (40, 576, 24, 3, 1),    # nine K blocks in four shares: 3, 3, 3 and none; tokens missing in the tile
-    (33, 576, 64, 6, 0),    # in two shares: 5 and 4; one token in the last tile
-    (65, 1024, 17, 1, 0), (130, 2048, 64, 8, 1)])
-def test_router_small_batch_sums_the_larger_batches_shares(T, d, E, k, renorm):
-    """A batch whose clusters fit on the SMs splits K into the shares that
-    every router launch of so few tokens takes (two above 32 experts, else
-    four): its logits are the partial logits of the shares, which a batch of a
-    128-token tile an SM accumulates whole, added in order, bit for bit. Targets,
-    weights and selection follow from those logits; a token with a NaN has none
-    and is reported."""
-    S = 2 if E > 32 else 4
+@pytest.mark.parametrize("T,d,E,S,k,renorm", [
+    # 17 experts and more: the kernel of small batches, or below d = 512 the larger batches'
+    (40, 576, 24, 4, 3, 1),    # nine K blocks in four shares: 3, 3, 3 and none; tokens missing in the tile
+    (33, 576, 64, 2, 6, 0),    # in two shares: 5 and 4; one token in the last tile
+    (65, 1024, 17, 4, 1, 0), (130, 2048, 64, 2, 8, 1),
+    (40, 320, 24, 4, 3, 0), (50, 448, 64, 2, 6, 1),  # 2, 2, 1 and none; 4 and 3
+    # up to 16 experts: 2, 2, 2, 2, 1 and none three times; 2 and 1; 2, 2, 1 and none over two tiles
+    (40, 576, 8, 8, 2, 1), (5, 192, 16, 2, 4, 0), (200, 320, 13, 4, 2, 1)])
+def test_router_sums_its_shares_of_k(T, d, E, S, k, renorm):
+    """A batch of few tokens splits K into S shares over a cluster: its logits
+    are the partial logits of the shares, which a batch of a 128-token tile an
+    SM accumulates whole, added in order, bit for bit. Targets, weights and
+    selection follow from those logits; a token with a NaN has none and is
+    reported."""
     w = synth.workload("tiny", T=T, d=d, E=E, n_clusters=1)
     inp = synth.layer_inputs(w, seed=T, with_ffn=False)
     X, Wr, home, M = inp["X"].to(DEV), inp["Wr"].to(DEV), inp["home"], w.M
