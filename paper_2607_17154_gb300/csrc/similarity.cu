@@ -1446,6 +1446,7 @@ __global__ void __launch_bounds__(kRepThreads) replicate_kernel(
       const double pj = s < nc ? __longlong_as_double(static_cast<long long>(key[s])) : 0.0;
       const uint32_t lg = rec >> 6;  // layer and group
       bool open = s < nc && !((cov[lg >> 6] >> (lg & 63u)) & 1ull);  // B = 0 once the group is local
+      __syncwarp();  // read before a lane below sets a bit
       for (;;) {
         const double b1 = __dadd_rn(b, pj);
         const unsigned bal = __ballot_sync(full, open && b1 <= cap);  // Eq. 35
@@ -1459,8 +1460,8 @@ __global__ void __launch_bounds__(kRepThreads) replicate_kernel(
           cov[lg >> 6] |= 1ull << (lg & 63u);
         }
         ++count;
+        __syncwarp();  // the next take may set a bit of the same word, and the next 32 read it
       }
-      __syncwarp();  // the groups covered here are seen by the next 32
     }
     if (lane == 0) {
       used[m] = b;

@@ -431,6 +431,29 @@ def test_replicate_bit_exact(L, E, M, ratio, seed):
         assert ref[2].sum() > 0
 
 
+@pytest.mark.parametrize("L,E,G,C", [(1, 64, 16, 1e9), (2, 64, 32, 1e9), (1, 64, 64, 1e9), (3, 40, 9, 120.0),
+                                     (20, 64, 16, 1e9)])  # the last: past the counted candidates
+def test_replicate_takes_groups_of_one_layer_in_a_window(L, E, G, C):
+    """Within a group the benefit and the memory fall together, so every
+    candidate stays until its group is covered: many takes of one layer lie in
+    one window of 32, and a group's later candidates in the next ones must find
+    it covered."""
+    rng = np.random.default_rng(L * E + G)
+    group = np.stack([rng.permutation(E) % G for _ in range(L)]).astype(np.int32)
+    order = rng.random((L, E))
+    p = 1.0 + np.round(order * 64) / 8        # larger importance, larger memory: none is passed over
+    imp = p * (1.0 + order)
+    M = 3
+    C = np.full(M, C)
+    x0 = np.zeros((L, M, E), np.uint8)
+    ref = oracle.replicate(group, imp, p, C, np.array([0.5, 0.3, 0.2]), x0, np.zeros(M))
+    got = gpu_replicate(group, imp, p, C, np.array([0.5, 0.3, 0.2]), x0, np.zeros(M))
+    for name, a, b in zip(("placement", "used", "replicas"), got, ref):
+        np.testing.assert_array_equal(a, b, err_msg=name)
+    if C[0] > 1e6:
+        assert (ref[2] == L * G).all()
+
+
 def test_replicate_largest_shape_and_errors():
     rng = np.random.default_rng(8)
     L, E, M = 256, 64, 4                          # L * E = 16384, the largest sort

@@ -1,6 +1,9 @@
-"""Distributed shared memory may be accessed once every CTA of the cluster is
+"""Barriers whose lack a run need not show, read from the sources.
+
+Distributed shared memory may be accessed once every CTA of the cluster is
 known to run: a kernel that maps an address of a peer CTA meets a cluster
-barrier first (read from the sources, since a run need not show its lack)."""
+barrier first. Votes and shuffles order no memory: lanes of a warp that change
+one shared word in turn need a warp barrier between them."""
 import glob
 import os
 import re
@@ -35,3 +38,17 @@ def test_kernels_with_peers_are_found():
 def test_cluster_barrier_before_the_first_access_to_a_peer(name, body):
     first = body.index("mapa_shared(")
     assert 0 <= body.find("cluster_sync()") < first, name
+
+
+def test_replicate_orders_the_takes_of_a_warp():
+    """Two takes of one window may set bits of the same layer's word, and the
+    lanes read those words at the window's start."""
+    body = dict(kernels())["replicate_kernel"]
+    window = body[body.index("for (int base = 0; base < nc; base += 32)"):]
+    read = window.index("cov[lg >> 6] >>")
+    loop = window.index("for (;;)")
+    take = window.index("cov[lg >> 6] |=")
+    assert read < window.index("__syncwarp()", read) < loop < take
+    count = window.index("++count;", take)  # runs in every lane, once a take
+    end = window.index("if (lane == 0)", count)
+    assert window[count:end].split("}")[0].count("__syncwarp()") == 1
