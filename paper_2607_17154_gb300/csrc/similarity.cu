@@ -6,6 +6,8 @@
 //     importance (Eqs. 27-28) and mandatory placement (Eqs. 29-31);
 //   ordermoe_replicate: redundant deployment (Eqs. 32-35);
 //   ordermoe_coverage: local group coverage (Eq. 32).
+#include <cstddef>
+
 #include "common.cuh"
 
 namespace om {
@@ -397,8 +399,8 @@ __device__ __forceinline__ unsigned long long rank_key(double x) {
   return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
 
-// One layer's scratch of the grouping.
-struct GroupSmem {
+// One layer's scratch of the grouping (cnt is read 16 bytes at a time).
+struct alignas(16) GroupSmem {
   unsigned long long kp[64];  // rank_key of p and of I, for the placement order
   unsigned long long ki[64];
   unsigned long long members[64];  // of each group
@@ -411,6 +413,8 @@ struct GroupSmem {
   int nan;  // a similarity is NaN
   int pad[2];
 };
+static_assert(alignof(GroupSmem) % 16 == 0 && offsetof(GroupSmem, cnt) % 16 == 0, "vector loads of cnt");
+static_assert(sizeof(GroupSmem) % 16 == 0, "the similarity keys follow it in a slice");
 // The similarities are kept as integer keys that order like them (-0 as +0),
 // so that the greedy scan is one integer maximum per expert; 0: no value.
 __device__ __forceinline__ uint32_t sim_key(float s) {
