@@ -946,21 +946,32 @@ __device__ __forceinline__ float la_value_lanes(const LaCtx<D>& c, int m, int kt
   return all_min(best);
 }
 
-// Dynamic shared memory for servers up to Mcap, NW warps, level rows of wcap
-// floats (Wa of every level, Cn of all but the last).
-__host__ __device__ inline size_t la_smem_fixed(int E, int D, int Mcap, int NW) {
-  return sizeof(float) * ((size_t)64 * NW + 2 * D * E * (E | 1) + (size_t)(2 * D + 2) * Mcap * E +
-                          la_max_loss(E)) +
-         (size_t)(la_max_loss(E) + 1) * la_class_pitch(E);
+// Dynamic shared memory for M servers and NW warps: what every block needs, the
+// class table, and the levels' rows where none is shorter than it can be (Wa of
+// every level, Cn of all but the last).
+__host__ __device__ constexpr size_t la_smem_fixed(int E, int D, int M, int NW) {
+  return sizeof(float) * ((size_t)64 * NW + 2 * D * E * (E | 1) + (size_t)(2 * D + 2) * M * E);
 }
-__host__ __device__ inline size_t la_smem_bytes(int E, int D, int Mcap, int NW, int wcap) {
-  return la_smem_fixed(E, D, Mcap, NW) + sizeof(float) * (size_t)(2 * D - 1) * wcap;
+__host__ __device__ inline size_t la_smem_classes(int E) {
+  return la_max_loss(E) == 0 ? 0
+                             : sizeof(float) * la_max_loss(E) + (size_t)(la_max_loss(E) + 1) * la_class_pitch(E);
 }
+__host__ __device__ inline size_t la_smem_rows(int E, int D, int M) {
+  return sizeof(float) * (size_t)(2 * D - 1) * E * ((E * M) | 1);
+}
+// The most a block asks for: the launch gives what the servers that the table
+// stride has room for can use, up to this, and the block lays it out for the
+// servers that there are: the class table where it fits beside the fixed part,
+// the rows in what is left where theirs fit.
+constexpr size_t kLaSmem = 200 * 1024;
+constexpr size_t kLaStatic = 27 * 1024;  // of the 227 KB a block can have; checked at the first launch
+static_assert(la_smem_fixed(64, 3, 32, 16) <= kLaSmem && kLaSmem + kLaStatic <= 227 * 1024,
+              "every shape that is taken can be launched");
 
 template <int D, int NW>
 __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
     const int32_t* __restrict__ topk_idx, int T, int E, int k, const uint8_t* __restrict__ tab,
-    Lookahead la, int Mcap, int wcap, int tpb, const uint8_t* __restrict__ home,
+    Lookahead la, int Mcap, int smem, int tpb, const uint8_t* __restrict__ home,
     uint8_t* __restrict__ loc, float* __restrict__ qhat, int32_t* __restrict__ chosen_expert,
     uint8_t* __restrict__ chosen_server, uint8_t* __restrict__ kind_out,
     int32_t* __restrict__ counters) {
@@ -1041,12 +1052,17 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     c.Ua[i] = U[2 * i] = sp;
-    c.Un[i] = U[2 * i + 1] = sp + Mcap * E;
-    sp += 2 * Mcap * E;
+    c.Un[i] = U[2 * i + 1] = sp + M * E;
+    sp += 2 * M * E;
   }
   float* Va = sp;
-  float* Vn = Va + Mcap * E;
-  sp = Vn + Mcap * E;
+  float* Vn = Va + M * E;
+  sp = Vn + M * E;
+  // what is left: the class table, then rows of wcap floats
+  const int left = smem - static_cast<int>(la_smem_fixed(E, D, M, NW));
+  const int class_bytes = static_cast<int>(la_smem_classes(E));
+  const bool class_room = class_bytes > 0 && class_bytes <= left;
+  const int wcap = (left - (class_room ? class_bytes : 0)) / ((2 * D - 1) * static_cast<int>(sizeof(float)));
 #pragma unroll
   for (int i = 0; i < D; ++i) {
     c.Wa[i] = Wa[i] = sp;
@@ -1202,7 +1218,7 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
     first0 = in - n0 - n1;
     first1 = in - n1;
     c.n_loss = __shfl_sync(0xffffffffu, in, 31);
-    c.classes = E > kLaNarrow && c.n_loss > 0 && c.n_loss <= la_max_loss(E);
+    c.classes = class_room && c.n_loss > 0 && c.n_loss <= la_max_loss(E);
   }
   auto first_of = [&](int kt) { return __shfl_sync(0xffffffffu, kt & 1 ? first1 : first0, kt >> 1); };
   if (c.classes) {
@@ -2230,16 +2246,11 @@ static cudaError_t lookahead_launch(int T, int E, int Mcap, int k, const int32_t
                                     uint8_t* loc, float* qhat, int32_t* chosen_expert,
                                     uint8_t* chosen_server, uint8_t* kind, int32_t* counters,
                                     cudaStream_t stream) {
-  // rows for every substitute set there can be, or as many as fit beside the
-  // rest of a block's shared memory (200 KB of the 227; the static arrays
-  // take up to 26 KB more)
-  const size_t fixed = la_smem_fixed(E, D, Mcap, NW);
-  long long wcap = (long long)E * ((E * Mcap) | 1);
-  const long long room = (200 * 1024 - (long long)fixed) / ((2 * D - 1) * (long long)sizeof(float));
-  if (wcap > room) wcap = room > 0 ? room : 0;
-  const size_t smem = la_smem_bytes(E, D, Mcap, NW, static_cast<int>(wcap));
-  cudaFuncSetAttribute(lookahead_select_kernel<D, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)smem);
+  const size_t full = la_smem_fixed(E, D, Mcap, NW) + la_smem_classes(E) + la_smem_rows(E, D, Mcap);
+  const size_t smem = full < kLaSmem ? full : kLaSmem;
+  const cudaError_t ae = cudaFuncSetAttribute(
+      lookahead_select_kernel<D, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (ae != cudaSuccess) return ae;
   // a token a warp until the blocks of one wave (one an SM) are full, then
   // more tokens a block, which share its tables
   const long long wave = (long long)num_sms() * NW;
@@ -2249,7 +2260,7 @@ static cudaError_t lookahead_launch(int T, int E, int Mcap, int k, const int32_t
   const long long blocks = T / tpb + Mcap;
   return launch_pdl(lookahead_select_kernel<D, NW>, dim3(static_cast<unsigned>(blocks)),
                     dim3(32 * NW), smem, stream, topk_idx, T, E, k, tb, la, Mcap,
-                    static_cast<int>(wcap), static_cast<int>(tpb), home, loc, qhat, chosen_expert,
+                    static_cast<int>(smem), static_cast<int>(tpb), home, loc, qhat, chosen_expert,
                     chosen_server, kind, counters);
 }
 

@@ -182,6 +182,57 @@ def test_lookahead_tokens_by_home_bit_exact(T, E, M, k, H, skew):
     np.testing.assert_array_equal(cnt.cpu().numpy(), np.bincount(ref[2].ravel(), minlength=4))
 
 
+@pytest.mark.parametrize("T,E,M,M_stride,k,H,groups", [
+    (30, 64, 32, 32, 2, 4, 64),   # the most of everything: no class table, no rows; no substitutes
+    (30, 64, 32, 32, 2, 4, 16),   # the same with substitutes: open evaluations by the whole block
+    (40, 64, 8, 32, 2, 4, 32),    # a stride with room for more servers than the tables have
+    (40, 64, 3, 32, 3, 3, 16), (40, 33, 8, 32, 2, 2, 8), (50, 8, 4, 32, 2, 4, 4),
+    (40, 64, 16, 16, 2, 4, 32), (20, 64, 20, 25, 2, 3, 16)])
+def test_lookahead_at_the_limits_of_shared_memory(T, E, M, M_stride, k, H, groups):
+    """Every E <= 64, M <= 32 and H <= 4, and any stride that holds the tables:
+    what does not fit in a block's shared memory is done without. Two servers
+    an expert and three successors a transition row, so that the oracle's
+    recursion stays small."""
+    rng = np.random.default_rng(E + M + M_stride + H + groups)
+    qbar = 0.25
+    used = B.ordermoe_tables_bytes(E, M)
+    stride = B.ordermoe_tables_bytes(E, M_stride)
+    buf = torch.zeros(H * stride, dtype=torch.uint8, device=DEV)
+    group = (np.arange(E) % groups).astype(np.int32)
+    otabs = []
+    for l in range(H):
+        sim = (0.4 + 0.6 * rng.random((E, E))).astype(np.float32)
+        np.fill_diagonal(sim, 1.0)
+        x = np.zeros((M, E), np.uint8)
+        x[rng.integers(0, M, E), np.arange(E)] = 1
+        x[rng.integers(0, M, E), np.arange(E)] = 1
+        sp = synth.server_params(M, 4096, 14336, seed=l)
+        sp.tau[:] *= 1e-3
+        build_tables(sim, group, x, 0.2, qbar, sp, DEV, out=buf[l * stride:l * stride + used])
+        otabs.append(oracle.tables(sim, group, x, 0.2, qbar, sp.F, sp.B, sp.tau, sp.z, sp.c, sp.omega_T,
+                                   sp.omega_Q))
+    P = np.zeros((H - 1, E, E), np.float32)
+    for h in range(H - 1):
+        for e in range(E):
+            P[h, e, rng.choice(E, 3, replace=False)] = (0.5, 0.25, 0.25)
+    logits = rng.standard_normal((T, E)).astype(np.float32)
+    home = rng.integers(0, M, T).astype(np.uint8)
+    loc = np.where(rng.random(T) < 0.5, home, rng.integers(0, M, T)).astype(np.uint8)
+    qhat = (rng.random(T) * qbar).astype(np.float32)
+    g = [torch.empty(T, k, dtype=dt, device=DEV)
+         for dt in (torch.int32, torch.float32, torch.int32, torch.uint8, torch.uint8)]
+    gl = torch.as_tensor(loc).to(DEV); gq = torch.as_tensor(qhat).to(DEV)
+    B.ordermoe_route_select_lookahead(None, None, torch.as_tensor(logits).to(DEV), T, E, 0, k, 1, buf,
+                                      stride, H, torch.as_tensor(P).to(DEV),
+                                      torch.as_tensor(home).to(DEV), gl, gq, None, *g)
+    idx, _ = oracle.topk(logits, k)
+    ref = oracle.select_lookahead(idx, otabs, P, home, loc, qhat)
+    for name, got, want in zip(("chosen", "server", "kind"), (g[2], g[3], g[4]), ref[:3]):
+        np.testing.assert_array_equal(got.cpu().numpy(), want, err_msg=name)
+    np.testing.assert_array_equal(gl.cpu().numpy(), ref[3])
+    np.testing.assert_array_equal(gq.cpu().numpy(), ref[4])
+
+
 def test_lookahead_horizon_one_equals_route_select():
     rng = np.random.default_rng(5)
     E, M, k, T = 8, 4, 2, 200
