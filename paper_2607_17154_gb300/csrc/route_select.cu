@@ -2248,9 +2248,13 @@ static cudaError_t lookahead_launch(int T, int E, int Mcap, int k, const int32_t
                                     cudaStream_t stream) {
   const size_t full = la_smem_fixed(E, D, Mcap, NW) + la_smem_classes(E) + la_smem_rows(E, D, Mcap);
   const size_t smem = full < kLaSmem ? full : kLaSmem;
-  const cudaError_t ae = cudaFuncSetAttribute(
-      lookahead_select_kernel<D, NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (ae != cudaSuccess) return ae;
+  static PerDevice attr;
+  const int ae = per_device(attr, [] {
+    return static_cast<int>(cudaFuncSetAttribute(lookahead_select_kernel<D, NW>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 static_cast<int>(kLaSmem)));
+  });
+  if (ae != cudaSuccess) return static_cast<cudaError_t>(ae);
   // a token a warp until the blocks of one wave (one an SM) are full, then
   // more tokens a block, which share its tables
   const long long wave = (long long)num_sms() * NW;
@@ -2296,12 +2300,35 @@ static int launch_select_lanes(const int32_t* topk_idx, int T, int E, int k, con
   long long blocks = (T + per_block - 1) / per_block;
   const long long cap = 4LL * num_sms();
   if (blocks > cap) blocks = cap;
-  cudaFuncSetAttribute(select_lanes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)tab_smem);
   OM_LAUNCH_PDL("select_lanes_kernel", select_lanes_kernel, dim3(static_cast<int>(blocks)),
                 dim3(kLaneThreads), tab_smem, stream, topk_idx, T, E, k, tb, home, loc, qhat,
                 chosen_expert, chosen_server, kind, counters);
   return ORDERMOE_OK;
+}
+
+// Selection from given logits: the tables, the staged delay table and the
+// logits' chunks in shared memory.
+template <int EM>
+constexpr size_t select_smem(int E) {
+  return sizeof(float) * (2 * (size_t)E * E + kDelayStage + EM * 128);
+}
+
+template <int EM>
+static cudaError_t launch_select(const float* logits_in, int T, int E, int k, int renorm,
+                                 const uint8_t* tb, const Lookahead& la, const uint8_t* home,
+                                 uint8_t* loc, float* qhat, float* logits_out, int32_t* topk_idx,
+                                 float* topk_w, int32_t* chosen_expert, uint8_t* chosen_server,
+                                 uint8_t* kind, int32_t* counters, cudaStream_t stream) {
+  static PerDevice attr;
+  const int ae = per_device(attr, [] {
+    return static_cast<int>(cudaFuncSetAttribute(select_kernel<EM>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 static_cast<int>(select_smem<EM>(EM))));
+  });
+  if (ae != cudaSuccess) return static_cast<cudaError_t>(ae);
+  return launch_pdl(select_kernel<EM>, dim3((T + 127) / 128), dim3(128), select_smem<EM>(E), stream,
+                    logits_in, T, E, k, renorm, tb, home, loc, qhat, logits_out, topk_idx, topk_w,
+                    chosen_expert, chosen_server, kind, counters, la);
 }
 
 template <int NE>
@@ -2340,25 +2367,15 @@ static int route_select_impl(const uint16_t* X, const uint16_t* W_r, const float
     return fail(ORDERMOE_ERR_INVALID_ARG, "route_select: tables buffer smaller than E needs");
   if (T == 0) return ORDERMOE_OK;
   const uint8_t* tb = static_cast<const uint8_t*>(tables);
-  const size_t tab_smem = sizeof(float) * 2 * E * E;  // the look-ahead and lane kernels'
-  const size_t sel_smem = tab_smem + sizeof(float) * kDelayStage;  // + the staged delay table
+  const size_t tab_smem = sizeof(float) * 2 * E * E;  // the lane kernel's
+  static_assert(sizeof(float) * 2 * 64 * 64 + sizeof(SelSmem) <= 48 * 1024, "launches without an attribute");
   const int blocks = (T + 127) / 128;
   if (logits_in != nullptr) {
-    cudaError_t sel_err = cudaSuccess;
-#define OM_SEL_LAUNCH(EM)                                                                        \
-  do {                                                                                           \
-    const size_t lg_smem = sel_smem + sizeof(float) * EM * 128; /* + the logits' chunks */      \
-    cudaFuncSetAttribute(select_kernel<EM>, cudaFuncAttributeMaxDynamicSharedMemorySize,         \
-                         (int)lg_smem);                                                          \
-    sel_err = launch_pdl(select_kernel<EM>, dim3(blocks), dim3(128), lg_smem, stream,            \
-                         logits_in, T, E, k, renorm, tb, home, loc, qhat, logits_out, topk_idx,   \
-                         topk_w, chosen_expert, chosen_server, kind, counters, la);              \
-  } while (0)
-    if (E <= 8) OM_SEL_LAUNCH(8);
-    else if (E <= 16) OM_SEL_LAUNCH(16);
-    else if (E <= 32) OM_SEL_LAUNCH(32);
-    else OM_SEL_LAUNCH(64);
-#undef OM_SEL_LAUNCH
+    const auto launch = E <= 8 ? launch_select<8> : E <= 16 ? launch_select<16>
+                        : E <= 32 ? launch_select<32> : launch_select<64>;
+    const cudaError_t sel_err = launch(logits_in, T, E, k, renorm, tb, la, home, loc, qhat, logits_out,
+                                       topk_idx, topk_w, chosen_expert, chosen_server, kind, counters,
+                                       stream);
     if (sel_err != cudaSuccess) return cuda_fail(sel_err, "select_kernel");
     return la.H > 1 ? launch_lookahead_select(topk_idx, T, E, k, tb, la, home, loc, qhat,
                                               chosen_expert, chosen_server, kind, counters, stream)

@@ -233,6 +233,56 @@ def test_lookahead_at_the_limits_of_shared_memory(T, E, M, M_stride, k, H, group
     np.testing.assert_array_equal(gq.cpu().numpy(), ref[4])
 
 
+def test_threads_with_calls_of_different_sizes():
+    """Two host threads whose calls share a kernel and ask for different
+    amounts of shared memory, each on its own stream: both succeed at every
+    call and give what they give alone."""
+    import threading
+
+    def prepare(E, M, H, T, seed):
+        rng = np.random.default_rng(seed)
+        buf, stride, _ = stack_tables(rng, H, E, M, 0.2, True)
+        P = rng.random((H - 1, E, E)).astype(np.float32)
+        P = torch.as_tensor((P / P.sum(axis=2, keepdims=True)).astype(np.float32)).to(DEV)
+        logits = torch.as_tensor(rng.standard_normal((T, E)).astype(np.float32)).to(DEV)
+        home = torch.as_tensor(rng.integers(0, M, T).astype(np.uint8)).to(DEV)
+        out = [torch.empty(T, 2, dtype=dt, device=DEV)
+               for dt in (torch.int32, torch.float32, torch.int32, torch.uint8, torch.uint8)]
+        stream = torch.cuda.Stream()
+
+        def call():
+            B.ordermoe_route_select_lookahead(None, None, logits, T, E, 0, 2, 1, buf, stride, H, P, home,
+                                              None, None, None, *out, None, stream)
+        return call, out
+
+    # one instantiation each: the selection of 33-64 experts (H = 2) or of 9-16 (H = 4)
+    for small, large in (((33, 2, 2), (64, 8, 2)), ((9, 2, 4), (16, 8, 4))):
+        pairs = [prepare(*small, 4, 1), prepare(*large, 4, 2)]
+        torch.cuda.synchronize()
+        want = []
+        for call, out in pairs:
+            call()
+            torch.cuda.synchronize()
+            want.append([o.clone() for o in out])
+        errors = []
+
+        def loop(call):
+            try:
+                for _ in range(400):
+                    call()
+            except Exception as e:  # noqa: BLE001
+                errors.append(e)
+
+        ts = [threading.Thread(target=loop, args=(call,)) for call, _ in pairs]
+        [t.start() for t in ts]
+        [t.join() for t in ts]
+        torch.cuda.synchronize()
+        assert not errors, errors[0]
+        for (_, out), w in zip(pairs, want):
+            for a, b in zip(out, w):
+                assert torch.equal(a, b)
+
+
 def test_lookahead_horizon_one_equals_route_select():
     rng = np.random.default_rng(5)
     E, M, k, T = 8, 4, 2, 200

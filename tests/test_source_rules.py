@@ -1,9 +1,14 @@
-"""Barriers whose lack a run need not show, read from the sources.
+"""Barriers and limits whose lack a run need not show, read from the sources.
 
 Distributed shared memory may be accessed once every CTA of the cluster is
 known to run: a kernel that maps an address of a peer CTA meets a cluster
 barrier first. Votes and shuffles order no memory: lanes of a warp that change
-one shared word in turn need a warp barrier between them."""
+one shared word in turn need a warp barrier between them.
+
+A kernel's limit of dynamic shared memory belongs to the function, not to the
+call: set by every call to its own size, one host thread lowers it between
+another's attribute and launch. It is set once per device, to the largest size.
+"""
 import glob
 import os
 import re
@@ -52,3 +57,21 @@ def test_replicate_orders_the_takes_of_a_warp():
     count = window.index("++count;", take)  # runs in every lane, once a take
     end = window.index("if (lane == 0)", count)
     assert window[count:end].split("}")[0].count("__syncwarp()") == 1
+
+
+def test_limits_of_shared_memory_are_set_once_per_device():
+    n = 0
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        text = re.sub(r"//[^\n]*", "", open(path).read())
+        for m in re.finditer(r"cudaFuncSetAttribute\((?!\w*\))", text):
+            function = text[text.rindex("\n}", 0, m.start()):m.start()]
+            assert "per_device(" in function or re.search(r"\w+_attr\(\) \{", function), (path, function[-300:])
+            n += 1
+    assert n >= 20
+    for helper in ("ffn_attr", "router_attr", "router_lanes_attr", "place_attr"):
+        calls = []
+        for path in glob.glob(os.path.join(CSRC, "*.cu")):
+            text = open(path).read()
+            calls += [text[text.rindex("\n}", 0, m.start()):m.start()]
+                      for m in re.finditer(helper + r"(<[^>]*>)?\(\)(?! \{)", text)]
+        assert calls and all("per_device(" in c for c in calls), helper
