@@ -699,6 +699,20 @@ __host__ __device__ inline size_t place_score_bytes(int M, int experts) {
   return 8 * ((size_t)M * place_depth(M, experts) + 2) * place_cols(M);
 }
 
+// Whether n experts of one size take the tables. The placement of one expert must
+// take longer than the producer's row, and a short range does not win back the
+// wait for the first rows. Tables against the general loop, us of a call with one
+// group and with eight groups a layer:
+//   servers, experts   1, 1536          2, 1536      2, 64      3, 64      4, 1536
+//                      1053 1041 / 705 694  799 667 / 842 832  92 61 / 65 53  83 63 / 67 55  507 363 / 717 705
+//                      4, 64      4, 32    4, 8      8, 64      12, 64
+//                      59 41 / 65 55  26 26 / 32 32  21 19 / 19 18  63 41 / 67 55  63-96 45-47 / 69 57
+//                      16, 128    16, 64    32, 1536     32, 128    32, 64
+//                      69 66 / 86 82  92 71 / 69 57  553 524 / 799 789  78 74 / 90 87  98 86 / 77 65
+__host__ __device__ inline bool place_tabulated(int M, int n) {
+  return M >= 2 && (n >= 96 || (n >= 32 && M >= 4 && M <= 8));
+}
+
 constexpr unsigned long long kNoServer = ~0ull;           // the expert does not fit
 constexpr unsigned long long kOddScore = 0x7FF0ull << 48;  // not a plain non-negative number
 
@@ -1059,11 +1073,11 @@ __global__ void __launch_bounds__(kPlaceThreads) place_kernel(
   unsigned long long* score = reinterpret_cast<unsigned long long*>(s_pl + sizeof(PlaceSmem));
   __shared__ int s_over;
   const int n = (l1 - l0) * E;
-  const bool uniform = place_uniform(p + (size_t)l0 * E, n, threadIdx.x, blockDim.x);
-  const int depth = uniform ? place_depth(M, n) : 0, cols = place_cols(M);
+  const bool tables = place_tabulated(M, n) && place_uniform(p + (size_t)l0 * E, n, threadIdx.x, blockDim.x);
+  const int depth = tables ? place_depth(M, n) : 0, cols = place_cols(M);
   place_tables_init(sm, score, M, depth, cols, pp.lambda2, threadIdx.x, blockDim.x);
   __syncthreads();
-  if (uniform && (threadIdx.x >> 5) == 1)
+  if (tables && (threadIdx.x >> 5) == 1)
     place_produce(sm, score, threadIdx.x & 31, M, depth, cols, p[(size_t)l0 * E], first, pp.lambda1, C, used);
   place_range(sm, score, cols, &s_over, group, porder, L, E, M, l0, l1, first, pp, p, C, placement, used, status,
               depth);
@@ -1101,8 +1115,8 @@ __global__ void __launch_bounds__(kGroupThreads + 32) group_place_kernel(
   unsigned long long* score = reinterpret_cast<unsigned long long*>(&ps + 1);
   __shared__ int s_over;
   const int n = (l1 - l0) * E;
-  const bool uniform = place_uniform(p + (size_t)l0 * E, n, threadIdx.x, blockDim.x);
-  const int depth = uniform ? place_depth(M, n) : 0, cols = place_cols(M);
+  const bool tables = place_tabulated(M, n) && place_uniform(p + (size_t)l0 * E, n, threadIdx.x, blockDim.x);
+  const int depth = tables ? place_depth(M, n) : 0, cols = place_cols(M);
   const int slice = threadIdx.x / nt;
   unsigned char* own = s_gp + (slice < slices ? slice : 0) * group_slice_bytes(E);
   GroupSmem& gs = *reinterpret_cast<GroupSmem*>(own);
@@ -1110,7 +1124,7 @@ __global__ void __launch_bounds__(kGroupThreads + 32) group_place_kernel(
   place_tables_init(ps, score, M, depth, cols, pp.lambda2, threadIdx.x, blockDim.x);
   __syncthreads();
   if (slice >= slices) {  // the last warp
-    if (uniform)
+    if (tables)
       place_produce(ps, score, threadIdx.x & 31, M, depth, cols, p[(size_t)l0 * E], first, pp.lambda1, C, used);
   } else {
     for (int lb = l0; lb < l1; lb += slices) {

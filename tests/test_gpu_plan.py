@@ -332,7 +332,11 @@ def test_placement_quotient_is_correctly_rounded():
     (6, 24, 5, 0.3, "tight"),     # fractional sizes, waiting lists, an overflow
     (3, 33, 7, 1.7, "loose"), (2, 1, 1, 1.0, "tight"), (40, 8, 4, 1.0, "loose"),
     (4, 16, 3, 0.0, "loose"),     # size 0: nothing fills up
-    (4, 64, 1, 1.0, "mates"),     # more experts of a group on a server than it has columns
+    (4, 64, 1, 1.0, "mates"),     # one server, which takes no tables
+    (4, 64, 2, 1.0, "mates"),     # more experts of a group on a server than it has columns
+    (8, 16, 3, 0.0, "loose"),     # size 0 in the tables
+    (4, 8, 4, 1.0, "tight"), (4, 8, 8, 1.0, "loose"), (12, 8, 2, 1.0, "tight"),  # the fewest that take them
+    (1, 31, 4, 1.0, "tight"), (4, 8, 9, 1.0, "tight"), (1, 63, 3, 1.0, "tight"),  # and those just off
     (20, 64, 3, 0.7, "mates")])   # ranges of 512 experts, the last one shorter
 def test_place_uniform_sizes_bit_exact(L, E, M, size, caps):
     """Experts of one size, whose servers' states are tabulated by the number of
