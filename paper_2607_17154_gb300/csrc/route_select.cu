@@ -970,7 +970,7 @@ static_assert(la_smem_fixed(64, 3, 32, 16) <= kLaSmem && kLaSmem + kLaStatic <= 
 
 template <int D, int NW>
 __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
-    const int32_t* __restrict__ topk_idx, int T, int E, int k, const uint8_t* __restrict__ tab,
+    const int32_t* __restrict__ topk_idx, int t0, int T, int E, int k, const uint8_t* __restrict__ tab,
     Lookahead la, int Mcap, int smem, int tpb, const uint8_t* __restrict__ home,
     uint8_t* __restrict__ loc, float* __restrict__ qhat, int32_t* __restrict__ chosen_expert,
     uint8_t* __restrict__ chosen_server, uint8_t* __restrict__ kind_out,
@@ -1101,7 +1101,7 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
   scan_homes([&](int t, int a) {
     const unsigned peers = __match_any_sync(0xffffffffu, a);
     if (a >= 0 && a < M && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[a], __popc(peers));
-    if (a >= M && blockIdx.x == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, t);
+    if (a >= M && blockIdx.x == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, t0 + t);
   });
   __syncthreads();
   if (warp == 0) {
@@ -1390,7 +1390,7 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
     float q = live && qhat != nullptr ? qhat[t] : 0.0f;
     const int idx = live && lane < k ? topk_idx[(size_t)t * k + lane] : 0;
     if (live && s >= M) {
-      if (lane == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, t);
+      if (lane == 0) report(&g_err_route, ORDERMOE_DEV_BAD_INDEX, t0 + t);
       live = false;
     }
     if (__any_sync(0xffffffffu, idx < 0 || idx >= E)) live = false;  // -1: a NaN token (reported)
@@ -1538,7 +1538,7 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
       best = s_best[warp];
       int kstar, mstar, kd;
       if (best == ~0ull) {
-        if (lane == 0) report(&g_err_route, ORDERMOE_DEV_NO_CANDIDATE, t);
+        if (lane == 0) report(&g_err_route, ORDERMOE_DEV_NO_CANDIDATE, t0 + t);
         kstar = r; mstar = s; kd = 0;
       } else {
         const uint32_t mlo = static_cast<uint32_t>(best);
@@ -2241,7 +2241,7 @@ extern "C" int ordermoe_build_tables(const float* sim, const int32_t* group,
 }
 
 template <int D, int NW>
-static cudaError_t lookahead_launch(int T, int E, int Mcap, int k, const int32_t* topk_idx,
+static cudaError_t lookahead_launch(int t0, int T, int E, int Mcap, int k, const int32_t* topk_idx,
                                     const uint8_t* tb, const Lookahead& la, const uint8_t* home,
                                     uint8_t* loc, float* qhat, int32_t* chosen_expert,
                                     uint8_t* chosen_server, uint8_t* kind, int32_t* counters,
@@ -2263,7 +2263,7 @@ static cudaError_t lookahead_launch(int T, int E, int Mcap, int k, const int32_t
   // a home's last block may be partly filled: at most one more block a home
   const long long blocks = T / tpb + Mcap;
   return launch_pdl(lookahead_select_kernel<D, NW>, dim3(static_cast<unsigned>(blocks)),
-                    dim3(32 * NW), smem, stream, topk_idx, T, E, k, tb, la, Mcap,
+                    dim3(32 * NW), smem, stream, topk_idx, t0, T, E, k, tb, la, Mcap,
                     static_cast<int>(smem), static_cast<int>(tpb), home, loc, qhat, chosen_expert,
                     chosen_server, kind, counters);
 }
@@ -2278,17 +2278,23 @@ static int launch_lookahead_select(const int32_t* topk_idx, int T, int E, int k,
   // number; one that does not fit is reported)
   int Mcap = 1;
   while (Mcap < ORDERMOE_MAX_SERVERS && om::tables_bytes(E, Mcap + 1) <= la.stride) ++Mcap;
-  cudaError_t e;
-#define OM_LA_LAUNCH(D)                                                                         \
-  (E > kLaNarrow ? lookahead_launch<D, 16>(T, E, Mcap, k, topk_idx, tb, la, home, loc, qhat,           \
-                                    chosen_expert, chosen_server, kind, counters, stream)       \
-          : lookahead_launch<D, 8>(T, E, Mcap, k, topk_idx, tb, la, home, loc, qhat,            \
-                                   chosen_expert, chosen_server, kind, counters, stream))
-  if (la.H == 2) e = OM_LA_LAUNCH(1);
-  else if (la.H == 3) e = OM_LA_LAUNCH(2);
-  else e = OM_LA_LAUNCH(3);
-#undef OM_LA_LAUNCH
-  return e == cudaSuccess ? ORDERMOE_OK : cuda_fail(e, "lookahead_select_kernel");
+  // Every block ranks the homes of all tokens of its launch, so the tokens go in
+  // launches of at most kLaTokens: 1000000 tokens of 8 experts, 4 servers, H = 2
+  // took 8.5 ms in one, 2.3 so (300000 of 64, 8 servers: 1.92 and 1.68).
+  constexpr int kLaTokens = 131072;
+  for (int t0 = 0; t0 < T; t0 += kLaTokens) {
+    const int n = T - t0 < kLaTokens ? T - t0 : kLaTokens;
+    const size_t at = (size_t)t0 * k;
+    const bool wide = E > kLaNarrow;
+    const auto launch = la.H == 2 ? (wide ? lookahead_launch<1, 16> : lookahead_launch<1, 8>)
+                        : la.H == 3 ? (wide ? lookahead_launch<2, 16> : lookahead_launch<2, 8>)
+                                    : (wide ? lookahead_launch<3, 16> : lookahead_launch<3, 8>);
+    const cudaError_t e = launch(t0, n, E, Mcap, k, topk_idx + at, tb, la, home + t0,
+                                 loc != nullptr ? loc + t0 : nullptr, qhat != nullptr ? qhat + t0 : nullptr,
+                                 chosen_expert + at, chosen_server + at, kind + at, counters, stream);
+    if (e != cudaSuccess) return cuda_fail(e, "lookahead_select_kernel");
+  }
+  return ORDERMOE_OK;
 }
 
 static int launch_select_lanes(const int32_t* topk_idx, int T, int E, int k, const uint8_t* tb,

@@ -233,6 +233,40 @@ def test_lookahead_at_the_limits_of_shared_memory(T, E, M, M_stride, k, H, group
     np.testing.assert_array_equal(gq.cpu().numpy(), ref[4])
 
 
+def test_lookahead_of_many_tokens_in_several_launches():
+    """More tokens than one launch takes (131072): the last launch has 77, and
+    reports the index of the token in the call."""
+    rng = np.random.default_rng(11)
+    T, E, M, k, H, qbar = 131072 + 77, 8, 4, 2, 2, 0.2
+    buf, stride, otabs = stack_tables(rng, H, E, M, qbar, True)
+    P = rng.random((H - 1, E, E)).astype(np.float32)
+    P = (P / P.sum(axis=2, keepdims=True)).astype(np.float32)
+    logits = rng.standard_normal((T, E)).astype(np.float32)
+    home = rng.integers(0, M, T).astype(np.uint8)
+    loc = rng.integers(0, M, T).astype(np.uint8)
+    qhat = (rng.random(T) * qbar).astype(np.float32)
+    g = [torch.empty(T, k, dtype=dt, device=DEV)
+         for dt in (torch.int32, torch.float32, torch.int32, torch.uint8, torch.uint8)]
+    idx, _ = oracle.topk(logits, k)
+    ref = oracle.select_lookahead(idx, otabs, P, home, loc, qhat)
+    for bad in (False, True):
+        loc_in = loc.copy()
+        if bad:
+            loc_in[T - 3] = M
+        gl = torch.as_tensor(loc_in).to(DEV); gq = torch.as_tensor(qhat).to(DEV)
+        cnt = torch.zeros(4, dtype=torch.int32, device=DEV)
+        B.ordermoe_route_select_lookahead(None, None, torch.as_tensor(logits).to(DEV), T, E, 0, k, 1, buf,
+                                          stride, H, torch.as_tensor(P).to(DEV),
+                                          torch.as_tensor(home).to(DEV), gl, gq, None, *g, cnt)
+        assert B.ordermoe_device_error() == ((B.DEV_BAD_INDEX, T - 3) if bad else (0, 0))
+        ok = np.arange(T) != (T - 3 if bad else -1)
+        for name, got, want in zip(("chosen", "server", "kind"), (g[2], g[3], g[4]), ref[:3]):
+            np.testing.assert_array_equal(got.cpu().numpy()[ok], want[ok], err_msg=name)
+        np.testing.assert_array_equal(gl.cpu().numpy()[ok], ref[3][ok])
+        np.testing.assert_array_equal(gq.cpu().numpy()[ok], ref[4][ok])
+        np.testing.assert_array_equal(cnt.cpu().numpy(), np.bincount(ref[2][ok].ravel(), minlength=4))
+
+
 def test_threads_with_calls_of_different_sizes():
     """Two host threads whose calls share a kernel and ask for different
     amounts of shared memory, each on its own stream: both succeed at every
