@@ -1296,6 +1296,9 @@ extern "C" int ordermoe_expert_counts(const float* logits, int64_t N, int E, int
 namespace om {
 
 constexpr int kRepThreads = 512;
+// Counting against sorting: 32 candidates 6.6 and 8.3 us, 128 12.2 and 11.2, 448
+// 39 and 19 (a graph of calls, with the copies that reset their state).
+constexpr int kRepCount = 64;
 constexpr int kRepMaxCand = 16384;
 constexpr int kRepMaxLayers = 1024;
 
@@ -1310,17 +1313,20 @@ constexpr int kRepMaxLayers = 1024;
 // so a candidate that fails against the initial state fails always. Of two
 // candidates of one group, the later is never taken when its p is at least the
 // earlier's: when the earlier was taken the group is covered, and when it did
-// not fit the later does not either. Up to kRepThreads candidates are ordered
-// by counting those before each, more by a bitonic sort in shared memory. One
-// warp then tests 32 at a time against the current state and takes the first
-// that passes: every candidate it passes over failed under the same state it
-// would have met one at a time.
+// not fit the later does not either. Up to kRepCount candidates are ordered by
+// counting those before each, more by a bitonic sort in shared memory. One warp
+// then tests 32 at a time against the current state and takes the first that
+// passes: every candidate it passes over failed under the same state it would
+// have met one at a time.
 //
 // Bound: latency of one block a server (barriers of the sort, fp64 chain of the
-// takes). All candidates in one bitonic sort, and a window read again after
-// each take, took 54.6 us for 24 layers x 64 experts on 8 full servers and 24.0
-// us for 32 x 8 on 4 servers with room for as many again; this takes 8.2
-// and 17.9 (ncu).
+// takes). In a graph of calls with the two copies that reset its state: layers x
+// experts, groups a layer, servers, all candidates in one sort with a window read
+// again after each take against this: 24 x 64, 8 groups, 8 servers with room for as
+// many again 54.1 and 7.9 us; 32 x 8, 4, 4 24.8 and 17.1; 24 x 64, 16, 8 91.3 and
+// 40.5; every expert its own group, 8 x 64 on 32 servers 22.1 and 20.2. (Candidates
+// compared with the whole layer instead of their group's, and up to 512 of them
+// ordered by counting those before each: 65.5 and 48.8 us for the last two.)
 __global__ void __launch_bounds__(kRepThreads) replicate_kernel(
     const int32_t* __restrict__ group, const double* __restrict__ importance,
     const double* __restrict__ p, const double* __restrict__ C, const double* __restrict__ pi,
@@ -1331,6 +1337,7 @@ __global__ void __launch_bounds__(kRepThreads) replicate_kernel(
   unsigned long long* cov = key + Np;  // [L]: bit g = group g covered (Eq. 32)
   uint32_t* cid = reinterpret_cast<uint32_t*>(cov + L);
   __shared__ int n_cand;
+  __shared__ unsigned long long mates[kRepThreads / 32][64];  // a layer's candidates by group
   const int m = blockIdx.x;
   const int t = threadIdx.x;
   const int lane = t & 31;
@@ -1364,29 +1371,46 @@ __global__ void __launch_bounds__(kRepThreads) replicate_kernel(
     cid[i] = static_cast<uint32_t>(g);
   }
   __syncthreads();
-  // kept: not after another of its group that asks for no more memory
-  uint32_t keep = 0;  // bit r: candidate r kRepThreads + t
-  static_assert(kRepMaxCand <= 32 * kRepThreads, "a bit a candidate of the thread");
-  for (int i = t, r = 0; i < N; i += kRepThreads, ++r) {
-    const unsigned long long k = key[i];
-    if (k == 0) continue;
-    const uint32_t g = cid[i];
-    const double pj = p[i];
-    const int l0 = i / E * E;
-    bool stays = true;
-    for (int o = l0; o < l0 + E && stays; ++o) {
-      const unsigned long long ko = key[o];
-      if ((ko > k || (ko == k && o < i)) && cid[o] == g) stays = !(p[o] <= pj);
+  // kept: not after another of its group that asks for no more memory. A warp a
+  // layer, an expert against the candidates of its own group
+  for (int l = t >> 5; l < L; l += kRepThreads / 32) {
+    unsigned long long* const mate = mates[t >> 5];
+    const unsigned long long own[2] = {lane < E ? key[l * E + lane] : 0ull,
+                                       lane + 32 < E ? key[l * E + lane + 32] : 0ull};
+    if (!__any_sync(full, (own[0] | own[1]) != 0)) continue;
+    mate[lane] = mate[lane + 32] = 0ull;
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (own[h] != 0) atomicOr(&mate[cid[l * E + lane + 32 * h]], 1ull << (lane + 32 * h));
+    __syncwarp();
+    uint32_t drop = 0;  // of this lane's two experts
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = lane + 32 * h, i = l * E + e;
+      const unsigned long long k = own[h];
+      if (k == 0) continue;
+      const double pj = p[i];
+      for (unsigned long long b = mate[cid[i]] & ~(1ull << e); b; b &= b - 1) {
+        const int o = l * E + __ffsll(static_cast<long long>(b)) - 1;
+        if ((key[o] > k || (key[o] == k && o < i)) && p[o] <= pj) {
+          drop |= 1u << h;
+          break;
+        }
+      }
     }
-    if (stays) keep |= 1u << r;
+    __syncwarp();  // the layer's keys are read
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if ((drop >> h) & 1u) key[l * E + lane + 32 * h] = 0ull;
   }
   __syncthreads();
   // their keys and ids moved to the front, kRepThreads candidates at a time (a
   // round writes only where it and the rounds before it have been read)
   for (int r = 0; r * kRepThreads < N; ++r) {
-    const bool mine = (keep >> r) & 1u;
     const int i = r * kRepThreads + t;
-    const unsigned long long k = mine ? key[i] : 0ull;
+    const unsigned long long k = i < N ? key[i] : 0ull;
+    const bool mine = k != 0;
     const unsigned bal = __ballot_sync(full, mine);
     int at = 0;
     if (lane == 0 && bal != 0u) at = atomicAdd(&n_cand, __popc(bal));
@@ -1399,7 +1423,7 @@ __global__ void __launch_bounds__(kRepThreads) replicate_kernel(
     __syncthreads();
   }
   const int nc = n_cand;
-  if (nc > kRepThreads) {
+  if (nc > kRepCount) {
     int ns = 1;
     while (ns < nc) ns <<= 1;  // <= Np
     for (int i = nc + t; i < ns; i += kRepThreads) {
@@ -1428,7 +1452,7 @@ __global__ void __launch_bounds__(kRepThreads) replicate_kernel(
     }
   }
   // each sorted slot holds (l, g, j) and the bits of p_{l,j}
-  if (nc <= kRepThreads) {
+  if (nc <= kRepCount) {
     int rank = 0, i = 0;
     if (t < nc) {
       const unsigned long long k = key[t];

@@ -436,7 +436,7 @@ def test_replicate_bit_exact(L, E, M, ratio, seed):
 
 
 @pytest.mark.parametrize("L,E,G,C", [(1, 64, 16, 1e9), (2, 64, 32, 1e9), (1, 64, 64, 1e9), (3, 40, 9, 120.0),
-                                     (20, 64, 16, 1e9)])  # the last: past the counted candidates
+                                     (20, 64, 16, 1e9)])  # the last: 1280 candidates
 def test_replicate_takes_groups_of_one_layer_in_a_window(L, E, G, C):
     """Within a group the benefit and the memory fall together, so every
     candidate stays until its group is covered: many takes of one layer lie in
