@@ -39,7 +39,9 @@ def test_transitions_given_logits_bit_exact(N, L, E, kf):
 
 @pytest.mark.parametrize("N,L,E,kf", [
     (78500, 2, 12, 3),   # two tiles of tokens a block, the last one ragged
-    (257, 9, 17, 1), (700, 3, 64, 8), (300, 3, 33, 9), (1, 2, 1, 1), (513, 4, 40, 5)])
+    (257, 9, 17, 1), (700, 3, 64, 8), (300, 3, 33, 9), (1, 2, 1, 1), (513, 4, 40, 5),
+    (300, 2, 64, 64), (260, 3, 7, 7), (300, 2, 12, 12),  # every expert
+    (300, 2, 63, 4), (520, 2, 33, 2), (300, 3, 5, 2)])   # rows that 16-byte loads do not fit
 def test_topk_sets_with_ties_infinities_and_nan(N, L, E, kf):
     """The counts and transitions against the rule itself (kf passes, each
     taking the first unused maximum): equal logits across the boundary, -inf
