@@ -53,16 +53,13 @@ struct Smem {
   uint32_t tmem_base;
   int abort;
   int zero;
-  int max_rows;  // the largest row tile
-  int mt_start[ORDERMOE_MAX_EXPERTS + 1];
-  int offs[ORDERMOE_MAX_EXPERTS + 1];
 };
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + static_cast<int>(sizeof(Smem));
 
 enum { GATEUP = 0, DOWN = 1 };
 
 struct Args {
-  const int32_t* offsets;  // [E+1] row ranges (0 <= ... <= rows); null: one group of `rows` rows
+  const int32_t* offsets;  // FFN: [E+1] row ranges (0 <= ... <= rows)
   int rows;
   int n_valid;       // LOGITS: number of valid output columns
   float* out_f32;    // LOGITS: H [rows][n_valid] fp32
@@ -73,7 +70,6 @@ struct Args {
   uint16_t* out;     // H [R][d_ff] or Y [R][d]
   int ldo;           // row length of out
   uint64_t limit_ns; // bounded-wait limit
-  int m_major;       // 1: all N slices of an M tile back to back (A read once from HBM)
   int fast_div;      // gate/up: SwiGLU's quotient by the fast reciprocal
 };
 
@@ -89,10 +85,7 @@ struct Tile {
 template <class S>
 __device__ __forceinline__ void load_row_tiles(S& s, const Args& args, int bm, int lane) {
   const int E = args.E;
-  auto off = [&](int e) {
-    e = min(e, E);
-    return args.offsets ? args.offsets[e] : (e == 0 ? 0 : args.rows);
-  };
+  auto off = [&](int e) { return args.offsets[min(e, E)]; };
   const int o0 = off(lane), o1 = off(lane + 32), o2 = off(64);
   const int top = __shfl_sync(0xffffffffu, o1, 0);
   int n0 = __shfl_down_sync(0xffffffffu, o0, 1), n1 = __shfl_down_sync(0xffffffffu, o1, 1);
@@ -130,30 +123,11 @@ __device__ __forceinline__ void load_row_tiles(S& s, const Args& args, int bm, i
   if (bad && lane == 0 && blockIdx.x == 0) report(&g_err_gemm, ORDERMOE_DEV_BAD_INDEX, -2);
 }
 
-__device__ __forceinline__ Tile decode(int tile, const Smem& s, int E, int n_tiles, int m_major) {
-  // the last expert whose first tile is <= tile (binary search: the row-tile
-  // starts never decrease; empty experts share their successor's start)
-  int e = 0, hi = E - 1;
-  while (e < hi) {
-    const int mid = (e + hi + 1) >> 1;
-    if (s.mt_start[mid] * n_tiles <= tile) e = mid;
-    else hi = mid - 1;
-  }
-  const int local = tile - s.mt_start[e] * n_tiles;
-  const int n_mt = s.mt_start[e + 1] - s.mt_start[e];
-  Tile t;
-  t.e = e;
-  int mt;
-  if (m_major) {
-    mt = local / n_tiles;
-    t.n = local - mt * n_tiles;
-  } else {
-    t.n = local / n_mt;
-    mt = local - t.n * n_mt;
-  }
-  t.m0 = s.offs[e] + mt * BM;
-  t.m_end = s.offs[e + 1];
-  return t;
+// A tile of the logits: all column slices of a row tile back to back, so that the
+// rows are read once from HBM (the stacked router rows stay in L2).
+__device__ __forceinline__ Tile decode(int tile, const Args& args) {
+  const int mt = tile / args.n_tiles;
+  return Tile{0, mt * BM, args.rows, tile - mt * args.n_tiles};
 }
 
 __global__ void __launch_bounds__(THREADS, 1)
@@ -192,16 +166,12 @@ __global__ void __launch_bounds__(THREADS, 1)
     tmem_alloc(&s.tmem_base, TMEM_COLS);
     tmem_relinquish();
   }
-  if (warp == 2) {
-    pdl_wait();  // the offsets come from the permutation
-    load_row_tiles(s, args, BM, lane);
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   pdl_wait();  // every thread: the previous kernel's outputs are visible
   const uint32_t tmem_base = s.tmem_base;
-  const int total = s.mt_start[args.E] * args.n_tiles;
+  const int total = (args.rows + BM - 1) / BM * args.n_tiles;
   const int kblocks = args.K / BK;
   volatile int* abort = &s.abort;
 
@@ -219,7 +189,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint32_t phase = 0;
     bool ok = true;
     for (int tile = blockIdx.x; tile < total && ok; tile += gridDim.x) {
-      const Tile t = decode(tile, s, args.E, args.n_tiles, args.m_major);
+      const Tile t = decode(tile, args);
       for (int kb = 0; kb < kblocks; ++kb) {
         if (!__all_sync(0xffffffffu, mbar_wait(&s.empty[stage], phase ^ 1u, args.limit_ns, abort))) {
           if (issuer && !*abort) report(&g_err_gemm, ORDERMOE_DEV_WAIT_TIMEOUT, 1);
@@ -298,7 +268,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         break;
       }
       tc_fence_after();
-      const Tile t = decode(tile, s, args.E, args.n_tiles, args.m_major);
+      const Tile t = decode(tile, args);
       const int row = t.m0 + lrow;
       const bool valid = row < t.m_end;
       const uint32_t tb = tmem_base + slot * BN + (static_cast<uint32_t>(q * 32) << 16);
@@ -389,10 +359,11 @@ __global__ void __launch_bounds__(THREADS, 1)
 // shared-memory exchange, and the decision to stop is a barrier reduction over
 // all epilogue warps (barrier 3), so they always leave together.
 constexpr int P_BM = 256;            // permuted rows (N side) per tile
-constexpr int P_MAX_STAGES = 20;
 constexpr int P_W_BYTES = 128 * BK * 2;   // 128 weight rows per CTA and K block
 constexpr int P_T_BYTES = 128 * BK * 2;   // one box of 128 permuted rows per CTA
 constexpr int P_STAGE_BYTES = P_W_BYTES + P_T_BYTES;
+// the most stages a ring has: a single CTA's with boxes of 16 rows, in the space of six of 128
+constexpr int P_MAX_STAGES = 6 * P_STAGE_BYTES / (P_W_BYTES + 16 * BK * 2);
 constexpr int P_X_PITCH = 17;             // floats per exchange row (odd: no bank conflicts)
 constexpr int P_XBUF_FLOATS = 128 * P_X_PITCH;
 constexpr int P_EPI_GROUP_BYTES = 2 * (P_XBUF_FLOATS * 4 + 32 * 64 * 2);  // gate/up, double-buffered
@@ -932,7 +903,11 @@ static int make_row_maps(gg::RowMaps* rm, const void* base, uint64_t rows, uint6
 // 128 + 67 against 133 + 69, 112 rows (139) 125 + 73 against 135 + 70, 131
 // rows (156) 157 + 85 against 136 + 72; 8 experts, d 4096, d_ff 14336: 107
 // rows (119) 287 + 155 against 302 + 161, 127 rows (142) 370 + 210 against
-// 305 + 162: the line is where the fuller experts pass 128 rows.
+// 305 + 162: the line is where the fuller experts pass 128 rows. (It sees the
+// average: with every row on one expert, single tiles of 128 x 128 move more of
+// the rows than the 256-column tiles they took the place of: gate/up + down of 64
+// experts, 96 rows on average, 100 against 91 us, of 16 experts, d 1024, d_ff 4096,
+// 111 rows, 66 against 57. By zipf 1.1 101 against 96 there, faster elsewhere.)
 constexpr int kPairRows = 112;
 static bool use_pairs(int R, int E) { return (long long)R >= (long long)kPairRows * E; }
 
@@ -1008,12 +983,10 @@ int logits_gemm_launch(const uint16_t* X, int N, const uint16_t* W, int C, int d
   a.rows = N;
   a.n_valid = C;
   a.out_f32 = H;
-  a.E = 1;
   a.K = d;
   a.n_tiles = n_tiles;
   a.b_rows = width;
   a.limit_ns = wait_limit_ns();
-  a.m_major = 1;  // the stacked router rows (a few MB) stay in L2; X_cal streams once
   const long long tiles = (long long)((N + BM - 1) / BM) * a.n_tiles;
   const int sms = num_sms();
   const int grid = static_cast<int>(tiles < sms ? tiles : sms);

@@ -1164,7 +1164,7 @@ int sim_tc_launch(const uint16_t* X, int N, const uint16_t* W, int L, int E, int
 }  // namespace om
 
 // Workspace: H [N][L E] fp32 | the hi/lo bf16 planes of H^T [L E][ldT] (tensor-core
-// path) | partial Grams [L][parts][64][64] fp32 | G [L][64][64] fp64.
+// path) | partial Grams [L][parts][64][64] fp32.
 static int64_t sim_ldT(int64_t N) { return (N + 7) / 8 * 8; }
 
 // Partial Grams per layer the workspace holds: one per 1024-token chunk on
@@ -1177,16 +1177,15 @@ static int64_t sim_parts(int L, int E, int64_t N) {
 }
 
 // Workspace of the similarity: H [N][L E] fp32 (with_H; the CUDA-core path
-// and the logits-keeping call need it), the hi/lo planes (tensor-core path),
-// the partial Grams and G.
+// and the logits-keeping call need it), the hi/lo planes (tensor-core path) and
+// the partial Grams.
 static size_t sim_ws_bytes(int L, int E, int64_t N, bool with_H) {
   if (L <= 0 || E <= 0 || E > ORDERMOE_MAX_EXPERTS || N <= 0) return 0;
   auto up = [](size_t v) { return (v + 255) & ~size_t(255); };
   const size_t h = with_H ? up((size_t)N * L * E * sizeof(float)) : 0;
   const size_t planes = sim_tc_supported(L, E) ? 2 * up((size_t)L * E * sim_ldT(N) * 2) : 0;
   const size_t g = (size_t)L * sim_parts(L, E, N) * 64 * 64 * sizeof(float);
-  const size_t gd = (size_t)L * 64 * 64 * sizeof(double);
-  return h + planes + up(g) + up(gd);
+  return h + planes + up(g);
 }
 
 extern "C" size_t ordermoe_similarity_workspace_bytes(int L, int E, int64_t N) {
