@@ -634,10 +634,18 @@ __global__ void __launch_bounds__(kLaneThreads) select_lanes_kernel(
 // One block a token, with the tables rebuilt for each and V folded into every
 // term, took 15.7 ms for 2048 tokens of 64 experts, 8 servers, top-6, H = 3,
 // and 14.6 us for 128 tokens of 8 experts, 4 servers, top-2 (ncu); this takes
-// 98 us and 10.7 us (351 us with every token's evaluations left to its warp).
+// 84 us and 11.5 us (351 us with every token's evaluations left to its warp).
 constexpr int kLaMaxTok = 512;   // tokens of a block
 constexpr int kLaTasks = 512;    // evaluations listed in a step
-constexpr int kLaMaxLoss = 512;  // losses of the last level that the class table takes
+// Losses of the last level that the class table takes: 37 KB at 64 experts, beside
+// which the rows of groups of 8 on 8 servers fit at H = 3 (beside a table for 1024,
+// 74 KB, they do not). Where the rows or the classes have no room the open
+// evaluations go by direct minima. Calls with logits given, 2048 tokens of 64
+// experts: H = 3, 8 servers, groups of 4 103 us and of 8 157 (in the tables), of 16
+// 72 ms; groups of 8 on 16 servers 14.9 ms, on 32 12.2; H = 2, groups of 16, 52 us
+// on 8 servers, 85 on 32. (One block a token: 10.2, 27.4, 108, 28.4, 30.6, 3.7 and
+// 2.3 ms.)
+constexpr int kLaMaxLoss = 512;
 // Up to 16 experts a block has 8 warps and no class table: its set-up (2 us)
 // is longer than the few evaluations it would shorten (14.5 against 12.4 us
 // for 128 tokens of 8 experts). For 64 experts the table took the 2048-token
