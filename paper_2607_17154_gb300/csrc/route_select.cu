@@ -1069,7 +1069,7 @@ __global__ void __launch_bounds__(32 * NW, 1) lookahead_select_kernel(
   // what is left: the class table, then rows of wcap floats
   const int left = smem - static_cast<int>(la_smem_fixed(E, D, M, NW));
   const int class_bytes = static_cast<int>(la_smem_classes(E));
-  const bool class_room = class_bytes > 0 && class_bytes <= left;
+  const bool class_room = kEmax > kLaNarrow && class_bytes > 0 && class_bytes <= left;
   const int wcap = (left - (class_room ? class_bytes : 0)) / ((2 * D - 1) * static_cast<int>(sizeof(float)));
 #pragma unroll
   for (int i = 0; i < D; ++i) {
